@@ -20,7 +20,6 @@ using namespace pic;
 const float *mlp_params(const pic_mlp *m);
 const float *mlp_norm(const pic_mlp *m);
 
-int pic_set_smem_attrs(size_t s1, size_t s2, size_t s3);
 static thread_local std::string g_init_error;
 
 void pic::set_thread_error(const char *msg) { g_init_error = msg ? msg : ""; }
@@ -123,11 +122,12 @@ static void release(pic_handle *h)
     for (int b = 0; b < 2; ++b) {
         f(h->Pblk[b]);
         f(h->jb[b]); f(h->sy[b]); f(h->sz[b]);
+        f(h->m1[b]); f(h->my[b]); f(h->mz[b]);
     }
     f(h->delta); f(h->pnew); f(h->a0);
     f(h->spx); f(h->spy); f(h->spz); f(h->sdy); f(h->sdz); f(h->red);
-    double *arr[] = {h->ex, h->ey, h->ez, h->ay, h->az, h->ek, h->ebar, h->ga_y, h->ga_z,
-                     h->eky, h->ekz, h->aky, h->akz, h->by, h->bz, h->r0y, h->r0z, h->rho,
+    double *arr[] = {h->ex, h->ey, h->ez, h->ay, h->az, h->ek, h->ebar,
+                     h->eky, h->ekz, h->aky, h->akz, h->by, h->bz, h->mdep, h->gtab, h->rho,
                      h->work, h->diag, h->d_rowM0, h->d_rowM1, h->d_rowK, h->d_rowPm,
                      h->d_tapM1, h->d_tapP};
     for (double *a : arr) f(a);
@@ -135,7 +135,7 @@ static void release(pic_handle *h)
     f(h->ctrl);
     f(h->d_count);
     drop_graphs(h);
-    f(h->img.a); f(h->img.f); f(h->img.an); f(h->img.ak); f(h->img.lo);
+    f(h->T.A); f(h->T.E); f(h->T.Kt); f(h->T.L);
     for (int m = 0; m < kMaxStartOrder; ++m) { f(h->fh.x[m]); f(h->fh.y[m]); f(h->fh.z[m]); }
     cudaStreamSynchronize(s);
     if (h->h_flag) cudaFreeHost(h->h_flag);
@@ -264,13 +264,13 @@ pic::RunDesc pic::handle_desc(pic_handle *h)
     d.M = h->M; d.K = h->K; d.fp32 = h->fp32; d.np = h->np; d.dx = h->dx; d.dt = h->cfg.dt;
     d.P = cur_parts(h);
     d.ex = h->ex; d.ek = h->ek; d.ebar = h->ebar; d.ay = h->ay; d.az = h->az;
-    d.ga_y = h->ga_y; d.ga_z = h->ga_z; d.j0 = h->jb[0]; d.j1 = h->jb[1];
+    d.m1[0] = h->m1[0]; d.m1[1] = h->m1[1];
     d.rowPm = h->d_rowPm; d.rowK = h->d_rowK;
     d.ey = h->ey; d.ez = h->ez; d.by = h->by; d.bz = h->bz;
     d.eky = h->eky; d.ekz = h->ekz; d.aky = h->aky; d.akz = h->akz;
-    d.sy0 = h->sy[0]; d.sz0 = h->sz[0]; d.sy1 = h->sy[1]; d.sz1 = h->sz[1];
+    for (int b = 0; b < 2; ++b) { d.my[b] = h->my[b]; d.mz[b] = h->mz[b]; }
     d.ctrl = h->ctrl;
-    d.img = h->img;
+    d.T = h->T;
     d.fh = h->fh;
     return d;
 }
@@ -278,14 +278,15 @@ pic::RunDesc pic::handle_desc(pic_handle *h)
 // ------------------------------------------------------------------ charge + Poisson
 static int deposit_charge(pic_handle *h, double *out)
 {
-    CK(cudaMemsetAsync(out, 0, sizeof(double) * h->M, h->stream));
+    CK(cudaMemsetAsync(h->mdep, 0, sizeof(double) * h->M * (h->K + 1), h->stream));
     DiagArgs a{};
     a.M = h->M; a.K = h->K; a.fp32 = h->fp32; a.np = h->np; a.dx = h->dx; a.w = h->cfg.weight;
     a.P = cur_parts(h);
-    a.out = out;
-    if (launch_charge(a, particle_grid(h), 256, charge_smem(h->M, h->K + 1), h->stream))
-        return fail(h, PIC_ERR_INVALID, "charge: bad degree");
+    a.mom = h->mdep;
+    if (launch_charge(a, h->grid2, h->stream)) return fail(h, PIC_ERR_INVALID, "charge: bad degree");
     CKL_N("launch_charge");
+    launch_moments_to_nodes(h->M, h->K, false, h->cfg.weight, h->mdep, out, h->stream);
+    CKL_N("launch_moments_to_nodes");
     return PIC_OK;
 }
 
@@ -293,7 +294,7 @@ static int conv_plain(pic_handle *h, const double *taps, int d_start, int ntap,
                       const double *in0, double *out0, const double *in1, double *out1)
 {
     ConvArgs c{};
-    c.M = h->M; c.d_start = d_start; c.ntap = ntap; c.mode = CONV_PLAIN; c.ncomp = in1 ? 2 : 1;
+    c.M = h->M; c.K = h->K; c.d_start = d_start; c.ntap = ntap; c.mode = CONV_PLAIN; c.ncomp = in1 ? 2 : 1;
     c.taps = taps;
     c.in[0] = in0; c.in[1] = in1;
     c.out[0] = out0; c.out[1] = out1;
@@ -318,6 +319,16 @@ extern "C" int pic_init(const pic_config *cfg, const pic_arrays *in, int32_t mem
                         pic_handle **out)
 {
     return pic_init_split(cfg, in, mem, stream, nullptr, nullptr, out);
+}
+
+// Bytes of a grid of M cells with a halo of H, its deposit rows and the marker stages of
+// a block of 512 threads: the limit on the grid size (pic.h).
+static size_t staged_grid_bytes(int M, int H, int fp32)
+{
+    const size_t W = (size_t)M + 2 * (size_t)H, stages = fp32 ? 4 : 2, r = fp32 ? 4 : 8;
+    const size_t one = 128 + stages * 512 * (4 + 3 * r) + (W + 32) * 8 + W * 24;
+    const size_t two = 128 + stages * 512 * (4 + 2 * r) + 2 * W * 8 + (fp32 ? 24 : 32) * W;
+    return std::max(one, two);
 }
 
 extern "C" int pic_init_split(const pic_config *cfg, const pic_arrays *in, int32_t mem, void *stream,
@@ -378,7 +389,6 @@ extern "C" int pic_init_split(const pic_config *cfg, const pic_arrays *in, int32
     }
     // |x^{n+1} - x^n| < dt because |p|/gamma < 1: at most ceil(dt/dx) cells
     h->Dlim = (int)std::ceil(c.dt / dx) + 1;
-    h->H = h->K + h->Dlim + 2;
     int rc = PIC_OK;
     auto bail = [&](int code) {
         g_init_error = h->err.empty() ? "pic_init failed" : h->err;
@@ -405,9 +415,12 @@ extern "C" int pic_init_split(const pic_config *cfg, const pic_arrays *in, int32
         h->P[b].t = h->Pblk[b] + off_t;
         h->P[b].p = h->Pblk[b] + off_p;
         h->P[b].id = reinterpret_cast<int32_t *>(h->Pblk[b] + off_id);
-        if ((rc = dalloc(h, &h->jb[b], M))) return bail(rc);
-        if ((rc = dalloc(h, &h->sy[b], M))) return bail(rc);
-        if ((rc = dalloc(h, &h->sz[b], M))) return bail(rc);
+        if ((rc = dalloc(h, &h->m1[b], M * c.degree)) || (rc = dalloc(h, &h->my[b], M * (c.degree + 1))) ||
+            (rc = dalloc(h, &h->mz[b], M * (c.degree + 1))))
+            return bail(rc);
+        if (reduce_fn && ((rc = dalloc(h, &h->jb[b], M)) || (rc = dalloc(h, &h->sy[b], M)) ||
+                          (rc = dalloc(h, &h->sz[b], M))))
+            return bail(rc);
     }
     if ((rc = dalloc(h, (char **)&h->delta, npa * h->rsize))) return bail(rc);
     if ((rc = dalloc(h, (char **)&h->pnew, npa * h->rsize))) return bail(rc);
@@ -415,9 +428,8 @@ extern "C" int pic_init_split(const pic_config *cfg, const pic_arrays *in, int32
     // FP64 pipe: 311 -> 287 ms a step on C2); in the FP32 form the extra 16 bytes a
     // marker cost more than the instructions they save (1.98 -> 2.04 ms a sweep)
     if (!h->fp32 && (rc = dalloc(h, (char **)&h->a0, npa * 4 * h->rsize))) return bail(rc);
-    double **grid_arrays[] = {&h->ex, &h->ey, &h->ez, &h->ay, &h->az, &h->ek, &h->ebar, &h->ga_y,
-                              &h->ga_z, &h->eky, &h->ekz, &h->aky, &h->akz, &h->by, &h->bz,
-                              &h->r0y, &h->r0z, &h->rho, &h->work};
+    double **grid_arrays[] = {&h->ex, &h->ey, &h->ez, &h->ay, &h->az, &h->ek, &h->ebar,
+                              &h->eky, &h->ekz, &h->aky, &h->akz, &h->by, &h->bz, &h->rho, &h->work};
     for (double **a : grid_arrays)
         if ((rc = dalloc(h, a, M))) return bail(rc);
     // starting fields: subsystem I from e_x^n (its changes are dominated by marker
@@ -446,14 +458,15 @@ extern "C" int pic_init_split(const pic_config *cfg, const pic_arrays *in, int32
         cudaMemcpyAsync(h->spz, in->sz, np * sizeof(double), k, h->stream);
         if (spin_optin(h->M)) return bail(fail(h, PIC_ERR_CUDA, "spin deposit shared-memory opt-in failed"));
     }
-    if (h->fp32) {
-        if ((rc = dalloc(h, &h->img.a, M)) || (rc = dalloc(h, &h->img.f, M)) || (rc = dalloc(h, &h->img.an, M)) ||
-            (rc = dalloc(h, &h->img.ak, M)) || (rc = dalloc(h, &h->img.lo, M)))
+    {
+        const size_t pa = coef_pad(h->fp32, c.degree + 1), pe = coef_pad(h->fp32, c.degree);
+        if ((rc = dalloc(h, (char **)&h->T.A, 2 * M * pa * h->rsize)) ||
+            (rc = dalloc(h, (char **)&h->T.Kt, 2 * M * pa * h->rsize)) ||
+            (rc = dalloc(h, (char **)&h->T.E, M * pe * h->rsize)) ||
+            (h->fp32 && (rc = dalloc(h, &h->T.L, 2 * M * pa))) ||
+            (rc = dalloc(h, &h->mdep, 2 * M * (c.degree + 1))) ||
+            (rc = dalloc(h, &h->gtab, M * coef_pad(0, c.degree + 1))))
             return bail(rc);
-        double fact = 1.0;
-        for (int d = 2; d <= c.degree; ++d) fact *= d;
-        h->img.inv_fact = 1.0 / fact;
-        h->img.escale = dx / (double)mean_scale(c.degree - 1);
     }
     if ((rc = dalloc(h, &h->counts, 2 * M * kVelBinsBase * bins_per_cell((long long)np, (int)M)))) return bail(rc);
     if ((rc = dalloc(h, &h->ctrl, 1))) return bail(rc);
@@ -497,25 +510,23 @@ extern "C" int pic_init_split(const pic_config *cfg, const pic_arrays *in, int32
     if (cudaMemcpy(h->d_tapP, taps.data(), sizeof(double) * h->tapP_n, cudaMemcpyHostToDevice) != cudaSuccess)
         return bail(PIC_ERR_CUDA);
 
-    // shared-memory budgets and persistent grid size
-    h->smem1 = sweep1_smem(h->M, h->H, h->fp32);
-    h->smem2 = sweep2_smem(h->M, h->H, h->fp32);
+    // grids that a block's shared memory could not stage with its markers are refused
+    // (the documented limit)
     int maxsm = 0;
     cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
-    if (h->smem1 > (size_t)maxsm || h->smem2 > (size_t)maxsm) {
-        fail(h, PIC_ERR_INVALID, "grid too large for shared memory (%zu > %d)", h->smem1, maxsm);
+    const size_t staged = staged_grid_bytes(h->M, h->K + h->Dlim + 2, h->fp32);
+    if (staged > (size_t)maxsm) {
+        fail(h, PIC_ERR_INVALID, "grid too large for shared memory (%zu > %d)", staged, maxsm);
         return bail(PIC_ERR_INVALID);
     }
-    // opt in to large dynamic shared memory (per kernel instantiation), then size the
-    // persistent sweep grids as SMs x resident blocks per SM
-    if (pic_set_smem_attrs(std::max(h->smem1, h->smem2), std::max(h->smem1, h->smem2),
-                           charge_smem(h->M, h->H)))
-        return bail(fail(h, PIC_ERR_CUDA, "cudaFuncSetAttribute failed"));
     {
-        const int b1 = sweep_blocks_per_sm(h->K, h->fp32, h->acc, 1, h->sweep_block, h->smem1);
-        const int b2 = sweep_blocks_per_sm(h->K, h->fp32, h->acc, 2, h->sweep_block, h->smem2);
+        // persistent sweeps: SMs x resident blocks, fewer when a warp step (32 markers) a
+        // block is all there is
+        const int b1 = sweep_blocks_per_sm(h->K, h->fp32, h->acc, 1), b2 = sweep_blocks_per_sm(h->K, h->fp32, h->acc, 2);
         if (b1 < 1 || b2 < 1) return bail(fail(h, PIC_ERR_INVALID, "sweep kernels do not fit on an SM"));
-        h->sweep_grid = h->num_sms * std::min(b1, b2);
+        const long long most = std::max<long long>(1, (h->np + 31) / 32);
+        h->grid1 = (int)std::min<long long>((long long)h->num_sms * b1, most);
+        h->grid2 = (int)std::min<long long>((long long)h->num_sms * b2, most);
     }
 
     // inputs
@@ -646,64 +657,68 @@ static int substep3(pic_handle *h)
 }
 
 // Subsystem I over a time step dt (the handle's dt, or half of it in a Strang step).
-static Sweep1Args sweep1_args(pic_handle *h, double dt)
+Sweep1Args pic::make_sweep1_args(pic_handle *h, double dt)
 {
     Sweep1Args a{};
-    a.M = h->M; a.H = h->H; a.Dlim = h->Dlim; a.K = h->K; a.fp32 = h->fp32; a.acc = h->acc; a.np = h->np;
-    a.dx = h->dx; a.dt = dt; a.w = h->cfg.weight;
+    a.M = h->M; a.Dlim = h->Dlim; a.K = h->K; a.fp32 = h->fp32; a.acc = h->acc; a.np = h->np;
+    a.dx = h->dx; a.dt = dt;
     a.P = cur_parts(h);
-    a.ebar = h->ebar; a.ga_y = h->ga_y; a.ga_z = h->ga_z; a.ay = h->ay; a.az = h->az;
+    a.T = h->T;
     a.ctrl = h->ctrl;
-    a.img = h->img;
     a.a0 = h->a0;
+    a.zforce = h->cfg.hbar != 0.0;
     a.hbar = h->cfg.hbar;
     a.sy = h->spy;
     a.sz = h->spz;
-    a.jpair[0] = h->jb[0]; a.jpair[1] = h->jb[1];
+    a.mom = h->m1[0];
+    a.mpair[0] = h->m1[0]; a.mpair[1] = h->m1[1];
     return a;
 }
 
-static ConvArgs conv1_args(pic_handle *h, double dt)
+ConvArgs pic::make_conv1_args(pic_handle *h, double dt)
 {
     ConvArgs c{};
-    c.img = h->img;
-    c.M = h->M; c.d_start = h->tapM1_start; c.ntap = h->tapM1_n; c.mode = CONV_SOLVE1; c.ncomp = 1;
+    c.T = h->T;
+    c.M = h->M; c.K = h->K; c.d_start = h->tapM1_start; c.ntap = h->tapM1_n; c.mode = CONV_SOLVE1; c.ncomp = 1;
     c.taps = h->d_tapM1;
+    c.scale = h->cfg.weight * h->dx;
     c.en[0] = h->ex; c.ek[0] = h->ek; c.aux[0] = h->ebar;
     c.dt = dt; c.dx = h->dx; c.tol = h->cfg.tol; c.dtol = 1e-6;   // FP32: estimated position error, cells relative to max(1, |delta|)
     c.erel = h->cfg.warm_field ? kFieldIncrementRelPredicted : kFieldIncrementRel;
     c.max_iter = h->cfg.max_iter; c.fp32 = h->fp32; c.subsystem = 1; c.ctrl = h->ctrl;
-    c.pair[0][0] = h->jb[0]; c.pair[0][1] = h->jb[1];
+    c.pair[0][0] = h->m1[0]; c.pair[0][1] = h->m1[1];
     return c;
 }
 
-static Sweep2Args sweep2_args(pic_handle *h)
+Sweep2Args pic::make_sweep2_args(pic_handle *h)
 {
     Sweep2Args a{};
-    a.status = &h->ctrl->status;
-    a.M = h->M; a.H = h->H; a.K = h->K; a.fp32 = h->fp32; a.acc = h->acc; a.np = h->np; a.w = h->cfg.weight;
+    a.M = h->M; a.K = h->K; a.fp32 = h->fp32; a.acc = h->acc; a.np = h->np;
     a.P = cur_parts(h);
-    a.an_y = h->ay; a.an_z = h->az; a.ak_y = h->aky; a.ak_z = h->akz;
-    a.img = h->img;
+    a.T = h->T;
     a.ctrl = h->ctrl;
-    a.sypair[0] = h->sy[0]; a.sypair[1] = h->sy[1];
-    a.szpair[0] = h->sz[0]; a.szpair[1] = h->sz[1];
+    a.a0 = h->a0;
+    a.zforce = h->cfg.hbar != 0.0;
+    a.mom_y = h->my[0]; a.mom_z = h->mz[0];
+    a.mypair[0] = h->my[0]; a.mypair[1] = h->my[1];
+    a.mzpair[0] = h->mz[0]; a.mzpair[1] = h->mz[1];
     return a;
 }
 
-static ConvArgs conv2_args(pic_handle *h)
+ConvArgs pic::make_conv2_args(pic_handle *h)
 {
     ConvArgs c{};
-    c.img = h->img;
-    c.M = h->M; c.d_start = h->tapP_start; c.ntap = h->tapP_n; c.mode = CONV_SOLVE2; c.ncomp = 2;
+    c.T = h->T;
+    c.M = h->M; c.K = h->K; c.d_start = h->tapP_start; c.ntap = h->tapP_n; c.mode = CONV_SOLVE2; c.ncomp = 2;
     c.taps = h->d_tapP;
+    c.scale = h->cfg.weight;
     c.en[0] = h->ey; c.en[1] = h->ez; c.ek[0] = h->eky; c.ek[1] = h->ekz;
     c.aux[0] = h->aky; c.aux[1] = h->akz; c.an[0] = h->ay; c.an[1] = h->az;
-    c.r0[0] = h->r0y; c.r0[1] = h->r0z;
+    c.b[0] = h->by; c.b[1] = h->bz;
     c.dt = h->cfg.dt; c.dx = h->dx; c.tol = h->cfg.tol; c.dtol = 0.0;
     c.max_iter = h->cfg.max_iter; c.fp32 = h->fp32; c.subsystem = 2; c.ctrl = h->ctrl;
-    c.pair[0][0] = h->sy[0]; c.pair[0][1] = h->sy[1];
-    c.pair[1][0] = h->sz[0]; c.pair[1][1] = h->sz[1];
+    c.pair[0][0] = h->my[0]; c.pair[0][1] = h->my[1];
+    c.pair[1][0] = h->mz[0]; c.pair[1][1] = h->mz[1];
     return c;
 }
 
@@ -718,22 +733,35 @@ static WarmArgs warm_args(pic_handle *h, double dt)
     return wa;
 }
 
-// The predicted start of subsystem I (warm_field): delta^(0) and j^(0) into jb[1]
-// (cleared by the preparation; the first sweep deposits into jb[0] and its solve
-// clears jb[1]), then e^(0) = e^n - M1^{-1} j^(0) and ebar^(0).
+// Split runs: the moments of a deposit as nodes, summed over the processes, become the
+// solve's input.  (Single-process runs read the moments in the solve itself.)
+static int reduce_moments(pic_handle *h, ConvArgs &c, int comp, const double *mom, double *nodes)
+{
+    c.mom[comp] = mom;
+    if (!h->reduce) return PIC_OK;
+    const bool path = c.subsystem == 1;
+    launch_moments_to_nodes(h->M, path ? h->K - 1 : h->K, path, c.scale, mom, nodes, h->stream);
+    CKL_N("launch_moments_to_nodes");
+    c.mom[comp] = nullptr;
+    c.in[comp] = nodes;
+    return reduce(h, PIC_REDUCE_SUM, nodes, h->M);
+}
+
+// The predicted start of subsystem I (warm_field): delta^(0) and j^(0) into m1[1]
+// (cleared by the preparation; the first sweep deposits into m1[0] and its solve
+// clears m1[1]), then e^(0) = e^n - M1^{-1} j^(0) and ebar^(0).
 static int predicted_start(pic_handle *h, double dt, cudaStream_t s)
 {
-    Sweep1Args a = sweep1_args(h, dt);
+    Sweep1Args a = make_sweep1_args(h, dt);
     a.warm = h->cfg.warm_start == PIC_WARM_EXPLICIT ? 1 : 0;   // else the network's delta is there
-    a.j = h->jb[1];
+    a.mom = h->m1[1];
     a.first = 1;
-    if (launch_predeposit(a, h->sweep_grid, h->sweep_block, h->smem1, s))
-        return fail(h, PIC_ERR_INVALID, "predeposit");
-    int rc;
-    if (s == h->stream && (rc = reduce(h, PIC_REDUCE_SUM, h->jb[1], h->M))) return rc;   // split runs
-    ConvArgs c = conv1_args(h, dt);
+    if (launch_predeposit(a, h->grid1, s)) return fail(h, PIC_ERR_INVALID, "predeposit");
+    ConvArgs c = make_conv1_args(h, dt);
     c.mode = CONV_START1;
-    c.in[0] = h->jb[1];
+    c.mom[0] = h->m1[1];
+    int rc;
+    if (s == h->stream && (rc = reduce_moments(h, c, 0, h->m1[1], h->jb[1]))) return rc;
     if (launch_conv(c, s)) return fail(h, PIC_ERR_CUDA, "k_conv launch");
     return PIC_OK;
 }
@@ -744,8 +772,8 @@ static int substep1(pic_handle *h, int *iters, double dt)
     const RunDesc desc = handle_desc(h);
     launch_prep1(desc, h->stream);
     CKL_N("launch_prep1");
-    Sweep1Args a = sweep1_args(h, dt);
-    ConvArgs c = conv1_args(h, dt);
+    Sweep1Args a = make_sweep1_args(h, dt);
+    ConvArgs c = make_conv1_args(h, dt);
     if (h->cfg.warm_start == PIC_WARM_MLP) {
         // learned proposal for delta^(0), written over the zero iterate
         if (!h->mlp) return fail(h, PIC_ERR_INVALID, "warm_start = PIC_WARM_MLP but no network attached");
@@ -763,18 +791,17 @@ static int substep1(pic_handle *h, int *iters, double dt)
     }
     int it = 0;
     for (;;) {
-        a.j = h->jb[it & 1];
+        a.mom = h->m1[it & 1];
         a.warm = (it == 0 && h->cfg.warm_start == PIC_WARM_EXPLICIT && !h->cfg.warm_field) ? 1 : 0;
         a.first = it == 0 ? 1 : 0;
         if ((rc = timed_begin(h))) return rc;
-        if (launch_sweep1(a, h->sweep_grid, h->sweep_block, h->smem1, h->stream))
+        if (launch_sweep1(a, h->grid1, h->stream))
             return fail(h, PIC_ERR_INVALID, "sweep1: bad degree");
         CKL_N("launch_sweep1");
         if ((rc = timed_end(h, 0))) return rc;
         h->marker_sweeps += h->np;
-        if ((rc = reduce(h, PIC_REDUCE_SUM, h->jb[it & 1], h->M)) || (rc = reduce_ctrl(h))) return rc;
-        c.in[0] = h->jb[it & 1];
-        c.zero[0] = h->jb[(it + 1) & 1];
+        if ((rc = reduce_moments(h, c, 0, h->m1[it & 1], h->jb[it & 1])) || (rc = reduce_ctrl(h))) return rc;
+        c.zero[0] = h->m1[(it + 1) & 1];
         if ((rc = timed_begin(h))) return rc;
         if (launch_conv(c, h->stream)) return fail(h, PIC_ERR_CUDA, "k_conv shared-memory opt-in failed");
         CKL_N("launch_conv");
@@ -811,25 +838,22 @@ static int substep2(pic_handle *h, int *iters)
         launch_spin_rhs(h->M, h->dx, h->cfg.dt, h->cfg.hbar, h->sdy, h->sdz, h->by, h->bz, h->stream);
         CKL_N("launch_spin_rhs");
     }
-    if ((rc = conv_plain(h, h->d_tapP, h->tapP_start, h->tapP_n, h->by, h->r0y, h->bz, h->r0z))) return rc;
-    Sweep2Args a = sweep2_args(h);
-    ConvArgs c = conv2_args(h);
+    Sweep2Args a = make_sweep2_args(h);
+    ConvArgs c = make_conv2_args(h);
     int it = 0;
     for (;;) {
-        a.s_y = h->sy[it & 1];
-        a.s_z = h->sz[it & 1];
+        a.mom_y = h->my[it & 1];
+        a.mom_z = h->mz[it & 1];
+        a.first = it == 0 ? 1 : 0;
         if ((rc = timed_begin(h))) return rc;
-        if (launch_sweep2(a, h->sweep_grid, h->sweep_block, h->smem2, h->stream))
-            return fail(h, PIC_ERR_INVALID, "sweep2: bad degree");
+        if (launch_sweep2(a, h->grid2, h->stream)) return fail(h, PIC_ERR_INVALID, "sweep2: bad degree");
         CKL_N("launch_sweep2");
         if ((rc = timed_end(h, 1))) return rc;
-        if ((rc = reduce(h, PIC_REDUCE_SUM, h->sy[it & 1], h->M)) ||
-            (rc = reduce(h, PIC_REDUCE_SUM, h->sz[it & 1], h->M)) || (rc = reduce_ctrl(h)))
+        if ((rc = reduce_moments(h, c, 0, h->my[it & 1], h->sy[it & 1])) ||
+            (rc = reduce_moments(h, c, 1, h->mz[it & 1], h->sz[it & 1])) || (rc = reduce_ctrl(h)))
             return rc;
-        c.in[0] = h->sy[it & 1];
-        c.in[1] = h->sz[it & 1];
-        c.zero[0] = h->sy[(it + 1) & 1];
-        c.zero[1] = h->sz[(it + 1) & 1];
+        c.zero[0] = h->my[(it + 1) & 1];
+        c.zero[1] = h->mz[(it + 1) & 1];
         if ((rc = timed_begin(h))) return rc;
         if (launch_conv(c, h->stream)) return fail(h, PIC_ERR_CUDA, "k_conv shared-memory opt-in failed");
         CKL_N("launch_conv");
@@ -917,14 +941,7 @@ static int seg_sub1_tail(pic_handle *h, cudaStream_t s, int *nodes)
 static int seg_sub2_head(pic_handle *h, cudaStream_t s, int *nodes)
 {
     launch_prep2(handle_desc(h), s);
-    ConvArgs c{};
-    c.M = h->M; c.d_start = h->tapP_start; c.ntap = h->tapP_n; c.mode = CONV_PLAIN; c.ncomp = 2;
-    c.taps = h->d_tapP;
-    c.in[0] = h->by; c.in[1] = h->bz;
-    c.out[0] = h->r0y; c.out[1] = h->r0z;
-    c.ctrl = h->ctrl;
-    if (launch_conv(c, s)) return fail(h, PIC_ERR_CUDA, "k_conv launch");
-    *nodes += 2;
+    *nodes += 1;
     return PIC_OK;
 }
 
@@ -938,23 +955,20 @@ static int seg_sub2_tail(pic_handle *h, cudaStream_t s, int *nodes)
 static int loop_body(pic_handle *h, cudaStream_t s, int which, double dt, unsigned long long cond)
 {
     if (which == 1) {
-        Sweep1Args a = sweep1_args(h, dt);
+        Sweep1Args a = make_sweep1_args(h, dt);
         a.graph = 1;
         a.warm = (h->cfg.warm_start == PIC_WARM_EXPLICIT && !h->cfg.warm_field) ? 1 : 0;   // applied when iter == 0
-        a.j = h->jb[0];
-        if (launch_sweep1(a, h->sweep_grid, h->sweep_block, h->smem1, s)) return fail(h, PIC_ERR_INVALID, "sweep1");
-        ConvArgs c = conv1_args(h, dt);
+        if (launch_sweep1(a, h->grid1, s)) return fail(h, PIC_ERR_INVALID, "sweep1");
+        ConvArgs c = make_conv1_args(h, dt);
         c.graph = 1;
         c.cond_handle = cond;
         c.count = h->d_count;
         if (launch_conv(c, s)) return fail(h, PIC_ERR_CUDA, "k_conv launch");
     } else {
-        Sweep2Args a = sweep2_args(h);
+        Sweep2Args a = make_sweep2_args(h);
         a.graph = 1;
-        a.s_y = h->sy[0];
-        a.s_z = h->sz[0];
-        if (launch_sweep2(a, h->sweep_grid, h->sweep_block, h->smem2, s)) return fail(h, PIC_ERR_INVALID, "sweep2");
-        ConvArgs c = conv2_args(h);
+        if (launch_sweep2(a, h->grid2, s)) return fail(h, PIC_ERR_INVALID, "sweep2");
+        ConvArgs c = make_conv2_args(h);
         c.graph = 1;
         c.cond_handle = cond;
         c.count = h->d_count + 1;
@@ -1193,15 +1207,16 @@ extern "C" int pic_deposit(pic_handle *h, int32_t kind, const double *aux, doubl
     }
     if (kind == PIC_DEP_CURRENT) {
         if (!aux) return fail(h, PIC_ERR_INVALID, "CURRENT needs the displacements");
-        CK(cudaMemsetAsync(out, 0, sizeof(double) * h->M, h->stream));
+        CK(cudaMemsetAsync(h->mdep, 0, sizeof(double) * h->M * h->K, h->stream));
         launch_ctrl_reset(h->ctrl, h->stream);
         CKL_N("launch_ctrl_reset");
         CurrentArgs a{};
-        a.M = h->M; a.H = h->H; a.Dlim = h->Dlim; a.K = h->K; a.fp32 = h->fp32; a.np = h->np;
-        a.dx = h->dx; a.w = h->cfg.weight; a.P = cur_parts(h); a.disp = aux; a.out = out; a.ctrl = h->ctrl;
-        if (launch_current(a, particle_grid(h), 256, charge_smem(h->M, h->H), h->stream))
-            return fail(h, PIC_ERR_INVALID, "bad degree");
+        a.M = h->M; a.Dlim = h->Dlim; a.K = h->K; a.fp32 = h->fp32; a.np = h->np;
+        a.dx = h->dx; a.P = cur_parts(h); a.disp = aux; a.mom = h->mdep; a.ctrl = h->ctrl;
+        if (launch_current(a, h->grid1, h->stream)) return fail(h, PIC_ERR_INVALID, "bad degree");
         CKL_N("launch_current");
+        launch_moments_to_nodes(h->M, h->K - 1, true, h->cfg.weight * h->dx, h->mdep, out, h->stream);
+        CKL_N("launch_moments_to_nodes");
         if ((rc = read_ctrl(h))) return rc;
         if (h->h_ctrl->status & STATUS_NUMERIC)
             return fail(h, PIC_ERR_NUMERIC, "displacement beyond the halo or not finite");
@@ -1209,16 +1224,19 @@ extern "C" int pic_deposit(pic_handle *h, int32_t kind, const double *aux, doubl
     }
     if (kind == PIC_DEP_SUSCEPT) {
         if (!aux) return fail(h, PIC_ERR_INVALID, "SUSCEPT needs a*");
-        CK(cudaMemsetAsync(out, 0, sizeof(double) * 2 * h->M, h->stream));
-        Sweep2Args a{};
-        a.status = &h->ctrl->status;
-        a.M = h->M; a.H = h->H; a.K = h->K; a.fp32 = h->fp32; a.acc = h->acc; a.np = h->np; a.w = h->cfg.weight;
-        a.P = cur_parts(h);
-        a.an_y = h->ay; a.an_z = h->az; a.ak_y = aux; a.ak_z = aux + h->M;
-        a.s_y = out; a.s_z = out + h->M;
-        if (launch_sweep2(a, h->sweep_grid, h->sweep_block, h->smem2, h->stream))
-            return fail(h, PIC_ERR_INVALID, "bad degree");
+        const size_t n = (size_t)h->M * (h->K + 1);
+        CK(cudaMemsetAsync(h->mdep, 0, sizeof(double) * 2 * n, h->stream));
+        launch_tables2(h->M, h->K, h->fp32, h->ay, h->az, aux, aux + h->M, h->T, h->stream);
+        CKL_N("launch_tables2");
+        Sweep2Args a = make_sweep2_args(h);
+        a.mom_y = h->mdep; a.mom_z = h->mdep + n;
+        a.a0 = nullptr;
+        a.zforce = 1;
+        if (launch_sweep2(a, h->grid2, h->stream)) return fail(h, PIC_ERR_INVALID, "sweep2: bad degree");
         CKL_N("launch_sweep2");
+        launch_moments_to_nodes(h->M, h->K, false, h->cfg.weight, h->mdep, out, h->stream);
+        launch_moments_to_nodes(h->M, h->K, false, h->cfg.weight, h->mdep + n, out + h->M, h->stream);
+        CKL_N("launch_moments_to_nodes");
         return sync(h);
     }
     return fail(h, PIC_ERR_INVALID, "unknown deposit kind %d", kind);
@@ -1234,7 +1252,9 @@ extern "C" int pic_gather(pic_handle *h, int32_t field, double *out)
         DiagArgs a{};
         a.M = h->M; a.K = h->K; a.fp32 = h->fp32; a.np = h->np; a.dx = h->dx; a.w = h->cfg.weight;
         a.P = cur_parts(h);
-        a.c0 = h->ex;
+        launch_cell_coefs(h->M, h->K - 1, true, h->ex, h->gtab, h->stream);
+        CKL_N("launch_cell_coefs");
+        a.tab = h->gtab;
         a.out = out;
         a.Dlim = h->Dlim;
         a.status = &h->ctrl->status;
@@ -1259,7 +1279,9 @@ extern "C" int pic_gather(pic_handle *h, int32_t field, double *out)
     DiagArgs a{};
     a.M = h->M; a.K = h->K; a.fp32 = h->fp32; a.np = h->np; a.dx = h->dx; a.w = h->cfg.weight;
     a.P = cur_parts(h);
-    a.c0 = coef;
+    launch_cell_coefs(h->M, d, false, coef, h->gtab, h->stream);
+    CKL_N("launch_cell_coefs");
+    a.tab = h->gtab;
     a.out = out;
     if (launch_gather(a, d, particle_grid(h), 256, h->stream)) return fail(h, PIC_ERR_INVALID, "bad degree");
     CKL_N("launch_gather");

@@ -30,6 +30,7 @@ struct DevCtrl {
     int status;                        // error bits, see STATUS_*
     unsigned int ticket;               // last-block election in multi-block grid kernels
     int hist1, hist2;                  // field changes stored for the starting fields
+    int zany;                          // a_z or e_z was non-zero at some node
     double acc[4];                     // reductions for diagnostics (energy, residual)
 };
 
@@ -38,6 +39,13 @@ enum : int {
     STATUS_NOCONV  = 2,
     STATUS_TIMEOUT = 4,    // a bounded wait on a bulk copy gave up
 };
+
+// accumulator kinds of the sweeps (pic_config.deposit)
+enum : int { ACC_NATIVE = 0, ACC_COMP = 1, ACC_DOUBLE = 2 };
+
+// numbers a row of n polynomial coefficients takes (pic_poly.cuh): rows are read by
+// 16-byte loads
+__host__ __device__ inline int coef_pad(int fp32, int n) { return fp32 ? (n <= 4 ? 4 : 8) : ((n + 1) & ~1); }
 
 // ---------------------------------------------------------------------------
 // Bulk asynchronous copies (the TMA engine's 1-D bulk mode) into shared memory,
@@ -65,28 +73,6 @@ __device__ __forceinline__ void fence_mbar_init()
 __device__ __forceinline__ void fence_proxy_async()
 {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(unsigned long long *bar, unsigned bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes)
-                 : "memory");
-}
-
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, unsigned bytes, unsigned long long *bar)
-{
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_u32(dst)),
-        "l"(src), "r"(bytes), "r"(smem_u32(bar))
-        : "memory");
-}
-
-// one arrival (release semantics: this thread's earlier shared-memory reads are
-// ordered before the barrier's phase completes)
-__device__ __forceinline__ void mbar_arrive(unsigned long long *bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
 __device__ __forceinline__ bool mbar_wait(unsigned long long *bar, unsigned parity)
@@ -271,237 +257,6 @@ __device__ __forceinline__ int walk_path(R t0, R d, Visit &&visit)
 }
 
 // ---------------------------------------------------------------------------
-// Accumulators of the per-lane deposit windows.  A lane adds the contributions of
-// the markers it holds between two flushes (about a hundred at 5e4 markers a
-// cell); what it adds are float values in the float form.
-//  AccNative<R>: a plain R sum (the double form; the float form's fastest choice,
-//                whose rounding grows with the number of markers a lane adds).
-//  AccComp:      a compensated float pair (hi, lo): each add is an error-free
-//                two-sum, so hi + lo carries the lane's sum to about double
-//                accuracy (Knuth's TwoSum; the pair is read out in double).
-//  AccDouble:    a double sum of float values (exact adds of the products,
-//                on the FP64 pipe).
-// warp_part() sums a slot over the warp in the accumulator's own type; value()
-// converts such a sum to double (done by the one lane that writes it).
-// ---------------------------------------------------------------------------
-template <typename R>
-struct AccNative {
-    R v;
-    __device__ __forceinline__ void clear() { v = R(0); }
-    template <typename T> __device__ __forceinline__ void add(T x) { v += x; }
-    // sum over the warp, in every lane, in the accumulator's own precision;
-    // value() reads a sum out in double (called by the writing lane only)
-    using Part = R;
-    __device__ __forceinline__ Part warp_part() const
-    {
-        R t = v;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        return t;
-    }
-    __device__ __forceinline__ static double value(Part t) { return (double)t; }
-};
-
-// Knuth's TwoSum: a + b = s + e exactly (float, any magnitudes)
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
-{
-    s = a + b;
-    const float bp = s - a;
-    e = (a - (s - bp)) + (b - bp);
-}
-
-// Compensated float pair with a bias: hi starts at 2^BL, far above any lane sum
-// of the deposits it collects, so every add satisfies |hi| >= |x| and Dekker's
-// Fast2Sum (three operations) recovers its rounding error exactly into lo, and
-// hi - 2^BL is exact at read-out (Sterbenz, as long as the lane sum stays below
-// 2^(BL-1)).  The sweeps take 2^BL = 4096 K! (rounded up to a power of two): their
-// values are at most about K! in the scaled units of bspline_scaled, so a lane may
-// collect some two thousand full-size values between flushes.  The error left is
-// lo's own rounding: each add's error is at most ulp(2^BL)/2 (about 1e-3 K!), so
-// lo stays a small random sum whose rounding is near 1e-11 of the lane sum, against
-// about eps sqrt(n) of the sum for a plain float sum of n markers.
-template <int BL>
-struct AccComp {
-    float hi, lo;
-    static constexpr float bias() { return (float)(1u << BL); }
-    __device__ __forceinline__ void clear() { hi = bias(); lo = 0.f; }
-    __device__ __forceinline__ void add(float x)
-    {
-        const float s = hi + x;
-        lo += x - (s - hi);
-        hi = s;
-    }
-    // the warp sum of (hi - bias) + lo as a float pair (the butterfly adds pairs
-    // with TwoSum, so no float rounding of the partial sums is lost); value()
-    // reads the pair out in double
-    using Part = float2;
-    __device__ __forceinline__ Part warp_part() const
-    {
-        float h = hi - bias(), l = lo;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float h2 = __shfl_xor_sync(0xffffffffu, h, o);
-            const float l2 = __shfl_xor_sync(0xffffffffu, l, o);
-            float sum, e;
-            two_sum(h, h2, sum, e);
-            h = sum;
-            l = (l + l2) + e;
-        }
-        return make_float2(h, l);
-    }
-    __device__ __forceinline__ static double value(Part t) { return (double)t.x + (double)t.y; }
-};
-
-// log2 of the bias for degree K: 12 + ceil(log2 K!)
-template <int K> struct CompBias;
-template <> struct CompBias<2> { static constexpr int v = 13; };
-template <> struct CompBias<3> { static constexpr int v = 15; };
-template <> struct CompBias<4> { static constexpr int v = 17; };
-template <> struct CompBias<5> { static constexpr int v = 19; };
-
-struct AccDouble {
-    double v;
-    __device__ __forceinline__ void clear() { v = 0.0; }
-    __device__ __forceinline__ void add(float x) { v += (double)x; }
-    __device__ __forceinline__ void add(double x) { v += x; }
-    using Part = double;
-    __device__ __forceinline__ Part warp_part() const
-    {
-        double t = v;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-        return t;
-    }
-    __device__ __forceinline__ static double value(Part t) { return t; }
-};
-
-// accumulator kinds of the sweeps (pic_config.deposit), for degree K
-enum : int { ACC_NATIVE = 0, ACC_COMP = 1, ACC_DOUBLE = 2 };
-template <typename R, int ACC, int K> struct AccOf;
-template <typename R, int K> struct AccOf<R, ACC_NATIVE, K> { using T = AccNative<R>; };
-template <typename R, int K> struct AccOf<R, ACC_COMP, K> { using T = AccComp<CompBias<K>::v>; };
-template <typename R, int K> struct AccOf<R, ACC_DOUBLE, K> { using T = AccDouble; };
-// the accumulator a form uses unless asked otherwise
-template <typename R> struct DefaultAcc { static constexpr int v = std::is_same<R, float>::value ? ACC_COMP : ACC_NATIVE; };
-
-// ---------------------------------------------------------------------------
-// Per-warp register window for deposits of cell-sorted markers.  Each lane keeps
-// NS partial sums for the consecutive grid nodes b0 .. b0+NS-1 around the warp's
-// base cell; a piece whose NV values fall on nodes cp - r (r = 0..NV-1) goes to
-// slots (cp - base) + OFF - r, chosen by a switch so that the array stays in
-// registers.  When the warp's base cell advances by one (the common case for
-// sorted markers) only the lowest slot leaves the window: it is summed over the
-// warp and added to the block's shared-memory row, and the other slots move
-// down; any other change of base flushes every slot.  Warp sums of the plain
-// float accumulator are formed in float; those of the compensated pair as float
-// pairs; only the one value written per node is converted to double (GB300's
-// FP64 pipe is narrow, so the window keeps double arithmetic out of its loop).
-// ---------------------------------------------------------------------------
-template <typename R, int NS, int NV, int OFF, int OMIN, int OMAX, typename A = AccNative<R>, bool TRACK = false>
-struct DepWindow {
-    A acc[NS];
-    // with TRACK: this lane added to the window since its last full flush, so that
-    // moves and flushes of a window nobody wrote to (e.g. A_z = 0) cost one vote
-    bool dirty;
-    __device__ __forceinline__ void clear()
-    {
-#pragma unroll
-        for (int s = 0; s < NS; ++s) acc[s].clear();
-        dirty = false;
-    }
-    template <int O>
-    __device__ __forceinline__ void add_at(const R *v)
-    {
-#pragma unroll
-        for (int r = 0; r < NV; ++r) acc[O + OFF - r].add(v[r]);
-        dirty = true;
-    }
-    // returns false when the piece lies outside the window (caller takes the slow path)
-    __device__ __forceinline__ bool put(int o, const R *v)
-    {
-        static_assert(OMIN >= -3 && OMAX <= 3 && OMIN <= 0 && OMAX >= 0, "window offsets");
-        switch (o) {
-        case -3: if (OMIN <= -3) { add_at<(OMIN <= -3 ? -3 : 0)>(v); return true; } return false;
-        case -2: if (OMIN <= -2) { add_at<(OMIN <= -2 ? -2 : 0)>(v); return true; } return false;
-        case -1: if (OMIN <= -1) { add_at<(OMIN <= -1 ? -1 : 0)>(v); return true; } return false;
-        case 0: add_at<0>(v); return true;
-        case 1: if (OMAX >= 1) { add_at<(OMAX >= 1 ? 1 : 0)>(v); return true; } return false;
-        case 2: if (OMAX >= 2) { add_at<(OMAX >= 2 ? 2 : 0)>(v); return true; } return false;
-        case 3: if (OMAX >= 3) { add_at<(OMAX >= 3 ? 3 : 0)>(v); return true; } return false;
-        default: return false;
-        }
-    }
-    // slot S summed over the warp, added (times `scale`, in double) to s_row[row0 + S]
-    // by lane 0; all 32 lanes must call.  The warp sum stays in the accumulator's
-    // own type and only the writing lane converts it: the double arithmetic of a
-    // flush is then one lane's, not the warp's.
-    template <int S>
-    __device__ __forceinline__ void flush_slot(double *s_row, int row0, double scale)
-    {
-        const typename A::Part t = acc[S].warp_part();
-        if ((threadIdx.x & 31) == 0) {
-            const double v = A::value(t);
-            if (v != 0.0) atomicAdd(&s_row[row0 + S], scale * v);
-        }
-        acc[S].clear();
-    }
-    // every slot to the row (row0 = shared-memory index of slot 0): lane s keeps the
-    // warp sum of slot s, and lanes 0..NS-1 convert and write in one step; all
-    // lanes call
-    __device__ __forceinline__ void flush(double *s_row, int row0, double scale)
-    {
-        if (TRACK && !__any_sync(0xffffffffu, dirty)) return;     // every slot is clear
-        dirty = false;
-        const int lane = threadIdx.x & 31;
-        typename A::Part mine{};
-#pragma unroll
-        for (int q = 0; q < NS; ++q) {
-            const typename A::Part t = acc[q].warp_part();
-            if (lane == q) mine = t;
-            acc[q].clear();
-        }
-        if (lane < NS) {
-            const double v = A::value(mine);
-            if (v != 0.0) atomicAdd(&s_row[row0 + lane], scale * v);
-        }
-    }
-    // the warp's base cell moved by `d` (warp-uniform); row0 = index of slot 0 for
-    // the old base.  All lanes must call.
-    __device__ __forceinline__ void advance(int d, double *s_row, int row0, double scale)
-    {
-        if (TRACK && !__any_sync(0xffffffffu, dirty)) return;     // nothing to move
-        if (d == 1) {
-            flush_slot<0>(s_row, row0, scale);
-#pragma unroll
-            for (int q = 0; q + 1 < NS; ++q) acc[q] = acc[q + 1];
-            acc[NS - 1].clear();
-        } else if (d == -1) {
-            flush_slot<NS - 1>(s_row, row0, scale);
-#pragma unroll
-            for (int q = NS - 1; q > 0; --q) acc[q] = acc[q - 1];
-            acc[0].clear();
-        } else {
-            flush(s_row, row0, scale);
-        }
-    }
-};
-
-// Cell of a marker as its warp's deposit window sees it.  Markers are sorted by
-// cell, but between sorts a marker that crossed the periodic boundary carries
-// cell 0, 1, .. among neighbours at cell M-1 (or the reverse): the warp's lowest
-// cell is then 0, and every marker at the top end would miss the window and take
-// the slow shared-atomic path.  In a warp that holds cells in the upper half of
-// the grid, cells below U are shifted by +M.  Shared arrays staged with a periodic
-// halo of H cells hold cell c at index c + H for -H <= c < M + H, so a kernel whose
-// accesses reach at most `reach` cells above a marker's cell passes
-// U = H - reach: every index stays below M + 2H.  All lanes must call.
-__device__ __forceinline__ int warp_unwrap_cell(int c, bool act, int M, int U)
-{
-    const int hi = __reduce_max_sync(0xffffffffu, act ? c : INT_MIN);
-    return (act && hi >= M / 2 && c < U) ? c + M : c;
-}
-
-// ---------------------------------------------------------------------------
 // Scaled B-spline arithmetic for the sweep kernels.  A rounded reciprocal such
 // as 1/3 (in float 1 + 3e-8 too large) would scale every basis value by the same
 // factor; through the discrete-gradient identity such a systematic bias becomes a
@@ -594,61 +349,6 @@ __device__ __forceinline__ void piece_means_scaled(R tm, R h, R *m)
             }
             m[r] += h4 * s;
         }
-    }
-}
-
-// Number of pieces of the path from local offset t0 by d cells: 1 + knots crossed.
-template <typename R>
-__device__ __forceinline__ int path_pieces(R t0, R d)
-{
-    return abs((int)floor_(t0 + d)) + 1;
-}
-
-template <typename R> __device__ __forceinline__ R clamp01(R v) { return v < R(0) ? R(0) : (v > R(1) ? R(1) : v); }
-
-// Branch-free walk of the path t0 -> s = t0 + d split at knots.  Piece p lies in
-// cell c = sign(d) p relative to the start cell.  The piece lengths are formed
-// from d and the knot distances, never as differences of clamped coordinates,
-// so a single-piece path has length exactly d:
-//   one piece:   t0 -> s                       (h = d)
-//   first piece: t0 -> the knot ahead           (h = 1 - t0, or -t0 moving left)
-//   middle:      a whole cell                   (h = +-1, midpoint 1/2)
-//   last piece:  the knot behind -> tl = s - floor(s)  (h = tl, or tl - 1 moving left)
-// The caller passes the warp maximum of the piece counts, so every lane runs the
-// same trip count; pieces beyond a lane's own count have zero length.
-// visit(c, h, m, p) gets the signed piece length h (cells) and the scaled means
-// m[r] = S_{K-1} * mean of the degree-(K-1) pieces over it (piece_means_scaled).
-template <int K, typename R, class Visit>
-__device__ __forceinline__ void walk_uniform(R t0, R d, int npc, Visit &&visit)
-{
-    constexpr int D = K - 1;
-    const R s = t0 + d;
-    const R fl = floor_(s);
-    const int n = abs((int)fl) + 1;          // this lane's piece count
-    const R tl = s - fl;                     // local offset of the end point
-    const bool right = d >= R(0);
-    const int sg = right ? 1 : -1;
-    R m[D + 1];
-    for (int p = 0; p < npc; ++p) {
-        R h, tm;
-        if (n == 1) {
-            h = (p == 0) ? d : R(0);
-            tm = R(0.5) * (t0 + s);
-        } else if (p == 0) {
-            h = right ? R(1) - t0 : -t0;
-            tm = t0 + R(0.5) * h;
-        } else if (p == n - 1) {
-            h = right ? tl : tl - R(1);
-            tm = R(0.5) * (right ? tl : R(1) + tl);
-        } else if (p < n) {
-            h = R(sg);
-            tm = R(0.5);
-        } else {
-            h = R(0);
-            tm = R(0.5);
-        }
-        piece_means_scaled<D, R>(tm, h, m);
-        visit(sg * p, h, m, p);
     }
 }
 

@@ -40,12 +40,12 @@ struct pic_ensemble {
     std::vector<RunDesc> desc;
     std::vector<Sweep1Args> a1, a1p;
     std::vector<Sweep2Args> a2;
-    std::vector<ConvArgs> c1, c2, cp, c1p;
+    std::vector<ConvArgs> c1, c2, c1p;
     std::vector<EnsRun> er;
     RunDesc *d_desc = nullptr;
     Sweep1Args *d_a1 = nullptr, *d_a1p = nullptr;
     Sweep2Args *d_a2 = nullptr;
-    ConvArgs *d_c1 = nullptr, *d_c2 = nullptr, *d_cp = nullptr, *d_c1p = nullptr;
+    ConvArgs *d_c1 = nullptr, *d_c2 = nullptr, *d_c1p = nullptr;
     EnsRun *d_er = nullptr;
     EnsQueue *d_q = nullptr;
     int *d_sweeps = nullptr, *d_status = nullptr;
@@ -54,7 +54,6 @@ struct pic_ensemble {
     int sort_grid = 1;
     int *h_buf = nullptr;               // pinned readback: sweeps (2 nruns), status (nruns), Q fields
 
-    size_t smem1 = 0, smem2 = 0;
     int bps_max = 1;                    // resident sweep blocks per SM (launch grid = SMs x bps_max)
     int item_markers = 65536, bps = 1;  // schedule (the autotuner's choice)
     int fin_grid = 1;
@@ -111,86 +110,37 @@ static void build_tables(pic_ensemble *e)
 {
     for (int r = 0; r < e->nruns; ++r) {
         pic_handle *h = e->runs[r];
-        const PartPtrs P = handle_parts(h);
-
         e->desc[r] = handle_desc(h);
 
         Sweep1Args &a = e->a1[r];
-        a = Sweep1Args{};
-        a.M = h->M; a.H = h->H; a.Dlim = h->Dlim; a.K = h->K; a.fp32 = h->fp32; a.acc = h->acc; a.np = h->np;
-        a.dx = h->dx; a.dt = h->cfg.dt; a.w = h->cfg.weight;
-        a.P = P;
-        a.ebar = h->ebar; a.ga_y = h->ga_y; a.ga_z = h->ga_z; a.ay = h->ay; a.az = h->az;
-        a.ctrl = h->ctrl;
-        a.j = h->jb[0];
+        a = make_sweep1_args(h, h->cfg.dt);
         // with a predicted start the proposal is already in delta when the loop starts
         a.warm = (h->cfg.warm_start == PIC_WARM_EXPLICIT && !h->cfg.warm_field) ? 1 : 0;
-        a.a0 = h->a0;
         a.graph = 1;
-        a.jpair[0] = h->jb[0]; a.jpair[1] = h->jb[1];
-        a.img = h->img;
 
-        // the predicted start: the explicit proposal and its current into jb[1]
+        // the predicted start: the explicit proposal and its current into m1[1]
         Sweep1Args &ap = e->a1p[r];
         ap = a;
         ap.warm = h->cfg.warm_start == PIC_WARM_EXPLICIT ? 1 : 0;
         ap.graph = 0;
         ap.first = 1;
-        ap.j = h->jb[1];
+        ap.mom = h->m1[1];
 
         ConvArgs &c = e->c1[r];
-        c = ConvArgs{};
-        c.M = h->M; c.d_start = h->tapM1_start; c.ntap = h->tapM1_n; c.mode = CONV_SOLVE1; c.ncomp = 1;
-        c.taps = h->d_tapM1;
-        c.en[0] = h->ex; c.ek[0] = h->ek; c.aux[0] = h->ebar;
-        c.dt = h->cfg.dt; c.dx = h->dx; c.tol = h->cfg.tol; c.dtol = 1e-6;
-        c.erel = h->cfg.warm_field ? kFieldIncrementRelPredicted : kFieldIncrementRel;
-        c.max_iter = h->cfg.max_iter; c.fp32 = h->fp32; c.subsystem = 1; c.ctrl = h->ctrl;
-        c.graph = 1;
-        c.pair[0][0] = h->jb[0]; c.pair[0][1] = h->jb[1];
-        c.cond_handle = 0;      // the ensemble ends the loop, not the run
-        c.img = h->img;
+        c = make_conv1_args(h, h->cfg.dt);
+        c.graph = 1;            // the ensemble ends the loop, not the run (cond_handle = 0)
 
         // e^(0) = e^n - M1^{-1} j^(0) from the predicted start's current
         ConvArgs &cs = e->c1p[r];
         cs = c;
         cs.mode = CONV_START1;
         cs.graph = 0;
-        cs.in[0] = h->jb[1];
+        cs.mom[0] = h->m1[1];
 
-        Sweep2Args &b = e->a2[r];
-        b = Sweep2Args{};
-        b.status = &h->ctrl->status;
-        b.M = h->M; b.H = h->H; b.K = h->K; b.fp32 = h->fp32; b.acc = h->acc; b.np = h->np; b.w = h->cfg.weight;
-        b.P = P;
-        b.an_y = h->ay; b.an_z = h->az; b.ak_y = h->aky; b.ak_z = h->akz;
-        b.s_y = h->sy[0]; b.s_z = h->sz[0];
-        b.graph = 1; b.ctrl = h->ctrl;
-        b.sypair[0] = h->sy[0]; b.sypair[1] = h->sy[1];
-        b.szpair[0] = h->sz[0]; b.szpair[1] = h->sz[1];
-        b.img = h->img;
-
-        ConvArgs &g = e->c2[r];
-        g = ConvArgs{};
-        g.M = h->M; g.d_start = h->tapP_start; g.ntap = h->tapP_n; g.mode = CONV_SOLVE2; g.ncomp = 2;
-        g.taps = h->d_tapP;
-        g.en[0] = h->ey; g.en[1] = h->ez; g.ek[0] = h->eky; g.ek[1] = h->ekz;
-        g.aux[0] = h->aky; g.aux[1] = h->akz; g.an[0] = h->ay; g.an[1] = h->az;
-        g.r0[0] = h->r0y; g.r0[1] = h->r0z;
-        g.dt = h->cfg.dt; g.dx = h->dx; g.tol = h->cfg.tol; g.dtol = 0.0;
-        g.max_iter = h->cfg.max_iter; g.fp32 = h->fp32; g.subsystem = 2; g.ctrl = h->ctrl;
-        g.graph = 1;
-        g.pair[0][0] = h->sy[0]; g.pair[0][1] = h->sy[1];
-        g.pair[1][0] = h->sz[0]; g.pair[1][1] = h->sz[1];
-        g.cond_handle = 0;
-        g.img = h->img;
-
-        ConvArgs &p = e->cp[r];
-        p = ConvArgs{};
-        p.M = h->M; p.d_start = h->tapP_start; p.ntap = h->tapP_n; p.mode = CONV_PLAIN; p.ncomp = 2;
-        p.taps = h->d_tapP;
-        p.in[0] = h->by; p.in[1] = h->bz; p.out[0] = h->r0y; p.out[1] = h->r0z;
-        p.ctrl = h->ctrl;
+        e->a2[r] = make_sweep2_args(h);
+        e->a2[r].graph = 1;
+        e->c2[r] = make_conv2_args(h);
+        e->c2[r].graph = 1;
 
         e->er[r].np = h->np;
         e->er[r].ctrl = h->ctrl;
@@ -205,7 +155,6 @@ static int upload_tables(pic_ensemble *e)
     ECK(cudaMemcpyAsync(e->d_a2, e->a2.data(), n * sizeof(Sweep2Args), cudaMemcpyHostToDevice, e->stream));
     ECK(cudaMemcpyAsync(e->d_c1, e->c1.data(), n * sizeof(ConvArgs), cudaMemcpyHostToDevice, e->stream));
     ECK(cudaMemcpyAsync(e->d_c2, e->c2.data(), n * sizeof(ConvArgs), cudaMemcpyHostToDevice, e->stream));
-    ECK(cudaMemcpyAsync(e->d_cp, e->cp.data(), n * sizeof(ConvArgs), cudaMemcpyHostToDevice, e->stream));
     ECK(cudaMemcpyAsync(e->d_a1p, e->a1p.data(), n * sizeof(Sweep1Args), cudaMemcpyHostToDevice, e->stream));
     ECK(cudaMemcpyAsync(e->d_c1p, e->c1p.data(), n * sizeof(ConvArgs), cudaMemcpyHostToDevice, e->stream));
     ECK(cudaMemcpyAsync(e->d_er, e->er.data(), n * sizeof(EnsRun), cudaMemcpyHostToDevice, e->stream));
@@ -228,12 +177,12 @@ static int loop_body(pic_ensemble *e, int which, cudaStream_t s, unsigned long l
     const int grid = e->num_sms * e->bps_max;
     ELAUNCH(launch_ens_plan(e->d_q, e->d_er, e->nruns, cond, s), "ensemble plan");
     if (which == 1) {
-        ELAUNCH(launch_sweep1_ens(e->K, e->fp32, e->d_a1, e->nruns, e->d_q, grid, e->smem1, s), "ensemble sweep I");
-        ELAUNCH(launch_conv_ens(e->d_c1, e->nruns, e->Mmax, 1, e->ntap1, e->d_q, e->d_sweeps, cond, s),
+        ELAUNCH(launch_sweep1_ens(e->K, e->fp32, e->d_a1, e->nruns, e->d_q, grid, s), "ensemble sweep I");
+        ELAUNCH(launch_conv_ens(e->d_c1, e->nruns, e->Mmax, e->K, 1, e->ntap1, e->d_q, e->d_sweeps, cond, s),
                 "ensemble solve I");
     } else {
-        ELAUNCH(launch_sweep2_ens(e->K, e->fp32, e->d_a2, e->nruns, e->d_q, grid, e->smem2, s), "ensemble sweep II");
-        ELAUNCH(launch_conv_ens(e->d_c2, e->nruns, e->Mmax, 2, e->ntap2, e->d_q, e->d_sweeps, cond, s),
+        ELAUNCH(launch_sweep2_ens(e->K, e->fp32, e->d_a2, e->nruns, e->d_q, grid, s), "ensemble sweep II");
+        ELAUNCH(launch_conv_ens(e->d_c2, e->nruns, e->Mmax, e->K, 2, e->ntap2, e->d_q, e->d_sweeps, cond, s),
                 "ensemble solve II");
     }
     return PIC_OK;
@@ -247,9 +196,9 @@ static int seg_prep1(pic_ensemble *e, cudaStream_t s)
         // and their currents (work queue), e^(0) per run
         const int grid = e->num_sms * e->bps_max;
         ELAUNCH(launch_ens_plan(e->d_q, e->d_er, e->nruns, 0ull, s), "ensemble plan");
-        ELAUNCH(launch_predeposit_ens(e->K, e->fp32, e->d_a1p, e->nruns, e->d_q, grid, e->smem1, s),
+        ELAUNCH(launch_predeposit_ens(e->K, e->fp32, e->d_a1p, e->nruns, e->d_q, grid, s),
                 "ensemble predicted start");
-        ELAUNCH(launch_conv_ens(e->d_c1p, e->nruns, e->Mmax, 1, e->ntap1, e->d_q, e->d_sweeps, 0ull, s),
+        ELAUNCH(launch_conv_ens(e->d_c1p, e->nruns, e->Mmax, e->K, 1, e->ntap1, e->d_q, e->d_sweeps, 0ull, s),
                 "ensemble start field");
     }
     return PIC_OK;
@@ -260,8 +209,6 @@ static int seg_mid(pic_ensemble *e, cudaStream_t s)
     ELAUNCH(launch_finalize1_ens(e->fp32, e->d_desc, e->nruns, e->fin_grid, s), "ensemble finalize I");
     ELAUNCH(launch_commit_ens(e->d_desc, e->nruns, e->Mmax, 1, s), "ensemble commit I");
     ELAUNCH(launch_prep2_ens(e->d_desc, e->nruns, e->Mmax, s), "ensemble prep II");
-    ELAUNCH(launch_conv_ens(e->d_cp, e->nruns, e->Mmax, 2, e->ntap2, e->d_q, e->d_sweeps, 0ull, s),
-            "ensemble P solve");
     return PIC_OK;
 }
 
@@ -272,7 +219,7 @@ static int seg_end(pic_ensemble *e, cudaStream_t s)
 }
 
 // kernels launched per step outside the loops, and per loop sweep
-static constexpr int kStepLaunches = 6, kLoopLaunches = 3, kStartLaunches = 3;
+static constexpr int kStepLaunches = 5, kLoopLaunches = 3, kStartLaunches = 3;
 
 // Build the step graph: linear segments as child graphs, loops as WHILE nodes
 // whose bodies are captured on the private stream.
@@ -357,7 +304,7 @@ static void ens_release(pic_ensemble *e)
     if (e->exec) cudaGraphExecDestroy(e->exec);
     if (e->graph) cudaGraphDestroy(e->graph);
     auto f = [](void *p) { if (p) cudaFree(p); };
-    f(e->d_desc); f(e->d_a1); f(e->d_a2); f(e->d_c1); f(e->d_c2); f(e->d_cp); f(e->d_er); f(e->d_q);
+    f(e->d_desc); f(e->d_a1); f(e->d_a2); f(e->d_c1); f(e->d_c2); f(e->d_er); f(e->d_q);
     f(e->d_a1p); f(e->d_c1p); f(e->d_sorts);
     f(e->d_sweeps); f(e->d_status);
     if (e->h_buf) cudaFreeHost(e->h_buf);
@@ -422,14 +369,12 @@ extern "C" int pic_ensemble_create(const pic_config *cfgs, const pic_arrays *ins
         e->Mmax = std::max(e->Mmax, h->M);
         e->ntap1 = std::max(e->ntap1, h->tapM1_n);
         e->ntap2 = std::max(e->ntap2, h->tapP_n);
-        e->smem1 = std::max(e->smem1, h->smem1);
-        e->smem2 = std::max(e->smem2, h->smem2);
         npmax = std::max(npmax, h->np);
     }
     e->fin_grid = (int)std::min<long long>(std::max<long long>((npmax + 255) / 256, 1), 64);
     {
-        const int b1 = sweep_blocks_per_sm(e->K, e->fp32, e->fp32 ? ACC_COMP : ACC_NATIVE, 1, kSweepThreads, e->smem1);
-        const int b2 = sweep_blocks_per_sm(e->K, e->fp32, e->fp32 ? ACC_COMP : ACC_NATIVE, 2, kSweepThreads, e->smem2);
+        const int b1 = sweep_blocks_per_sm(e->K, e->fp32, e->fp32 ? ACC_COMP : ACC_NATIVE, 1);
+        const int b2 = sweep_blocks_per_sm(e->K, e->fp32, e->fp32 ? ACC_COMP : ACC_NATIVE, 2);
         e->bps_max = std::max(1, std::min(b1, b2));
         e->bps = e->bps_max;
     }
@@ -437,10 +382,10 @@ extern "C" int pic_ensemble_create(const pic_config *cfgs, const pic_arrays *ins
     e->sort_grid = (int)std::min<long long>(std::max<long long>((npmax + 1023) / 1024, 1), 4LL * e->num_sms);
     const size_t n = (size_t)nruns;
     e->desc.resize(n); e->a1.resize(n); e->a2.resize(n); e->c1.resize(n); e->c2.resize(n);
-    e->cp.resize(n); e->er.resize(n); e->a1p.resize(n); e->c1p.resize(n);
+    e->er.resize(n); e->a1p.resize(n); e->c1p.resize(n);
     int rc;
     if ((rc = ealloc(e, &e->d_desc, n)) || (rc = ealloc(e, &e->d_a1, n)) || (rc = ealloc(e, &e->d_a2, n)) ||
-        (rc = ealloc(e, &e->d_c1, n)) || (rc = ealloc(e, &e->d_c2, n)) || (rc = ealloc(e, &e->d_cp, n)) ||
+        (rc = ealloc(e, &e->d_c1, n)) || (rc = ealloc(e, &e->d_c2, n)) ||
         (rc = ealloc(e, &e->d_er, n)) || (rc = ealloc(e, &e->d_q, 1)) || (rc = ealloc(e, &e->d_sweeps, 2 * n)) ||
         (rc = ealloc(e, &e->d_status, n)) || (rc = ealloc(e, &e->d_a1p, n)) || (rc = ealloc(e, &e->d_c1p, n)) ||
         (rc = ealloc(e, &e->d_sorts, n)))
@@ -450,7 +395,7 @@ extern "C" int pic_ensemble_create(const pic_config *cfgs, const pic_arrays *ins
     if (cudaMemsetAsync(e->d_q, 0, sizeof(EnsQueue), e->stream) != cudaSuccess ||
         cudaMemsetAsync(e->d_sweeps, 0, 2 * n * sizeof(int), e->stream) != cudaSuccess)
         return bail(PIC_ERR_CUDA);
-    if (conv_ens_optin(e->Mmax, std::max(e->ntap1, e->ntap2)))
+    if (conv_ens_optin(std::max(e->ntap1, e->ntap2)))
         return bail(efail(e, PIC_ERR_CUDA, "solve kernel shared-memory opt-in failed"));
     build_tables(e);
     if ((rc = upload_tables(e)) || (rc = upload_schedule(e))) return bail(rc);

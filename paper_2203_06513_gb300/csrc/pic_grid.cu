@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "pic_internal.h"
+#include "pic_poly.cuh"
 
 namespace pic {
 
@@ -33,12 +34,6 @@ static double cardinal_tp(int n, double s)
         binom = binom * (n + 1 - i) / (i + 1);
     }
     return acc / fact;
-}
-
-int mean_scale(int d)
-{
-    static const int S[] = {1, 1, 6, 6, 120};
-    return (d >= 0 && d <= 4) ? S[d] : 0;
 }
 
 void mass_band(int d, double dx, double *band)
@@ -221,131 +216,217 @@ __device__ void decide(const ConvArgs &A)
         cudaGraphSetConditional((cudaGraphConditionalHandle)A.cond_handle, stop ? 0u : 1u);
 }
 
-// float images of sweep I: a / K! rounded, their differences, ebar dx / S1 rounded
-__device__ __forceinline__ void image1_at(int i, int M, const double *ay, const double *az, double ebar,
-                                          const StageImages &img)
+// Spline pieces of every degree (pic_poly.cuh).  Grid kernels take the degree at run time.
+__constant__ SplineTab c_spline = make_spline_tab();
+
+// Stores coefficient m of row `row` (pad numbers a row) in the form's type.
+__device__ __forceinline__ void put_coef(void *tab, int fp32, size_t row, int pad, int m, double v)
 {
-    const int im = (i == 0) ? M - 1 : i - 1;
-    const float y = (float)(ay[i] * img.inv_fact), ym = (float)(ay[im] * img.inv_fact);
-    const float z = (float)(az[i] * img.inv_fact), zm = (float)(az[im] * img.inv_fact);
-    img.a[i] = make_float2(y, z);
-    img.f[i] = make_float4((float)(ebar * img.escale), y - ym, z - zm, 0.f);
+    if (fp32) static_cast<float *>(tab)[row * pad + m] = (float)v;
+    else static_cast<double *>(tab)[row * pad + m] = v;
 }
 
-// float images of sweep II for one component c: a^(k) / K! rounded and the residue
-// of the sum a^n / K! + a^(k) / K! after both roundings
-__device__ __forceinline__ void image2_at(int i, int c, double an, double ak, const StageImages &img)
+// Coefficient m of the degree-D polynomial in the cell whose node r steps down has value at(r).
+template <class At>
+__device__ __forceinline__ double cell_coef(int D, int m, At &&at)
 {
-    const double n = an * img.inv_fact, k = ak * img.inv_fact;
-    const float hn = (float)n, hk = (float)k;
-    const float lo = (float)((n - (double)hn) + (k - (double)hk));
-    float *pk = reinterpret_cast<float *>(&img.ak[i]), *pl = reinterpret_cast<float *>(&img.lo[i]);
-    pk[c] = hk;
-    pl[c] = lo;
+    double s = 0.0;
+    for (int r = 0; r <= D; ++r) s = fma(c_spline.b[D][r][m], at(r), s);
+    return s;
 }
 
-// y_i = sum_n taps[n] in[(i - (d_start + n)) mod M], one output per thread,
-// input and taps staged in shared memory (input twice, so no index wraps).
-// Block bx of component comp; returns true in the one block that finished the
-// run's solve last (after the convergence decision, in the solve modes).
-__device__ bool conv_block(const ConvArgs &A, int bx, int comp, double *s_conv, double *s_red)
+// Value of a deposit at node j from the moments of degree D (path: coefficient m over m + 1).
+__device__ __forceinline__ double node_value(int M, int D, bool path, const double *mom, int j)
 {
-    const int M = A.M;
-    double *s_in = s_conv;              // 2M
-    double *s_tap = s_conv + 2 * M;     // ntap
-    const double *in = A.in[comp];
+    const int NV = D + 1;
+    double s[kMaxDegree + 1] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    int c = j;
+    for (int r = 0; r < NV; ++r) {
+        const double *row = mom + (size_t)c * NV;
+#pragma unroll
+        for (int m = 0; m <= kMaxDegree; ++m)
+            if (m < NV) s[m] = fma(c_spline.b[D][r][m], row[m], s[m]);
+        c = c + 1 == M ? 0 : c + 1;
+    }
+    double v = 0.0;
+#pragma unroll
+    for (int m = 0; m <= kMaxDegree; ++m)
+        if (m < NV) v += path ? s[m] * (1.0 / (m + 1)) : s[m];
+    return v;
+}
+
+// The residue of a^n + a^(k) after both coefficients were rounded to float.
+__device__ __forceinline__ float sum_residue(double n, double k)
+{
+    return (float)((n - (double)(float)n) + (k - (double)(float)k));
+}
+
+// y_i = sum_n taps[n] in[(i - (d_start + n)) mod M] for the kConvOut nodes
+// i0 - K .. i0 - K + kConvOut - 1 of block bx, i0 = bx (kConvOut - K): the block owns the
+// last kConvOut - K of them and recomputes the K below, which the polynomials of
+// its cells need.  One warp computes a quarter of the taps for all nodes (lane =
+// node): with a few dozen nodes a block the solve spreads over the SMs instead of
+// waiting on one SM's FP64 pipe, and only the block's part of the deposit is staged
+// (M = 2048, cubic: 35 us with one thread a node and the whole row staged twice by every
+// block, 18 us so; both with cold caches).
+// Returns true in the one block that finished the run's solve last (after the
+// convergence decision, in the solve modes).
+constexpr int kConvOut = 32, kConvThreads = 128;
+
+inline size_t conv_smem(int ntap)
+{
+    const int nq = kConvOut + ntap - 1;
+    return ((size_t)nq + ntap + 4 * kConvOut + 2 * kConvOut) * sizeof(double);
+}
+inline int conv_blocks(int M, int K) { return (M + kConvOut - K - 1) / (kConvOut - K); }
+
+__device__ bool conv_block(const ConvArgs &A, int bx, int comp, double *sm)
+{
+    const int M = A.M, K = A.K, TB = kConvOut - K, i0 = bx * TB;
+    const int D = A.subsystem == 1 ? K - 1 : K, NV = D + 1;
+    const int nq = kConvOut + A.ntap - 1;
+    double *s_in = sm, *s_tap = s_in + nq, *s_part = s_tap + A.ntap;
+    double *s_val = s_part + 4 * kConvOut, *s_an = s_val + kConvOut;
+    const double *mom = A.mom[comp];
     double *zero = A.zero[comp];
     if (A.graph && A.mode != CONV_PLAIN) {   // replayed by a graph: buffers by sweep parity
         const int it = *reinterpret_cast<volatile const int *>(&A.ctrl->iter);
-        in = A.pair[comp][it & 1];
+        mom = A.pair[comp][it & 1];
         zero = A.pair[comp][(it + 1) & 1];
     }
-    const int off = M / 2;              // s_in[q] = in[(q - off) mod M], q in [0, 2M)
-    for (int q = threadIdx.x; q < 2 * M; q += blockDim.x) {
-        int g = q - off;
-        g = g < 0 ? g + M : (g >= M ? g - M : g);
-        s_in[q] = in[g];
+    // s_in[q]: node (g0 + q) mod M
+    const int g0 = wrap_cell(i0 - K - (A.d_start + A.ntap - 1), M);
+    for (int n = threadIdx.x; n < A.ntap; n += kConvThreads) s_tap[n] = A.taps[n];
+    if (mom) {
+        for (int q = threadIdx.x; q < nq; q += kConvThreads) {
+            const int g = (g0 + q) % M;
+            double s = A.scale * node_value(M, D, A.subsystem == 1, mom, g);
+            if (A.mode == CONV_SOLVE2) s = fma(A.dt, s, A.b[comp][g]);
+            s_in[q] = s;
+        }
+    } else {
+        for (int q = threadIdx.x; q < nq; q += kConvThreads) {
+            const int g = (g0 + q) % M;
+            const double s = A.in[comp][g];
+            s_in[q] = A.mode == CONV_SOLVE2 ? fma(A.dt, s, A.b[comp][g]) : s;
+        }
     }
-    for (int n = threadIdx.x; n < A.ntap; n += blockDim.x) s_tap[n] = A.taps[n];
     __syncthreads();
-    const int i = bx * blockDim.x + threadIdx.x;
-    double diff = 0.0, mag = 0.0;
-    if (i < M) {
-        // offsets d = d_start + n lie in [-(M-1)/2, M/2], so i - d + off is in [0, 2M)
-        const double *base = s_in + (i - A.d_start + off);
-        double acc0 = 0.0, acc1 = 0.0;
-        int n = 0;
-        for (; n + 1 < A.ntap; n += 2) {
-            acc0 = fma(s_tap[n], base[-n], acc0);
-            acc1 = fma(s_tap[n + 1], base[-n - 1], acc1);
+    const int o = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    {
+        const int per = (A.ntap + 3) >> 2, n0 = wid * per, n1 = min(A.ntap, n0 + per);
+        const double *base = s_in + o + A.ntap - 1;
+        double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+        int n = n0;
+        for (; n + 3 < n1; n += 4) {
+            a0 = fma(s_tap[n], base[-n], a0);
+            a1 = fma(s_tap[n + 1], base[-n - 1], a1);
+            a2 = fma(s_tap[n + 2], base[-n - 2], a2);
+            a3 = fma(s_tap[n + 3], base[-n - 3], a3);
         }
-        if (n < A.ntap) acc0 = fma(s_tap[n], base[-n], acc0);
-        const double y = acc0 + acc1;
+        for (; n < n1; ++n) a0 = fma(s_tap[n], base[-n], a0);
+        s_part[wid * kConvOut + o] = (a0 + a1) + (a2 + a3);
+    }
+    __syncthreads();
+    double diff = 0.0, mag = 0.0;
+    if (wid == 0) {
+        const double y = (s_part[o] + s_part[kConvOut + o]) + (s_part[2 * kConvOut + o] + s_part[3 * kConvOut + o]);
+        const int i = i0 - K + o;
+        const bool own = o >= K && i < M;
+        const int iw = wrap_cell(i, M);
         if (A.mode == CONV_PLAIN) {
-            A.out[comp][i] = y;
-        } else if (A.mode == CONV_START1) {
-            const double en = A.en[0][i];
-            const double e0 = en - y;                    // e^(0) = e^n - M1^{-1} j^(0)
-            A.ek[0][i] = e0;
-            A.aux[0][i] = 0.5 * (en + e0);
-            if (A.img.f) reinterpret_cast<float *>(A.img.f)[4 * i] = (float)(0.5 * (en + e0) * A.img.escale);
-        } else if (A.mode == CONV_SOLVE1) {
-            const double en = A.en[0][i];
+            if (own) A.out[comp][i] = y;
+        } else if (A.mode != CONV_SOLVE2) {              // START1, SOLVE1
+            const double en = A.en[0][iw];
             const double enew = en - y;                  // e^(k+1) = e^n - M1^{-1} j
-            diff = fabs(enew - A.ek[0][i]);
-            mag = fabs(enew);
-            A.ek[0][i] = enew;
-            A.aux[0][i] = 0.5 * (en + enew);             // ebar for the next sweep
-            if (A.img.f) reinterpret_cast<float *>(A.img.f)[4 * i] = (float)(0.5 * (en + enew) * A.img.escale);
-            zero[i] = 0.0;
-        } else {                                         // CONV_SOLVE2
-            const double en = A.en[comp][i];
-            const double enew = A.r0[comp][i] + A.dt * y;   // P e^(k+1) = b + dt s
-            diff = fabs(enew - A.ek[comp][i]);
-            mag = fabs(enew);
-            A.ek[comp][i] = enew;
-            const double ak = A.an[comp][i] - 0.5 * A.dt * (en + enew);   // a^(k+1)
-            A.aux[comp][i] = ak;
-            if (A.img.ak) image2_at(i, comp, A.an[comp][i], ak, A.img);
-            zero[i] = 0.0;
+            const double eb = 0.5 * (en + enew);         // ebar for the next sweep
+            s_val[o] = eb;
+            if (own) {
+                if (A.mode == CONV_SOLVE1) {
+                    diff = fabs(enew - A.ek[0][i]);
+                    mag = fabs(enew);
+                }
+                A.ek[0][i] = enew;
+                A.aux[0][i] = eb;
+            }
+        } else {                                         // P e^(k+1) = b + dt s
+            const double en = A.en[comp][iw], an = A.an[comp][iw];
+            const double enew = y;
+            const double ak = an - 0.5 * A.dt * (en + enew);   // a^(k+1)
+            s_val[o] = ak;
+            s_an[o] = an;
+            if (own) {
+                diff = fabs(enew - A.ek[comp][i]);
+                mag = fabs(enew);
+                A.ek[comp][i] = enew;
+                A.aux[comp][i] = ak;
+            }
         }
     }
-    if (A.mode == CONV_PLAIN || A.mode == CONV_START1) return false;
-    block_max_to(&A.ctrl->emax_bits, diff, s_red);
-    block_max_to(&A.ctrl->emag_bits, mag, s_red);
+    if (A.mode == CONV_PLAIN) return false;
+    __syncthreads();
+    // the cells' polynomials of the new field, and the next sweep's moments cleared
+    const int ncell = min(TB, M - i0);
+    if (A.mode != CONV_SOLVE2) {
+        const int pad = coef_pad(A.fp32, K);
+        for (int q = threadIdx.x; q < ncell * K; q += kConvThreads) {
+            const int j = q / K, m = q % K;
+            const double v = cell_coef(K - 1, m, [&](int r) { return s_val[K + j - r]; });
+            put_coef(A.T.E, A.fp32, (size_t)(i0 + j), pad, m, v * A.dx / (double)(m + 1));
+        }
+    } else {
+        const int pad = coef_pad(A.fp32, K + 1);
+        for (int q = threadIdx.x; q < ncell * (K + 1); q += kConvThreads) {
+            const int j = q / (K + 1), m = q % (K + 1);
+            const size_t row = 2 * (size_t)(i0 + j) + comp;
+            const double k = cell_coef(K, m, [&](int r) { return s_val[K + j - r]; });
+            put_coef(A.T.Kt, A.fp32, row, pad, m, k);
+            if (A.fp32) {
+                const double n = cell_coef(K, m, [&](int r) { return s_an[K + j - r]; });
+                A.T.L[row * pad + m] = sum_residue(n, k);
+            }
+        }
+    }
+    if (A.mode == CONV_START1) return false;
+    if (zero)
+        for (int q = threadIdx.x; q < ncell * NV; q += kConvThreads) zero[(size_t)i0 * NV + q] = 0.0;
     __shared__ int s_last;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const unsigned int nblk = (unsigned)(((M + blockDim.x - 1) / blockDim.x) * A.ncomp);
-        const unsigned int t = atomicAdd(&A.ctrl->ticket, 1u);
-        s_last = (t == nblk - 1) ? 1 : 0;
-        if (s_last) decide(A);
+    if (wid == 0) {
+        diff = warp_max(diff);
+        mag = warp_max(mag);
+        if (o == 0) {
+            atomic_max_nonneg(&A.ctrl->emax_bits, diff);
+            atomic_max_nonneg(&A.ctrl->emag_bits, mag);
+            __threadfence();
+            const unsigned int nblk = (unsigned)(((M + TB - 1) / TB) * A.ncomp);
+            const unsigned int t = atomicAdd(&A.ctrl->ticket, 1u);
+            s_last = (t == nblk - 1) ? 1 : 0;
+            if (s_last) decide(A);
+        }
     }
     __syncthreads();
     return s_last != 0;
 }
 
-__global__ void __launch_bounds__(64) k_conv(ConvArgs A)
+__global__ void __launch_bounds__(kConvThreads) k_conv(ConvArgs A)
 {
     extern __shared__ __align__(16) double s_conv[];
-    __shared__ double s_red[32];
-    conv_block(A, blockIdx.x, blockIdx.y, s_conv, s_red);
+    conv_block(A, blockIdx.x, blockIdx.y, s_conv);
 }
 
 // Batched solves of an ensemble: block (bx, run, comp).  Runs that are not in
 // the current sweep (converged, or stopped by an error) are skipped.  After a
 // run's decision, the last run to decide in this sweep records whether any run
 // goes on, and sets the loop's conditional handle (graph mode).
-__global__ void __launch_bounds__(64) k_conv_ens(const ConvArgs *runs, EnsQueue *Q, int *sweeps,
-                                                 unsigned long long cond)
+__global__ void __launch_bounds__(kConvThreads) k_conv_ens(const ConvArgs *runs, EnsQueue *Q, int *sweeps,
+                                                           unsigned long long cond)
 {
     extern __shared__ __align__(16) double s_conv[];
-    __shared__ double s_red[32];
     const int r = blockIdx.y, comp = blockIdx.z;
     const ConvArgs &A = runs[r];
     if (A.mode != CONV_PLAIN && !Q->active[r]) return;
-    if (comp >= A.ncomp || (int)(blockIdx.x * blockDim.x) >= A.M) return;
-    const bool last = conv_block(A, blockIdx.x, comp, s_conv, s_red);
+    if (comp >= A.ncomp || (int)blockIdx.x * (kConvOut - A.K) >= A.M) return;
+    const bool last = conv_block(A, blockIdx.x, comp, s_conv);
     if (!last || threadIdx.x != 0) return;
     atomicAdd(&sweeps[2 * r + A.subsystem - 1], 1);
     if (!A.ctrl->converged) atomicAdd(&Q->n_continue, 1);
@@ -360,8 +441,12 @@ __global__ void __launch_bounds__(64) k_conv_ens(const ConvArgs *runs, EnsQueue 
     }
 }
 
+// Raises a solve kernel's dynamic shared-memory limit (never lowers it).  Inverse rows
+// that decay slowly (large dt/dx in subsystem II) may keep as many taps as nodes.
 static int conv_optin(const void *fn, size_t smem, size_t &opted)
 {
+    static std::mutex mu;
+    std::lock_guard<std::mutex> lock(mu);
     if (smem > 48 * 1024 && smem > opted) {
         if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
             return 1;
@@ -373,30 +458,27 @@ static int conv_optin(const void *fn, size_t smem, size_t &opted)
 static size_t g_conv_ens_opted = 0;
 
 // raise the shared-memory limit of k_conv_ens before any capture of it
-int conv_ens_optin(int Mmax, int ntap_max)
+int conv_ens_optin(int ntap_max)
 {
-    const size_t smem = (2 * (size_t)Mmax + (size_t)ntap_max) * sizeof(double);
-    return conv_optin((const void *)k_conv_ens, smem, g_conv_ens_opted);
+    return conv_optin((const void *)k_conv_ens, conv_smem(ntap_max), g_conv_ens_opted);
 }
 
-int launch_conv_ens(const ConvArgs *runs, int nruns, int Mmax, int ncomp, int ntap_max, EnsQueue *Q,
+int launch_conv_ens(const ConvArgs *runs, int nruns, int Mmax, int K, int ncomp, int ntap_max, EnsQueue *Q,
                     int *sweeps, unsigned long long cond, cudaStream_t s)
 {
-    const size_t smem = (2 * (size_t)Mmax + (size_t)ntap_max) * sizeof(double);
+    const size_t smem = conv_smem(ntap_max);
     if (smem > 48 * 1024 && smem > g_conv_ens_opted) return 1;   // conv_ens_optin first
-    dim3 grid((Mmax + 63) / 64, nruns, ncomp);
-    k_conv_ens<<<grid, 64, smem, s>>>(runs, Q, sweeps, cond);
+    dim3 grid(conv_blocks(Mmax, K), nruns, ncomp);
+    k_conv_ens<<<grid, kConvThreads, smem, s>>>(runs, Q, sweeps, cond);
     return 0;
 }
 
 int launch_conv(const ConvArgs &a, cudaStream_t s)
 {
-    const int threads = 64;
-    dim3 grid((a.M + threads - 1) / threads, a.ncomp);
-    const size_t smem = (2 * (size_t)a.M + (size_t)a.ntap) * sizeof(double);
+    const size_t smem = conv_smem(a.ntap);
     static size_t opted = 0;   // largest dynamic shared memory opted in so far
     if (conv_optin((const void *)k_conv, smem, opted)) return 1;
-    k_conv<<<grid, threads, smem, s>>>(a);
+    k_conv<<<dim3(conv_blocks(a.M, a.K), a.ncomp), kConvThreads, smem, s>>>(a);
     return 0;
 }
 
@@ -429,25 +511,36 @@ __device__ __forceinline__ double start_field(double e, double *const d[kMaxStar
 }
 
 // ---------------------------------------------------------------------------
-// Subsystem I preparation: e^(0), ebar^(0) = (e^n + e^(0)) / 2, the gradients
-// (G a)_i = (a_i - a_{i-1}) / dx, cleared deposits, the float images, the
-// control block reset for the loop.
+// Subsystem I preparation: e^(0), ebar^(0) = (e^n + e^(0)) / 2, the cells' polynomials
+// of a^n and ebar^(0), cleared moments, the control block reset for the loop.
 // ---------------------------------------------------------------------------
+// both rows of the polynomials of (cy, cz) in cell i, and whether cz has a non-zero
+__device__ __forceinline__ void a_rows(int i, int M, int K, int fp32, const double *cy, const double *cz, void *tab)
+{
+    const int pad = coef_pad(fp32, K + 1);
+    for (int m = 0; m <= K; ++m) {
+        put_coef(tab, fp32, 2 * (size_t)i, pad, m, cell_coef(K, m, [&](int r) { return cy[wrap_cell(i - r, M)]; }));
+        put_coef(tab, fp32, 2 * (size_t)i + 1, pad, m, cell_coef(K, m, [&](int r) { return cz[wrap_cell(i - r, M)]; }));
+    }
+}
+
 __device__ __forceinline__ void prep1_at(int i, const RunDesc &R)
 {
-    const int M = R.M;
+    const int M = R.M, K = R.K;
     const int q = min(R.ctrl->hist1, R.fh.order1);    // hist1: written only by the commit kernel
     if (i < M) {
-        const double e0 = start_field(R.ex[i], R.fh.x, i, q);
-        const double eb = 0.5 * (R.ex[i] + e0);
-        if (R.img.a) image1_at(i, M, R.ay, R.az, eb, R.img);
-        const int im = (i == 0) ? M - 1 : i - 1;
-        R.ga_y[i] = (R.ay[i] - R.ay[im]) / R.dx;
-        R.ga_z[i] = (R.az[i] - R.az[im]) / R.dx;
-        R.ek[i] = e0;
-        R.ebar[i] = eb;
-        R.j0[i] = 0.0;
-        R.j1[i] = 0.0;
+        auto ebar = [&](int g) { return 0.5 * (R.ex[g] + start_field(R.ex[g], R.fh.x, g, q)); };
+        R.ek[i] = start_field(R.ex[i], R.fh.x, i, q);
+        R.ebar[i] = ebar(i);
+        a_rows(i, M, K, R.fp32, R.ay, R.az, R.T.A);
+        const int pad = coef_pad(R.fp32, K);
+        for (int m = 0; m < K; ++m) {
+            const double v = cell_coef(K - 1, m, [&](int r) { return ebar(wrap_cell(i - r, M)); });
+            put_coef(R.T.E, R.fp32, (size_t)i, pad, m, v * R.dx / (double)(m + 1));
+            R.m1[0][(size_t)i * K + m] = 0.0;
+            R.m1[1][(size_t)i * K + m] = 0.0;
+        }
+        if (R.az[i] != 0.0) R.ctrl->zany = 1;
     }
     if (i == 0) ctrl_loop_reset(R.ctrl);
 }
@@ -461,20 +554,20 @@ __global__ void k_prep1_ens(const RunDesc *runs)
 
 int launch_prep1_ens(const RunDesc *R, int nruns, int Mmax, cudaStream_t s)
 {
-    k_prep1_ens<<<dim3((Mmax + 255) / 256, nruns), 256, 0, s>>>(R);
+    k_prep1_ens<<<dim3((Mmax + 63) / 64, nruns), 64, 0, s>>>(R);
     return 0;
 }
 
 int launch_prep1(const RunDesc &R, cudaStream_t s)
 {
-    k_prep1<<<(R.M + 255) / 256, 256, 0, s>>>(R);
+    k_prep1<<<(R.M + 63) / 64, 64, 0, s>>>(R);
     return 0;
 }
 
 // ---------------------------------------------------------------------------
 // Subsystem II preparation: b = (M0 - dt^2/4 K) e^n + dt K a^n (banded
 // circulant products), e^(0), a^(0) = a^n - dt/2 (e^n + e^(0)), cleared
-// deposits, the float images, the control block reset for the loop.
+// moments, the cells' polynomials, the control block reset for the loop.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void prep2_at(int i, const RunDesc &R)
 {
@@ -483,13 +576,32 @@ __device__ __forceinline__ void prep2_at(int i, const RunDesc &R)
     const int q = min(R.ctrl->hist2, R.fh.order2);    // hist2: written only by the commit kernel
     if (i < M) {
         const double *ey = R.ey, *ez = R.ez, *ay = R.ay, *az = R.az;
+        auto a0 = [&](const double *a, const double *e, double *const d[kMaxStartOrder], int g) {
+            return a[g] - 0.5 * dt * (e[g] + start_field(e[g], d, g, q));
+        };
         const double ey0 = start_field(ey[i], R.fh.y, i, q);
         const double ez0 = start_field(ez[i], R.fh.z, i, q);
-        const double ay0 = ay[i] - 0.5 * dt * (ey[i] + ey0), az0 = az[i] - 0.5 * dt * (ez[i] + ez0);
-        if (R.img.an) {
-            R.img.an[i] = make_float2((float)(ay[i] * R.img.inv_fact), (float)(az[i] * R.img.inv_fact));
-            image2_at(i, 0, ay[i], ay0, R.img);
-            image2_at(i, 1, az[i], az0, R.img);
+        const double ay0 = a0(ay, ey, R.fh.y, i), az0 = a0(az, ez, R.fh.z, i);
+        {
+            double kn[2][kMaxDegree + 1], kk[2][kMaxDegree + 1];     // nodes i, i - 1, .. i - K
+            for (int r = 0; r <= K; ++r) {
+                const int g = wrap_cell(i - r, M);
+                kn[0][r] = ay[g];
+                kn[1][r] = az[g];
+                kk[0][r] = a0(ay, ey, R.fh.y, g);
+                kk[1][r] = a0(az, ez, R.fh.z, g);
+            }
+            const int pad = coef_pad(R.fp32, K + 1);
+            for (int c = 0; c < 2; ++c) {
+                const size_t row = 2 * (size_t)i + c;
+                for (int m = 0; m <= K; ++m) {
+                    const double n = cell_coef(K, m, [&](int r) { return kn[c][r]; });
+                    const double k = cell_coef(K, m, [&](int r) { return kk[c][r]; });
+                    put_coef(R.T.A, R.fp32, row, pad, m, n);
+                    put_coef(R.T.Kt, R.fp32, row, pad, m, k);
+                    if (R.fp32) R.T.L[row * pad + m] = sum_residue(n, k);
+                }
+            }
         }
         double vy = R.rowPm[0] * ey[i] + dt * R.rowK[0] * ay[i];
         double vz = R.rowPm[0] * ez[i] + dt * R.rowK[0] * az[i];
@@ -504,7 +616,12 @@ __device__ __forceinline__ void prep2_at(int i, const RunDesc &R)
         R.ekz[i] = ez0;
         R.aky[i] = ay0;
         R.akz[i] = az0;
-        R.sy0[i] = 0.0; R.sz0[i] = 0.0; R.sy1[i] = 0.0; R.sz1[i] = 0.0;
+        for (int m = 0; m <= K; ++m)
+            for (int b = 0; b < 2; ++b) {
+                R.my[b][(size_t)i * (K + 1) + m] = 0.0;
+                R.mz[b][(size_t)i * (K + 1) + m] = 0.0;
+            }
+        if (az[i] != 0.0 || ez[i] != 0.0) R.ctrl->zany = 1;
     }
     if (i == 0) ctrl_loop_reset(R.ctrl);
 }
@@ -518,13 +635,13 @@ __global__ void k_prep2_ens(const RunDesc *runs)
 
 int launch_prep2_ens(const RunDesc *R, int nruns, int Mmax, cudaStream_t s)
 {
-    k_prep2_ens<<<dim3((Mmax + 255) / 256, nruns), 256, 0, s>>>(R);
+    k_prep2_ens<<<dim3((Mmax + 63) / 64, nruns), 64, 0, s>>>(R);
     return 0;
 }
 
 int launch_prep2(const RunDesc &R, cudaStream_t s)
 {
-    k_prep2<<<(R.M + 255) / 256, 256, 0, s>>>(R);
+    k_prep2<<<(R.M + 63) / 64, 64, 0, s>>>(R);
     return 0;
 }
 
@@ -647,6 +764,61 @@ int launch_ens_plan(EnsQueue *Q, const EnsRun *runs, int nruns, unsigned long lo
     return 0;
 }
 
+__global__ void k_moments_to_nodes(int M, int D, bool path, double scale, const double *mom, double *out)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= M) return;
+    out[j] = scale * node_value(M, D, path, mom, j);
+}
+
+int launch_moments_to_nodes(int M, int D, bool path, double scale, const double *mom, double *out, cudaStream_t s)
+{
+    k_moments_to_nodes<<<(M + 63) / 64, 64, 0, s>>>(M, D, path, scale, mom, out);
+    return 0;
+}
+
+__global__ void k_cell_coefs(int M, int D, bool path, const double *c, double *tab)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= M) return;
+    const int pad = coef_pad(0, D + 1);
+    for (int m = 0; m <= D; ++m) {
+        const double v = cell_coef(D, m, [&](int r) { return c[wrap_cell(i - r, M)]; });
+        tab[(size_t)i * pad + m] = path ? v / (double)(m + 1) : v;
+    }
+}
+
+int launch_cell_coefs(int M, int D, bool path, const double *c, double *tab, cudaStream_t s)
+{
+    k_cell_coefs<<<(M + 63) / 64, 64, 0, s>>>(M, D, path, c, tab);
+    return 0;
+}
+
+__global__ void k_tables2(int M, int K, int fp32, const double *an_y, const double *an_z, const double *ak_y,
+                          const double *ak_z, CoefTables T)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= M) return;
+    a_rows(i, M, K, fp32, an_y, an_z, T.A);
+    a_rows(i, M, K, fp32, ak_y, ak_z, T.Kt);
+    if (!fp32) return;
+    const int pad = coef_pad(fp32, K + 1);
+    for (int c = 0; c < 2; ++c) {
+        const double *n = c ? an_z : an_y, *k = c ? ak_z : ak_y;
+        for (int m = 0; m <= K; ++m)
+            T.L[(2 * (size_t)i + c) * pad + m] =
+                sum_residue(cell_coef(K, m, [&](int r) { return n[wrap_cell(i - r, M)]; }),
+                            cell_coef(K, m, [&](int r) { return k[wrap_cell(i - r, M)]; }));
+    }
+}
+
+int launch_tables2(int M, int K, int fp32, const double *an_y, const double *an_z, const double *ak_y,
+                   const double *ak_z, CoefTables T, cudaStream_t s)
+{
+    k_tables2<<<(M + 63) / 64, 64, 0, s>>>(M, K, fp32, an_y, an_z, ak_y, ak_z, T);
+    return 0;
+}
+
 // Discrete Poisson right side: with r = -rho + dx, d = M1 e_x solves
 // (d_j - d_{j+1}) / dx = r_j (Remark 2, Sec. 4.2): a running sum made mean-free.
 __global__ void k_poisson_rhs(int M, double dx, const double *rho, double *d)
@@ -743,6 +915,7 @@ __global__ void k_ctrl_reset(DevCtrl *c)
     c->ticket = 0u;
     c->hist1 = 0;
     c->hist2 = 0;
+    c->zany = 0;
     c->acc[0] = c->acc[1] = c->acc[2] = c->acc[3] = 0.0;
 }
 

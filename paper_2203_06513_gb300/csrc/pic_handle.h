@@ -11,13 +11,13 @@
 using pic::PartPtrs;
 using pic::DevCtrl;
 using pic::kSweepThreads;
-using pic::StageImages;
+using pic::CoefTables;
 
 struct pic_handle {
     pic_config cfg{};
     cudaStream_t stream = nullptr;
     int device = 0, num_sms = 0;
-    int M = 0, K = 0, H = 0, Dlim = 0, fp32 = 0;
+    int M = 0, K = 0, Dlim = 0, fp32 = 0;
     int acc = 0;                    // deposit window accumulator of the sweeps (pic::ACC_*)
     long long np = 0;
     double dx = 0.0;
@@ -31,7 +31,7 @@ struct pic_handle {
     char *Pblk[2] = {nullptr, nullptr};
     int cur = 0;
     void *delta = nullptr, *pnew = nullptr;
-    void *a0 = nullptr;             // subsystem-I start-point cache (4 reals a marker; FP64 form)
+    void *a0 = nullptr;             // start-point cache of a fixed-point loop (4 reals a marker; FP64 form)
     // spin (hbar != 0, FP64 form): components in caller order, and the spin deposits
     double *spx = nullptr, *spy = nullptr, *spz = nullptr;
     double *sdy = nullptr, *sdz = nullptr;
@@ -52,10 +52,14 @@ struct pic_handle {
 
     // grid state (double)
     double *ex = nullptr, *ey = nullptr, *ez = nullptr, *ay = nullptr, *az = nullptr;
-    double *ek = nullptr, *ebar = nullptr, *ga_y = nullptr, *ga_z = nullptr, *jb[2] = {nullptr, nullptr};
+    double *ek = nullptr, *ebar = nullptr, *jb[2] = {nullptr, nullptr};
     double *eky = nullptr, *ekz = nullptr, *aky = nullptr, *akz = nullptr;
-    double *by = nullptr, *bz = nullptr, *r0y = nullptr, *r0z = nullptr;
-    double *sy[2] = {nullptr, nullptr}, *sz[2] = {nullptr, nullptr};
+    double *by = nullptr, *bz = nullptr;
+    double *sy[2] = {nullptr, nullptr}, *sz[2] = {nullptr, nullptr};    // node deposits (split runs)
+    // moments of the sweeps' deposits (M x K and, per component, M x (K + 1)), by sweep
+    // parity, and of the deposit entry points; double cell polynomials of the gathers
+    double *m1[2] = {nullptr, nullptr}, *my[2] = {nullptr, nullptr}, *mz[2] = {nullptr, nullptr};
+    double *mdep = nullptr, *gtab = nullptr;
     double *rho = nullptr, *work = nullptr, *diag = nullptr;
     int32_t *counts = nullptr;
 
@@ -64,14 +68,13 @@ struct pic_handle {
     double *d_tapM1 = nullptr, *d_tapP = nullptr;
     int tapM1_start = 0, tapM1_n = 0, tapP_start = 0, tapP_n = 0;
 
-    StageImages img{};              // float staging images (FP32 form)
+    CoefTables T{};                 // cell polynomials of the sweeps' fields
     pic::FieldHist fh{};            // field changes of the last solves (starting fields)
     DevCtrl *ctrl = nullptr;
     int *h_flag = nullptr;          // pinned: converged flag readback
     DevCtrl *h_ctrl = nullptr;      // pinned: full control block readback
 
-    int sweep_grid = 0, sweep_block = kSweepThreads;
-    size_t smem1 = 0, smem2 = 0;
+    int grid1 = 0, grid2 = 0;       // blocks of the sweeps of subsystems I and II
 
     // timing: event pairs recorded around the timed launches, read back (and the
     // pairs reused) by pic_timing_read or when kMaxTimedLaunches are pending
@@ -98,4 +101,9 @@ int handle_sort(pic_handle *h);
 PartPtrs handle_parts(pic_handle *h);
 // the grid-side pointers of one handle (preparation and commit kernels)
 RunDesc handle_desc(pic_handle *h);
+// kernel arguments of the sweeps and solves of one handle (time step dt of subsystem I)
+Sweep1Args make_sweep1_args(pic_handle *h, double dt);
+Sweep2Args make_sweep2_args(pic_handle *h);
+ConvArgs make_conv1_args(pic_handle *h, double dt);
+ConvArgs make_conv2_args(pic_handle *h);
 }  // namespace pic

@@ -18,8 +18,18 @@ namespace pic {
 // cells.
 constexpr int kVelBinsBase = 16;
 inline int bins_per_cell(long long np, int M) { return np >= 8192LL * M ? 4 : 1; }
-// threads per block of the sweep kernels (two blocks per SM)
-constexpr int kSweepThreads = 512;
+// threads per block of the sweep kernels
+constexpr int kSweepThreads = 256;
+constexpr int kSweepWarps = kSweepThreads / 32;
+// cells a warp's deposit window holds: subsystem I (paths of sorted markers visit two
+// or three cells, one more after a step without a sort), subsystem II without and with
+// the z component (whose window doubles the registers)
+constexpr int kWin1 = 4, kWin2 = 3, kWin2z = 2;
+// resident blocks per SM the sweeps are compiled for (registers a thread: 65536 /
+// (256 x blocks)): the windows of the higher degrees need more registers
+template <typename R, int K> struct SweepOcc { static constexpr int v1 = 2, v2 = 2; };
+template <> struct SweepOcc<float, 2> { static constexpr int v1 = 3, v2 = 3; };
+template <> struct SweepOcc<float, 3> { static constexpr int v1 = 3, v2 = 3; };
 
 // ---------------------------------------------------------------- particles
 struct PartPtrs {
@@ -31,68 +41,65 @@ struct PartPtrs {
     int32_t *id;        // caller index of each stored marker
 };
 
-// Float staging images of the grid fields for the float-form sweeps, built on the
-// grid side (prep kernels once per substep, solve epilogues once per sweep) so that
-// the sweep blocks copy them instead of converting doubles per block range.  All
-// pointers null in the double form.
-struct StageImages {
-    float2 *a;          // sweep I: fl(a_y / K!), fl(a_z / K!)
-    float4 *f;          // sweep I: fl(ebar dx / S1), fl(a_j) - fl(a_{j-1}) for y and z, 0
-    float2 *an;         // sweep II: fl(a^n / K!)
-    float2 *ak;         // sweep II: fl(a^(k) / K!)
-    float2 *lo;         // sweep II: fl((a^n/K! - an) + (a^(k)/K! - ak))
-    double inv_fact;    // 1 / K!
-    double escale;      // dx / S1 (S1: scale of the degree-(K-1) path means)
+// Coefficient tables of the sweeps (pic_poly.cuh): per cell one row of the field's
+// polynomial in the cell, of the form's real type (float rows are rounded once from
+// double coefficients).  Rows are padded for 16-byte loads (coef_pad).
+struct CoefTables {
+    void *A;            // a^n: y row, z row (K + 1 coefficients each)
+    void *E;            // ebar dx, coefficient m divided by m + 1 (K coefficients)
+    void *Kt;           // a^(k): y row, z row
+    float *L;           // float form: residues of a^n + a^(k) after both roundings
 };
 
 struct Sweep1Args {
-    int M, H, Dlim, K, fp32;
+    int M, Dlim, K, fp32;
     int acc;            // deposit window accumulator (ACC_*)
     long long np;
-    double dx, dt, w;
+    double dx, dt;
     PartPtrs P;
-    const double *ebar, *ga_y, *ga_z, *ay, *az;
-    double *j;
+    CoefTables T;
+    double *mom;        // deposit: M x K moments h S_m (without w dx)
     DevCtrl *ctrl;
     int warm;           // 1: delta^(0) = explicit predictor, computed in-kernel (first sweep)
     int first;          // 1: the first sweep of the loop (writes the start-point cache)
     // graph mode (the launch is replayed by a CUDA graph): the deposit buffer is
-    // jpair[iter & 1], and the explicit warm start and the first-sweep role apply
+    // mpair[iter & 1], and the explicit warm start and the first-sweep role apply
     // when iter == 0, with iter read from ctrl at kernel start
     int graph;
-    double *jpair[2];
-    StageImages img;
-    // start-point cache, 4 reals a marker (A_y(x^n), A_z(x^n), gamma(p^n, A(x^n)),
-    // unused): written by the loop's first sweep, read by the later ones; NULL: none
+    double *mpair[2];
+    // double form: start-point cache, 4 reals a marker (A_y(x^n), A_z(x^n),
+    // gamma(p^n, A(x^n)), unused): written by the loop's first sweep, read by the later
+    // ones; NULL: none
     void *a0;
+    int zforce;         // 1: treat the z component as present whatever ctrl->zany says
     // spin (double form, hbar != 0): spin components in caller order (indexed by id)
     double hbar;
     const double *sy, *sz;
 };
 
 struct Sweep2Args {
-    int M, H, K, fp32;
+    int M, K, fp32;
     int acc;            // deposit window accumulator (ACC_*)
     long long np;
-    double w;
     PartPtrs P;
-    const double *an_y, *an_z, *ak_y, *ak_z;
-    double *s_y, *s_z;
-    int *status;        // error bits (STATUS_TIMEOUT)
-    // graph mode: deposits go to sypair/szpair[iter & 1], iter read from ctrl
+    CoefTables T;
+    double *mom_y, *mom_z;      // deposits: M x (K + 1) moments f v^m (without w)
+    int first;
+    // graph mode: deposits go to mypair/mzpair[iter & 1], iter read from ctrl
     int graph;
     const DevCtrl *ctrl;
-    double *sypair[2], *szpair[2];
-    StageImages img;
+    double *mypair[2], *mzpair[2];
+    void *a0;           // double form: (A_y, A_z, gamma) at a^n, as in subsystem I
+    int zforce;
 };
 
 struct CurrentArgs {
-    int M, H, Dlim, K, fp32;
+    int M, Dlim, K, fp32;
     long long np;
-    double dx, w;
+    double dx;
     PartPtrs P;
     const double *disp;     // caller order, length units
-    double *out;
+    double *mom;            // M x K moments
     DevCtrl *ctrl;
 };
 
@@ -101,23 +108,22 @@ struct DiagArgs {
     long long np;
     double dx, w;
     PartPtrs P;
-    const double *c0, *c1;  // field coefficients (gather: c0; kinetic: a_y, a_z)
-    double *out;            // gather output (caller order) or rho
+    const double *c0, *c1;  // field coefficients (kinetic: a_y, a_z)
+    const double *tab;      // gathers: cell polynomials (launch_cell_coefs)
+    double *out;            // gather output (caller order)
+    double *mom;            // charge: M x (K + 1) moments
     double *acc;            // kinetic sum
     int Dlim;               // path gathers: largest displacement (cells)
     int *status;            // path gathers: error bits (STATUS_NUMERIC)
 };
 
-int launch_sweep1(const Sweep1Args &a, int grid, int block, size_t smem, cudaStream_t s);
+int launch_sweep1(const Sweep1Args &a, int grid, cudaStream_t s);
 // the predicted start of subsystem I: delta^(0) (explicit when a.warm) and its current
-// into a.j; the sweep's launch shape and shared memory
-int launch_predeposit(const Sweep1Args &a, int grid, int block, size_t smem, cudaStream_t s);
-size_t sweep1_smem(int M, int H, int fp32);
-int launch_sweep2(const Sweep2Args &a, int grid, int block, size_t smem, cudaStream_t s);
-size_t sweep2_smem(int M, int H, int fp32);
-int launch_current(const CurrentArgs &a, int grid, int block, size_t smem, cudaStream_t s);
-int launch_charge(const DiagArgs &a, int grid, int block, size_t smem, cudaStream_t s);
-size_t charge_smem(int M, int H);
+// into a.mom; the sweep's launch shape
+int launch_predeposit(const Sweep1Args &a, int grid, cudaStream_t s);
+int launch_sweep2(const Sweep2Args &a, int grid, cudaStream_t s);
+int launch_current(const CurrentArgs &a, int grid, cudaStream_t s);
+int launch_charge(const DiagArgs &a, int grid, cudaStream_t s);
 int launch_gather(const DiagArgs &a, int field_degree, int grid, int block, cudaStream_t s);
 int launch_gather_path(const DiagArgs &a, int grid, int block, cudaStream_t s);
 int launch_kinetic(const DiagArgs &a, int grid, int block, cudaStream_t s);
@@ -131,7 +137,7 @@ int launch_store(int fp32, long long np, double dx, PartPtrs P, double *x, doubl
 // scratch); consecutive writes, so x and p may be device addresses of page-locked host memory
 int launch_store_ordered(int fp32, long long np, double dx, PartPtrs P, int32_t *inv, double *x, double *p,
                          int grid, int block, cudaStream_t s);
-int sweep_blocks_per_sm(int K, int fp32, int acc, int which, int block, size_t smem);
+int sweep_blocks_per_sm(int K, int fp32, int acc, int which);
 // whether the sweep kernels are built for (degree, form, accumulator)
 bool sweep_variant_ok(int K, int fp32, int acc);
 // one run's counting sort in a batched launch (key: cell * nbins + velocity bin)
@@ -161,27 +167,31 @@ constexpr double kFieldIncrementRelPredicted = 3e-9;
 enum ConvMode { CONV_PLAIN = 0, CONV_SOLVE1 = 1, CONV_SOLVE2 = 2, CONV_START1 = 3 };
 
 struct ConvArgs {
-    int M, d_start, ntap, mode, ncomp;
+    int M, K, d_start, ntap, mode, ncomp;
     const double *taps;
+    // input: the moments of the deposit (mom, of degree K - 1 in subsystem I and K in II,
+    // times scale), or nodes (in) where mom is null
+    const double *mom[2];
     const double *in[2];
+    double scale;
     double *out[2];
     const double *en[2];    // e^n
     double *ek[2];          // e^(k) (in: previous, out: new)
     double *aux[2];         // SOLVE1: ebar out; SOLVE2: a^(k) out
     const double *an[2];    // SOLVE2: a^n
-    const double *r0[2];    // SOLVE2: P^{-1} b
-    double *zero[2];        // deposit buffers of the next sweep, cleared here
+    const double *b[2];     // SOLVE2: right side b of P e = b + dt s
+    double *zero[2];        // moments of the next sweep, cleared here
     double dt, dx, tol, dtol;
     double erel;        // FP32 subsystem I: field increment tolerance relative to the field's max-norm
     int max_iter, fp32, subsystem;
     DevCtrl *ctrl;
-    // graph mode: in[c] = pair[c][iter & 1], zero[c] = pair[c][(iter + 1) & 1]
+    // graph mode: mom[c] = pair[c][iter & 1], zero[c] = pair[c][(iter + 1) & 1]
     // (iter read from ctrl at kernel start), and the decision sets the loop's
     // conditional handle (1 = run another sweep)
     int graph;
     double *pair[2][2];
     unsigned long long cond_handle;
-    StageImages img;    // SOLVE1: f.x = ebar image; SOLVE2: ak, lo
+    CoefTables T;       // START1 / SOLVE1: E; SOLVE2: Kt, L
     int *count;         // graph mode of single runs: sweeps counted by the decision (or NULL)
 };
 
@@ -257,37 +267,40 @@ struct RunDesc {
     long long np;
     double dx, dt;
     PartPtrs P;
-    double *ex, *ek, *ebar, *ay, *az, *ga_y, *ga_z, *j0, *j1;
+    double *ex, *ek, *ebar, *ay, *az, *m1[2];        // m1: M x K moments of subsystem I
     const double *rowPm, *rowK;
-    double *ey, *ez, *by, *bz, *eky, *ekz, *aky, *akz, *sy0, *sz0, *sy1, *sz1;
+    double *ey, *ez, *by, *bz, *eky, *ekz, *aky, *akz, *my[2], *mz[2];   // M x (K + 1) moments
     DevCtrl *ctrl;
-    StageImages img;
+    CoefTables T;
     FieldHist fh;
 };
 
 int launch_ens_plan(EnsQueue *Q, const EnsRun *runs, int nruns, unsigned long long cond, cudaStream_t s);
 int launch_ens_status(const EnsRun *runs, int nruns, int *status, cudaStream_t s);
-int conv_ens_optin(int Mmax, int ntap_max);
-int launch_conv_ens(const ConvArgs *runs, int nruns, int Mmax, int ncomp, int ntap_max, EnsQueue *Q,
+int conv_ens_optin(int ntap_max);
+int launch_conv_ens(const ConvArgs *runs, int nruns, int Mmax, int K, int ncomp, int ntap_max, EnsQueue *Q,
                     int *sweeps, unsigned long long cond, cudaStream_t s);
 int launch_prep1_ens(const RunDesc *R, int nruns, int Mmax, cudaStream_t s);
 int launch_prep2_ens(const RunDesc *R, int nruns, int Mmax, cudaStream_t s);
 int launch_commit_ens(const RunDesc *R, int nruns, int Mmax, int which, cudaStream_t s);
-int launch_sweep1_ens(int K, int fp32, const Sweep1Args *runs, int nruns, EnsQueue *Q, int grid,
-                      size_t smem, cudaStream_t s);
-int launch_sweep2_ens(int K, int fp32, const Sweep2Args *runs, int nruns, EnsQueue *Q, int grid,
-                      size_t smem, cudaStream_t s);
-// the predicted start of every run in the queue (delta^(0) and its current into each run's a.j)
-int launch_predeposit_ens(int K, int fp32, const Sweep1Args *runs, int nruns, EnsQueue *Q, int grid,
-                          size_t smem, cudaStream_t s);
+int launch_sweep1_ens(int K, int fp32, const Sweep1Args *runs, int nruns, EnsQueue *Q, int grid, cudaStream_t s);
+int launch_sweep2_ens(int K, int fp32, const Sweep2Args *runs, int nruns, EnsQueue *Q, int grid, cudaStream_t s);
+// the predicted start of every run in the queue (delta^(0) and its current into each run's a.mom)
+int launch_predeposit_ens(int K, int fp32, const Sweep1Args *runs, int nruns, EnsQueue *Q, int grid, cudaStream_t s);
 int launch_finalize1_ens(int fp32, const RunDesc *R, int nruns, int grid_x, cudaStream_t s);
 int launch_prep1(const RunDesc &R, cudaStream_t s);
 int launch_prep2(const RunDesc &R, cudaStream_t s);
 // end of a substep (which = 1, 2): the converged iterate becomes the state, and
 // its change is recorded for the next starting field
 int launch_commit(const RunDesc &R, int which, cudaStream_t s);
-// scale S of the scaled path means of degree d (the sweeps' piece_means_scaled)
-int mean_scale(int d);
+// node values of a deposit from its moments of degree D (times scale; path: coefficient m
+// divided by m + 1): out[j] = scale sum_r sum_m B_D[r][m] mom[j + r][m]
+int launch_moments_to_nodes(int M, int D, bool path, double scale, const double *mom, double *out, cudaStream_t s);
+// double cell polynomials of the degree-D spline with coefficients c (path: m-th divided by m + 1)
+int launch_cell_coefs(int M, int D, bool path, const double *c, double *tab, cudaStream_t s);
+// the tables of a subsystem-II sweep with given a^n and a^(k) (T.A, T.Kt, T.L)
+int launch_tables2(int M, int K, int fp32, const double *an_y, const double *an_z, const double *ak_y,
+                   const double *ak_z, CoefTables T, cudaStream_t s);
 int launch_poisson_rhs(int M, double dx, const double *rho, double *d, cudaStream_t s);
 int launch_energy_grid(int M, int K, double dx, const double *rowM0, const double *rowM1,
                        const double *rowK, const double *ex, const double *ey, const double *ez,
