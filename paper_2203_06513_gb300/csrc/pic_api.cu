@@ -122,12 +122,12 @@ static void release(pic_handle *h)
     for (int b = 0; b < 2; ++b) {
         f(h->Pblk[b]);
         f(h->jb[b]); f(h->sy[b]); f(h->sz[b]);
-        f(h->m1[b]); f(h->my[b]); f(h->mz[b]);
+        f(h->m1[b]); f(h->my[b]); f(h->mz[b]); f(h->flux[b]);
     }
     f(h->delta); f(h->pnew); f(h->a0);
     f(h->spx); f(h->spy); f(h->spz); f(h->sdy); f(h->sdz); f(h->red);
     double *arr[] = {h->ex, h->ey, h->ez, h->ay, h->az, h->ek, h->ebar,
-                     h->eky, h->ekz, h->aky, h->akz, h->by, h->bz, h->mdep, h->gtab, h->rho,
+                     h->eky, h->ekz, h->aky, h->akz, h->by, h->bz, h->m0, h->mdep, h->gtab, h->rho,
                      h->work, h->diag, h->d_rowM0, h->d_rowM1, h->d_rowK, h->d_rowPm,
                      h->d_tapM1, h->d_tapP};
     for (double *a : arr) f(a);
@@ -264,7 +264,8 @@ pic::RunDesc pic::handle_desc(pic_handle *h)
     d.M = h->M; d.K = h->K; d.fp32 = h->fp32; d.np = h->np; d.dx = h->dx; d.dt = h->cfg.dt;
     d.P = cur_parts(h);
     d.ex = h->ex; d.ek = h->ek; d.ebar = h->ebar; d.ay = h->ay; d.az = h->az;
-    d.m1[0] = h->m1[0]; d.m1[1] = h->m1[1];
+    d.m0 = h->m0;
+    for (int b = 0; b < 2; ++b) { d.m1[b] = h->m1[b]; d.flux[b] = h->flux[b]; }
     d.rowPm = h->d_rowPm; d.rowK = h->d_rowK;
     d.ey = h->ey; d.ez = h->ez; d.by = h->by; d.bz = h->bz;
     d.eky = h->eky; d.ekz = h->ekz; d.aky = h->aky; d.akz = h->akz;
@@ -308,6 +309,9 @@ static int solve_poisson(pic_handle *h)
 {
     int rc;
     if ((rc = deposit_charge(h, h->rho))) return rc;
+    // the markers' moments, the start points of the first step
+    launch_start_moments(h->M, h->K, h->mdep, h->m0, h->stream);
+    CKL_N("launch_start_moments");
     if ((rc = reduce(h, PIC_REDUCE_SUM, h->rho, h->M))) return rc;
     launch_poisson_rhs(h->M, h->dx, h->rho, h->work, h->stream);
     CKL_N("launch_poisson_rhs");
@@ -416,7 +420,7 @@ extern "C" int pic_init_split(const pic_config *cfg, const pic_arrays *in, int32
         h->P[b].p = h->Pblk[b] + off_p;
         h->P[b].id = reinterpret_cast<int32_t *>(h->Pblk[b] + off_id);
         if ((rc = dalloc(h, &h->m1[b], M * c.degree)) || (rc = dalloc(h, &h->my[b], M * (c.degree + 1))) ||
-            (rc = dalloc(h, &h->mz[b], M * (c.degree + 1))))
+            (rc = dalloc(h, &h->mz[b], M * (c.degree + 1))) || (rc = dalloc(h, &h->flux[b], M)))
             return bail(rc);
         if (reduce_fn && ((rc = dalloc(h, &h->jb[b], M)) || (rc = dalloc(h, &h->sy[b], M)) ||
                           (rc = dalloc(h, &h->sz[b], M))))
@@ -464,7 +468,7 @@ extern "C" int pic_init_split(const pic_config *cfg, const pic_arrays *in, int32
             (rc = dalloc(h, (char **)&h->T.Kt, 2 * M * pa * h->rsize)) ||
             (rc = dalloc(h, (char **)&h->T.E, M * pe * h->rsize)) ||
             (h->fp32 && (rc = dalloc(h, &h->T.L, 2 * M * pa))) ||
-            (rc = dalloc(h, &h->mdep, 2 * M * (c.degree + 1))) ||
+            (rc = dalloc(h, &h->m0, M * c.degree)) || (rc = dalloc(h, &h->mdep, 2 * M * (c.degree + 1))) ||
             (rc = dalloc(h, &h->gtab, M * coef_pad(0, c.degree + 1))))
             return bail(rc);
     }
@@ -671,7 +675,8 @@ Sweep1Args pic::make_sweep1_args(pic_handle *h, double dt)
     a.sy = h->spy;
     a.sz = h->spz;
     a.mom = h->m1[0];
-    a.mpair[0] = h->m1[0]; a.mpair[1] = h->m1[1];
+    a.flux = h->flux[0];
+    for (int b = 0; b < 2; ++b) { a.mpair[b] = h->m1[b]; a.fpair[b] = h->flux[b]; }
     return a;
 }
 
@@ -686,7 +691,8 @@ ConvArgs pic::make_conv1_args(pic_handle *h, double dt)
     c.dt = dt; c.dx = h->dx; c.tol = h->cfg.tol; c.dtol = 1e-6;   // FP32: estimated position error, cells relative to max(1, |delta|)
     c.erel = h->cfg.warm_field ? kFieldIncrementRelPredicted : kFieldIncrementRel;
     c.max_iter = h->cfg.max_iter; c.fp32 = h->fp32; c.subsystem = 1; c.ctrl = h->ctrl;
-    c.pair[0][0] = h->m1[0]; c.pair[0][1] = h->m1[1];
+    c.mom0 = h->m0;
+    for (int b = 0; b < 2; ++b) { c.pair[0][b] = h->m1[b]; c.fpair[b] = h->flux[b]; }
     return c;
 }
 
@@ -739,8 +745,8 @@ static int reduce_moments(pic_handle *h, ConvArgs &c, int comp, const double *mo
 {
     c.mom[comp] = mom;
     if (!h->reduce) return PIC_OK;
-    const bool path = c.subsystem == 1;
-    launch_moments_to_nodes(h->M, path ? h->K - 1 : h->K, path, c.scale, mom, nodes, h->stream);
+    if (c.subsystem == 1) launch_path_nodes(h->M, h->K, c.scale, mom, h->m0, c.flux, nodes, h->stream);
+    else launch_moments_to_nodes(h->M, h->K, false, c.scale, mom, nodes, h->stream);
     CKL_N("launch_moments_to_nodes");
     c.mom[comp] = nullptr;
     c.in[comp] = nodes;
@@ -755,11 +761,13 @@ static int predicted_start(pic_handle *h, double dt, cudaStream_t s)
     Sweep1Args a = make_sweep1_args(h, dt);
     a.warm = h->cfg.warm_start == PIC_WARM_EXPLICIT ? 1 : 0;   // else the network's delta is there
     a.mom = h->m1[1];
+    a.flux = h->flux[1];
     a.first = 1;
     if (launch_predeposit(a, h->grid1, s)) return fail(h, PIC_ERR_INVALID, "predeposit");
     ConvArgs c = make_conv1_args(h, dt);
     c.mode = CONV_START1;
     c.mom[0] = h->m1[1];
+    c.flux = h->flux[1];
     int rc;
     if (s == h->stream && (rc = reduce_moments(h, c, 0, h->m1[1], h->jb[1]))) return rc;
     if (launch_conv(c, s)) return fail(h, PIC_ERR_CUDA, "k_conv launch");
@@ -792,6 +800,7 @@ static int substep1(pic_handle *h, int *iters, double dt)
     int it = 0;
     for (;;) {
         a.mom = h->m1[it & 1];
+        a.flux = h->flux[it & 1];
         a.warm = (it == 0 && h->cfg.warm_start == PIC_WARM_EXPLICIT && !h->cfg.warm_field) ? 1 : 0;
         a.first = it == 0 ? 1 : 0;
         if ((rc = timed_begin(h))) return rc;
@@ -800,8 +809,10 @@ static int substep1(pic_handle *h, int *iters, double dt)
         CKL_N("launch_sweep1");
         if ((rc = timed_end(h, 0))) return rc;
         h->marker_sweeps += h->np;
+        c.flux = h->flux[it & 1];
         if ((rc = reduce_moments(h, c, 0, h->m1[it & 1], h->jb[it & 1])) || (rc = reduce_ctrl(h))) return rc;
         c.zero[0] = h->m1[(it + 1) & 1];
+        c.zflux = h->flux[(it + 1) & 1];
         if ((rc = timed_begin(h))) return rc;
         if (launch_conv(c, h->stream)) return fail(h, PIC_ERR_CUDA, "k_conv shared-memory opt-in failed");
         CKL_N("launch_conv");
@@ -1161,7 +1172,7 @@ extern "C" int pic_get_state(pic_handle *h, const pic_arrays *o, int32_t mem)
     double *pp = (host && o->p) ? static_cast<double *>(const_cast<void *>(pinned_device_ptr(o->p))) : nullptr;
     if ((o->x || o->p) && (!o->x || px) && (!o->p || pp)) {
         int32_t *inv = reinterpret_cast<int32_t *>(h->Pblk[1 - h->cur]);
-        launch_store_ordered(h->fp32, h->np, h->dx, cur_parts(h), inv, px, pp, particle_grid(h), 256, h->stream);
+        launch_store_ordered(h->fp32, h->np, h->M, h->dx, cur_parts(h), inv, px, pp, particle_grid(h), 256, h->stream);
         cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
         if (e != cudaSuccess) return fail(h, PIC_ERR_CUDA, "get_state: %s", cudaGetErrorString(e));
@@ -1171,7 +1182,7 @@ extern "C" int pic_get_state(pic_handle *h, const pic_arrays *o, int32_t mem)
         // the store writes each marker to its input position (a permutation after the
         // sorts): scattered there in device memory, then copied to the host in bulk
         if (host) stage_doubles(h, 1 - h->cur, o->x ? &dx_out : nullptr, o->p ? &dp_out : nullptr);
-        launch_store(h->fp32, h->np, h->dx, cur_parts(h), dx_out, dp_out, particle_grid(h), 256, h->stream);
+        launch_store(h->fp32, h->np, h->M, h->dx, cur_parts(h), dx_out, dp_out, particle_grid(h), 256, h->stream);
         cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess && host) {
             if (o->x) e = cudaMemcpyAsync(o->x, dx_out, np * sizeof(double), cudaMemcpyDeviceToHost, h->stream);

@@ -54,7 +54,8 @@ struct pic_ensemble {
     int sort_grid = 1;
     int *h_buf = nullptr;               // pinned readback: sweeps (2 nruns), status (nruns), Q fields
 
-    int bps_max = 1;                    // resident sweep blocks per SM (launch grid = SMs x bps_max)
+    int grid1 = 1, grid2 = 1;           // launch grids of the sweeps: SMs x resident blocks
+    int bps_max = 1;                    // blocks per SM of the schedule: the smaller of both
     int item_markers = 65536, bps = 1;  // schedule (the autotuner's choice)
     int fin_grid = 1;
 
@@ -125,6 +126,7 @@ static void build_tables(pic_ensemble *e)
         ap.graph = 0;
         ap.first = 1;
         ap.mom = h->m1[1];
+        ap.flux = h->flux[1];
 
         ConvArgs &c = e->c1[r];
         c = make_conv1_args(h, h->cfg.dt);
@@ -136,6 +138,7 @@ static void build_tables(pic_ensemble *e)
         cs.mode = CONV_START1;
         cs.graph = 0;
         cs.mom[0] = h->m1[1];
+        cs.flux = h->flux[1];
 
         e->a2[r] = make_sweep2_args(h);
         e->a2[r].graph = 1;
@@ -164,7 +167,7 @@ static int upload_tables(pic_ensemble *e)
 // the schedule fields of the queue, read by the plan and sweep kernels at run time
 static int upload_schedule(pic_ensemble *e)
 {
-    int v[2] = {e->item_markers, e->num_sms * e->bps};
+    int v[3] = {e->item_markers, e->bps, e->bps_max};
     ECK(cudaMemcpyAsync(&e->d_q->item_markers, v, sizeof(v), cudaMemcpyHostToDevice, e->stream));
     ECK(cudaStreamSynchronize(e->stream));
     return PIC_OK;
@@ -174,14 +177,13 @@ static int upload_schedule(pic_ensemble *e)
 // The loop body: plan, batched sweep, batched solve (cond = 0: no graph).
 static int loop_body(pic_ensemble *e, int which, cudaStream_t s, unsigned long long cond)
 {
-    const int grid = e->num_sms * e->bps_max;
     ELAUNCH(launch_ens_plan(e->d_q, e->d_er, e->nruns, cond, s), "ensemble plan");
     if (which == 1) {
-        ELAUNCH(launch_sweep1_ens(e->K, e->fp32, e->d_a1, e->nruns, e->d_q, grid, s), "ensemble sweep I");
+        ELAUNCH(launch_sweep1_ens(e->K, e->fp32, e->d_a1, e->nruns, e->d_q, e->grid1, s), "ensemble sweep I");
         ELAUNCH(launch_conv_ens(e->d_c1, e->nruns, e->Mmax, e->K, 1, e->ntap1, e->d_q, e->d_sweeps, cond, s),
                 "ensemble solve I");
     } else {
-        ELAUNCH(launch_sweep2_ens(e->K, e->fp32, e->d_a2, e->nruns, e->d_q, grid, s), "ensemble sweep II");
+        ELAUNCH(launch_sweep2_ens(e->K, e->fp32, e->d_a2, e->nruns, e->d_q, e->grid2, s), "ensemble sweep II");
         ELAUNCH(launch_conv_ens(e->d_c2, e->nruns, e->Mmax, e->K, 2, e->ntap2, e->d_q, e->d_sweeps, cond, s),
                 "ensemble solve II");
     }
@@ -194,9 +196,8 @@ static int seg_prep1(pic_ensemble *e, cudaStream_t s)
     if (e->warm_field) {
         // predicted start of every run: plan (all runs are iterating), the proposals
         // and their currents (work queue), e^(0) per run
-        const int grid = e->num_sms * e->bps_max;
         ELAUNCH(launch_ens_plan(e->d_q, e->d_er, e->nruns, 0ull, s), "ensemble plan");
-        ELAUNCH(launch_predeposit_ens(e->K, e->fp32, e->d_a1p, e->nruns, e->d_q, grid, s),
+        ELAUNCH(launch_predeposit_ens(e->K, e->fp32, e->d_a1p, e->nruns, e->d_q, e->grid1, s),
                 "ensemble predicted start");
         ELAUNCH(launch_conv_ens(e->d_c1p, e->nruns, e->Mmax, e->K, 1, e->ntap1, e->d_q, e->d_sweeps, 0ull, s),
                 "ensemble start field");
@@ -376,6 +377,8 @@ extern "C" int pic_ensemble_create(const pic_config *cfgs, const pic_arrays *ins
         const int b1 = sweep_blocks_per_sm(e->K, e->fp32, e->fp32 ? ACC_COMP : ACC_NATIVE, 1);
         const int b2 = sweep_blocks_per_sm(e->K, e->fp32, e->fp32 ? ACC_COMP : ACC_NATIVE, 2);
         e->bps_max = std::max(1, std::min(b1, b2));
+        e->grid1 = e->num_sms * std::max(1, b1);
+        e->grid2 = e->num_sms * std::max(1, b2);
         e->bps = e->bps_max;
     }
     // sort blocks a run: about four sweeps of 256 markers a block for the largest

@@ -219,6 +219,18 @@ __device__ void decide(const ConvArgs &A)
 // Spline pieces of every degree (pic_poly.cuh).  Grid kernels take the degree at run time.
 __constant__ SplineTab c_spline = make_spline_tab();
 
+// Pieces of C_i = sum_{j >= i} Lambda^0_j in the cells i + r, r = 0 .. d - 1: the running
+// sums over r of the pieces of N^d.
+constexpr SplineTab make_cumulative_tab()
+{
+    SplineTab T = make_spline_tab();
+    for (int d = 0; d <= kMaxDegree; ++d)
+        for (int r = 1; r <= d; ++r)
+            for (int m = 0; m <= d; ++m) T.b[d][r][m] += T.b[d][r - 1][m];
+    return T;
+}
+__constant__ SplineTab c_cumulative = make_cumulative_tab();
+
 // Stores coefficient m of row `row` (pad numbers a row) in the form's type.
 __device__ __forceinline__ void put_coef(void *tab, int fp32, size_t row, int pad, int m, double v)
 {
@@ -255,6 +267,27 @@ __device__ __forceinline__ double node_value(int M, int D, bool path, const doub
     return v;
 }
 
+// Path current at node j over w dx (pic_poly.cuh): the polynomials of C_j on the change of
+// the moments in the cells j .. j + K - 1, and the crossings of the knot j + K.
+__device__ __forceinline__ double path_node_value(int M, int K, const double *mom, const double *mom0,
+                                                  const int *flux, int j)
+{
+    double s0 = 0.0, s1 = 0.0;
+    int c = j, f = flux[j];
+    for (int r = 0; r < K; ++r) {
+        const int cn = c + 1 == M ? 0 : c + 1;
+        const int fn = flux[cn];
+        s0 = fma(c_cumulative.b[K][r][0], (double)(f - fn), s0);
+        for (int m = 1; m <= K; ++m) {
+            const size_t q = (size_t)c * K + m - 1;
+            s1 = fma(c_cumulative.b[K][r][m], mom[q] - mom0[q], s1);
+        }
+        c = cn;
+        f = fn;
+    }
+    return (s0 + s1) + (double)f;
+}
+
 // The residue of a^n + a^(k) after both coefficients were rounded to float.
 __device__ __forceinline__ float sum_residue(double n, double k)
 {
@@ -283,16 +316,20 @@ inline int conv_blocks(int M, int K) { return (M + kConvOut - K - 1) / (kConvOut
 __device__ bool conv_block(const ConvArgs &A, int bx, int comp, double *sm)
 {
     const int M = A.M, K = A.K, TB = kConvOut - K, i0 = bx * TB;
-    const int D = A.subsystem == 1 ? K - 1 : K, NV = D + 1;
+    const int NV = A.subsystem == 1 ? K : K + 1;       // moments a cell
     const int nq = kConvOut + A.ntap - 1;
     double *s_in = sm, *s_tap = s_in + nq, *s_part = s_tap + A.ntap;
     double *s_val = s_part + 4 * kConvOut, *s_an = s_val + kConvOut;
     const double *mom = A.mom[comp];
     double *zero = A.zero[comp];
+    const int *flux = A.flux;
+    int *zflux = A.zflux;
     if (A.graph && A.mode != CONV_PLAIN) {   // replayed by a graph: buffers by sweep parity
         const int it = *reinterpret_cast<volatile const int *>(&A.ctrl->iter);
         mom = A.pair[comp][it & 1];
         zero = A.pair[comp][(it + 1) & 1];
+        flux = A.fpair[it & 1];
+        zflux = A.fpair[(it + 1) & 1];
     }
     // s_in[q]: node (g0 + q) mod M
     const int g0 = wrap_cell(i0 - K - (A.d_start + A.ntap - 1), M);
@@ -300,7 +337,8 @@ __device__ bool conv_block(const ConvArgs &A, int bx, int comp, double *sm)
     if (mom) {
         for (int q = threadIdx.x; q < nq; q += kConvThreads) {
             const int g = (g0 + q) % M;
-            double s = A.scale * node_value(M, D, A.subsystem == 1, mom, g);
+            double s = A.scale * (A.subsystem == 1 ? path_node_value(M, K, mom, A.mom0, flux, g)
+                                                   : node_value(M, K, false, mom, g));
             if (A.mode == CONV_SOLVE2) s = fma(A.dt, s, A.b[comp][g]);
             s_in[q] = s;
         }
@@ -390,6 +428,8 @@ __device__ bool conv_block(const ConvArgs &A, int bx, int comp, double *sm)
     if (A.mode == CONV_START1) return false;
     if (zero)
         for (int q = threadIdx.x; q < ncell * NV; q += kConvThreads) zero[(size_t)i0 * NV + q] = 0.0;
+    if (zflux && A.subsystem == 1)
+        for (int q = threadIdx.x; q < ncell; q += kConvThreads) zflux[i0 + q] = 0;
     __shared__ int s_last;
     if (wid == 0) {
         diff = warp_max(diff);
@@ -540,6 +580,8 @@ __device__ __forceinline__ void prep1_at(int i, const RunDesc &R)
             R.m1[0][(size_t)i * K + m] = 0.0;
             R.m1[1][(size_t)i * K + m] = 0.0;
         }
+        R.flux[0][i] = 0;
+        R.flux[1][i] = 0;
         if (R.az[i] != 0.0) R.ctrl->zany = 1;
     }
     if (i == 0) ctrl_loop_reset(R.ctrl);
@@ -663,6 +705,9 @@ __device__ __forceinline__ void commit_at(int i, const RunDesc &R, int which)
     if (i < R.M) {
         if (which == 1) {
             commit_field(i, R.ek, R.ex, R.fh.x, R.fh.order1);
+            // the end points of the last sweep are the next step's start points
+            const double *last = R.m1[(R.ctrl->iter - 1) & 1];
+            for (int m = 0; m < R.K; ++m) R.m0[(size_t)i * R.K + m] = last[(size_t)i * R.K + m];
         } else {
             commit_field(i, R.eky, R.ey, R.fh.y, R.fh.order2);
             commit_field(i, R.ekz, R.ez, R.fh.z, R.fh.order2);
@@ -774,6 +819,33 @@ __global__ void k_moments_to_nodes(int M, int D, bool path, double scale, const 
 int launch_moments_to_nodes(int M, int D, bool path, double scale, const double *mom, double *out, cudaStream_t s)
 {
     k_moments_to_nodes<<<(M + 63) / 64, 64, 0, s>>>(M, D, path, scale, mom, out);
+    return 0;
+}
+
+__global__ void k_path_nodes(int M, int K, double scale, const double *mom, const double *mom0, const int *flux,
+                             double *out)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < M) out[j] = scale * path_node_value(M, K, mom, mom0, flux, j);
+}
+
+int launch_path_nodes(int M, int K, double scale, const double *mom, const double *mom0, const int *flux, double *out,
+                      cudaStream_t s)
+{
+    k_path_nodes<<<(M + 63) / 64, 64, 0, s>>>(M, K, scale, mom, mom0, flux, out);
+    return 0;
+}
+
+__global__ void k_start_moments(int M, int K, const double *charge, double *mom0)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= M * K) return;
+    mom0[i] = charge[(size_t)(i / K) * (K + 1) + i % K + 1];
+}
+
+int launch_start_moments(int M, int K, const double *charge, double *mom0, cudaStream_t s)
+{
+    k_start_moments<<<(M * K + 255) / 256, 256, 0, s>>>(M, K, charge, mom0);
     return 0;
 }
 

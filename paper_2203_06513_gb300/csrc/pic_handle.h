@@ -57,7 +57,10 @@ struct pic_handle {
     double *by = nullptr, *bz = nullptr;
     double *sy[2] = {nullptr, nullptr}, *sz[2] = {nullptr, nullptr};    // node deposits (split runs)
     // moments of the sweeps' deposits (M x K and, per component, M x (K + 1)), by sweep
-    // parity, and of the deposit entry points; double cell polynomials of the gathers
+    // parity, with subsystem I's knot crossings and start-point moments; moments of the
+    // deposit entry points; double cell polynomials of the gathers
+    int *flux[2] = {nullptr, nullptr};
+    double *m0 = nullptr;
     double *m1[2] = {nullptr, nullptr}, *my[2] = {nullptr, nullptr}, *mz[2] = {nullptr, nullptr};
     double *mdep = nullptr, *gtab = nullptr;
     double *rho = nullptr, *work = nullptr, *diag = nullptr;

@@ -18,23 +18,40 @@ namespace pic {
 // cells.
 constexpr int kVelBinsBase = 16;
 inline int bins_per_cell(long long np, int M) { return np >= 8192LL * M ? 4 : 1; }
-// threads per block of the sweep kernels
+// most threads per block of the marker kernels that split their range by warps
 constexpr int kSweepThreads = 256;
 constexpr int kSweepWarps = kSweepThreads / 32;
 // cells a warp's deposit window holds: subsystem I (paths of sorted markers visit two
 // or three cells, one more after a step without a sort), subsystem II without and with
 // the z component (whose window doubles the registers)
 constexpr int kWin1 = 4, kWin2 = 3, kWin2z = 2;
-// resident blocks per SM the sweeps are compiled for (registers a thread: 65536 /
-// (256 x blocks)): the windows of the higher degrees need more registers
-template <typename R, int K> struct SweepOcc { static constexpr int v1 = 2, v2 = 2; };
-template <> struct SweepOcc<float, 2> { static constexpr int v1 = 3, v2 = 3; };
-template <> struct SweepOcc<float, 3> { static constexpr int v1 = 3, v2 = 3; };
+// markers a lane takes per step: two in float, whose steps are bound by issue and the
+// latency of their chains; one in double, bound by the FP64 pipe
+template <typename R> struct SweepU { static constexpr int v = 1; };
+template <> struct SweepU<float> { static constexpr int v = 2; };
+// Shape of the sweep kernels: threads a block and resident blocks an SM they are compiled
+// for, which set the registers a thread may take (65536 / (threads x blocks)).  The float
+// sweeps keep two markers and a window in registers; with fewer registers they spill, with
+// more the SM holds too few warps.  Measured, us a launch (sweep I / II; cubic: 1e8
+// markers, quintic: 5e7):
+//   cubic    256 x 3 (85 registers)  1822 /  607     quintic  256 x 2 (128)  834 / 440
+//            256 x 2 (128)            992 /  770              128 x 5 (102)    - / 378
+//            128 x 7 (73)               - /  570              128 x 4 (128)  833 / 440
+//            128 x 5 (102)           1606 /  662              128 x 3 (170)  624 /   -
+// The double form is bound by the FP64 pipe and does not mind (1513 / 672 us for 1e7
+// markers at 16 warps, cubic).
+template <typename R, int K> struct SweepShape {
+    static constexpr int threads1 = 256, blocks1 = 2, threads2 = 256, blocks2 = 2;
+};
+template <int K> struct SweepShape<float, K> {
+    static constexpr int threads1 = K <= 4 ? 256 : 128, blocks1 = K <= 4 ? 2 : 3;
+    static constexpr int threads2 = 128, blocks2 = K <= 3 ? 7 : 5;
+};
 
 // ---------------------------------------------------------------- particles
 struct PartPtrs {
     int32_t *cell;      // cell index in [0, M)
-    void *t;            // offset in [0,1): float or double
+    void *t;            // offset from the cell's centre in [-1/2, 1/2]: float or double
     void *p;            // momentum
     void *delta;        // subsystem-I iterate: displacement x^(k) - x^n, cell units
     void *pnew;         // subsystem-I iterate p^(k+1)
@@ -58,15 +75,17 @@ struct Sweep1Args {
     double dx, dt;
     PartPtrs P;
     CoefTables T;
-    double *mom;        // deposit: M x K moments h S_m (without w dx)
+    double *mom;        // deposit: M x K moments v, .. v^K of the paths' ends
+    int *flux;          // deposit: net crossings (to the right) of the left edge of each cell
     DevCtrl *ctrl;
     int warm;           // 1: delta^(0) = explicit predictor, computed in-kernel (first sweep)
     int first;          // 1: the first sweep of the loop (writes the start-point cache)
     // graph mode (the launch is replayed by a CUDA graph): the deposit buffer is
-    // mpair[iter & 1], and the explicit warm start and the first-sweep role apply
+    // mpair / fpair[iter & 1], and the explicit warm start and the first-sweep role apply
     // when iter == 0, with iter read from ctrl at kernel start
     int graph;
     double *mpair[2];
+    int *fpair[2];
     // double form: start-point cache, 4 reals a marker (A_y(x^n), A_z(x^n),
     // gamma(p^n, A(x^n)), unused): written by the loop's first sweep, read by the later
     // ones; NULL: none
@@ -131,11 +150,11 @@ int launch_finalize1(int fp32, long long np, int M, PartPtrs P, bool zero_delta,
                      cudaStream_t s);
 int launch_load(int fp32, long long np, int M, double dx, const double *x, const double *p,
                 PartPtrs P, int grid, int block, cudaStream_t s);
-int launch_store(int fp32, long long np, double dx, PartPtrs P, double *x, double *p,
+int launch_store(int fp32, long long np, int M, double dx, PartPtrs P, double *x, double *p,
                  int grid, int block, cudaStream_t s);
 // the same values in caller order through an inverse permutation (inv: np int32 of
 // scratch); consecutive writes, so x and p may be device addresses of page-locked host memory
-int launch_store_ordered(int fp32, long long np, double dx, PartPtrs P, int32_t *inv, double *x, double *p,
+int launch_store_ordered(int fp32, long long np, int M, double dx, PartPtrs P, int32_t *inv, double *x, double *p,
                          int grid, int block, cudaStream_t s);
 int sweep_blocks_per_sm(int K, int fp32, int acc, int which);
 // whether the sweep kernels are built for (degree, form, accumulator)
@@ -169,9 +188,11 @@ enum ConvMode { CONV_PLAIN = 0, CONV_SOLVE1 = 1, CONV_SOLVE2 = 2, CONV_START1 = 
 struct ConvArgs {
     int M, K, d_start, ntap, mode, ncomp;
     const double *taps;
-    // input: the moments of the deposit (mom, of degree K - 1 in subsystem I and K in II,
-    // times scale), or nodes (in) where mom is null
+    // input: the moments of the deposit times scale (subsystem I: mom, mom0 and flux of
+    // the paths, II: mom), or nodes (in) where mom is null
     const double *mom[2];
+    const double *mom0;     // subsystem I: moments of the start points
+    const int *flux;
     const double *in[2];
     double scale;
     double *out[2];
@@ -181,15 +202,18 @@ struct ConvArgs {
     const double *an[2];    // SOLVE2: a^n
     const double *b[2];     // SOLVE2: right side b of P e = b + dt s
     double *zero[2];        // moments of the next sweep, cleared here
+    int *zflux;
     double dt, dx, tol, dtol;
     double erel;        // FP32 subsystem I: field increment tolerance relative to the field's max-norm
     int max_iter, fp32, subsystem;
     DevCtrl *ctrl;
-    // graph mode: mom[c] = pair[c][iter & 1], zero[c] = pair[c][(iter + 1) & 1]
+    // graph mode: mom[c] = pair[c][iter & 1], zero[c] = pair[c][(iter + 1) & 1] (flux and
+    // zflux from fpair the same way)
     // (iter read from ctrl at kernel start), and the decision sets the loop's
     // conditional handle (1 = run another sweep)
     int graph;
     double *pair[2][2];
+    int *fpair[2];
     unsigned long long cond_handle;
     CoefTables T;       // START1 / SOLVE1: E; SOLVE2: Kt, L
     int *count;         // graph mode of single runs: sweeps counted by the decision (or NULL)
@@ -239,8 +263,8 @@ struct EnsQueue {
     int n_decided;           // runs that took their convergence decision in this sweep
     int n_continue;          // ... and go on
     int go;                  // 1: some run goes on after this sweep
-    int item_markers;        // markers per item (a multiple of the tile size)
-    int nblocks;             // sweep blocks that claim items (the rest leave at once)
+    int item_markers;        // markers per item (a multiple of 1024)
+    int share, shares;       // share of shares of a sweep's blocks claim items (the rest leave at once)
     int loops[2];            // sweeps of the loops of subsystems I and II (all runs together)
     int item_start[kEnsMaxRuns + 1];
     int active[kEnsMaxRuns];
@@ -267,7 +291,8 @@ struct RunDesc {
     long long np;
     double dx, dt;
     PartPtrs P;
-    double *ex, *ek, *ebar, *ay, *az, *m1[2];        // m1: M x K moments of subsystem I
+    double *ex, *ek, *ebar, *ay, *az, *m1[2], *m0;   // M x K moments of subsystem I: ends (by sweep parity), starts
+    int *flux[2];
     const double *rowPm, *rowK;
     double *ey, *ez, *by, *bz, *eky, *ekz, *aky, *akz, *my[2], *mz[2];   // M x (K + 1) moments
     DevCtrl *ctrl;
@@ -296,6 +321,11 @@ int launch_commit(const RunDesc &R, int which, cudaStream_t s);
 // node values of a deposit from its moments of degree D (times scale; path: coefficient m
 // divided by m + 1): out[j] = scale sum_r sum_m B_D[r][m] mom[j + r][m]
 int launch_moments_to_nodes(int M, int D, bool path, double scale, const double *mom, double *out, cudaStream_t s);
+// node values of the path current of subsystem I (ConvArgs: mom, mom0, flux, scale)
+int launch_path_nodes(int M, int K, double scale, const double *mom, const double *mom0, const int *flux, double *out,
+                      cudaStream_t s);
+// start-point moments (m = 1 .. K) from charge moments (m = 0 .. K)
+int launch_start_moments(int M, int K, const double *charge, double *mom0, cudaStream_t s);
 // double cell polynomials of the degree-D spline with coefficients c (path: m-th divided by m + 1)
 int launch_cell_coefs(int M, int D, bool path, const double *c, double *tab, cudaStream_t s);
 // the tables of a subsystem-II sweep with given a^n and a^(k) (T.A, T.Kt, T.L)

@@ -423,7 +423,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_warm_mlp(WarmArgs A)
         const bool act = a < A.np;
         float f[kIn], pn = 0.f, g0 = 1.f;
         const int c = nc;
-        const float t = (float)nt;
+        const float t = (float)nt + 0.5f;             // cell-relative position
         pn = act ? (float)np_ : 0.f;
         if (a + stride < A.np) {
             nc = A.P.cell[a + stride];

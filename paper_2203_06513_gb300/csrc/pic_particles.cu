@@ -1,6 +1,6 @@
 // pic_particles.cu -- marker kernels of libpic (sm_103a).
 //
-// Markers are stored as structure-of-arrays (cell int32, offset t, momentum p,
+// Markers are stored as structure-of-arrays (cell int32, offset t from the cell's centre, momentum p,
 // iterates delta and p_new, caller index id) and kept sorted by the key
 // (cell, velocity bin), so the 32 lanes of a warp hold markers of one or two
 // cells with similar displacements.  Each warp of a sweep owns one contiguous range
@@ -34,10 +34,6 @@ struct Real<float> { static constexpr bool fp32 = true; };
 template <>
 struct Real<double> { static constexpr bool fp32 = false; };
 
-// Correctly rounded division: an approximate reciprocal carries a systematic
-// bias that the discrete-gradient identity turns into a steady energy drift.
-template <typename R> __device__ __forceinline__ R fdiv_(R a, R b) { return a / b; }
-
 // Contiguous chunk of markers owned by one block (a multiple of 32, so every
 // warp's lanes see consecutive, sorted markers).
 __device__ __forceinline__ void block_chunk(long long np, long long &beg, long long &end)
@@ -62,7 +58,7 @@ __device__ __forceinline__ void warp_chunk(long long beg, long long end, long lo
 // number q * grid + b), so that a launch with fewer ranges than warps uses every SM.
 __device__ __forceinline__ void grid_warp_chunk(long long np, long long &wb, long long &we)
 {
-    const long long nw = (long long)gridDim.x * kSweepWarps;
+    const long long nw = (long long)gridDim.x * (blockDim.x >> 5);
     warp_chunk(0, np, (long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x, nw, wb, we);
 }
 
@@ -75,34 +71,36 @@ __device__ __forceinline__ void sweep_max_to(unsigned long long *dst, double v)
     __syncthreads();
     if (threadIdx.x == 0) {
         double u = s_max[0];
-        for (int i = 1; i < kSweepWarps; ++i) {
+        for (int i = 1; i < (int)(blockDim.x >> 5); ++i) {
             const double x = s_max[i];
             u = (x > u || x != x) ? x : u;
         }
-        if (u != 0.0) atomic_max_nonneg(dst, u);
+        if (u != 0.0) atomic_max_nonneg(dst, u);      // (a NaN is not equal to 0)
     }
     __syncthreads();
 }
 
-// Start-point cache of the double form: (A_y, A_z, gamma, unused) per marker, as two
-// 16-byte accesses.  A(x^n) and gamma(p^n, A(x^n)) do not change during a fixed-point
-// loop: its first sweep stores them and the later ones read them back (32 bytes a
-// marker against about 20 operations on the narrow FP64 pipe; in the float form the
-// bytes would cost more than the operations).
+// Start-point cache of the double form: (A_y, gamma) and, with the z component, (A_z, 0)
+// per marker, 16-byte accesses.  A(x^n) and gamma(p^n, A(x^n)) do not change during a
+// fixed-point loop: its first sweep stores them and the later ones read them back (the
+// bytes against a dozen operations on the narrow FP64 pipe; in the float form the bytes
+// would cost more than the operations).
+template <bool Z>
 __device__ __forceinline__ void start_cache_store(void *base, long long a, double y, double z, double g)
 {
     double2 *q = reinterpret_cast<double2 *>(base) + 2 * a;
-    q[0] = make_double2(y, z);
-    q[1] = make_double2(g, 0.0);
+    q[0] = make_double2(y, g);
+    if (Z) q[1] = make_double2(z, 0.0);
 }
 
+template <bool Z>
 __device__ __forceinline__ void start_cache_load(const void *base, long long a, double &y, double &z, double &g)
 {
     const double2 *q = reinterpret_cast<const double2 *>(base) + 2 * a;
-    const double2 u = q[0], w = q[1];
+    const double2 u = q[0];
     y = u.x;
-    z = u.y;
-    g = w.x;
+    g = u.y;
+    if (Z) z = q[1].x;
 }
 
 // ---------------------------------------------------------------------------
@@ -116,253 +114,280 @@ __device__ __forceinline__ void start_cache_load(const void *base, long long a, 
 // In cell units with tau = dt/dx: p^(k+1) = p^n + tau (Ebar dx - (A1+A0).D dx/(...)).
 // The path is split at the knots; a piece of length h in one cell contributes
 //   h sum_m E_m S_m to the integral of ebar and h sum_m A_{m+1} S_m to A1 - A0
-// (path_sums), and the deposit adds h S_m to the moments of that cell.
+// (path_sums); the deposit adds the end point's moments and the knots crossed.
 //
 // What bounds it: the FP32 form instruction issue, the FP64 form the FP64 pipe (1/64 of
-// the FP32 rate).  A sweep that evaluates the triangle of basis values at both ends and
-// the piece means of every path piece from nodes staged in shared memory, and deposits
-// two cumulative bases through a switch over window offsets, took 453 us in float
-// (2e7 markers, 2048 cells, cubic: 652 warp instructions per 32 markers) and 854 us in
-// double (2e6 markers); the cell polynomials take 336 us (458) and 537 us.
+// the FP32 rate).  us a launch, float (1e8 markers, 2048 cells, cubic) and double (1e7):
+//   basis triangles at both ends, piece means, node windows     2160   4200
+//   cell polynomials, path moments h S_m in every cell visited  1680   2680
+//   end-point moments and knot counts, centred offsets, roots
+//   and quotients without exception paths, two markers a lane    992   1513
 // PRE: the predicted start instead of a sweep -- the proposal delta^(0) (the
 // explicit predictor when A.warm, else the one already in delta) is written back
 // and its path current deposited into A.mom; no gather walk, no momentum update.
 // ---------------------------------------------------------------------------
-template <int K, typename R, int ACC, bool PRE>
-__device__ __forceinline__ void sweep1_range(const Sweep1Args &A, long long beg, long long end, double &dmax_out,
-                                             bool &bad_out)
+// Z: the z component is not identically zero (a linearly polarised wave keeps A_z = 0
+// exactly, and then none of its terms are needed).
+template <int K, typename R, int ACC, bool PRE, bool Z>
+__device__ __forceinline__ void sweep1_range_z(const Sweep1Args &A, long long beg, long long end, double &dmax_out,
+                                               bool &bad_out)
 {
     constexpr int NC = K + 1;                           // coefficients of A in a cell
     constexpr int PA = CoefPad<R, NC>::v, PE = CoefPad<R, K>::v;
+    constexpr int U = SweepU<R>::v;                     // markers a lane and step
+    constexpr bool kSpin = !Real<R>::fp32 && !PRE && Z;
     const R one = R(1), half = R(0.5);
     double *mom = A.mom;
+    int *flux = A.flux;
     bool warm = A.warm != 0;
     bool first = A.first != 0;
     if (!PRE && A.graph) {                  // replayed by a graph: buffers by sweep parity
         const int it = *reinterpret_cast<volatile const int *>(&A.ctrl->iter);
         mom = A.mpair[it & 1];
+        flux = A.fpair[it & 1];
         warm = warm && it == 0;
         first = it == 0;
     }
     const int M = A.M;
-    const bool hasz = A.zforce || *reinterpret_cast<volatile const int *>(&A.ctrl->zany) != 0;
     const int32_t *__restrict__ cp = A.P.cell;
-    const R *__restrict__ tp = static_cast<const R *>(A.P.t);
+    const R *__restrict__ vp = static_cast<const R *>(A.P.t);
     const R *__restrict__ pp = static_cast<const R *>(A.P.p);
     R *dp = static_cast<R *>(A.P.delta);
     R *pnp = static_cast<R *>(A.P.pnew);
     const R *TA = static_cast<const R *>(A.T.A), *TE = static_cast<const R *>(A.T.E);
     const R tau = (R)(A.dt / A.dx);
     const R dlim = (R)A.Dlim;
+    const bool spin = kSpin && A.hbar != 0.0;
+    const bool cached = !Real<R>::fp32 && !PRE && !first && A.a0 != nullptr;
+    const bool keep = !Real<R>::fp32 && !PRE && first && A.a0 != nullptr;
     const int lane = threadIdx.x & 31;
     R dmax = R(0);
     bool bad = false;
-    MomentWindow<kWin1, K, typename AccOf<R, ACC>::T> win;
-    win.start();
-    int adds = 0;
+    if (beg >= end) return;
+    PathDeposit<K, U, typename AccOf<R, ACC>::T> dep;
+    dep.start(mom, flux, M, cp[beg]);
 
     // the next step's markers are loaded while this one's are computed
-    int nc = 0;
-    R nt = half, npn = R(0), nd = R(0);
+    int nc[U];
+    R nv[U], npn[U], nd[U];
     auto fetch = [&](long long s) {
-        const long long a = s + lane;
-        if (a < end) {
-            nc = cp[a];
-            nt = tp[a];
-            npn = pp[a];
-            if (!warm) nd = dp[a];
-        } else {
-            nt = half;
-            npn = R(0);
-            nd = R(0);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const long long a = s + 32 * u + lane;
+            if (a < end) {
+                nc[u] = cp[a];
+                nv[u] = vp[a];
+                npn[u] = pp[a];
+                if (!warm) nd[u] = dp[a];
+            } else {
+                nv[u] = R(0);
+                npn[u] = R(0);
+                nd[u] = R(0);
+            }
         }
     };
-    if (beg < end) fetch(beg);
-    for (long long s = beg; s < end; s += 32) {
-        const long long a = s + lane;
-        const bool act = a < end;
-        const unsigned amask = __ballot_sync(0xffffffffu, act);
-        const int cw = nc;                               // in [0, M)
-        const R t0 = nt, pn = npn, dread = nd;
-        if (s + 32 < end) fetch(s + 32);
-        const R v0 = t0 - half;
-        // A(x^n), gamma(p^n, A(x^n))
-        R ay[NC], az[NC];
-        R A0y, A0z = R(0), g0;
-        load_coef<NC>(TA + (size_t)cw * (2 * PA), ay);
 #pragma unroll
-        for (int m = 0; m < NC; ++m) az[m] = R(0);
-        if (hasz) load_coef<NC>(TA + (size_t)cw * (2 * PA) + PA, az);
-        bool cached = false;
-        if constexpr (!Real<R>::fp32 && !PRE) cached = !first && A.a0 != nullptr;
-        if (cached) {
-            if constexpr (!Real<R>::fp32) {
-                if (act) start_cache_load(A.a0, a, A0y, A0z, g0);
-                else { A0y = R(0); g0 = one; }
-            }
-        } else {
-            A0y = horner<NC>(ay, v0);
-            R q0 = fma(A0y, A0y, fma(pn, pn, one));
-            if (hasz) {
-                A0z = horner<NC>(az, v0);
-                q0 = fma(A0z, A0z, q0);
-            }
-            g0 = sqrt_(q0);
-            if constexpr (!Real<R>::fp32 && !PRE)
-                if (A.a0 && act) start_cache_store(A.a0, a, A0y, A0z, g0);
+    for (int u = 0; u < U; ++u) { nc[u] = 0; nd[u] = R(0); }
+    fetch(beg);
+    for (long long s = beg; s < end; s += 32 * U) {
+        bool act[U];
+        int cw[U];
+        R v0[U], pn[U], dold[U], dnew[U], pnew[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            act[u] = s + 32 * u + lane < end;
+            cw[u] = nc[u];
+            v0[u] = nv[u];
+            pn[u] = npn[u];
+            dold[u] = nd[u];
         }
-        R dold = warm ? fdiv_(tau * pn, g0) : dread;
-        if (!(fabs(dold) <= dlim)) { bad = bad || act; dold = R(0); }
-        R dnew = R(0), pnew = R(0);
+        if (s + 32 * U < end) fetch(s + 32 * U);
+        // A(x^n), gamma(p^n, A(x^n))
+        R A0y[U], A0z[U], g0[U], ay[U][NC], az[U][NC];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const size_t row = (size_t)cw[u] * (2 * PA);
+            load_coef<NC>(TA + row, ay[u]);
+            if (Z) load_coef<NC>(TA + row + PA, az[u]);
+            A0z[u] = R(0);
+            if (cached) {
+                if constexpr (!Real<R>::fp32) {
+                    A0y[u] = R(0);
+                    g0[u] = one;
+                    if (act[u]) start_cache_load<Z>(A.a0, s + 32 * u + lane, A0y[u], A0z[u], g0[u]);
+                }
+            } else {
+                A0y[u] = horner<NC>(ay[u], v0[u]);
+                R q0 = fma(A0y[u], A0y[u], fma(pn[u], pn[u], one));
+                if (Z) {
+                    A0z[u] = horner<NC>(az[u], v0[u]);
+                    q0 = fma(A0z[u], A0z[u], q0);
+                }
+                g0[u] = root(q0);
+                if constexpr (!Real<R>::fp32)
+                    if (keep && act[u]) start_cache_store<Z>(A.a0, s + 32 * u + lane, A0y[u], A0z[u], g0[u]);
+            }
+            if (warm) dold[u] = quotient(tau * pn[u], g0[u]);
+            if (!within(dold[u], dlim)) { bad = bad || act[u]; dold[u] = R(0); }
+        }
         if constexpr (PRE) {
-            dnew = dold;
+#pragma unroll
+            for (int u = 0; u < U; ++u) dnew[u] = dold[u];
         } else {
-            int n;
-            R t1;
-            path_end(t0, dold, n, t1);
-            const int an = abs(n);
-            const bool right = n > 0;
-            // first piece (the whole path when no knot is crossed)
-            R h0, EI, Qy, Qz = R(0), W;
-            {
-                const R tb = an == 0 ? t1 : (right ? one : R(0));
-                h0 = tb - t0;
+            int n[U], g[U], an[U], nmax = 0;
+            bool right[U];
+            R v1[U], h0[U], EI[U], Qy[U], Qz[U], W[U], D2y[U], D2z[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                path_end(v0[u], dold[u], n[u], v1[u]);
+                an[u] = abs(n[u]);
+                right[u] = n[u] > 0;
+                nmax = max(nmax, an[u]);
+                g[u] = cw[u];
+                // first piece (the whole path when no knot is crossed)
+                const R vb = an[u] == 0 ? v1[u] : (right[u] ? half : -half);
+                h0[u] = vb - v0[u];
                 R S[K], ec[K];
-                path_sums<K, R>(v0, tb - half, S);
-                load_coef<K>(TE + (size_t)cw * PE, ec);
-                R e = ec[0], y = ay[1], z = az[1];
+                path_sums<K, R>(v0[u], vb, S);
+                load_coef<K>(TE + (size_t)cw[u] * PE, ec);
+                R e = ec[0], y = ay[u][1], z = Z ? az[u][1] : R(0);
 #pragma unroll
                 for (int m = 1; m < K; ++m) {
                     e = fma(ec[m], S[m], e);
-                    y = fma(ay[m + 1], S[m], y);
-                }
-                if (hasz) {
-#pragma unroll
-                    for (int m = 1; m < K; ++m) z = fma(az[m + 1], S[m], z);
+                    y = fma(ay[u][m + 1], S[m], y);
+                    if (Z) z = fma(az[u][m + 1], S[m], z);
                 }
                 // one piece: the means are e, y, z themselves (weight 1, no division by h)
-                const R hw = an == 0 ? one : h0;
-                EI = hw * e;
-                Qy = hw * y;
-                Qz = hw * z;
-                W = hw;
-            }
-            R D2y = R(0), D2z = R(0);
-            if constexpr (!Real<R>::fp32) {
-                if (A.hbar != 0.0) {
-                    // path integral of d^2A/dx^2 (cell units) for the Zeeman term:
-                    // the difference quotient of A' = sum_m m A_m v^(m-1)
-                    R S[K];
-                    path_sums<K, R>(v0, (an == 0 ? t1 : (right ? one : R(0))) - half, S);
+                const R hw = an[u] == 0 ? one : h0[u];
+                EI[u] = hw * e;
+                Qy[u] = hw * y;
+                Qz[u] = Z ? hw * z : R(0);
+                W[u] = hw;
+                D2y[u] = D2z[u] = R(0);
+                if constexpr (kSpin) {
+                    if (spin) {
+                        // path integral of d^2A/dx^2 (cell units) for the Zeeman term:
+                        // the difference quotient of A' = sum_m m A_m v^(m-1)
 #pragma unroll
-                    for (int m = 2; m <= K; ++m) {
-                        D2y = fma(R(m) * ay[m], S[m - 2], D2y);
-                        D2z = fma(R(m) * az[m], S[m - 2], D2z);
+                        for (int m = 2; m <= K; ++m) {
+                            D2y[u] = fma(R(m) * ay[u][m], S[m - 2], D2y[u]);
+                            D2z[u] = fma(R(m) * az[u][m], S[m - 2], D2z[u]);
+                        }
+                        D2y[u] *= hw;
+                        D2z[u] *= hw;
                     }
-                    const R hw = an == 0 ? one : h0;
-                    D2y *= hw;
-                    D2z *= hw;
                 }
             }
-            const int nmax = __reduce_max_sync(0xffffffffu, act ? an : 0);
-            int g = cw;
+            nmax = __reduce_max_sync(0xffffffffu, nmax);
             for (int q = 1; q <= nmax; ++q) {
-                g += right ? 1 : -1;
-                g = g >= M ? g - M : (g < 0 ? g + M : g);
-                const bool on = q <= an;
-                const R ta = right ? R(0) : one;
-                const R tb = q == an ? t1 : (right ? one : R(0));
-                const R h = on ? tb - ta : R(0);
-                R S[K], ec[K], by[NC];
-                path_sums<K, R>(ta - half, tb - half, S);
-                load_coef<K>(TE + (size_t)g * PE, ec);
-                load_coef<NC>(TA + (size_t)g * (2 * PA), by);
-                R e = ec[0], y = by[1];
 #pragma unroll
-                for (int m = 1; m < K; ++m) {
-                    e = fma(ec[m], S[m], e);
-                    y = fma(by[m + 1], S[m], y);
-                }
-                EI = fma(h, e, EI);
-                Qy = fma(h, y, Qy);
-                W += h;
-                if constexpr (!Real<R>::fp32) {
-                    if (A.hbar != 0.0) {
-                        R d2 = R(0);
+                for (int u = 0; u < U; ++u) {
+                    g[u] = wrap_once(g[u] + (right[u] ? 1 : -1), M);
+                    const R va = right[u] ? -half : half;
+                    const R vb = q == an[u] ? v1[u] : -va;
+                    const R h = q <= an[u] ? vb - va : R(0);
+                    R S[K], ec[K], by[NC];
+                    edge_sums<K, R>(right[u], va, vb, S);
+                    load_coef<K>(TE + (size_t)g[u] * PE, ec);
+                    load_coef<NC>(TA + (size_t)g[u] * (2 * PA), by);
+                    R e = ec[0], y = by[1];
 #pragma unroll
-                        for (int m = 2; m <= K; ++m) d2 = fma(R(m) * by[m], S[m - 2], d2);
-                        D2y = fma(h, d2, D2y);
+                    for (int m = 1; m < K; ++m) {
+                        e = fma(ec[m], S[m], e);
+                        y = fma(by[m + 1], S[m], y);
                     }
-                }
-                if (hasz) {
-                    R bz[NC];
-                    load_coef<NC>(TA + (size_t)g * (2 * PA) + PA, bz);
-                    R z = bz[1];
-#pragma unroll
-                    for (int m = 1; m < K; ++m) z = fma(bz[m + 1], S[m], z);
-                    Qz = fma(h, z, Qz);
-                    if constexpr (!Real<R>::fp32) {
-                        if (A.hbar != 0.0) {
+                    EI[u] = fma(h, e, EI[u]);
+                    Qy[u] = fma(h, y, Qy[u]);
+                    if (an[u] != 0) W[u] += h;
+                    if constexpr (kSpin) {
+                        if (spin) {
                             R d2 = R(0);
 #pragma unroll
-                            for (int m = 2; m <= K; ++m) d2 = fma(R(m) * bz[m], S[m - 2], d2);
-                            D2z = fma(h, d2, D2z);
+                            for (int m = 2; m <= K; ++m) d2 = fma(R(m) * by[m], S[m - 2], d2);
+                            D2y[u] = fma(h, d2, D2y[u]);
+                        }
+                    }
+                    if (Z) {
+                        R bz[NC];
+                        load_coef<NC>(TA + (size_t)g[u] * (2 * PA) + PA, bz);
+                        R z = bz[1];
+#pragma unroll
+                        for (int m = 1; m < K; ++m) z = fma(bz[m + 1], S[m], z);
+                        Qz[u] = fma(h, z, Qz[u]);
+                        if constexpr (kSpin) {
+                            if (spin) {
+                                R d2 = R(0);
+#pragma unroll
+                                for (int m = 2; m <= K; ++m) d2 = fma(R(m) * bz[m], S[m - 2], d2);
+                                D2z[u] = fma(h, d2, D2z[u]);
+                            }
                         }
                     }
                 }
             }
-            // A(x^(k)) = A(x^n) + the path integral of dA/dx, of the staged field
-            const R hs = an == 0 ? h0 : one;
-            const R A1y = fma(hs, Qy, A0y), A1z = fma(hs, Qz, A0z);
-
-            // p^(k+1) = p^n + tau (Ebar - (A1 + A0).D / (g1 + g0)) with Ebar = EI/W,
-            // D = Q/W (W the summed pieces, 1 for a single one), as one division
-            R q1 = fma(A1y, A1y, one), nm = (A1y + A0y) * Qy;
-            if (hasz) {
-                q1 = fma(A1z, A1z, q1);
-                nm = fma(A1z + A0z, Qz, nm);
-            }
-            const R g1 = sqrt_(fma(pn, pn, q1));
-            const R G = g1 + g0;
-            const R num = fma(EI, G, -nm);
-            R kick = fdiv_(num, W * G);
-            if constexpr (!Real<R>::fp32) {
-                if (A.hbar != 0.0 && act) {
-                    const int id = A.P.id[a];
-                    kick -= A.hbar / A.dx * ((A.sy[id] * D2z - A.sz[id] * D2y) / W);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                // A(x^(k)) = A(x^n) + the path integral of dA/dx, of the staged field
+                const R hs = an[u] == 0 ? h0[u] : one;
+                const R A1y = fma(hs, Qy[u], A0y[u]);
+                // p^(k+1) = p^n + tau (Ebar - (A1 + A0).D / (g1 + g0)) with Ebar = EI/W,
+                // D = Q/W (W the summed pieces, 1 for a single one), as one division
+                R q1 = fma(A1y, A1y, one), nm = (A1y + A0y[u]) * Qy[u];
+                if (Z) {
+                    const R A1z = fma(hs, Qz[u], A0z[u]);
+                    q1 = fma(A1z, A1z, q1);
+                    nm = fma(A1z + A0z[u], Qz[u], nm);
+                }
+                const R g1 = root(fma(pn[u], pn[u], q1));
+                const R G = g1 + g0[u];
+                R kick = quotient(fma(EI[u], G, -nm), W[u] * G);
+                if constexpr (kSpin) {
+                    if (spin && act[u]) {
+                        const int id = A.P.id[s + 32 * u + lane];
+                        kick -= A.hbar / A.dx * ((A.sy[id] * D2z[u] - A.sz[id] * D2y[u]) / W[u]);
+                    }
+                }
+                pnew[u] = fma(tau, kick, pn[u]);
+                const R g2 = root(fma(pnew[u], pnew[u], q1));
+                dnew[u] = quotient(tau * (pn[u] + pnew[u]), g1 + g2);
+                if (!within(dnew[u], dlim)) { bad = bad || act[u]; dnew[u] = R(0); }
+                if (act[u]) {
+                    R inc = fabs(dnew[u] - dold[u]);
+                    if constexpr (Real<R>::fp32) inc *= approx_rcp(fmaxf(one, fabsf(dnew[u])));   // convergence metric only
+                    dmax = max_nonneg(dmax, inc);
                 }
             }
-            pnew = fma(tau, kick, pn);
-            const R g2 = sqrt_(fma(pnew, pnew, q1));
-            dnew = fdiv_(tau * (pn + pnew), g1 + g2);
-            if (!(fabs(dnew) <= dlim)) { bad = bad || act; dnew = R(0); }
         }
-
         // deposit of the path x^n -> x^(k+1); its end is the position finalize stores
-        {
-            int n;
-            R t1;
-            path_end(t0, dnew, n, t1);
-            deposit_paths<kWin1, K>(win, mom, M, act, amask, warp_unwrap_cell(cw, act, M), t0, n, t1);
-            if (++adds == kMaxLaneAdds) { win.flush(mom, M); adds = 0; }
-        }
-        if (act) {
-            dp[a] = dnew;
-            if constexpr (!PRE) {
-                pnp[a] = pnew;
-                R inc = fabs(dnew - dold);
-                if (Real<R>::fp32) inc = __fdividef(inc, fmax(one, fabs(dnew)));   // convergence metric only
-                dmax = (inc > dmax || inc != inc) ? inc : dmax;
+        int n1[U];
+        R ve[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            path_end(v0[u], dnew[u], n1[u], ve[u]);
+            if (act[u]) {
+                const long long a = s + 32 * u + lane;
+                dp[a] = dnew[u];
+                if constexpr (!PRE) pnp[a] = pnew[u];
             }
         }
+        dep.step(act, cw, n1, ve);
     }
-    win.flush(mom, M);
-    dmax_out = (double)dmax > dmax_out || dmax != dmax ? (double)dmax : dmax_out;
+    dep.flush();
+    dmax_out = max_nonneg(dmax_out, (double)dmax);
     bad_out = bad_out || bad;
 }
 
+template <int K, typename R, int ACC, bool PRE>
+__device__ __forceinline__ void sweep1_range(const Sweep1Args &A, long long beg, long long end, double &dmax, bool &bad)
+{
+    if (A.zforce || *reinterpret_cast<volatile const int *>(&A.ctrl->zany) != 0)
+        sweep1_range_z<K, R, ACC, PRE, true>(A, beg, end, dmax, bad);
+    else
+        sweep1_range_z<K, R, ACC, PRE, false>(A, beg, end, dmax, bad);
+}
+
 template <int K, typename R, int ACC>
-__global__ void __launch_bounds__(kSweepThreads, SweepOcc<R, K>::v1) k_sweep1(Sweep1Args A)
+__global__ void __launch_bounds__(SweepShape<R, K>::threads1, SweepShape<R, K>::blocks1) k_sweep1(Sweep1Args A)
 {
     long long wb, we;
     grid_warp_chunk(A.np, wb, we);
@@ -382,7 +407,7 @@ __global__ void __launch_bounds__(kSweepThreads, SweepOcc<R, K>::v1) k_sweep1(Sw
 // the starting field sets how far the first sweep's kick is off.
 // ---------------------------------------------------------------------------
 template <int K, typename R, int ACC>
-__global__ void __launch_bounds__(kSweepThreads, SweepOcc<R, K>::v1) k_predeposit(Sweep1Args A)
+__global__ void __launch_bounds__(SweepShape<R, K>::threads1, SweepShape<R, K>::blocks1) k_predeposit(Sweep1Args A)
 {
     long long wb, we;
     grid_warp_chunk(A.np, wb, we);
@@ -412,7 +437,7 @@ int launch_sweep1(const Sweep1Args &a, int grid, cudaStream_t s)
 {
 #define L1(KK, RR, AA)                                                                              \
     if (a.K == KK && (a.fp32 != 0) == std::is_same<RR, float>::value && a.acc == AA) {              \
-        k_sweep1<KK, RR, AA><<<grid, kSweepThreads, 0, s>>>(a);                                     \
+        k_sweep1<KK, RR, AA><<<grid, SweepShape<RR, KK>::threads1, 0, s>>>(a);                      \
         return 0;                                                                                   \
     }
     PIC_FOR_SWEEP_VARIANTS(L1)
@@ -427,63 +452,85 @@ int launch_sweep1(const Sweep1Args &a, int grid, cudaStream_t s)
 // basis value to a shared-memory row by a double atomic (a compare-and-swap loop) took
 // 4.2 ms for 1e7 markers; the register window takes 0.32 ms.
 // ---------------------------------------------------------------------------
+// The deposit is the path's pieces cell by cell, h S_m in each (displacements may be tiny
+// here, which the difference of the end points' moments would not resolve).
 template <int K, typename R>
 __global__ void __launch_bounds__(kSweepThreads) k_current(CurrentArgs A)
 {
     const int32_t *__restrict__ cp = A.P.cell;
     const int32_t *__restrict__ id = A.P.id;
-    const R *__restrict__ tp = static_cast<const R *>(A.P.t);
+    const R *__restrict__ vp = static_cast<const R *>(A.P.t);
     const int lane = threadIdx.x & 31, M = A.M;
     const double inv = 1.0 / A.dx;
+    const R half = R(0.5);
     long long wb, we;
     grid_warp_chunk(A.np, wb, we);
+    if (wb >= we) return;
     MomentWindow<kWin1, K, AccNative<double>> win;
-    win.start();
+    win.clear();
+    int base = cp[wb];
+    unsigned used = 0u;
     bool bad = false;
     for (long long s = wb; s < we; s += 32) {
         const long long a = s + lane;
         const bool act = a < we;
         const unsigned amask = __ballot_sync(0xffffffffu, act);
-        const int cw = act ? cp[a] : 0;
-        const R t0 = act ? tp[a] : R(0.5);
+        const int c = act ? cp[a] : 0;
+        const R v0 = act ? vp[a] : R(0);
         R d = act ? (R)(A.disp[id[a]] * inv) : R(0);
         if (!(fabs(d) <= (R)A.Dlim)) { bad = true; d = R(0); }
         int n;
-        R t1;
-        path_end(t0, d, n, t1);
-        const int c0 = warp_unwrap_cell(cw, act, M), c1 = c0 + n;
-        const int lo = min(c0, c1), hi = max(c0, c1);
-        const int nb = window_base<kWin1>(win.base, lo, hi, act, amask);
-        if (nb != win.base) win.move(nb, A.mom, M);
-        const bool in = act && lo >= win.base && hi < win.base + kWin1;
-        const int rlo = __reduce_min_sync(0xffffffffu, in ? lo - win.base : kWin1);
-        const int rhi = __reduce_max_sync(0xffffffffu, in ? hi - win.base : -1);
-        const int b0 = in ? c0 - win.base : 4 * kWin1, b1 = in ? c1 - win.base : 4 * kWin1;
+        R v1;
+        path_end(v0, d, n, v1);
+        int r0 = rel_cell(c, base, M), r1 = r0 + n;
+        bool in = act && (unsigned)r0 < (unsigned)kWin1 && (unsigned)r1 < (unsigned)kWin1;
+        if (__popc(__ballot_sync(0xffffffffu, act && !in)) > kWindowMisses) {
+            int off = window_move<kWin1>(min(r0, r1), min(r0, r1), act, amask);
+            if (off > 0 && off < kWin1) {
+                for (; off > 0; --off) {
+                    win.shift(A.mom, base, used);
+                    used >>= 1;
+                    base = base + 1 == M ? 0 : base + 1;
+                }
+            } else if (off != 0) {
+                win.flush(A.mom, base, used, M);
+                used = 0u;
+                base = wrap_cell(base + off, M);
+            }
+            r0 = rel_cell(c, base, M);
+            r1 = r0 + n;
+            in = act && (unsigned)r0 < (unsigned)kWin1 && (unsigned)r1 < (unsigned)kWin1;
+        }
+        const int lo = min(r0, r1), hi = max(r0, r1);
+        const unsigned mine = in ? (2u << hi) - (1u << lo) : 0u;
+        const unsigned mask = __reduce_or_sync(0xffffffffu, mine);
+        used |= mask;
 #pragma unroll
         for (int w = 0; w < kWin1; ++w) {
-            if (w >= rlo && w <= rhi) {
-                win.used |= 1u << w;
-                const R ta = clip_end(b0 - w, t0), tb = clip_end(b1 - w, t1);
-                R S[K];
-                path_sums<K, R>(ta - R(0.5), tb - R(0.5), S);
-                const R h = (n == 0 && in && b0 == w) ? d : tb - ta;
+            if (mask & (1u << w)) {
+                if (mine & (1u << w)) {
+                    const R va = r0 == w ? v0 : (r0 < w ? -half : half), vb = r1 == w ? v1 : (r1 < w ? -half : half);
+                    R x[K];
+                    piece_moments<K, R>(va, vb, n == 0 ? d : vb - va, x);
 #pragma unroll
-                for (int m = 0; m < K; ++m) win.acc[w][m].add((double)(m == 0 ? h : h * S[m]));
+                    for (int m = 0; m < K; ++m) win.acc[w][m].add((double)x[m]);
+                }
             }
         }
         if (act && !in) {
-            if (n == 0) {
-                R S[K];
-                path_sums<K, R>(t0 - R(0.5), t1 - R(0.5), S);
+            int g = c;
+            for (int q = 0; q <= abs(n); ++q) {
+                const R va = q == 0 ? v0 : (n > 0 ? -half : half);
+                const R vb = q == abs(n) ? v1 : (n > 0 ? half : -half);
+                R x[K];
+                piece_moments<K, R>(va, vb, n == 0 ? d : vb - va, x);
 #pragma unroll
-                for (int m = 0; m < K; ++m)
-                    atomicAdd(&A.mom[(size_t)cw * K + m], (double)(m == 0 ? d : d * S[m]));
-            } else {
-                deposit_path_global<K, R>(A.mom, M, c0, t0, c1, t1);
+                for (int m = 0; m < K; ++m) atomicAdd(&A.mom[(size_t)g * K + m], (double)x[m]);
+                g = wrap_once(g + (n > 0 ? 1 : -1), M);
             }
         }
     }
-    win.flush(A.mom, M);
+    win.flush(A.mom, base, used, M);
     if (bad) atomicOr(&A.ctrl->status, STATUS_NUMERIC);
 }
 
@@ -509,12 +556,11 @@ int launch_current(const CurrentArgs &a, int grid, cudaStream_t s)
 // Subsystem II: one fixed-point sweep (Sec. 4.2).  Markers frozen at x; with
 // A0 = A^n_h(x), A1 = A^(k)_h(x):
 //   s_i += w (A0 + A1) Lambda^0_i(x) / (g(p,A0) + g(p,A1))   (y and z),
-// deposited as the moments f v^m of each cell.  Same warp ranges as subsystem I.  From
-// basis values and node windows: 287 us in float (2e7 markers, 2048 cells, cubic), 413 us
-// in double (2e6 markers); from cell polynomials and moments 153 us and 166 us.
-// Z: the z component is not identically zero (a linearly polarised wave keeps
-// A_z = 0 exactly, and then neither its gathers nor its moments are needed).
-// ---------------------------------------------------------------------------
+// deposited as the moments f v^m of each cell.  Same warp ranges as subsystem I.
+// us a launch, float (1e8 markers, cubic) and double (1e7): basis values and node windows
+// 1260 and 2060, cell polynomials and moments 767 and 830, as here (centred offsets, the
+// short root and quotient, two markers a lane) 570 and 672.
+// Z: the z component is not identically zero, as in subsystem I.
 template <int K, typename R, int ACC, bool Z>
 __device__ __forceinline__ void sweep2_range_z(const Sweep2Args &A, long long beg, long long end, double *my, double *mz,
                                                bool first)
@@ -522,127 +568,177 @@ __device__ __forceinline__ void sweep2_range_z(const Sweep2Args &A, long long be
     constexpr int NC = K + 1;
     constexpr int PA = CoefPad<R, NC>::v;
     constexpr int NW = Z ? kWin2z : kWin2;
-    const R one = R(1), half = R(0.5);
+    constexpr int U = SweepU<R>::v;
+    const R one = R(1);
     const int M = A.M;
     const int32_t *__restrict__ cp = A.P.cell;
-    const R *__restrict__ tp = static_cast<const R *>(A.P.t);
+    const R *__restrict__ vp = static_cast<const R *>(A.P.t);
     const R *__restrict__ pp = static_cast<const R *>(A.P.p);
     const R *TA = static_cast<const R *>(A.T.A), *TK = static_cast<const R *>(A.T.Kt);
     const float *TL = A.T.L;
+    const bool cached = !Real<R>::fp32 && !first && A.a0 != nullptr;
+    const bool keep = !Real<R>::fp32 && first && A.a0 != nullptr;
     const int lane = threadIdx.x & 31;
+    if (beg >= end) return;
     using Acc = typename AccOf<R, ACC>::T;
     MomentWindow<NW, NC, Acc> wy, wz;
-    wy.start();
-    if (Z) wz.start();
-    int adds = 0;
-    int nc = 0;
-    R nt = half, npn = R(0);
+    wy.clear();
+    if (Z) wz.clear();
+    int base = cp[beg], adds = 0;
+    unsigned used = 0u;
+    auto flush = [&]() {
+        wy.flush(my, base, used, M);
+        if (Z) wz.flush(mz, base, used, M);
+        used = 0u;
+        adds = 0;
+    };
+    int nc[U];
+    R nv[U], npn[U];
     auto fetch = [&](long long s) {
-        const long long a = s + lane;
-        if (a < end) {
-            nc = cp[a];
-            nt = tp[a];
-            npn = pp[a];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const long long a = s + 32 * u + lane;
+            if (a < end) {
+                nc[u] = cp[a];
+                nv[u] = vp[a];
+                npn[u] = pp[a];
+            }
         }
     };
-    if (beg < end) fetch(beg);
-    for (long long s = beg; s < end; s += 32) {
-        const long long a = s + lane;
-        const bool act = a < end;
-        const unsigned amask = __ballot_sync(0xffffffffu, act);
-        const int cw = nc;
-        const R v = nt - half, p = npn;
-        if (s + 32 < end) fetch(s + 32);
-        const R pp1 = fma(p, p, one);
-        const size_t row = (size_t)cw * (2 * PA);
-        R A0y, A1y, A0z = R(0), A1z = R(0), Ly = R(0), Lz = R(0), g0;
-        bool cached = false;
-        if constexpr (!Real<R>::fp32) cached = !first && A.a0 != nullptr;
-        if (cached) {
-            if constexpr (!Real<R>::fp32) {
-                if (act) start_cache_load(A.a0, a, A0y, A0z, g0);
-                else { A0y = R(0); g0 = one; }
-            }
-        } else {
+#pragma unroll
+    for (int u = 0; u < U; ++u) { nc[u] = 0; nv[u] = R(0); npn[u] = R(0); }
+    fetch(beg);
+    for (long long s = beg; s < end; s += 32 * U) {
+        bool act[U], in[U];
+        int cw[U], rel[U], miss = 0;
+        R v[U], p[U], fy[U], fz[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            act[u] = s + 32 * u + lane < end;
+            cw[u] = nc[u];
+            v[u] = nv[u];
+            p[u] = npn[u];
+        }
+        if (s + 32 * U < end) fetch(s + 32 * U);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const R pp1 = fma(p[u], p[u], one);
+            const size_t row = (size_t)cw[u] * (2 * PA);
+            R A0y, A1y, A0z = R(0), A1z = R(0), g0;
             R c[NC];
-            load_coef<NC>(TA + row, c);
-            A0y = horner<NC>(c, v);
-            R q = fma(A0y, A0y, pp1);
-            if (Z) {
-                load_coef<NC>(TA + row + PA, c);
-                A0z = horner<NC>(c, v);
-                q = fma(A0z, A0z, q);
+            if (cached) {
+                if constexpr (!Real<R>::fp32) {
+                    A0y = R(0);
+                    g0 = one;
+                    if (act[u]) start_cache_load<Z>(A.a0, s + 32 * u + lane, A0y, A0z, g0);
+                }
+            } else {
+                load_coef<NC>(TA + row, c);
+                A0y = horner<NC>(c, v[u]);
+                R q = fma(A0y, A0y, pp1);
+                if (Z) {
+                    load_coef<NC>(TA + row + PA, c);
+                    A0z = horner<NC>(c, v[u]);
+                    q = fma(A0z, A0z, q);
+                }
+                g0 = root(q);
+                if constexpr (!Real<R>::fp32)
+                    if (keep && act[u]) start_cache_store<Z>(A.a0, s + 32 * u + lane, A0y, A0z, g0);
             }
-            g0 = sqrt_(q);
-            if constexpr (!Real<R>::fp32)
-                if (A.a0 && act) start_cache_store(A.a0, a, A0y, A0z, g0);
-        }
-        R c[NC];
-        load_coef<NC>(TK + row, c);
-        A1y = horner<NC>(c, v);
-        R q1 = fma(A1y, A1y, pp1);
-        if (Z) {
-            load_coef<NC>(TK + row + PA, c);
-            A1z = horner<NC>(c, v);
-            q1 = fma(A1z, A1z, q1);
-        }
-        const R g1 = sqrt_(q1);
-        if constexpr (Real<R>::fp32) {
-            // The float rounding of a coefficient is the same for every marker of its
-            // cell, so it does not average out over markers: in the exchange term
-            // (A1 - A0)(A1 + A0)/(g0 + g1) it shows as an energy error of about 1e-11
-            // per step.  The residues of the sum a^n + a^(k) enter the numerator before
-            // its one rounding, which leaves only per-marker rounding.
-            load_coef<NC>(TL + row, c);
-            Ly = horner<NC>(c, v);
+            load_coef<NC>(TK + row, c);
+            A1y = horner<NC>(c, v[u]);
+            R q1 = fma(A1y, A1y, pp1);
             if (Z) {
-                load_coef<NC>(TL + row + PA, c);
-                Lz = horner<NC>(c, v);
+                load_coef<NC>(TK + row + PA, c);
+                A1z = horner<NC>(c, v[u]);
+                q1 = fma(A1z, A1z, q1);
+            }
+            const R cf = quotient(one, g0 + root(q1));
+            const R sy = A0y + A1y, sz = A0z + A1z;
+            if constexpr (Real<R>::fp32) {
+                // The float rounding of a coefficient is the same for every marker of its
+                // cell, so it does not average out over markers: in the exchange term
+                // (A1 - A0)(A1 + A0)/(g0 + g1) it shows as an energy error of about 1e-11
+                // per step.  The residues L of the sum a^n + a^(k) enter before its one
+                // rounding, which leaves only per-marker rounding: f = cf (s + L) rounded
+                // once, with the product's own rounding error (exact by an fma) and cf L
+                // added to it (L is far below half an ulp of s).
+                load_coef<NC>(TL + row, c);
+                const float py = cf * sy;
+                fy[u] = py + fmaf(cf, horner<NC>(c, v[u]), fmaf(cf, sy, -py));
+                if (Z) {
+                    load_coef<NC>(TL + row + PA, c);
+                    const float pz = cf * sz;
+                    fz[u] = pz + fmaf(cf, horner<NC>(c, v[u]), fmaf(cf, sz, -pz));
+                }
+            } else {
+                fy[u] = cf * sy;
+                if (Z) fz[u] = cf * sz;
+            }
+            rel[u] = rel_cell(cw[u], base, M);
+            in[u] = act[u] && (unsigned)rel[u] < (unsigned)NW;
+            miss += __popc(__ballot_sync(0xffffffffu, act[u] && !in[u]));
+        }
+        if (miss > kWindowMisses) {
+            int lo = INT_MAX;
+#pragma unroll
+            for (int u = 0; u < U; ++u) lo = act[u] ? min(lo, rel[u]) : lo;
+            const unsigned amask = __ballot_sync(0xffffffffu, act[0]);
+            int off = window_move<NW>(lo, rel[0], act[0], amask);
+            if (off > 0 && off < NW) {
+                for (; off > 0; --off) {
+                    wy.shift(my, base, used);
+                    if (Z) wz.shift(mz, base, used);
+                    used >>= 1;
+                    base = base + 1 == M ? 0 : base + 1;
+                }
+            } else if (off != 0) {
+                flush();
+                base = wrap_cell(base + off, M);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                rel[u] = rel_cell(cw[u], base, M);
+                in[u] = act[u] && (unsigned)rel[u] < (unsigned)NW;
             }
         }
-        const R cf = fdiv_(one, g0 + g1);
-        const R sy = A0y + A1y, sz = A0z + A1z;
-        R fy, fz = R(0);
-        if constexpr (Real<R>::fp32) {
-            // f = cf (s + L) rounded once: the residue L is far below half an ulp of s,
-            // so s + L in float would drop it.  The product's own rounding error (exact
-            // by an fma) and cf L are added before the one rounding.
-            const float py = cf * sy;
-            fy = py + (fmaf(cf, sy, -py) + cf * Ly);
-            if (Z) {
-                const float pz = cf * sz;
-                fz = pz + (fmaf(cf, sz, -pz) + cf * Lz);
+        unsigned bits = 0u;
+#pragma unroll
+        for (int u = 0; u < U; ++u) bits |= in[u] ? 1u << rel[u] : 0u;
+        const unsigned mask = __reduce_or_sync(0xffffffffu, bits);
+        used |= mask;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            R x[NC], pw = one;
+            x[0] = fy[u];
+            R pws[NC];
+            pws[0] = one;
+#pragma unroll
+            for (int m = 1; m < NC; ++m) { pw = m == 1 ? v[u] : pw * v[u]; pws[m] = pw; x[m] = fy[u] * pw; }
+            const int r = in[u] ? rel[u] : -1;
+            wy.add(mask, r, x);
+            if (act[u] && !in[u]) {
+                double *dst = my + (size_t)cw[u] * NC;
+#pragma unroll
+                for (int m = 0; m < NC; ++m)
+                    if (x[m] != R(0)) atomicAdd(&dst[m], (double)x[m]);
             }
-        } else {
-            fy = cf * sy;
-            fz = cf * sz;
-        }
-        const int cu = warp_unwrap_cell(cw, act, M);
-        const int nb = window_base<NW>(wy.base, cu, cu, act, amask);
-        if (nb != wy.base) {
-            wy.move(nb, my, M);
-            if (Z) wz.move(nb, mz, M);
-        }
-        R x[NC], pw[NC];
-        pw[0] = one;
+            if (Z) {
+                x[0] = fz[u];
 #pragma unroll
-        for (int m = 1; m < NC; ++m) pw[m] = pw[m - 1] * v;
+                for (int m = 1; m < NC; ++m) x[m] = fz[u] * pws[m];
+                wz.add(mask, r, x);
+                if (act[u] && !in[u]) {
+                    double *dst = mz + (size_t)cw[u] * NC;
 #pragma unroll
-        for (int m = 0; m < NC; ++m) x[m] = m == 0 ? fy : fy * pw[m];
-        deposit_points<NW, NC>(wy, my, M, act, cu, x);
-        if (Z) {
-#pragma unroll
-            for (int m = 0; m < NC; ++m) x[m] = m == 0 ? fz : fz * pw[m];
-            deposit_points<NW, NC>(wz, mz, M, act, cu, x);
+                    for (int m = 0; m < NC; ++m)
+                        if (x[m] != R(0)) atomicAdd(&dst[m], (double)x[m]);
+                }
+            }
         }
-        if (++adds == kMaxLaneAdds) {
-            wy.flush(my, M);
-            if (Z) wz.flush(mz, M);
-            adds = 0;
-        }
+        if (++adds == kMaxLaneAdds / U) flush();
     }
-    wy.flush(my, M);
-    if (Z) wz.flush(mz, M);
+    flush();
 }
 
 template <int K, typename R, int ACC>
@@ -663,7 +759,7 @@ __device__ __forceinline__ void sweep2_range(const Sweep2Args &A, long long beg,
 }
 
 template <int K, typename R, int ACC>
-__global__ void __launch_bounds__(kSweepThreads, SweepOcc<R, K>::v2) k_sweep2(Sweep2Args A)
+__global__ void __launch_bounds__(SweepShape<R, K>::threads2, SweepShape<R, K>::blocks2) k_sweep2(Sweep2Args A)
 {
     long long wb, we;
     grid_warp_chunk(A.np, wb, we);
@@ -682,7 +778,7 @@ int launch_predeposit(const Sweep1Args &a, int grid, cudaStream_t s)
 {
 #define LP(KK, RR, AA)                                                                              \
     if (a.K == KK && (a.fp32 != 0) == std::is_same<RR, float>::value) {                             \
-        k_predeposit<KK, RR, AA><<<grid, kSweepThreads, 0, s>>>(a);                                 \
+        k_predeposit<KK, RR, AA><<<grid, SweepShape<RR, KK>::threads1, 0, s>>>(a);                  \
         return 0;                                                                                   \
     }
     PIC_FOR_PREDEPOSIT_VARIANTS(LP)
@@ -694,7 +790,7 @@ int launch_sweep2(const Sweep2Args &a, int grid, cudaStream_t s)
 {
 #define L2(KK, RR, AA)                                                                              \
     if (a.K == KK && (a.fp32 != 0) == std::is_same<RR, float>::value && a.acc == AA) {              \
-        k_sweep2<KK, RR, AA><<<grid, kSweepThreads, 0, s>>>(a);                                     \
+        k_sweep2<KK, RR, AA><<<grid, SweepShape<RR, KK>::threads2, 0, s>>>(a);                      \
         return 0;                                                                                   \
     }
     PIC_FOR_SWEEP_VARIANTS(L2)
@@ -710,27 +806,52 @@ template <int K, typename R>
 __global__ void __launch_bounds__(kSweepThreads) k_charge(DiagArgs A)
 {
     const int32_t *__restrict__ cp = A.P.cell;
-    const R *__restrict__ tp = static_cast<const R *>(A.P.t);
+    const R *__restrict__ vp = static_cast<const R *>(A.P.t);
     const int lane = threadIdx.x & 31, M = A.M;
     long long wb, we;
     grid_warp_chunk(A.np, wb, we);
+    if (wb >= we) return;
     MomentWindow<kWin2, K + 1, AccNative<double>> win;
-    win.start();
+    win.clear();
+    int base = cp[wb];
+    unsigned used = 0u;
     for (long long s = wb; s < we; s += 32) {
         const long long a = s + lane;
         const bool act = a < we;
         const unsigned amask = __ballot_sync(0xffffffffu, act);
-        const int c = warp_unwrap_cell(act ? cp[a] : 0, act, M);
-        const double v = act ? (double)tp[a] - 0.5 : 0.0;
-        const int nb = window_base<kWin2>(win.base, c, c, act, amask);
-        if (nb != win.base) win.move(nb, A.mom, M);
+        const int c = act ? cp[a] : 0;
+        const double v = act ? (double)vp[a] : 0.0;
+        int rel = rel_cell(c, base, M);
+        bool in = act && (unsigned)rel < (unsigned)kWin2;
+        if (__popc(__ballot_sync(0xffffffffu, act && !in)) > kWindowMisses) {
+            int off = window_move<kWin2>(rel, rel, act, amask);
+            if (off > 0 && off < kWin2) {
+                for (; off > 0; --off) {
+                    win.shift(A.mom, base, used);
+                    used >>= 1;
+                    base = base + 1 == M ? 0 : base + 1;
+                }
+            } else if (off != 0) {
+                win.flush(A.mom, base, used, M);
+                used = 0u;
+                base = wrap_cell(base + off, M);
+            }
+            rel = rel_cell(c, base, M);
+            in = act && (unsigned)rel < (unsigned)kWin2;
+        }
+        const unsigned mask = __reduce_or_sync(0xffffffffu, in ? 1u << rel : 0u);
+        used |= mask;
         double x[K + 1];
         x[0] = 1.0;
 #pragma unroll
-        for (int m = 1; m <= K; ++m) x[m] = x[m - 1] * v;
-        deposit_points<kWin2, K + 1>(win, A.mom, M, act, c, x);
+        for (int m = 1; m <= K; ++m) x[m] = m == 1 ? v : x[m - 1] * v;
+        win.add(mask, in ? rel : -1, x);
+        if (act && !in) {
+#pragma unroll
+            for (int m = 0; m <= K; ++m) atomicAdd(&A.mom[(size_t)c * (K + 1) + m], x[m]);
+        }
     }
-    win.flush(A.mom, M);
+    win.flush(A.mom, base, used, M);
 }
 
 // A.tab: the field's polynomial of each cell in double (launch_cell_coefs)
@@ -742,7 +863,7 @@ __global__ void __launch_bounds__(256) k_gather(DiagArgs A)
     for (long long a = (long long)blockIdx.x * blockDim.x + threadIdx.x; a < A.np; a += stride) {
         double c[D + 1];
         load_coef<D + 1>(A.tab + (size_t)A.P.cell[a] * CoefPad<double, D + 1>::v, c);
-        A.out[A.P.id[a]] = horner<D + 1>(c, (double)tp[a] - 0.5);
+        A.out[A.P.id[a]] = horner<D + 1>(c, (double)tp[a]);
     }
 }
 
@@ -757,7 +878,7 @@ __global__ void __launch_bounds__(256) k_kinetic(DiagArgs A)
     for (long long a = (long long)blockIdx.x * blockDim.x + threadIdx.x; a < A.np; a += stride) {
         const int c = A.P.cell[a];
         double v[K + 1];
-        bspline_vals<K, double>((double)tp[a], v);
+        bspline_vals<K, double>((double)tp[a] + 0.5, v);
         double Ay = 0.0, Az = 0.0;
 #pragma unroll
         for (int r = 0; r <= K; ++r) {
@@ -828,27 +949,26 @@ __global__ void __launch_bounds__(256) k_gather_path(DiagArgs A)
         const int id = A.P.id[a];
         const double d = A.out[id] * inv;
         if (!(fabs(d) <= (double)A.Dlim)) { bad = true; A.out[id] = 0.0; continue; }
-        const double t0 = (double)tp[a];
+        const double v0 = (double)tp[a];
         int n;
-        double t1;
-        path_end(t0, d, n, t1);
+        double v1;
+        path_end(v0, d, n, v1);
         const int an = abs(n);
         const bool right = n > 0;
         double sum = 0.0, W = 0.0;
         for (int q = 0; q <= an; ++q) {
-            const double ta = q == 0 ? t0 : (right ? 0.0 : 1.0);
-            const double tb = q == an ? t1 : (right ? 1.0 : 0.0);
+            const double va = q == 0 ? v0 : (right ? -0.5 : 0.5);
+            const double vb = q == an ? v1 : (right ? 0.5 : -0.5);
             double S[K], c[K];
-            path_sums<K, double>(ta - 0.5, tb - 0.5, S);
+            path_sums<K, double>(va, vb, S);
             load_coef<K>(A.tab + (size_t)g * PE, c);
             double e = c[0];
 #pragma unroll
             for (int m = 1; m < K; ++m) e = fma(c[m], S[m], e);
-            const double h = an == 0 ? 1.0 : tb - ta;
+            const double h = an == 0 ? 1.0 : vb - va;
             sum = fma(h, e, sum);
             W += h;
-            g += right ? 1 : -1;
-            g = g >= A.M ? g - A.M : (g < 0 ? g + A.M : g);
+            g = wrap_once(g + (right ? 1 : -1), A.M);
         }
         A.out[id] = an == 0 ? sum : sum / W;
     }
@@ -862,10 +982,10 @@ __global__ void __launch_bounds__(256) k_gather_path(DiagArgs A)
 // ---------------------------------------------------------------------------
 // dA/dx at a marker: sum_i (G a)_i Lambda^1_i(x), (G a)_i = (a_i - a_{i-1}) / dx
 template <int K>
-__device__ __forceinline__ void spin_field_grad(const SpinArgs &A, int c, double t, double &Y, double &Z)
+__device__ __forceinline__ void spin_field_grad(const SpinArgs &A, int c, double off, double &Y, double &Z)
 {
     double v[K];
-    bspline_vals<K - 1, double>(t, v);
+    bspline_vals<K - 1, double>(off + 0.5, v);
     Y = 0.0;
     Z = 0.0;
 #pragma unroll
@@ -891,7 +1011,7 @@ __global__ void __launch_bounds__(256) k_spin_deposit(SpinArgs A)
         const int c = A.P.cell[a];
         const int id = A.P.id[a];
         double v[K];
-        bspline_vals<K - 1, double>(tp[a], v);
+        bspline_vals<K - 1, double>(tp[a] + 0.5, v);
         const double wy = A.w * A.sy[id], wz = A.w * A.sz[id];
 #pragma unroll
         for (int r = 0; r < K; ++r) {
@@ -1027,13 +1147,11 @@ __device__ __forceinline__ void finalize1_range(long long np, int M, const PartP
     R *dp = static_cast<R *>(P.delta);
     const R *pnp = static_cast<const R *>(P.pnew);
     for (long long a = a0; a < np; a += stride) {
-        const R s = tp[a] + dp[a];
-        const R f = floor_(s);
-        int c = P.cell[a] + (int)f;
-        R t = s - f;
-        if (t >= R(1)) { t -= R(1); c += 1; }
-        P.cell[a] = wrap_cell(c, M);
-        tp[a] = t;
+        int n;
+        R v;
+        path_end(tp[a], dp[a], n, v);
+        P.cell[a] = wrap_cell(P.cell[a] + n, M);
+        tp[a] = v;
         pp[a] = pnp[a];
         if (zero_delta) dp[a] = R(0);
     }
@@ -1069,11 +1187,8 @@ __global__ void __launch_bounds__(256) k_load(long long np, int M, double dx, co
     for (long long a = (long long)blockIdx.x * blockDim.x + threadIdx.x; a < np; a += stride) {
         const double u = x[a] / dx;
         const double f = ::floor(u);
-        int c = (int)f;
-        R t = (R)(u - f);
-        if (t >= R(1)) { t = R(0); c += 1; }
-        P.cell[a] = wrap_cell(c, M);
-        tp[a] = t;
+        P.cell[a] = wrap_cell((int)f, M);
+        tp[a] = (R)((u - f) - 0.5);
         pp[a] = (R)p[a];
         pnp[a] = (R)p[a];
         dp[a] = R(0);
@@ -1089,24 +1204,33 @@ int launch_load(int fp32, long long np, int M, double dx, const double *x, const
     return 0;
 }
 
+// position of a marker in [0, L): the centre of its cell plus its offset (an offset of a
+// whole half cell may reach L)
 template <typename R>
-__global__ void __launch_bounds__(256) k_store(long long np, double dx, PartPtrs P, double *x, double *p)
+__device__ __forceinline__ double position(int c, R v, double dx, double L)
+{
+    const double x = (((double)c + 0.5) + (double)v) * dx;
+    return x >= L ? x - L : x;
+}
+
+template <typename R>
+__global__ void __launch_bounds__(256) k_store(long long np, int M, double dx, PartPtrs P, double *x, double *p)
 {
     const R *tp = static_cast<const R *>(P.t);
     const R *pp = static_cast<const R *>(P.p);
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long a = (long long)blockIdx.x * blockDim.x + threadIdx.x; a < np; a += stride) {
         const long long i = P.id[a];
-        if (x) x[i] = ((double)P.cell[a] + (double)tp[a]) * dx;
+        if (x) x[i] = position(P.cell[a], tp[a], dx, M * dx);
         if (p) p[i] = (double)pp[a];
     }
 }
 
-int launch_store(int fp32, long long np, double dx, PartPtrs P, double *x, double *p,
+int launch_store(int fp32, long long np, int M, double dx, PartPtrs P, double *x, double *p,
                  int grid, int block, cudaStream_t s)
 {
-    if (fp32) k_store<float><<<grid, block, 0, s>>>(np, dx, P, x, p);
-    else k_store<double><<<grid, block, 0, s>>>(np, dx, P, x, p);
+    if (fp32) k_store<float><<<grid, block, 0, s>>>(np, M, dx, P, x, p);
+    else k_store<double><<<grid, block, 0, s>>>(np, M, dx, P, x, p);
     return 0;
 }
 
@@ -1123,7 +1247,7 @@ __global__ void __launch_bounds__(256) k_inverse_id(long long np, const int32_t 
 // consecutive, so the destination may be page-locked host memory written over the host
 // link (the same values as k_store)
 template <typename R>
-__global__ void __launch_bounds__(256) k_store_ordered(long long np, double dx, PartPtrs P,
+__global__ void __launch_bounds__(256) k_store_ordered(long long np, int M, double dx, PartPtrs P,
                                                        const int32_t *__restrict__ inv, double *x, double *p)
 {
     const R *tp = static_cast<const R *>(P.t);
@@ -1131,17 +1255,17 @@ __global__ void __launch_bounds__(256) k_store_ordered(long long np, double dx, 
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < np; i += stride) {
         const long long a = inv[i];
-        if (x) x[i] = ((double)P.cell[a] + (double)tp[a]) * dx;
+        if (x) x[i] = position(P.cell[a], tp[a], dx, M * dx);
         if (p) p[i] = (double)pp[a];
     }
 }
 
-int launch_store_ordered(int fp32, long long np, double dx, PartPtrs P, int32_t *inv, double *x, double *p,
+int launch_store_ordered(int fp32, long long np, int M, double dx, PartPtrs P, int32_t *inv, double *x, double *p,
                          int grid, int block, cudaStream_t s)
 {
     k_inverse_id<<<grid, block, 0, s>>>(np, P.id, inv);
-    if (fp32) k_store_ordered<float><<<grid, block, 0, s>>>(np, dx, P, inv, x, p);
-    else k_store_ordered<double><<<grid, block, 0, s>>>(np, dx, P, inv, x, p);
+    if (fp32) k_store_ordered<float><<<grid, block, 0, s>>>(np, M, dx, P, inv, x, p);
+    else k_store_ordered<double><<<grid, block, 0, s>>>(np, M, dx, P, inv, x, p);
     return 0;
 }
 
@@ -1359,15 +1483,15 @@ __device__ __forceinline__ bool ens_claim(EnsQueue *Q, const Args *runs, int nru
     const long long im = Q->item_markers;
     const long long ib = (long long)(item - Q->item_start[run]) * im;
     const long long ie = ib + im < runs[run].np ? ib + im : runs[run].np;
-    warp_chunk(ib, ie, threadIdx.x >> 5, kSweepWarps, beg, end);
+    warp_chunk(ib, ie, threadIdx.x >> 5, blockDim.x >> 5, beg, end);
     return true;
 }
 
 template <int K, typename R>
-__global__ void __launch_bounds__(kSweepThreads, SweepOcc<R, K>::v1)
+__global__ void __launch_bounds__(SweepShape<R, K>::threads1, SweepShape<R, K>::blocks1)
     k_sweep1_ens(const Sweep1Args *runs, int nruns, EnsQueue *Q)
 {
-    if ((int)blockIdx.x >= Q->nblocks) return;
+    if (blockIdx.x * Q->shares >= gridDim.x * Q->share) return;
     int run;
     long long beg, end;
     while (ens_claim(Q, runs, nruns, run, beg, end)) {
@@ -1381,10 +1505,10 @@ __global__ void __launch_bounds__(kSweepThreads, SweepOcc<R, K>::v1)
 
 // the predicted start of every run (sweep1_range's PRE mode over the work queue)
 template <int K, typename R>
-__global__ void __launch_bounds__(kSweepThreads, SweepOcc<R, K>::v1)
+__global__ void __launch_bounds__(SweepShape<R, K>::threads1, SweepShape<R, K>::blocks1)
     k_predeposit_ens(const Sweep1Args *runs, int nruns, EnsQueue *Q)
 {
-    if ((int)blockIdx.x >= Q->nblocks) return;
+    if (blockIdx.x * Q->shares >= gridDim.x * Q->share) return;
     int run;
     long long beg, end;
     while (ens_claim(Q, runs, nruns, run, beg, end)) {
@@ -1396,10 +1520,10 @@ __global__ void __launch_bounds__(kSweepThreads, SweepOcc<R, K>::v1)
 }
 
 template <int K, typename R>
-__global__ void __launch_bounds__(kSweepThreads, SweepOcc<R, K>::v2)
+__global__ void __launch_bounds__(SweepShape<R, K>::threads2, SweepShape<R, K>::blocks2)
     k_sweep2_ens(const Sweep2Args *runs, int nruns, EnsQueue *Q)
 {
-    if ((int)blockIdx.x >= Q->nblocks) return;
+    if (blockIdx.x * Q->shares >= gridDim.x * Q->share) return;
     int run;
     long long beg, end;
     while (ens_claim(Q, runs, nruns, run, beg, end)) sweep2_range<K, R, DefaultAcc<R>::v>(runs[run], beg, end);
@@ -1408,13 +1532,14 @@ __global__ void __launch_bounds__(kSweepThreads, SweepOcc<R, K>::v2)
 template <typename R>
 static int launch_sweep_ens_t(int which, int K, const void *runs, int nruns, EnsQueue *Q, int grid, cudaStream_t s)
 {
-    const int b = kSweepThreads;
 #define ENS(KK)                                                                                          \
-    case KK:                                                                                             \
-        if (which == 1) k_sweep1_ens<KK, R><<<grid, b, 0, s>>>((const Sweep1Args *)runs, nruns, Q);      \
-        else if (which == 2) k_sweep2_ens<KK, R><<<grid, b, 0, s>>>((const Sweep2Args *)runs, nruns, Q); \
-        else k_predeposit_ens<KK, R><<<grid, b, 0, s>>>((const Sweep1Args *)runs, nruns, Q);             \
-        break;
+    case KK: {                                                                                           \
+        constexpr int b1 = SweepShape<R, KK>::threads1, b2 = SweepShape<R, KK>::threads2;                \
+        if (which == 1) k_sweep1_ens<KK, R><<<grid, b1, 0, s>>>((const Sweep1Args *)runs, nruns, Q);     \
+        else if (which == 2) k_sweep2_ens<KK, R><<<grid, b2, 0, s>>>((const Sweep2Args *)runs, nruns, Q); \
+        else k_predeposit_ens<KK, R><<<grid, b1, 0, s>>>((const Sweep1Args *)runs, nruns, Q);            \
+        break;                                                                                           \
+    }
     switch (K) {
     ENS(2) ENS(3) ENS(4) ENS(5)
     default: return 1;
@@ -1487,8 +1612,8 @@ int sweep_blocks_per_sm(int K, int fp32, int acc, int which)
     cudaError_t e = cudaErrorInvalidValue;
 #define OCC(KK, RR, AA)                                                                                   \
     if (K == KK && (fp32 != 0) == std::is_same<RR, float>::value && acc == AA)                           \
-        e = which == 1 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sweep1<KK, RR, AA>, kSweepThreads, 0) \
-                       : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sweep2<KK, RR, AA>, kSweepThreads, 0);
+        e = which == 1 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sweep1<KK, RR, AA>, SweepShape<RR, KK>::threads1, 0) \
+                       : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_sweep2<KK, RR, AA>, SweepShape<RR, KK>::threads2, 0);
     PIC_FOR_SWEEP_VARIANTS(OCC)
 #undef OCC
     return e == cudaSuccess ? n : 0;
