@@ -365,8 +365,9 @@ extern "C" int pic_ensemble_create(const pic_config *cfgs, const pic_arrays *ins
     e->K = h0->K;
     e->fp32 = h0->fp32;
     e->num_sms = h0->num_sms;
-    long long npmax = 0;
+    long long npmax = 0, total = 0;
     for (pic_handle *h : e->runs) {
+        total += h->np;
         e->Mmax = std::max(e->Mmax, h->M);
         e->ntap1 = std::max(e->ntap1, h->tapM1_n);
         e->ntap2 = std::max(e->ntap2, h->tapP_n);
@@ -381,6 +382,10 @@ extern "C" int pic_ensemble_create(const pic_config *cfgs, const pic_arrays *ins
         e->grid2 = e->num_sms * std::max(1, b2);
         e->bps = e->bps_max;
     }
+    // about a dozen items a block of sweep I, so that the last items to be claimed end close
+    // together (64 runs, 1.4e7 markers: 2.6 ms a step at 4096 markers an item, 2.8 at 8192,
+    // 3.1 at 16384, 7.0 at 65536); fewer markers would cost a window flush per few steps
+    e->item_markers = (int)std::min<long long>(65536, std::max<long long>(2048, (total / (12LL * e->grid1) + 1023) / 1024 * 1024));
     // sort blocks a run: about four sweeps of 256 markers a block for the largest
     e->sort_grid = (int)std::min<long long>(std::max<long long>((npmax + 1023) / 1024, 1), 4LL * e->num_sms);
     const size_t n = (size_t)nruns;
@@ -557,7 +562,7 @@ extern "C" int pic_ensemble_tune(pic_ensemble *e, const char *cache_path, int32_
     long long np_total = 0;
     for (pic_handle *h : e->runs) np_total += h->np;
     std::vector<std::pair<int, int>> cands;
-    for (int im : {16384, 65536, 262144})
+    for (int im : {4096, 16384, 65536, 262144})
         for (int b = 1; b <= e->bps_max; ++b) cands.push_back({im, b});
     cudaEvent_t t0, t1;
     ECK(cudaEventCreate(&t0));
