@@ -1166,10 +1166,40 @@ extern "C" int pic_get_state(pic_handle *h, const pic_arrays *o, int32_t mem)
     if (mem != PIC_MEM_HOST && mem != PIC_MEM_DEVICE) return fail(h, PIC_ERR_INVALID, "bad mem");
     const size_t np = (size_t)h->np, M = (size_t)h->M;
     const bool host = mem == PIC_MEM_HOST;
+    if (!host) {
+        // device arrays: one launch, or for many markers the two passes of the dealt store
+        // (through the marker copy not in use) beside it
+        StateOut so{};
+        const bool deal = h->np > kDealMarkers && (o->x || o->p);
+        if (deal) {
+            if (launch_store_dealt(h->fp32, h->np, h->M, h->dx, cur_parts(h), h->Pblk[1 - h->cur], h->counts, o->x, o->p,
+                                   h->stream))
+                return fail(h, PIC_ERR_CUDA, "get_state: launch setup failed");
+            CKL_N("launch_store_dealt");
+            h->launches += 2;
+        } else {
+            so.x = o->x;
+            so.p = o->p;
+        }
+        auto add = [&](double *dst, const double *src, size_t len) {
+            if (!dst) return;
+            so.dst[so.n] = dst; so.src[so.n] = src; so.len[so.n] = (long long)len;
+            ++so.n;
+        };
+        add(o->ex, h->ex, M); add(o->ey, h->ey, M); add(o->ez, h->ez, M); add(o->ay, h->ay, M); add(o->az, h->az, M);
+        if (h->cfg.hbar != 0.0) { add(o->sx, h->spx, np); add(o->sy, h->spy, np); add(o->sz, h->spz, np); }
+        if (so.x || so.p || so.n) {
+            const long long most = std::max<long long>(deal ? 0 : h->np, h->cfg.hbar != 0.0 ? h->np : h->M);
+            const int grid = (int)std::min<long long>(particle_grid(h) * 2, (most + 255) / 256);
+            launch_store_state(h->fp32, h->np, h->M, h->dx, cur_parts(h), so, grid, 256, h->stream);
+            CKL_N("launch_store_state");
+        }
+        return sync(h);
+    }
     // page-locked host arrays: written in caller order over the host link by one
     // kernel, through the inverse of the markers' permutation (in the other marker copy)
-    double *px = (host && o->x) ? static_cast<double *>(const_cast<void *>(pinned_device_ptr(o->x))) : nullptr;
-    double *pp = (host && o->p) ? static_cast<double *>(const_cast<void *>(pinned_device_ptr(o->p))) : nullptr;
+    double *px = o->x ? static_cast<double *>(const_cast<void *>(pinned_device_ptr(o->x))) : nullptr;
+    double *pp = o->p ? static_cast<double *>(const_cast<void *>(pinned_device_ptr(o->p))) : nullptr;
     if ((o->x || o->p) && (!o->x || px) && (!o->p || pp)) {
         int32_t *inv = reinterpret_cast<int32_t *>(h->Pblk[1 - h->cur]);
         launch_store_ordered(h->fp32, h->np, h->M, h->dx, cur_parts(h), inv, px, pp, particle_grid(h), 256, h->stream);
@@ -1178,13 +1208,13 @@ extern "C" int pic_get_state(pic_handle *h, const pic_arrays *o, int32_t mem)
         if (e != cudaSuccess) return fail(h, PIC_ERR_CUDA, "get_state: %s", cudaGetErrorString(e));
         h->launches += 2;
     } else if (o->x || o->p) {
-        double *dx_out = o->x, *dp_out = o->p;
+        double *dx_out = nullptr, *dp_out = nullptr;
         // the store writes each marker to its input position (a permutation after the
         // sorts): scattered there in device memory, then copied to the host in bulk
-        if (host) stage_doubles(h, 1 - h->cur, o->x ? &dx_out : nullptr, o->p ? &dp_out : nullptr);
+        stage_doubles(h, 1 - h->cur, o->x ? &dx_out : nullptr, o->p ? &dp_out : nullptr);
         launch_store(h->fp32, h->np, h->M, h->dx, cur_parts(h), dx_out, dp_out, particle_grid(h), 256, h->stream);
         cudaError_t e = cudaGetLastError();
-        if (e == cudaSuccess && host) {
+        if (e == cudaSuccess) {
             if (o->x) e = cudaMemcpyAsync(o->x, dx_out, np * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
             if (e == cudaSuccess && o->p)
                 e = cudaMemcpyAsync(o->p, dp_out, np * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
@@ -1194,7 +1224,7 @@ extern "C" int pic_get_state(pic_handle *h, const pic_arrays *o, int32_t mem)
         if (e != cudaSuccess) return fail(h, PIC_ERR_CUDA, "get_state: %s", cudaGetErrorString(e));
         ++h->launches;
     }
-    const cudaMemcpyKind kind = host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
+    const cudaMemcpyKind kind = cudaMemcpyDeviceToHost;
     struct { double *dst; const double *src; } g[] = {
         {o->ex, h->ex}, {o->ey, h->ey}, {o->ez, h->ez}, {o->ay, h->ay}, {o->az, h->az}};
     for (auto &f : g)

@@ -152,6 +152,22 @@ int launch_load(int fp32, long long np, int M, double dx, const double *x, const
                 PartPtrs P, int grid, int block, cudaStream_t s);
 int launch_store(int fp32, long long np, int M, double dx, PartPtrs P, double *x, double *p,
                  int grid, int block, cudaStream_t s);
+// device destinations of a state: x and p in caller order (NULL: skipped) and n plain arrays
+struct StateOut {
+    double *x, *p;
+    int n;
+    double *dst[8];
+    const double *src[8];
+    long long len[8];
+};
+int launch_store_state(int fp32, long long np, int M, double dx, PartPtrs P, const StateOut &o, int grid, int block,
+                       cudaStream_t s);
+// x and p (device) through buckets of caller indices; rec: scratch of 16 (float) or 24
+// (double) bytes a marker, cursor: 256 int32
+int launch_store_dealt(int fp32, long long np, int M, double dx, PartPtrs P, void *rec, int *cursor, double *x, double *p,
+                       cudaStream_t s);
+// more markers than this are dealt: their x and p exceed half of L2
+constexpr long long kDealMarkers = 1LL << 22;
 // the same values in caller order through an inverse permutation (inv: np int32 of
 // scratch); consecutive writes, so x and p may be device addresses of page-locked host memory
 int launch_store_ordered(int fp32, long long np, int M, double dx, PartPtrs P, int32_t *inv, double *x, double *p,

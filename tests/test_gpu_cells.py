@@ -62,3 +62,27 @@ def test_steps_at_awkward_shapes(shape, precision):
     if precision == pic.PIC_FP64:
         assert g.energy()["gauss"] < 1e-12
     g.close()
+
+
+@pytest.mark.parametrize("precision", [pic.PIC_FP64, pic.PIC_FP32])
+@pytest.mark.parametrize("n", [1, 4099, (1 << 22) + 1, 5 * (1 << 20) + 77])
+def test_device_state_equals_host_state(n, precision):
+    """pic_get_state into device arrays (one launch, or dealt into buckets for many
+    markers) gives the bits of the host copy, for all members and for p alone."""
+    import torch
+    nx, k = 64, 3
+    g = torch.Generator(device="cuda").manual_seed(n)
+    L = 4 * np.pi
+    x = torch.rand(n, dtype=torch.float64, device="cuda", generator=g) * L
+    p = 0.1 * torch.randn(n, dtype=torch.float64, device="cuda", generator=g)
+    ay = 0.1 * torch.ones(nx, dtype=torch.float64, device="cuda")
+    sim = pic.Pic(pic.Config(L, nx, k, n, L / n, 0.05, precision=precision, sort_every=1), x, p, ay, 0.5 * ay)
+    ref = sim.state_numpy()
+    dev = {q: torch.full((v.size,), float("nan"), dtype=torch.float64, device="cuda") for q, v in ref.items()}
+    sim.get_state(**dev)
+    for q, v in ref.items():
+        np.testing.assert_array_equal(dev[q].cpu().numpy(), v, err_msg=q)
+    only = torch.empty(n, dtype=torch.float64, device="cuda")
+    sim.get_state(p=only)
+    np.testing.assert_array_equal(only.cpu().numpy(), ref["p"])
+    sim.close()
