@@ -128,12 +128,13 @@ static void release(pic_handle *h)
     f(h->spx); f(h->spy); f(h->spz); f(h->sdy); f(h->sdz); f(h->red);
     double *arr[] = {h->ex, h->ey, h->ez, h->ay, h->az, h->ek, h->ebar,
                      h->eky, h->ekz, h->aky, h->akz, h->by, h->bz, h->m0, h->mdep, h->gtab, h->rho,
-                     h->work, h->diag, h->d_rowM0, h->d_rowM1, h->d_rowK, h->d_rowPm,
+                     h->work, h->diag, h->d_rowM0, h->d_rowM1, h->d_rowK,
                      h->d_tapM1, h->d_tapP};
     for (double *a : arr) f(a);
     f(h->counts);
     f(h->ctrl);
     f(h->d_count);
+    f(h->small);
     drop_graphs(h);
     f(h->T.A); f(h->T.E); f(h->T.Kt); f(h->T.L);
     for (int m = 0; m < kMaxStartOrder; ++m) { f(h->fh.x[m]); f(h->fh.y[m]); f(h->fh.z[m]); }
@@ -266,7 +267,7 @@ pic::RunDesc pic::handle_desc(pic_handle *h)
     d.ex = h->ex; d.ek = h->ek; d.ebar = h->ebar; d.ay = h->ay; d.az = h->az;
     d.m0 = h->m0;
     for (int b = 0; b < 2; ++b) { d.m1[b] = h->m1[b]; d.flux[b] = h->flux[b]; }
-    d.rowPm = h->d_rowPm; d.rowK = h->d_rowK;
+    d.rowM0 = h->d_rowM0; d.rowM1 = h->d_rowM1;
     d.ey = h->ey; d.ez = h->ez; d.by = h->by; d.bz = h->bz;
     d.eky = h->eky; d.ekz = h->ekz; d.aky = h->aky; d.akz = h->akz;
     for (int b = 0; b < 2; ++b) { d.my[b] = h->my[b]; d.mz[b] = h->mz[b]; }
@@ -454,7 +455,7 @@ extern "C" int pic_init_split(const pic_config *cfg, const pic_arrays *in, int32
     if (reduce_fn && (rc = dalloc(h, &h->red, 4))) return bail(rc);
     if (c.hbar != 0.0) {
         if ((rc = dalloc(h, &h->spx, np)) || (rc = dalloc(h, &h->spy, np)) || (rc = dalloc(h, &h->spz, np)) ||
-            (rc = dalloc(h, &h->sdy, M)) || (rc = dalloc(h, &h->sdz, M)))
+            (rc = dalloc(h, &h->sdy, M * c.degree)) || (rc = dalloc(h, &h->sdz, M * c.degree)))
             return bail(rc);
         const cudaMemcpyKind k = mem == PIC_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
         cudaMemcpyAsync(h->spx, in->sx, np * sizeof(double), k, h->stream);
@@ -477,25 +478,23 @@ extern "C" int pic_init_split(const pic_config *cfg, const pic_arrays *in, int32
     if (cudaMallocHost((void **)&h->h_flag, sizeof(int)) != cudaSuccess) return bail(PIC_ERR_NOMEM);
     if (cudaMallocHost((void **)&h->h_ctrl, sizeof(DevCtrl)) != cudaSuccess) return bail(PIC_ERR_NOMEM);
 
-    // circulant bands: M0 (degree k), M1 (degree k-1), K = G^T M1 G, P = M0 +/- dt^2/4 K
+    // circulant bands: M0 (degree k), M1 (degree k-1), K = G^T M1 G, P = M0 + dt^2/4 K
     const int K = h->K;
-    std::vector<double> m0(K + 1, 0.0), m1(K + 1, 0.0), kr(K + 1, 0.0), pp(K + 1), pm(K + 1);
+    std::vector<double> m0(K + 1, 0.0), m1(K + 1, 0.0), kr(K + 1, 0.0), pp(K + 1);
     mass_band(K, dx, m0.data());
     mass_band(K - 1, dx, m1.data());
     // K_d = (2 m1_d - m1_{d-1} - m1_{d+1}) / dx^2 with m1_{-d} = m1_d
     auto m1at = [&](int d) { d = std::abs(d); return d <= K - 1 ? m1[d] : 0.0; };
     for (int d = 0; d <= K; ++d) kr[d] = (2.0 * m1at(d) - m1at(d - 1) - m1at(d + 1)) / (dx * dx);
     const double q = c.dt * c.dt / 4.0;
-    for (int d = 0; d <= K; ++d) { pp[d] = m0[d] + q * kr[d]; pm[d] = m0[d] - q * kr[d]; }
+    for (int d = 0; d <= K; ++d) pp[d] = m0[d] + q * kr[d];
     std::vector<double> gfull(M), taps(M);
     if ((rc = dalloc(h, &h->d_rowM0, K + 1))) return bail(rc);
     if ((rc = dalloc(h, &h->d_rowM1, K + 1))) return bail(rc);
     if ((rc = dalloc(h, &h->d_rowK, K + 1))) return bail(rc);
-    if ((rc = dalloc(h, &h->d_rowPm, K + 1))) return bail(rc);
     cudaMemcpyAsync(h->d_rowM0, m0.data(), sizeof(double) * (K + 1), cudaMemcpyHostToDevice, h->stream);
     cudaMemcpyAsync(h->d_rowM1, m1.data(), sizeof(double) * (K + 1), cudaMemcpyHostToDevice, h->stream);
     cudaMemcpyAsync(h->d_rowK, kr.data(), sizeof(double) * (K + 1), cudaMemcpyHostToDevice, h->stream);
-    cudaMemcpyAsync(h->d_rowPm, pm.data(), sizeof(double) * (K + 1), cudaMemcpyHostToDevice, h->stream);
     {
         cudaError_t e = cudaStreamSynchronize(h->stream);
         if (e == cudaSuccess) e = cudaGetLastError();
@@ -577,7 +576,7 @@ extern "C" int pic_init_split(const pic_config *cfg, const pic_arrays *in, int32
 static int check_status(pic_handle *h, int which)
 {
     if (h->h_ctrl->status & STATUS_TIMEOUT)
-        return fail(h, PIC_ERR_CUDA, "subsystem %d: a bounded wait on a bulk copy gave up", which);
+        return fail(h, PIC_ERR_CUDA, "subsystem %d: a bounded wait gave up", which);
     if (h->h_ctrl->status & STATUS_NUMERIC)
         return fail(h, PIC_ERR_NUMERIC, "subsystem %d: non-finite value or displacement beyond c dt", which);
     if (h->h_ctrl->status & STATUS_NOCONV)
@@ -1057,14 +1056,83 @@ static int build_step_graph(pic_handle *h)
     return PIC_OK;
 }
 
+// ------------------------------------------------------------------ small plasmas
+// With a thread a marker the steps run in one cooperative kernel (pic_small.cuh).
+static bool small_eligible(const pic_handle *h)
+{
+    return h->np <= (long long)h->num_sms * kSmallThreads && !h->reduce && !h->timing && !debug_sync() &&
+           h->cfg.warm_start != PIC_WARM_MLP && h->acc == (h->fp32 ? ACC_COMP : ACC_NATIVE) &&
+           getenv("PIC_NO_GRAPH") == nullptr;
+}
+
+static int step_counts(pic_handle *h)
+{
+    if (h->d_count) return PIC_OK;
+    int rc;
+    if ((rc = dalloc(h, &h->d_count, 2))) return rc;
+    GCK(cudaMallocHost((void **)&h->h_count, 2 * sizeof(int)));
+    return PIC_OK;
+}
+
+static int step_small(pic_handle *h, int nsteps, long long *s1, long long *s2)
+{
+    int rc;
+    if ((rc = step_counts(h))) return rc;
+    if (!h->small && (rc = dalloc(h, &h->small, 1))) return rc;
+    GCK(cudaMemsetAsync(h->d_count, 0, 2 * sizeof(int), h->stream));
+    const bool strang = h->cfg.splitting == PIC_SPLIT_STRANG;
+    const double dt1 = strang ? 0.5 * h->cfg.dt : h->cfg.dt;
+    for (int n = 0; n < nsteps;) {
+        SmallArgs a{};
+        // as many steps as fit before the next sort
+        const int every = h->cfg.sort_every;
+        const int room = std::min(nsteps - n, kSmallSteps);
+        const int m = every > 0 ? (int)std::min<long long>(room, every - h->steps_done % every) : room;
+        a.d = handle_desc(h);
+        a.a1 = make_sweep1_args(h, dt1);
+        a.c1 = make_conv1_args(h, dt1);
+        a.c1p = a.c1;
+        a.c1.graph = 1;
+        a.c1.count = h->d_count;
+        a.c1p.mode = CONV_START1;
+        a.c1p.mom[0] = h->m1[1];
+        a.c1p.flux = h->flux[1];
+        a.c2 = make_conv2_args(h);
+        a.c2.graph = 1;
+        a.c2.count = h->d_count + 1;
+        a.warm = h->cfg.warm_start == PIC_WARM_EXPLICIT;
+        a.nsteps = m;
+        a.strang = strang;
+        a.warm_field = h->cfg.warm_field;
+        a.zero_delta = h->cfg.warm_start == PIC_WARM_NONE;
+        a.sync = h->small;
+        a.w = h->cfg.weight;
+        a.hbar = h->cfg.hbar;
+        a.sx = h->spx; a.sy = h->spy; a.sz = h->spz;
+        a.sm_y = h->sdy; a.sm_z = h->sdz;
+        GCK(cudaMemsetAsync(h->small, 0, sizeof(SmallSync), h->stream));
+        if ((h->fp32 ? launch_small_f32 : launch_small_f64)(a, h->num_sms, h->stream)) return fail(h, PIC_ERR_CUDA, "step kernel: launch failed");
+        CKL_N("launch_small");
+        n += m;
+        h->steps_done += m;
+        if (every > 0 && h->steps_done % every == 0)
+            if ((rc = sort_markers(h))) return rc;
+    }
+    GCK(cudaMemcpyAsync(h->h_count, h->d_count, 2 * sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    if ((rc = read_ctrl(h))) return rc;
+    *s1 = h->h_count[0];
+    *s2 = h->h_count[1];
+    h->marker_sweeps += *s1 * h->np;
+    for (int which = 1; which <= 2; ++which)
+        if ((rc = check_status(h, which))) return rc;
+    return PIC_OK;
+}
+
 // nsteps steps as graph launches; counts and status read back once at the end
 static int step_graphs(pic_handle *h, int nsteps, long long *s1, long long *s2)
 {
     int rc;
-    if (!h->d_count) {
-        if ((rc = dalloc(h, &h->d_count, 2))) return rc;
-        GCK(cudaMallocHost((void **)&h->h_count, 2 * sizeof(int)));
-    }
+    if ((rc = step_counts(h))) return rc;
     GCK(cudaMemsetAsync(h->d_count, 0, 2 * sizeof(int), h->stream));
     for (int n = 0; n < nsteps; ++n) {
         if (!h->step_exec[h->cur] && (rc = build_step_graph(h))) return rc;
@@ -1092,6 +1160,13 @@ extern "C" int pic_step(pic_handle *h, int32_t nsteps, int64_t *iters_I, int64_t
     long long s1 = 0, s2 = 0;
     int rc = PIC_OK;
     for (int n = 0; n < nsteps; ++n) {
+        if (small_eligible(h)) {
+            long long g1 = 0, g2 = 0;
+            rc = step_small(h, nsteps - n, &g1, &g2);
+            s1 += g1;
+            s2 += g2;
+            break;
+        }
         // graph steps once a host-loop step has opted the kernels in to their shared memory
         if (h->host_steps > 0 && graph_eligible(h)) {
             long long g1 = 0, g2 = 0;

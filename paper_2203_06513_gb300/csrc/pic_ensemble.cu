@@ -192,7 +192,7 @@ static int loop_body(pic_ensemble *e, int which, cudaStream_t s, unsigned long l
 
 static int seg_prep1(pic_ensemble *e, cudaStream_t s)
 {
-    ELAUNCH(launch_prep1_ens(e->d_desc, e->nruns, e->Mmax, s), "ensemble prep I");
+    ELAUNCH(launch_prep1_ens(e->d_desc, e->nruns, e->K, e->Mmax, s), "ensemble prep I");
     if (e->warm_field) {
         // predicted start of every run: plan (all runs are iterating), the proposals
         // and their currents (work queue), e^(0) per run
@@ -209,7 +209,7 @@ static int seg_mid(pic_ensemble *e, cudaStream_t s)
 {
     ELAUNCH(launch_finalize1_ens(e->fp32, e->d_desc, e->nruns, e->fin_grid, s), "ensemble finalize I");
     ELAUNCH(launch_commit_ens(e->d_desc, e->nruns, e->Mmax, 1, s), "ensemble commit I");
-    ELAUNCH(launch_prep2_ens(e->d_desc, e->nruns, e->Mmax, s), "ensemble prep II");
+    ELAUNCH(launch_prep2_ens(e->d_desc, e->nruns, e->K, e->Mmax, s), "ensemble prep II");
     return PIC_OK;
 }
 
@@ -403,7 +403,7 @@ extern "C" int pic_ensemble_create(const pic_config *cfgs, const pic_arrays *ins
     if (cudaMemsetAsync(e->d_q, 0, sizeof(EnsQueue), e->stream) != cudaSuccess ||
         cudaMemsetAsync(e->d_sweeps, 0, 2 * n * sizeof(int), e->stream) != cudaSuccess)
         return bail(PIC_ERR_CUDA);
-    if (conv_ens_optin(std::max(e->ntap1, e->ntap2)))
+    if (conv_ens_optin(e->K, std::max(e->ntap1, e->ntap2)))
         return bail(efail(e, PIC_ERR_CUDA, "solve kernel shared-memory opt-in failed"));
     build_tables(e);
     if ((rc = upload_tables(e)) || (rc = upload_schedule(e))) return bail(rc);

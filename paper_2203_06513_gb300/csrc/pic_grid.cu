@@ -13,6 +13,7 @@
 
 #include "pic_internal.h"
 #include "pic_poly.cuh"
+#include "pic_solve.cuh"
 
 namespace pic {
 
@@ -147,317 +148,28 @@ void inverse_taps(const double *band, int bw, int M, double cut, double *g, int 
                           *ntap});
 }
 
-// ---------------------------------------------------------------------------
-// Convergence decision, made by the last block of a solve kernel.
-// FP64 form (Sec. 5, tolerance tol): max |x^(k+1) - x^(k)| <= tol (length) and
-// max |e^(k+1) - e^(k)| <= tol.  FP32 form: position increments at the float
-// resolution of the offset (dtol, relative to max(1, |delta|)) and field
-// increments below tol or no longer shrinking (stagnation at float noise).
-// ---------------------------------------------------------------------------
-__device__ void decide(const ConvArgs &A)
-{
-    DevCtrl *c = A.ctrl;
-    __threadfence();
-    if (A.count) *A.count += 1;
-    const double d = (A.subsystem == 1) ? bits_to_double(c->dmax_bits) : 0.0;
-    const double e = bits_to_double(c->emax_bits);
-    const double ep = bits_to_double(c->eprev_bits);
-    c->iter += 1;
-    bool ok;
-    if (!A.fp32) {
-        ok = (d * A.dx <= A.tol) && (e <= A.tol);
-    } else {
-        // Float iterates stop improving at rounding noise, so increments alone never
-        // reach a tight tolerance.  Estimate the remaining error of the new iterate
-        // from the increment v_k and the observed contraction r = v_k / v_{k-1}
-        // (geometric tail v_k r / (1 - r), r capped at 0.9), and stop when both the
-        // position and field estimates are below tolerance, or when both increments
-        // have stopped shrinking at noise level.
-        const double dp = bits_to_double(c->dprev_bits);
-        auto est = [](double v, double vprev) {
-            if (v == 0.0) return 0.0;
-            // no previous increment (first sweep): no contraction estimate yet
-            double r = (vprev < 1e300) ? v / vprev : 0.9;
-            if (!(r < 0.9)) r = 0.9;
-            return v * r / (1.0 - r);
-        };
-        // field tolerance.  Subsystem I: the absolute tol, or erel of the field's
-        // max-norm when that is larger, on the last increment itself: the markers'
-        // momenta were updated with the field of the sweep before, and that
-        // mismatch is proportional to the last increment (not to the estimated
-        // remaining error), with a sign that does not average out over steps: a
-        // rule on the estimate accepted increments near 1e-7 of the field and let
-        // the energy drift by 1e-12 of the total a step on C2.
-        // Subsystem II: the estimated remaining error below the absolute tol.  Its
-        // markers do not move, the sweep is deterministic, and the remaining field
-        // error enters the transverse energy directly.
-        const double emag = bits_to_double(c->emag_bits);
-        const bool dok = (A.subsystem == 1) ? (est(d, dp) <= A.dtol) : true;
-        const bool eok = (A.subsystem == 1) ? (e <= fmax(A.tol, A.erel * emag)) : (est(e, ep) <= A.tol);
-        const bool dstag = (A.subsystem == 1) ? (d >= 0.5 * dp && d <= 1e-4) : true;
-        const bool estag = e >= 0.5 * ep && e <= 1e-8;
-        ok = (dok && eok) || (c->iter >= 3 && dstag && estag);
+// the body for the degree K (a compile-time constant in it)
+#define PIC_FOR_DEGREE(K_, ...)                                                           \
+    switch (K_) {                                                                         \
+    case 2: { constexpr int K = 2; __VA_ARGS__; break; }                                  \
+    case 3: { constexpr int K = 3; __VA_ARGS__; break; }                                  \
+    case 4: { constexpr int K = 4; __VA_ARGS__; break; }                                  \
+    case 5: { constexpr int K = 5; __VA_ARGS__; break; }                                  \
+    default: break;                                                                       \
     }
-    bool stop = ok;
-    if (!ok && c->iter >= A.max_iter) {
-        c->status |= STATUS_NOCONV;
-        stop = true;
-    }
-    if (c->status & (STATUS_NUMERIC | STATUS_TIMEOUT)) stop = true;
-    c->converged = stop ? 1 : 0;
-    c->dprev_bits = c->dmax_bits;
-    c->eprev_bits = c->emax_bits;
-    c->dmax_bits = 0ull;
-    c->emax_bits = 0ull;
-    c->emag_bits = 0ull;
-    c->ticket = 0u;
-    __threadfence();
-    if (A.graph && A.cond_handle)
-        cudaGraphSetConditional((cudaGraphConditionalHandle)A.cond_handle, stop ? 0u : 1u);
-}
 
-// Spline pieces of every degree (pic_poly.cuh).  Grid kernels take the degree at run time.
-__constant__ SplineTab c_spline = make_spline_tab();
-
-// Pieces of C_i = sum_{j >= i} Lambda^0_j in the cells i + r, r = 0 .. d - 1: the running
-// sums over r of the pieces of N^d.
-constexpr SplineTab make_cumulative_tab()
-{
-    SplineTab T = make_spline_tab();
-    for (int d = 0; d <= kMaxDegree; ++d)
-        for (int r = 1; r <= d; ++r)
-            for (int m = 0; m <= d; ++m) T.b[d][r][m] += T.b[d][r - 1][m];
-    return T;
-}
-__constant__ SplineTab c_cumulative = make_cumulative_tab();
-
-// Stores coefficient m of row `row` (pad numbers a row) in the form's type.
-__device__ __forceinline__ void put_coef(void *tab, int fp32, size_t row, int pad, int m, double v)
-{
-    if (fp32) static_cast<float *>(tab)[row * pad + m] = (float)v;
-    else static_cast<double *>(tab)[row * pad + m] = v;
-}
-
-// Coefficient m of the degree-D polynomial in the cell whose node r steps down has value at(r).
-template <class At>
-__device__ __forceinline__ double cell_coef(int D, int m, At &&at)
-{
-    double s = 0.0;
-    for (int r = 0; r <= D; ++r) s = fma(c_spline.b[D][r][m], at(r), s);
-    return s;
-}
-
-// Value of a deposit at node j from the moments of degree D (path: coefficient m over m + 1).
-__device__ __forceinline__ double node_value(int M, int D, bool path, const double *mom, int j)
-{
-    const int NV = D + 1;
-    double s[kMaxDegree + 1] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    int c = j;
-    for (int r = 0; r < NV; ++r) {
-        const double *row = mom + (size_t)c * NV;
-#pragma unroll
-        for (int m = 0; m <= kMaxDegree; ++m)
-            if (m < NV) s[m] = fma(c_spline.b[D][r][m], row[m], s[m]);
-        c = c + 1 == M ? 0 : c + 1;
-    }
-    double v = 0.0;
-#pragma unroll
-    for (int m = 0; m <= kMaxDegree; ++m)
-        if (m < NV) v += path ? s[m] * (1.0 / (m + 1)) : s[m];
-    return v;
-}
-
-// Path current at node j over w dx (pic_poly.cuh): the polynomials of C_j on the change of
-// the moments in the cells j .. j + K - 1, and the crossings of the knot j + K.
-__device__ __forceinline__ double path_node_value(int M, int K, const double *mom, const double *mom0,
-                                                  const int *flux, int j)
-{
-    double s0 = 0.0, s1 = 0.0;
-    int c = j, f = flux[j];
-    for (int r = 0; r < K; ++r) {
-        const int cn = c + 1 == M ? 0 : c + 1;
-        const int fn = flux[cn];
-        s0 = fma(c_cumulative.b[K][r][0], (double)(f - fn), s0);
-        for (int m = 1; m <= K; ++m) {
-            const size_t q = (size_t)c * K + m - 1;
-            s1 = fma(c_cumulative.b[K][r][m], mom[q] - mom0[q], s1);
-        }
-        c = cn;
-        f = fn;
-    }
-    return (s0 + s1) + (double)f;
-}
-
-// The residue of a^n + a^(k) after both coefficients were rounded to float.
-__device__ __forceinline__ float sum_residue(double n, double k)
-{
-    return (float)((n - (double)(float)n) + (k - (double)(float)k));
-}
-
-// y_i = sum_n taps[n] in[(i - (d_start + n)) mod M] for the kConvOut nodes
-// i0 - K .. i0 - K + kConvOut - 1 of block bx, i0 = bx (kConvOut - K): the block owns the
-// last kConvOut - K of them and recomputes the K below, which the polynomials of
-// its cells need.  One warp computes a quarter of the taps for all nodes (lane =
-// node): with a few dozen nodes a block the solve spreads over the SMs instead of
-// waiting on one SM's FP64 pipe, and only the block's part of the deposit is staged
-// (M = 2048, cubic: 35 us with one thread a node and the whole row staged twice by every
-// block, 18 us so; both with cold caches).
-// Returns true in the one block that finished the run's solve last (after the
-// convergence decision, in the solve modes).
-constexpr int kConvOut = 32, kConvThreads = 128;
-
-inline size_t conv_smem(int ntap)
-{
-    const int nq = kConvOut + ntap - 1;
-    return ((size_t)nq + ntap + 4 * kConvOut + 2 * kConvOut) * sizeof(double);
-}
-inline int conv_blocks(int M, int K) { return (M + kConvOut - K - 1) / (kConvOut - K); }
-
-__device__ bool conv_block(const ConvArgs &A, int bx, int comp, double *sm)
-{
-    const int M = A.M, K = A.K, TB = kConvOut - K, i0 = bx * TB;
-    const int NV = A.subsystem == 1 ? K : K + 1;       // moments a cell
-    const int nq = kConvOut + A.ntap - 1;
-    double *s_in = sm, *s_tap = s_in + nq, *s_part = s_tap + A.ntap;
-    double *s_val = s_part + 4 * kConvOut, *s_an = s_val + kConvOut;
-    const double *mom = A.mom[comp];
-    double *zero = A.zero[comp];
-    const int *flux = A.flux;
-    int *zflux = A.zflux;
-    if (A.graph && A.mode != CONV_PLAIN) {   // replayed by a graph: buffers by sweep parity
-        const int it = *reinterpret_cast<volatile const int *>(&A.ctrl->iter);
-        mom = A.pair[comp][it & 1];
-        zero = A.pair[comp][(it + 1) & 1];
-        flux = A.fpair[it & 1];
-        zflux = A.fpair[(it + 1) & 1];
-    }
-    // s_in[q]: node (g0 + q) mod M
-    const int g0 = wrap_cell(i0 - K - (A.d_start + A.ntap - 1), M);
-    for (int n = threadIdx.x; n < A.ntap; n += kConvThreads) s_tap[n] = A.taps[n];
-    if (mom) {
-        for (int q = threadIdx.x; q < nq; q += kConvThreads) {
-            const int g = (g0 + q) % M;
-            double s = A.scale * (A.subsystem == 1 ? path_node_value(M, K, mom, A.mom0, flux, g)
-                                                   : node_value(M, K, false, mom, g));
-            if (A.mode == CONV_SOLVE2) s = fma(A.dt, s, A.b[comp][g]);
-            s_in[q] = s;
-        }
-    } else {
-        for (int q = threadIdx.x; q < nq; q += kConvThreads) {
-            const int g = (g0 + q) % M;
-            const double s = A.in[comp][g];
-            s_in[q] = A.mode == CONV_SOLVE2 ? fma(A.dt, s, A.b[comp][g]) : s;
-        }
-    }
-    __syncthreads();
-    const int o = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    {
-        const int per = (A.ntap + 3) >> 2, n0 = wid * per, n1 = min(A.ntap, n0 + per);
-        const double *base = s_in + o + A.ntap - 1;
-        double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-        int n = n0;
-        for (; n + 3 < n1; n += 4) {
-            a0 = fma(s_tap[n], base[-n], a0);
-            a1 = fma(s_tap[n + 1], base[-n - 1], a1);
-            a2 = fma(s_tap[n + 2], base[-n - 2], a2);
-            a3 = fma(s_tap[n + 3], base[-n - 3], a3);
-        }
-        for (; n < n1; ++n) a0 = fma(s_tap[n], base[-n], a0);
-        s_part[wid * kConvOut + o] = (a0 + a1) + (a2 + a3);
-    }
-    __syncthreads();
-    double diff = 0.0, mag = 0.0;
-    if (wid == 0) {
-        const double y = (s_part[o] + s_part[kConvOut + o]) + (s_part[2 * kConvOut + o] + s_part[3 * kConvOut + o]);
-        const int i = i0 - K + o;
-        const bool own = o >= K && i < M;
-        const int iw = wrap_cell(i, M);
-        if (A.mode == CONV_PLAIN) {
-            if (own) A.out[comp][i] = y;
-        } else if (A.mode != CONV_SOLVE2) {              // START1, SOLVE1
-            const double en = A.en[0][iw];
-            const double enew = en - y;                  // e^(k+1) = e^n - M1^{-1} j
-            const double eb = 0.5 * (en + enew);         // ebar for the next sweep
-            s_val[o] = eb;
-            if (own) {
-                if (A.mode == CONV_SOLVE1) {
-                    diff = fabs(enew - A.ek[0][i]);
-                    mag = fabs(enew);
-                }
-                A.ek[0][i] = enew;
-                A.aux[0][i] = eb;
-            }
-        } else {                                         // P e^(k+1) = b + dt s
-            const double en = A.en[comp][iw], an = A.an[comp][iw];
-            const double enew = y;
-            const double ak = an - 0.5 * A.dt * (en + enew);   // a^(k+1)
-            s_val[o] = ak;
-            s_an[o] = an;
-            if (own) {
-                diff = fabs(enew - A.ek[comp][i]);
-                mag = fabs(enew);
-                A.ek[comp][i] = enew;
-                A.aux[comp][i] = ak;
-            }
-        }
-    }
-    if (A.mode == CONV_PLAIN) return false;
-    __syncthreads();
-    // the cells' polynomials of the new field, and the next sweep's moments cleared
-    const int ncell = min(TB, M - i0);
-    if (A.mode != CONV_SOLVE2) {
-        const int pad = coef_pad(A.fp32, K);
-        for (int q = threadIdx.x; q < ncell * K; q += kConvThreads) {
-            const int j = q / K, m = q % K;
-            const double v = cell_coef(K - 1, m, [&](int r) { return s_val[K + j - r]; });
-            put_coef(A.T.E, A.fp32, (size_t)(i0 + j), pad, m, v * A.dx / (double)(m + 1));
-        }
-    } else {
-        const int pad = coef_pad(A.fp32, K + 1);
-        for (int q = threadIdx.x; q < ncell * (K + 1); q += kConvThreads) {
-            const int j = q / (K + 1), m = q % (K + 1);
-            const size_t row = 2 * (size_t)(i0 + j) + comp;
-            const double k = cell_coef(K, m, [&](int r) { return s_val[K + j - r]; });
-            put_coef(A.T.Kt, A.fp32, row, pad, m, k);
-            if (A.fp32) {
-                const double n = cell_coef(K, m, [&](int r) { return s_an[K + j - r]; });
-                A.T.L[row * pad + m] = sum_residue(n, k);
-            }
-        }
-    }
-    if (A.mode == CONV_START1) return false;
-    if (zero)
-        for (int q = threadIdx.x; q < ncell * NV; q += kConvThreads) zero[(size_t)i0 * NV + q] = 0.0;
-    if (zflux && A.subsystem == 1)
-        for (int q = threadIdx.x; q < ncell; q += kConvThreads) zflux[i0 + q] = 0;
-    __shared__ int s_last;
-    if (wid == 0) {
-        diff = warp_max(diff);
-        mag = warp_max(mag);
-        if (o == 0) {
-            atomic_max_nonneg(&A.ctrl->emax_bits, diff);
-            atomic_max_nonneg(&A.ctrl->emag_bits, mag);
-            __threadfence();
-            const unsigned int nblk = (unsigned)(((M + TB - 1) / TB) * A.ncomp);
-            const unsigned int t = atomicAdd(&A.ctrl->ticket, 1u);
-            s_last = (t == nblk - 1) ? 1 : 0;
-            if (s_last) decide(A);
-        }
-    }
-    __syncthreads();
-    return s_last != 0;
-}
-
+template <int K>
 __global__ void __launch_bounds__(kConvThreads) k_conv(ConvArgs A)
 {
     extern __shared__ __align__(16) double s_conv[];
-    conv_block(A, blockIdx.x, blockIdx.y, s_conv);
+    conv_block<K>(A, A.T, conv_iter(A), blockIdx.x, blockIdx.y, s_conv, nullptr);
 }
 
 // Batched solves of an ensemble: block (bx, run, comp).  Runs that are not in
 // the current sweep (converged, or stopped by an error) are skipped.  After a
 // run's decision, the last run to decide in this sweep records whether any run
 // goes on, and sets the loop's conditional handle (graph mode).
+template <int K>
 __global__ void __launch_bounds__(kConvThreads) k_conv_ens(const ConvArgs *runs, EnsQueue *Q, int *sweeps,
                                                            unsigned long long cond)
 {
@@ -465,8 +177,8 @@ __global__ void __launch_bounds__(kConvThreads) k_conv_ens(const ConvArgs *runs,
     const int r = blockIdx.y, comp = blockIdx.z;
     const ConvArgs &A = runs[r];
     if (A.mode != CONV_PLAIN && !Q->active[r]) return;
-    if (comp >= A.ncomp || (int)blockIdx.x * (kConvOut - A.K) >= A.M) return;
-    const bool last = conv_block(A, blockIdx.x, comp, s_conv);
+    if (comp >= A.ncomp || (int)blockIdx.x * (kConvOut - K) >= A.M) return;
+    const bool last = conv_block<K>(A, A.T, conv_iter(A), blockIdx.x, comp, s_conv, nullptr);
     if (!last || threadIdx.x != 0) return;
     atomicAdd(&sweeps[2 * r + A.subsystem - 1], 1);
     if (!A.ctrl->converged) atomicAdd(&Q->n_continue, 1);
@@ -495,233 +207,94 @@ static int conv_optin(const void *fn, size_t smem, size_t &opted)
     return 0;
 }
 
-static size_t g_conv_ens_opted = 0;
+static size_t g_conv_ens_opted[kMaxDegree + 1];
 
 // raise the shared-memory limit of k_conv_ens before any capture of it
-int conv_ens_optin(int ntap_max)
+int conv_ens_optin(int K_, int ntap_max)
 {
-    return conv_optin((const void *)k_conv_ens, conv_smem(ntap_max), g_conv_ens_opted);
+    PIC_FOR_DEGREE(K_, return conv_optin((const void *)k_conv_ens<K>, conv_smem(K, ntap_max), g_conv_ens_opted[K]))
+    return 1;
 }
 
-int launch_conv_ens(const ConvArgs *runs, int nruns, int Mmax, int K, int ncomp, int ntap_max, EnsQueue *Q,
+int launch_conv_ens(const ConvArgs *runs, int nruns, int Mmax, int K_, int ncomp, int ntap_max, EnsQueue *Q,
                     int *sweeps, unsigned long long cond, cudaStream_t s)
 {
-    const size_t smem = conv_smem(ntap_max);
-    if (smem > 48 * 1024 && smem > g_conv_ens_opted) return 1;   // conv_ens_optin first
-    dim3 grid(conv_blocks(Mmax, K), nruns, ncomp);
-    k_conv_ens<<<grid, kConvThreads, smem, s>>>(runs, Q, sweeps, cond);
+    const size_t smem = conv_smem(K_, ntap_max);
+    if (smem > 48 * 1024 && smem > g_conv_ens_opted[K_]) return 1;   // conv_ens_optin first
+    dim3 grid(conv_blocks(Mmax, K_), nruns, ncomp);
+    PIC_FOR_DEGREE(K_, (k_conv_ens<K><<<grid, kConvThreads, smem, s>>>(runs, Q, sweeps, cond)))
     return 0;
 }
 
 int launch_conv(const ConvArgs &a, cudaStream_t s)
 {
-    const size_t smem = conv_smem(a.ntap);
-    static size_t opted = 0;   // largest dynamic shared memory opted in so far
-    if (conv_optin((const void *)k_conv, smem, opted)) return 1;
-    k_conv<<<dim3(conv_blocks(a.M, a.K), a.ncomp), kConvThreads, smem, s>>>(a);
+    const size_t smem = conv_smem(a.K, a.ntap);
+    static size_t opted[kMaxDegree + 1];   // largest dynamic shared memory opted in so far
+    const dim3 grid(conv_blocks(a.M, a.K), a.ncomp);
+    PIC_FOR_DEGREE(a.K, {
+        if (conv_optin((const void *)k_conv<K>, smem, opted[K])) return 1;
+        k_conv<K><<<grid, kConvThreads, smem, s>>>(a);
+    })
     return 0;
 }
 
-// Control block at the start of a fixed-point loop (the error bits and the field
-// history counts stay).
-__device__ __forceinline__ void ctrl_loop_reset(DevCtrl *ctrl)
+// preparation WHICH, task t = blockIdx.x blockDim.x + threadIdx.x = (q, cell), cells fastest
+template <int K, int WHICH>
+__device__ __forceinline__ void prep_thread(int t, const RunDesc &R)
 {
-    ctrl->dmax_bits = 0ull;
-    ctrl->emax_bits = 0ull;
-    ctrl->emag_bits = 0ull;
-    ctrl->dprev_bits = 0x7ff0000000000000ull;
-    ctrl->eprev_bits = 0x7ff0000000000000ull;
-    ctrl->iter = 0;
-    ctrl->converged = 0;
-    ctrl->ticket = 0u;
+    constexpr int n = WHICH == 1 ? prep1_tasks<K> : prep2_tasks<K>;
+    const int q = t / R.M, i = t - q * R.M;
+    if (q >= n) return;
+    if (WHICH == 1) prep1_task<K>(i, q, R);
+    else prep2_task<K>(i, q, R);
 }
 
-// Starting field of a fixed-point iteration.  The fixed point does not depend on
-// it, only the number of sweeps to reach it does: e^n extrapolated in time by the
-// polynomial through the last q + 1 states, q = min(stored changes, order):
-// e^n, e^n + d0, e^n + 2 d0 - d1, e^n + 3 d0 - 3 d1 + d2.
-__device__ __forceinline__ double start_field(double e, double *const d[kMaxStartOrder], int i, int q)
+template <int K, int WHICH>
+__global__ void __launch_bounds__(128) k_prep(RunDesc R)
 {
-    switch (q) {
-    case 0: return e;
-    case 1: return e + d[0][i];
-    case 2: return e + (2.0 * d[0][i] - d[1][i]);
-    default: return e + (3.0 * (d[0][i] - d[1][i]) + d[2][i]);
-    }
+    prep_thread<K, WHICH>(blockIdx.x * blockDim.x + threadIdx.x, R);
 }
 
-// ---------------------------------------------------------------------------
-// Subsystem I preparation: e^(0), ebar^(0) = (e^n + e^(0)) / 2, the cells' polynomials
-// of a^n and ebar^(0), cleared moments, the control block reset for the loop.
-// ---------------------------------------------------------------------------
-// both rows of the polynomials of (cy, cz) in cell i, and whether cz has a non-zero
-__device__ __forceinline__ void a_rows(int i, int M, int K, int fp32, const double *cy, const double *cz, void *tab)
+template <int K, int WHICH>
+__global__ void __launch_bounds__(128) k_prep_ens(const RunDesc *runs)
 {
-    const int pad = coef_pad(fp32, K + 1);
-    for (int m = 0; m <= K; ++m) {
-        put_coef(tab, fp32, 2 * (size_t)i, pad, m, cell_coef(K, m, [&](int r) { return cy[wrap_cell(i - r, M)]; }));
-        put_coef(tab, fp32, 2 * (size_t)i + 1, pad, m, cell_coef(K, m, [&](int r) { return cz[wrap_cell(i - r, M)]; }));
-    }
+    prep_thread<K, WHICH>(blockIdx.x * blockDim.x + threadIdx.x, runs[blockIdx.y]);
 }
 
-__device__ __forceinline__ void prep1_at(int i, const RunDesc &R)
+template <int K, int WHICH>
+static int prep_grid(int M)
 {
-    const int M = R.M, K = R.K;
-    const int q = min(R.ctrl->hist1, R.fh.order1);    // hist1: written only by the commit kernel
-    if (i < M) {
-        auto ebar = [&](int g) { return 0.5 * (R.ex[g] + start_field(R.ex[g], R.fh.x, g, q)); };
-        R.ek[i] = start_field(R.ex[i], R.fh.x, i, q);
-        R.ebar[i] = ebar(i);
-        a_rows(i, M, K, R.fp32, R.ay, R.az, R.T.A);
-        const int pad = coef_pad(R.fp32, K);
-        for (int m = 0; m < K; ++m) {
-            const double v = cell_coef(K - 1, m, [&](int r) { return ebar(wrap_cell(i - r, M)); });
-            put_coef(R.T.E, R.fp32, (size_t)i, pad, m, v * R.dx / (double)(m + 1));
-            R.m1[0][(size_t)i * K + m] = 0.0;
-            R.m1[1][(size_t)i * K + m] = 0.0;
-        }
-        R.flux[0][i] = 0;
-        R.flux[1][i] = 0;
-        if (R.az[i] != 0.0) R.ctrl->zany = 1;
-    }
-    if (i == 0) ctrl_loop_reset(R.ctrl);
+    return (M * (WHICH == 1 ? prep1_tasks<K> : prep2_tasks<K>) + 127) / 128;
 }
 
-__global__ void k_prep1(RunDesc R) { prep1_at(blockIdx.x * blockDim.x + threadIdx.x, R); }
-
-__global__ void k_prep1_ens(const RunDesc *runs)
+int launch_prep1_ens(const RunDesc *R, int nruns, int K_, int Mmax, cudaStream_t s)
 {
-    prep1_at(blockIdx.x * blockDim.x + threadIdx.x, runs[blockIdx.y]);
-}
-
-int launch_prep1_ens(const RunDesc *R, int nruns, int Mmax, cudaStream_t s)
-{
-    k_prep1_ens<<<dim3((Mmax + 63) / 64, nruns), 64, 0, s>>>(R);
+    PIC_FOR_DEGREE(K_, (k_prep_ens<K, 1><<<dim3(prep_grid<K, 1>(Mmax), nruns), 128, 0, s>>>(R)))
     return 0;
 }
 
 int launch_prep1(const RunDesc &R, cudaStream_t s)
 {
-    k_prep1<<<(R.M + 63) / 64, 64, 0, s>>>(R);
+    PIC_FOR_DEGREE(R.K, (k_prep<K, 1><<<prep_grid<K, 1>(R.M), 128, 0, s>>>(R)))
     return 0;
 }
 
-// ---------------------------------------------------------------------------
-// Subsystem II preparation: b = (M0 - dt^2/4 K) e^n + dt K a^n (banded
-// circulant products), e^(0), a^(0) = a^n - dt/2 (e^n + e^(0)), cleared
-// moments, the cells' polynomials, the control block reset for the loop.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ void prep2_at(int i, const RunDesc &R)
+int launch_prep2_ens(const RunDesc *R, int nruns, int K_, int Mmax, cudaStream_t s)
 {
-    const int M = R.M, K = R.K;
-    const double dt = R.dt;
-    const int q = min(R.ctrl->hist2, R.fh.order2);    // hist2: written only by the commit kernel
-    if (i < M) {
-        const double *ey = R.ey, *ez = R.ez, *ay = R.ay, *az = R.az;
-        auto a0 = [&](const double *a, const double *e, double *const d[kMaxStartOrder], int g) {
-            return a[g] - 0.5 * dt * (e[g] + start_field(e[g], d, g, q));
-        };
-        const double ey0 = start_field(ey[i], R.fh.y, i, q);
-        const double ez0 = start_field(ez[i], R.fh.z, i, q);
-        const double ay0 = a0(ay, ey, R.fh.y, i), az0 = a0(az, ez, R.fh.z, i);
-        {
-            double kn[2][kMaxDegree + 1], kk[2][kMaxDegree + 1];     // nodes i, i - 1, .. i - K
-            for (int r = 0; r <= K; ++r) {
-                const int g = wrap_cell(i - r, M);
-                kn[0][r] = ay[g];
-                kn[1][r] = az[g];
-                kk[0][r] = a0(ay, ey, R.fh.y, g);
-                kk[1][r] = a0(az, ez, R.fh.z, g);
-            }
-            const int pad = coef_pad(R.fp32, K + 1);
-            for (int c = 0; c < 2; ++c) {
-                const size_t row = 2 * (size_t)i + c;
-                for (int m = 0; m <= K; ++m) {
-                    const double n = cell_coef(K, m, [&](int r) { return kn[c][r]; });
-                    const double k = cell_coef(K, m, [&](int r) { return kk[c][r]; });
-                    put_coef(R.T.A, R.fp32, row, pad, m, n);
-                    put_coef(R.T.Kt, R.fp32, row, pad, m, k);
-                    if (R.fp32) R.T.L[row * pad + m] = sum_residue(n, k);
-                }
-            }
-        }
-        double vy = R.rowPm[0] * ey[i] + dt * R.rowK[0] * ay[i];
-        double vz = R.rowPm[0] * ez[i] + dt * R.rowK[0] * az[i];
-        for (int d = 1; d <= K; ++d) {
-            const int ip = (i + d) % M, im = (i - d + M) % M;
-            vy += R.rowPm[d] * (ey[ip] + ey[im]) + dt * R.rowK[d] * (ay[ip] + ay[im]);
-            vz += R.rowPm[d] * (ez[ip] + ez[im]) + dt * R.rowK[d] * (az[ip] + az[im]);
-        }
-        R.by[i] = vy;
-        R.bz[i] = vz;
-        R.eky[i] = ey0;
-        R.ekz[i] = ez0;
-        R.aky[i] = ay0;
-        R.akz[i] = az0;
-        for (int m = 0; m <= K; ++m)
-            for (int b = 0; b < 2; ++b) {
-                R.my[b][(size_t)i * (K + 1) + m] = 0.0;
-                R.mz[b][(size_t)i * (K + 1) + m] = 0.0;
-            }
-        if (az[i] != 0.0 || ez[i] != 0.0) R.ctrl->zany = 1;
-    }
-    if (i == 0) ctrl_loop_reset(R.ctrl);
-}
-
-__global__ void k_prep2(RunDesc R) { prep2_at(blockIdx.x * blockDim.x + threadIdx.x, R); }
-
-__global__ void k_prep2_ens(const RunDesc *runs)
-{
-    prep2_at(blockIdx.x * blockDim.x + threadIdx.x, runs[blockIdx.y]);
-}
-
-int launch_prep2_ens(const RunDesc *R, int nruns, int Mmax, cudaStream_t s)
-{
-    k_prep2_ens<<<dim3((Mmax + 63) / 64, nruns), 64, 0, s>>>(R);
+    PIC_FOR_DEGREE(K_, (k_prep_ens<K, 2><<<dim3(prep_grid<K, 2>(Mmax), nruns), 128, 0, s>>>(R)))
     return 0;
 }
 
 int launch_prep2(const RunDesc &R, cudaStream_t s)
 {
-    k_prep2<<<(R.M + 63) / 64, 64, 0, s>>>(R);
+    PIC_FOR_DEGREE(R.K, (k_prep<K, 2><<<prep_grid<K, 2>(R.M), 128, 0, s>>>(R)))
     return 0;
 }
 
-// e^{n+1} = e^(k) replaces e^n; its change enters the history (d[2] = d[1],
-// d[1] = d[0], d[0] = e^{n+1} - e^n), as deep as the extrapolation order needs.
-__device__ __forceinline__ void commit_field(int i, const double *ek, double *e, double *const d[kMaxStartOrder],
-                                             int order)
+__global__ void k_commit(RunDesc R, int which) 
 {
-    const double v = ek[i];
-    for (int m = order - 1; m > 0; --m) d[m][i] = d[m - 1][i];
-    if (order > 0) d[0][i] = v - e[i];
-    e[i] = v;
+    commit_at(blockIdx.x * blockDim.x + threadIdx.x, R, which, R.ctrl->iter - 1);
 }
-
-// End of a substep: I: e_x = e^(k); II: e_perp = e^(k), a_perp = a^(k).  Thread
-// 0 counts the stored changes (up to kMaxStartOrder) for the next preparation.
-__device__ __forceinline__ void commit_at(int i, const RunDesc &R, int which)
-{
-    if (i < R.M) {
-        if (which == 1) {
-            commit_field(i, R.ek, R.ex, R.fh.x, R.fh.order1);
-            // the end points of the last sweep are the next step's start points
-            const double *last = R.m1[(R.ctrl->iter - 1) & 1];
-            for (int m = 0; m < R.K; ++m) R.m0[(size_t)i * R.K + m] = last[(size_t)i * R.K + m];
-        } else {
-            commit_field(i, R.eky, R.ey, R.fh.y, R.fh.order2);
-            commit_field(i, R.ekz, R.ez, R.fh.z, R.fh.order2);
-            R.ay[i] = R.aky[i];
-            R.az[i] = R.akz[i];
-        }
-    }
-    if (i == 0) {
-        int *h = which == 1 ? &R.ctrl->hist1 : &R.ctrl->hist2;
-        if (*h < kMaxStartOrder) *h += 1;
-    }
-}
-
-__global__ void k_commit(RunDesc R, int which) { commit_at(blockIdx.x * blockDim.x + threadIdx.x, R, which); }
 
 int launch_commit(const RunDesc &R, int which, cudaStream_t s)
 {
@@ -735,7 +308,7 @@ __global__ void k_commit_ens(const RunDesc *runs, int which)
 {
     const RunDesc &R = runs[blockIdx.y];
     if (R.ctrl->status & (STATUS_NUMERIC | STATUS_TIMEOUT)) return;
-    commit_at(blockIdx.x * blockDim.x + threadIdx.x, R, which);
+    commit_at(blockIdx.x * blockDim.x + threadIdx.x, R, which, R.ctrl->iter - 1);
 }
 
 int launch_commit_ens(const RunDesc *R, int nruns, int Mmax, int which, cudaStream_t s)
@@ -822,17 +395,23 @@ int launch_moments_to_nodes(int M, int D, bool path, double scale, const double 
     return 0;
 }
 
-__global__ void k_path_nodes(int M, int K, double scale, const double *mom, const double *mom0, const int *flux,
-                             double *out)
+template <int K>
+__global__ void k_path_nodes(int M, double scale, const double *mom, const double *mom0, const int *flux, double *out)
 {
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j < M) out[j] = scale * path_node_value(M, K, mom, mom0, flux, j);
+    if (j >= M) return;
+    out[j] = scale * path_node_value<K>(
+                         [&](int r, int m) {
+                             const size_t q = (size_t)wrap_cell(j + r, M) * K + m;
+                             return mom[q] - mom0[q];
+                         },
+                         [&](int r) { return flux[wrap_cell(j + r, M)]; });
 }
 
-int launch_path_nodes(int M, int K, double scale, const double *mom, const double *mom0, const int *flux, double *out,
+int launch_path_nodes(int M, int K_, double scale, const double *mom, const double *mom0, const int *flux, double *out,
                       cudaStream_t s)
 {
-    k_path_nodes<<<(M + 63) / 64, 64, 0, s>>>(M, K, scale, mom, mom0, flux, out);
+    PIC_FOR_DEGREE(K_, (k_path_nodes<K><<<(M + 63) / 64, 64, 0, s>>>(M, scale, mom, mom0, flux, out)))
     return 0;
 }
 
@@ -849,45 +428,49 @@ int launch_start_moments(int M, int K, const double *charge, double *mom0, cudaS
     return 0;
 }
 
-__global__ void k_cell_coefs(int M, int D, bool path, const double *c, double *tab)
+template <int D>
+__global__ void k_cell_coefs(int M, bool path, const double *c, double *tab)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, i = t / (D + 1), m = t % (D + 1);
     if (i >= M) return;
-    const int pad = coef_pad(0, D + 1);
-    for (int m = 0; m <= D; ++m) {
-        const double v = cell_coef(D, m, [&](int r) { return c[wrap_cell(i - r, M)]; });
-        tab[(size_t)i * pad + m] = path ? v / (double)(m + 1) : v;
-    }
+    const double v = cell_coef<D>(m, [&](int r) { return c[wrap_cell(i - r, M)]; });
+    tab[(size_t)i * coef_pad(0, D + 1) + m] = path ? v / (double)(m + 1) : v;
 }
 
 int launch_cell_coefs(int M, int D, bool path, const double *c, double *tab, cudaStream_t s)
 {
-    k_cell_coefs<<<(M + 63) / 64, 64, 0, s>>>(M, D, path, c, tab);
+    const int grid = (M * (D + 1) + 127) / 128;
+    switch (D) {
+    case 1: k_cell_coefs<1><<<grid, 128, 0, s>>>(M, path, c, tab); break;
+    case 2: k_cell_coefs<2><<<grid, 128, 0, s>>>(M, path, c, tab); break;
+    case 3: k_cell_coefs<3><<<grid, 128, 0, s>>>(M, path, c, tab); break;
+    case 4: k_cell_coefs<4><<<grid, 128, 0, s>>>(M, path, c, tab); break;
+    case 5: k_cell_coefs<5><<<grid, 128, 0, s>>>(M, path, c, tab); break;
+    default: return 1;
+    }
     return 0;
 }
 
-__global__ void k_tables2(int M, int K, int fp32, const double *an_y, const double *an_z, const double *ak_y,
+template <int K>
+__global__ void k_tables2(int M, int fp32, const double *an_y, const double *an_z, const double *ak_y,
                           const double *ak_z, CoefTables T)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, i = t / (2 * (K + 1)), c = t / (K + 1) & 1, m = t % (K + 1);
     if (i >= M) return;
-    a_rows(i, M, K, fp32, an_y, an_z, T.A);
-    a_rows(i, M, K, fp32, ak_y, ak_z, T.Kt);
-    if (!fp32) return;
+    const double *a = c ? an_z : an_y, *b = c ? ak_z : ak_y;
     const int pad = coef_pad(fp32, K + 1);
-    for (int c = 0; c < 2; ++c) {
-        const double *n = c ? an_z : an_y, *k = c ? ak_z : ak_y;
-        for (int m = 0; m <= K; ++m)
-            T.L[(2 * (size_t)i + c) * pad + m] =
-                sum_residue(cell_coef(K, m, [&](int r) { return n[wrap_cell(i - r, M)]; }),
-                            cell_coef(K, m, [&](int r) { return k[wrap_cell(i - r, M)]; }));
-    }
+    const size_t row = 2 * (size_t)i + c;
+    const double n = cell_coef<K>(m, [&](int r) { return a[wrap_cell(i - r, M)]; });
+    const double k = cell_coef<K>(m, [&](int r) { return b[wrap_cell(i - r, M)]; });
+    put_coef(T.A, fp32, row, pad, m, n);
+    put_coef(T.Kt, fp32, row, pad, m, k);
+    if (fp32) T.L[row * pad + m] = sum_residue(n, k);
 }
 
-int launch_tables2(int M, int K, int fp32, const double *an_y, const double *an_z, const double *ak_y,
+int launch_tables2(int M, int K_, int fp32, const double *an_y, const double *an_z, const double *ak_y,
                    const double *ak_z, CoefTables T, cudaStream_t s)
 {
-    k_tables2<<<(M + 63) / 64, 64, 0, s>>>(M, K, fp32, an_y, an_z, ak_y, ak_z, T);
+    PIC_FOR_DEGREE(K_, (k_tables2<K><<<(M * 2 * (K + 1) + 127) / 128, 128, 0, s>>>(M, fp32, an_y, an_z, ak_y, ak_z, T)))
     return 0;
 }
 

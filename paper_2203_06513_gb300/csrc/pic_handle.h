@@ -34,7 +34,7 @@ struct pic_handle {
     void *a0 = nullptr;             // start-point cache of a fixed-point loop (4 reals a marker; FP64 form)
     // spin (hbar != 0, FP64 form): components in caller order, and the spin deposits
     double *spx = nullptr, *spy = nullptr, *spz = nullptr;
-    double *sdy = nullptr, *sdz = nullptr;
+    double *sdy = nullptr, *sdz = nullptr;      // M x K each (moments, or M nodes)
 
     // split run: the markers of one plasma spread over several processes; marker
     // sums and maxima go through this reduction (NULL: all markers are here)
@@ -49,6 +49,7 @@ struct pic_handle {
     int *d_count = nullptr;             // sweeps of subsystems I and II (graph mode)
     int *h_count = nullptr;             // pinned readback of d_count
     int host_steps = 0;                 // steps taken by host loops (the first one opts kernels in)
+    pic::SmallSync *small = nullptr;    // barrier of the one-kernel steps of small plasmas
 
     // grid state (double)
     double *ex = nullptr, *ey = nullptr, *ez = nullptr, *ay = nullptr, *az = nullptr;
@@ -67,7 +68,7 @@ struct pic_handle {
     int32_t *counts = nullptr;
 
     // circulant bands and inverse taps
-    double *d_rowM0 = nullptr, *d_rowM1 = nullptr, *d_rowK = nullptr, *d_rowPm = nullptr;
+    double *d_rowM0 = nullptr, *d_rowM1 = nullptr, *d_rowK = nullptr;
     double *d_tapM1 = nullptr, *d_tapP = nullptr;
     int tapM1_start = 0, tapM1_n = 0, tapP_start = 0, tapP_n = 0;
 

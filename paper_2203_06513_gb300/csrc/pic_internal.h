@@ -309,7 +309,7 @@ struct RunDesc {
     PartPtrs P;
     double *ex, *ek, *ebar, *ay, *az, *m1[2], *m0;   // M x K moments of subsystem I: ends (by sweep parity), starts
     int *flux[2];
-    const double *rowPm, *rowK;
+    const double *rowM0, *rowM1;
     double *ey, *ez, *by, *bz, *eky, *ekz, *aky, *akz, *my[2], *mz[2];   // M x (K + 1) moments
     DevCtrl *ctrl;
     CoefTables T;
@@ -318,17 +318,40 @@ struct RunDesc {
 
 int launch_ens_plan(EnsQueue *Q, const EnsRun *runs, int nruns, unsigned long long cond, cudaStream_t s);
 int launch_ens_status(const EnsRun *runs, int nruns, int *status, cudaStream_t s);
-int conv_ens_optin(int ntap_max);
+int conv_ens_optin(int K, int ntap_max);
 int launch_conv_ens(const ConvArgs *runs, int nruns, int Mmax, int K, int ncomp, int ntap_max, EnsQueue *Q,
                     int *sweeps, unsigned long long cond, cudaStream_t s);
-int launch_prep1_ens(const RunDesc *R, int nruns, int Mmax, cudaStream_t s);
-int launch_prep2_ens(const RunDesc *R, int nruns, int Mmax, cudaStream_t s);
+int launch_prep1_ens(const RunDesc *R, int nruns, int K, int Mmax, cudaStream_t s);
+int launch_prep2_ens(const RunDesc *R, int nruns, int K, int Mmax, cudaStream_t s);
 int launch_commit_ens(const RunDesc *R, int nruns, int Mmax, int which, cudaStream_t s);
 int launch_sweep1_ens(int K, int fp32, const Sweep1Args *runs, int nruns, EnsQueue *Q, int grid, cudaStream_t s);
 int launch_sweep2_ens(int K, int fp32, const Sweep2Args *runs, int nruns, EnsQueue *Q, int grid, cudaStream_t s);
 // the predicted start of every run in the queue (delta^(0) and its current into each run's a.mom)
 int launch_predeposit_ens(int K, int fp32, const Sweep1Args *runs, int nruns, EnsQueue *Q, int grid, cudaStream_t s);
 int launch_finalize1_ens(int fp32, const RunDesc *R, int nruns, int grid_x, cudaStream_t s);
+// ---------------------------------------------------------------- small plasmas
+// Whole steps in one cooperative kernel (pic_small.cuh), one marker a thread: up to
+// num_sms * kSmallThreads markers.
+constexpr int kSmallThreads = 256;
+constexpr int kSmallSteps = 256;        // most steps a launch
+struct SmallSync {
+    // by subsystem and sweep mod 3: marker increment, field increment, field
+    unsigned long long maxima[2][3][3];
+    unsigned arrived;       // barrier arrivals since the launch (zeroed before it)
+    int abort;
+};
+struct SmallArgs {
+    RunDesc d;
+    Sweep1Args a1;
+    ConvArgs c1, c1p, c2;   // c1p: the predicted start (warm_field)
+    int nsteps, strang, warm, warm_field, zero_delta;
+    SmallSync *sync;
+    double w, hbar;
+    double *sx, *sy, *sz;   // spins, caller order (hbar != 0)
+    double *sm_y, *sm_z;    // M x K moments of the spin deposit
+};
+int launch_small_f32(const SmallArgs &a, int num_sms, cudaStream_t s);
+int launch_small_f64(const SmallArgs &a, int num_sms, cudaStream_t s);
 int launch_prep1(const RunDesc &R, cudaStream_t s);
 int launch_prep2(const RunDesc &R, cudaStream_t s);
 // end of a substep (which = 1, 2): the converged iterate becomes the state, and

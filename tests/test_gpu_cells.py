@@ -86,3 +86,47 @@ def test_device_state_equals_host_state(n, precision):
     sim.get_state(p=only)
     np.testing.assert_array_equal(only.cpu().numpy(), ref["p"])
     sim.close()
+
+
+@pytest.mark.parametrize("n,k,kw", [
+    (1, 3, {}), (31, 2, dict(warm_start=1, warm_field=1)), (33, 5, dict(splitting=1)),
+    (5003, 4, dict(sort_every=2, warm_start=1)), (38912, 3, dict(warm_start=1, warm_field=1, sort_every=3)),
+    (38913, 3, dict(warm_start=1, warm_field=1)), (4001, 3, dict(splitting=1, warm_start=1, warm_field=1)),
+    (2003, 3, dict(hbar=0.1)), (2003, 2, dict(hbar=0.1, sort_every=1))])
+def test_one_kernel_steps_equal_host_loops(n, k, kw, monkeypatch):
+    """Steps of a small plasma (one cooperative kernel, or just above its limit the graph)
+    against the same steps driven from the host: the same iteration, so rounding order
+    apart the same state and sweep counts."""
+    w = I.Workload("s", nx=50, degree=k, np=n, vth=0.2, pump=0.2, seed=n)
+    x, p = I.particles(w)
+    ay, az, ey, ez = I.fields(w)
+    az = 0.05 * np.random.default_rng(k).normal(size=w.nx)
+    spin = None
+    if "hbar" in kw:
+        s = np.random.default_rng(n).normal(size=(3, n))
+        spin = tuple(np.ascontiguousarray(v) for v in s / np.linalg.norm(s, axis=0))
+    cfg = pic.Config.from_workload(w, **kw)
+    a = pic.Pic(cfg, x, p, ay, az, ey, ez, spin=spin)
+    got_it = a.step(5)
+    got = a.state_numpy()
+    monkeypatch.setenv("PIC_NO_GRAPH", "1")
+    b = pic.Pic(cfg, x, p, ay, az, ey, ez, spin=spin)
+    ref_it = b.step(5)
+    ref = b.state_numpy()
+    assert max(abs(got_it[0] - ref_it[0]), abs(got_it[1] - ref_it[1])) <= 1
+    d = np.mod(got["x"] - ref["x"] + 0.5 * w.L, w.L) - 0.5 * w.L
+    assert np.max(np.abs(d)) / w.L < 1e-12
+    for key in ref:
+        if key != "x":
+            assert np.max(np.abs(got[key] - ref[key])) <= 1e-11 * max(np.max(np.abs(ref[key])), 1e-2), key
+    a.close()
+    b.close()
+
+
+def test_one_kernel_steps_report_no_convergence():
+    w = I.Workload("n", nx=32, degree=3, np=1000, pump=0.2)
+    x, p = I.particles(w)
+    g = pic.Pic(pic.Config.from_workload(w, max_iter=1, tol=1e-30), x, p, *I.fields(w))
+    with pytest.raises(pic.NoConvergence):
+        g.step(3)
+    g.close()
