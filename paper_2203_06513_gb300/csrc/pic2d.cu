@@ -2,21 +2,26 @@
 //
 // Spaces (Sec. 3.2): tensor-product B-splines on a uniform periodic M1 x M2 grid,
 // node i = i1 * M2 + i2; A_z on N^k x N^k, the 1-form e_xy as e_x on N^{k-1} x N^k
-// and e_y on N^k x N^{k-1}.  One thread per marker and sweep:
-//   * the path means of both V1 components along x^n -> x^(k) (the straight path
-//     split at every knot crossing of either coordinate, k-point Gauss--Legendre on
-//     each piece: the integrand is a polynomial of degree 2k - 1 there), gathered
-//     against e_bar;
-//   * the coordinate-increment difference quotients D of A_z as exact path means of
-//     dA/dx1 along x1 (at x2^(k)) and of dA/dx2 along x2 (at x1^n);
+// and e_y on N^k x N^{k-1}.  As in one dimension (pic_poly.cuh) every field is one
+// polynomial per cell, here in both centred offsets (v1, v2) with coefficients
+// sum_{r1, r2} c_{c1-r1, c2-r2} B[r1][a] B[r2][b], and deposits are moments v1^a v2^b of
+// the cell: the marker kernel evaluates no basis function, and the grid kernels convert
+// between nodes and cells once per sweep.  One thread per marker and sweep:
+//   * the path means of both V1 components along x^n -> x^(k) (the straight path split at
+//     every knot crossing of either coordinate, k-point Gauss--Legendre on each piece: the
+//     integrand is a polynomial of degree 2k - 1 there), e_bar evaluated by Horner's rule
+//     at the quadrature points;
+//   * the coordinate-increment difference quotients D of A_z: along x1 at x2^(k) the
+//     polynomial contracted over v2 (which gives A(x^(k)) as well) and its exact divided
+//     difference, along x2 at x1^n the same with the contraction over v1, which does not
+//     change during the fixed point and is kept from its first sweep;
 //   * with spins (hbar != 0), the quotients of the Zeeman term hbar s . B,
-//     B = (dA/dx2, -dA/dx1, b_z), the same way: path means of the second
-//     differences of A_z and the first differences of b_z along each coordinate;
+//     B = (dA/dx2, -dA/dx1, b_z), the same way from the contracted derivatives;
 //   * the momentum and position updates of the discrete-gradient scheme;
-//   * the current of the new path x^n -> x^(k+1), accumulated per block in shared
-//     memory over the whole grid and added to the global deposit once per node.
+//   * the moments of the new path x^n -> x^(k+1), added to the cells in global memory.
 // The grid side applies M1^{-1} = diag(M1_x^{-1} (x) M0_y^{-1}, M0_x^{-1} (x) M1_y^{-1})
 // as two circulant passes with the exact inverse rows of the 1D mass matrices.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -26,34 +31,46 @@
 #include <vector>
 
 #include "pic2d.h"
+#include "pic_hostcopy.h"
 #include "pic_internal.h"
+#include "pic_poly.cuh"
 
 namespace pic {
 namespace {
 
-constexpr int kMax2DNodes = 4096;     // M1 * M2: the block's shared-memory deposit rows
+constexpr int kMax2DNodes = 4096;     // largest M1 * M2
 constexpr int kMaxCross = 16;         // knot crossings per coordinate and path
+
+__constant__ SplineTab c_spline2 = make_spline_tab();
+
+// coefficients per cell, rows padded to 16 bytes: A (K+1)^2, e_x K (K+1) as [a][b], e_y
+// (K+1) K, b_z K^2; moments of the two current components like e_x and e_y, unpadded
+template <int K> struct Dim2 {
+    static constexpr int nA = (K + 1) * (K + 1), nE = K * (K + 1), nB = K * K;
+    static constexpr int pA = (nA + 1) & ~1, pE = (nE + 1) & ~1, pB = (nB + 1) & ~1;
+    static constexpr int nCache = K + 2;    // contraction over v1 (b = 1 .. K), A(x^n), gamma
+};
+inline int pad2(int n) { return (n + 1) & ~1; }
 
 struct Args2D {
     int M1, M2;
     long long np;
     double dx1, dx2, dt, w;
     double idx1, idx2;      // 1 / dx1, 1 / dx2
-    const double *x;        // np x 2, in the box
-    double *a0;             // np: A_z(x^n), written by the first sweep of a step
+    int2 *cell;
+    double2 *v;             // centred offsets
+    double *cache;          // nCache x np, written by the first sweep of a step
     int first;              // this is the step's first sweep
-    const double *pn;       // np x 2
-    double *d;              // np x 2 displacement iterate (length units), in/out
-    double *pk;             // np x 2 momentum iterate, in/out
-    const double *ebx, *eby;
-    const double *az, *gax, *gay;
-    double *jx, *jy;        // deposits of this sweep (zeroed before)
+    const double2 *pn;
+    double2 *d;             // displacement iterate (cell units), in/out
+    double2 *pk;            // momentum iterate, in/out
+    const double *TA, *TEx, *TEy, *TB;
+    double *mx, *my;        // moments of this sweep (zeroed before)
     double hbar;            // Zeeman terms on when non-zero (spins given)
     const double *s;        // np x 3 spins
-    const double *gxy, *gxx, *gyy, *gbx, *gby;   // G_x G_y a, G_x G_x a, G_y G_y a, G_x b_z, G_y b_z
     unsigned long long *dmax_bits, *pmax_bits;
     int *status;
-    double glx[5], glw[5];  // K-point Gauss--Legendre on [-1, 1]
+    double gls[5], glw[5];  // K-point Gauss--Legendre on [0, 1]
 };
 
 __device__ __forceinline__ int wrapi(int i, int M)
@@ -62,307 +79,200 @@ __device__ __forceinline__ int wrapi(int i, int M)
     return r < 0 ? r + M : r;
 }
 
-// [N^D(r + t)], r = 0..D: the normalised B-spline values of one cell
-template <int D>
-__device__ __forceinline__ void bsp(double t, double *v)
-{
-    bspline_scaled<D, double>(t, v);
-    const double s = 1.0 / (double)Fact<D>::v;
-#pragma unroll
-    for (int r = 0; r <= D; ++r) v[r] *= s;
-}
-
-// Pieces of the path u0 -> u0 + du (cell units, both coordinates) between knot
-// crossings: f(sa, sb) for consecutive parameter values 0 = s_0 < ... = 1.
-// Returns false when a coordinate crosses more than kMaxCross knots.
+// Pieces of the path (v1, v2) -> + (d1, d2) between knot crossings, n1 and n2 cells over:
+// f(sa, sb, k1, k2) for consecutive parameter values 0 = s_0 < ... = 1, in the cell k1, k2
+// over.
 template <class F>
-__device__ __forceinline__ bool walk2(double u0x, double u0y, double dux, double duy, F &&f)
+__device__ __forceinline__ void walk2(double v1, double v2, double d1, double d2, int n1, int n2, F &&f)
 {
-    const double ex = u0x + dux, ey = u0y + duy;
-    const int tx = dux > 0.0 ? (int)ceil(ex) - 1 - (int)floor(u0x) : (dux < 0.0 ? (int)ceil(u0x) - 1 - (int)floor(ex) : 0);
-    const int ty = duy > 0.0 ? (int)ceil(ey) - 1 - (int)floor(u0y) : (duy < 0.0 ? (int)ceil(u0y) - 1 - (int)floor(ey) : 0);
-    if (tx > kMaxCross || ty > kMaxCross) return false;
-    // next knot index and its step in each coordinate; crossing parameters by the
-    // reciprocal of the increment
-    int nx = dux > 0.0 ? (int)floor(u0x) + 1 : (int)ceil(u0x) - 1;
-    int ny = duy > 0.0 ? (int)floor(u0y) + 1 : (int)ceil(u0y) - 1;
-    const int sx = dux > 0.0 ? 1 : -1, sy = duy > 0.0 ? 1 : -1;
-    const double rx = tx > 0 ? 1.0 / dux : 0.0, ry = ty > 0 ? 1.0 / duy : 0.0;
-    int cx = 0, cy = 0;
-    double sa = 0.0;
+    double sa = 0.0, sb = 1.0, r1 = 0.0, r2 = 0.0;
+    int k1 = 0, k2 = 0;
+    const bool multi = n1 != 0 || n2 != 0;
+    const int g1 = n1 > 0 ? 1 : -1, g2 = n2 > 0 ? 1 : -1;
+    if (multi) {
+        r1 = n1 != 0 ? 1.0 / d1 : 0.0;
+        r2 = n2 != 0 ? 1.0 / d2 : 0.0;
+    }
     for (int guard = 0; guard < 2 * kMaxCross + 2; ++guard) {
-        const double bx = cx < tx ? ((double)nx - u0x) * rx : 2.0;
-        const double by = cy < ty ? ((double)ny - u0y) * ry : 2.0;
-        const double sb = fmin(fmin(bx, by), 1.0);
-        if (sb > sa) f(sa, sb);
-        if (sb >= 1.0) return true;
-        if (bx <= sb) { nx += sx; ++cx; }
-        if (by <= sb) { ny += sy; ++cy; }
-        sa = sb;
-    }
-    return true;
-}
-
-// 1D pieces of u0 -> u0 + du
-template <class F>
-__device__ __forceinline__ bool walk1(double u0, double du, F &&f)
-{
-    return walk2(u0, 0.0, du, 0.0, [&](double sa, double sb) { f(sa, sb); });
-}
-
-// One triangle for two degrees: vk[r] = D! N^D(r + t) (r = 0..D) and
-// vm[r] = (D-1)! N^{D-1}(r + t) (r = 0..D-1), both left unnormalised
-template <int D>
-__device__ __forceinline__ void bsp_pair(double t, double *vk, double *vm)
-{
-    vk[0] = 1.0;
-    if (D == 1) vm[0] = 1.0;
-#pragma unroll
-    for (int n = 1; n <= D; ++n) {
-        vk[n] = (1.0 - t) * vk[n - 1];
-#pragma unroll
-        for (int r = n - 1; r >= 1; --r) vk[r] = (t + (double)r) * vk[r] + ((double)(n + 1 - r) - t) * vk[r - 1];
-        vk[0] = t * vk[0];
-        if (n == D - 1) {
-#pragma unroll
-            for (int r = 0; r < D; ++r) vm[r] = vk[r];
+        double b1 = 2.0, b2 = 2.0;
+        if (multi) {
+            if (k1 != n1) b1 = ((double)k1 + 0.5 * g1 - v1) * r1;
+            if (k2 != n2) b2 = ((double)k2 + 0.5 * g2 - v2) * r2;
+            sb = fmin(fmin(b1, b2), 1.0);
         }
+        if (sb > sa) f(sa, sb, k1, k2);
+        if (sb >= 1.0) return;
+        if (b1 <= sb) k1 += g1;
+        if (b2 <= sb) k2 += g2;
+        sa = fmax(sa, sb);
     }
 }
 
-// sum_i c_i N^{D1}(u1 - i1) N^{D2}(u2 - i2) at one point (cell coordinates)
-template <int D1, int D2>
-__device__ __forceinline__ double value_dd(const double *c, int M1, int M2, double u1, double u2)
+// row[q] = sum_b c[q][b] y^b for the rows q = 0 .. NR - 1 of NC coefficients at `c`
+template <int NR, int NC>
+__device__ __forceinline__ void contract_rows(const double *c, double y, double (&row)[NR])
 {
-    const double c1 = floor(u1), c2 = floor(u2);
-    double v1[D1 + 1], v2[D2 + 1];
-    bspline_scaled<D1, double>(u1 - c1, v1);
-    bspline_scaled<D2, double>(u2 - c2, v2);
-    int o2[D2 + 1];
+    double q[NR * NC];
+    load_coef<NR * NC>(c, q);
 #pragma unroll
-    for (int r2 = 0; r2 <= D2; ++r2) o2[r2] = wrapi((int)c2 - r2, M2);
-    double s = 0.0;
+    for (int a = 0; a < NR; ++a) {
+        double s = q[a * NC + NC - 1];
 #pragma unroll
-    for (int r1 = 0; r1 <= D1; ++r1) {
-        const double *row = c + wrapi((int)c1 - r1, M1) * M2;
-        double t = 0.0;
-#pragma unroll
-        for (int r2 = 0; r2 <= D2; ++r2) t = fma(v2[r2], row[o2[r2]], t);
-        s = fma(v1[r1], t, s);
-    }
-    return s * (1.0 / ((double)Fact<D1>::v * (double)Fact<D2>::v));
-}
-
-template <int K>
-__device__ __forceinline__ double value0(const double *a, int M1, int M2, double u1, double u2)
-{
-    return value_dd<K, K>(a, M1, M2, u1, u2);
-}
-
-// The basis weights of one knot piece [sa, sb] of the path u0 -> u0 + du (inside
-// the cell (c1, c2)): mx[r1][r2] = (sb - sa) x the mean over the piece of the
-// x-component basis N^{K-1} x N^K at node (c1 - r1, c2 - r2), my likewise for the
-// y-component N^K x N^{K-1}, both times (K-1)! K! (unnormalised B-splines).
-// K-point Gauss--Legendre is exact: the integrand is a polynomial of degree
-// 2K - 1 in the path parameter.
-template <int K>
-__device__ __forceinline__ void piece_weights(const Args2D &A, double u0x, double u0y, double dux, double duy,
-                                              double sa, double sb, double c1, double c2, double (&mx)[K][K + 1],
-                                              double (&my)[K + 1][K])
-{
-    const double sm = 0.5 * (sa + sb), hs = 0.5 * (sb - sa);
-#pragma unroll
-    for (int g = 0; g < K; ++g) {
-        const double s = fma(hs, A.glx[g], sm);
-        const double wq = hs * A.glw[g];
-        double b1k[K + 1], b1m[K], b2k[K + 1], b2m[K];
-        bsp_pair<K>(fma(s, dux, u0x) - c1, b1k, b1m);
-        bsp_pair<K>(fma(s, duy, u0y) - c2, b2k, b2m);
-#pragma unroll
-        for (int r1 = 0; r1 < K; ++r1) {
-            const double f = wq * b1m[r1];
-#pragma unroll
-            for (int r2 = 0; r2 <= K; ++r2) mx[r1][r2] = g == 0 ? f * b2k[r2] : fma(f, b2k[r2], mx[r1][r2]);
-        }
-#pragma unroll
-        for (int r1 = 0; r1 <= K; ++r1) {
-            const double f = wq * b1k[r1];
-#pragma unroll
-            for (int r2 = 0; r2 < K; ++r2) my[r1][r2] = g == 0 ? f * b2m[r2] : fma(f, b2m[r2], my[r1][r2]);
-        }
+        for (int b = NC - 2; b >= 0; --b) s = fma(s, y, q[a * NC + b]);
+        row[a] = s;
     }
 }
 
-// node offsets of the cell (c1, c2): o1[r] = ((c1 - r) mod M1) M2, o2[r] = (c2 - r) mod M2
-template <int K>
-__device__ __forceinline__ void cell_offsets(const Args2D &A, double c1, double c2, int *o1, int *o2)
+// col[q] = sum_a c[a][q] x^a
+template <int NR, int NC>
+__device__ __forceinline__ void contract_cols(const double *c, double x, double (&col)[NC])
 {
+    double q[NR * NC];
+    load_coef<NR * NC>(c, q);
 #pragma unroll
-    for (int r = 0; r <= K; ++r) {
-        o1[r] = wrapi((int)c1 - r, A.M1) * A.M2;
-        o2[r] = wrapi((int)c2 - r, A.M2);
+    for (int b = 0; b < NC; ++b) {
+        double s = q[(NR - 1) * NC + b];
+#pragma unroll
+        for (int a = NR - 2; a >= 0; --a) s = fma(s, x, q[a * NC + b]);
+        col[b] = s;
     }
 }
 
-// (Ex, Ey) = the path means of e_bar's two components along u0 -> u0 + du
-template <int K>
-__device__ __forceinline__ bool gather_path(const Args2D &A, double u0x, double u0y, double dux, double duy,
-                                            double &Ex, double &Ey)
+// d/dy of the rows: row[q] = sum_{b >= 1} b c[q][b] y^(b-1)
+template <int NR, int NC>
+__device__ __forceinline__ void contract_rows_dy(const double *c, double y, double (&row)[NR])
 {
-    double sx = 0.0, sy = 0.0;
-    const bool ok = walk2(u0x, u0y, dux, duy, [&](double sa, double sb) {
-        const double sm = 0.5 * (sa + sb);
-        const double c1 = floor(fma(sm, dux, u0x)), c2 = floor(fma(sm, duy, u0y));
-        double mx[K][K + 1], my[K + 1][K];
-        piece_weights<K>(A, u0x, u0y, dux, duy, sa, sb, c1, c2, mx, my);
-        int o1[K + 1], o2[K + 1];
-        cell_offsets<K>(A, c1, c2, o1, o2);
 #pragma unroll
-        for (int r1 = 0; r1 <= K; ++r1) {
-            const double *rx = A.ebx + o1[r1], *ry = A.eby + o1[r1];
+    for (int a = 0; a < NR; ++a) {
+        double s = (double)(NC - 1) * c[a * NC + NC - 1];
 #pragma unroll
-            for (int r2 = 0; r2 <= K; ++r2) {
-                if (r1 < K) sx = fma(mx[r1 < K ? r1 : 0][r2], rx[o2[r2]], sx);
-                if (r2 < K) sy = fma(my[r1][r2 < K ? r2 : 0], ry[o2[r2]], sy);
-            }
-        }
-    });
-    const double scale = 1.0 / ((double)Fact<K - 1>::v * (double)Fact<K>::v);
-    Ex = sx * scale;
-    Ey = sy * scale;
-    return ok;
+        for (int b = NC - 2; b >= 1; --b) s = fma(s, y, (double)b * c[a * NC + b]);
+        row[a] = s;
+    }
 }
 
-// s_j[x | y] += (wx, wy) x the path means of the two basis components along
-// u0 -> u0 + du, one shared-memory add per node and knot piece
-template <int K>
-__device__ __forceinline__ bool deposit_path(const Args2D &A, double *s_j, int N, double u0x, double u0y, double dux,
-                                             double duy, double wx, double wy)
+template <int NR, int NC>
+__device__ __forceinline__ void contract_cols_dx(const double *c, double x, double (&col)[NC])
 {
-    const double scale = 1.0 / ((double)Fact<K - 1>::v * (double)Fact<K>::v);
-    const double cx = wx * scale, cy = wy * scale;
-    return walk2(u0x, u0y, dux, duy, [&](double sa, double sb) {
-        const double sm = 0.5 * (sa + sb);
-        const double c1 = floor(fma(sm, dux, u0x)), c2 = floor(fma(sm, duy, u0y));
-        double mx[K][K + 1], my[K + 1][K];
-        piece_weights<K>(A, u0x, u0y, dux, duy, sa, sb, c1, c2, mx, my);
-        int o1[K + 1], o2[K + 1];
-        cell_offsets<K>(A, c1, c2, o1, o2);
 #pragma unroll
-        for (int r1 = 0; r1 <= K; ++r1) {
+    for (int b = 0; b < NC; ++b) {
+        double s = (double)(NR - 1) * c[(NR - 1) * NC + b];
 #pragma unroll
-            for (int r2 = 0; r2 <= K; ++r2) {
-                const int i = o1[r1] + o2[r2];
-                if (r1 < K && cx != 0.0) atomicAdd(&s_j[i], cx * mx[r1 < K ? r1 : 0][r2]);
-                if (r2 < K && cy != 0.0) atomicAdd(&s_j[N + i], cy * my[r1][r2 < K ? r2 : 0]);
-            }
-        }
-    });
+        for (int a = NR - 2; a >= 1; --a) s = fma(s, x, (double)a * c[a * NC + b]);
+        col[b] = s;
+    }
 }
 
-// mean of dA/dx1 along x1 from u0 to u0 + du at fixed x2 (cell coordinate uo):
-// sum (G_x a)_i (mean of N^{K-1}(x1 - i1)) N^K(x2 - i2); and the same along x2.
-// The across factor is contracted once per knot piece; the along factor is the
-// exact piece mean of the midpoint form (no quadrature nodes).
-template <int K>
-__device__ __forceinline__ double dA_mean(const Args2D &A, int axis, double u0, double du, double uo)
+// One piece of a coordinate-increment quotient: the sums of a path along one coordinate
+// (n cells over, from v0 to the end offset ve), piece q of 0 .. |n|.  h: its length, or 1
+// for a path in one cell (the mean itself).
+template <int N>
+__device__ __forceinline__ double quotient_piece(int q, int n, double v0, double ve, double (&S)[N])
 {
-    const double co = floor(uo);
-    double vo[K + 1];
-    bspline_scaled<K, double>(uo - co, vo);
-    const double *ga = axis == 0 ? A.gax : A.gay;
-    const int Ma = axis == 0 ? A.M1 : A.M2, Mo = axis == 0 ? A.M2 : A.M1;
-    const int sa_ = axis == 0 ? A.M2 : 1, so = axis == 0 ? 1 : A.M2;
-    int io[K + 1];
-#pragma unroll
-    for (int ro = 0; ro <= K; ++ro) io[ro] = wrapi((int)co - ro, Mo) * so;
-    double s = 0.0;
-    walk1(u0, du, [&](double pa, double pb) {
-        const double sm = 0.5 * (pa + pb), hs = 0.5 * (pb - pa);
-        const double c = floor(fma(sm, du, u0));
-        double col[K];
-#pragma unroll
-        for (int r = 0; r < K; ++r) {
-            const double *q = ga + wrapi((int)c - r, Ma) * sa_;
-            double acc = 0.0;
-#pragma unroll
-            for (int ro = 0; ro <= K; ++ro) acc = fma(q[io[ro]], vo[ro], acc);
-            col[r] = acc;
-        }
-        // the exact mean of the degree-(K-1) pieces over this piece (midpoint form,
-        // S_{K-1} times the mean), times its parameter length and (K-1)! / S_{K-1}
-        double m[K];
-        piece_means_scaled<K - 1, double>(fma(sm, du, u0) - c, 2.0 * hs * du, m);
-        double v = 0.0;
-#pragma unroll
-        for (int r = 0; r < K; ++r) v = fma(m[r], col[r], v);
-        constexpr double kPM = (double)Fact<K - 1>::v / (double)MeanScale<K - 1>::S;
-        s = fma(2.0 * hs * kPM, v, s);
-    });
-    return s * (1.0 / ((double)Fact<K - 1>::v * (double)Fact<K>::v));
+    const int an = abs(n);
+    const double edge = n > 0 ? 0.5 : -0.5;
+    const double va = q == 0 ? v0 : -edge, vb = q == an ? ve : edge;
+    path_sums<N, double>(va, vb, S);
+    return an == 0 ? 1.0 : vb - va;
 }
 
-// One coordinate-increment quotient of the Zeeman term along `axis`: the mean over
-// u_axis in [u0, u0 + du] (the other coordinate fixed at uo) of
-//   wm dF_m/du + wp dF_p/du + wb dF_b/du,
-// given the derivative coefficients on their own degrees (along, across):
-// cm on (K-1, K-1), cp on (K-2, K), cb on (K-2, K-1).  Along x1 these are
-// G_x G_y a, G_x G_x a and G_x b_z; along x2, G_x G_y a, G_y G_y a and G_y b_z.
-template <int K>
-__device__ __forceinline__ double zee_mean(const Args2D &A, int axis, double u0, double du, double uo,
-                                           const double *cm, double wm, const double *cp, double wp,
-                                           const double *cb, double wb)
+// sum_{q >= 1} c_q S_{q-1}: the divided difference of the polynomial c
+template <int N>
+__device__ __forceinline__ double divided(const double (&c)[N], const double (&S)[N - 1])
 {
-    const double co = floor(uo);
-    double vk[K + 1], vm[K];
-    bsp_pair<K>(uo - co, vk, vm);
-    // normalisations of the unnormalised values folded into the weights
-    constexpr double fk = (double)Fact<K>::v, fm = (double)Fact<K - 1>::v, f2 = (double)Fact<K - 2>::v;
-    const double em = wm * (1.0 / (fm * fm)), ep = wp * (1.0 / (f2 * fk)), eb = wb * (1.0 / (f2 * fm));
-    const int Ma = axis == 0 ? A.M1 : A.M2, Mo = axis == 0 ? A.M2 : A.M1;
-    const int sa = axis == 0 ? A.M2 : 1, so = axis == 0 ? 1 : A.M2;
-    int io[K + 1];
+    double s = c[1];
 #pragma unroll
-    for (int ro = 0; ro <= K; ++ro) io[ro] = wrapi((int)co - ro, Mo) * so;
-    double s = 0.0;
-    walk1(u0, du, [&](double pa, double pb) {
-        const double sm = 0.5 * (pa + pb), hs = 0.5 * (pb - pa);
-        const double c = floor(fma(sm, du, u0));
-        double colm[K], colq[K - 1];
-#pragma unroll
-        for (int r = 0; r < K; ++r) {
-            const int ia = wrapi((int)c - r, Ma) * sa;
-            double am = 0.0;
-#pragma unroll
-            for (int ro = 0; ro < K; ++ro) am = fma(cm[ia + io[ro]], vm[ro], am);
-            colm[r] = em * am;
-            if (r < K - 1) {
-                double ap = 0.0, ab = 0.0;
-#pragma unroll
-                for (int ro = 0; ro <= K; ++ro) ap = fma(cp[ia + io[ro]], vk[ro], ap);
-#pragma unroll
-                for (int ro = 0; ro < K; ++ro) ab = fma(cb[ia + io[ro]], vm[ro], ab);
-                colq[r < K - 1 ? r : 0] = ep * ap + eb * ab;
-            }
-        }
-        // exact means of the degree-(K-1) and degree-(K-2) pieces over this piece
-        // (midpoint form, S_D times the mean; degree 0 is 1 inside one cell), each
-        // times D! / S_D to match the unnormalised values the weights expect
-        const double tm = fma(sm, du, u0) - c, hh = 2.0 * hs * du;
-        double m1[K], m2[K - 1];
-        piece_means_scaled<K - 1, double>(tm, hh, m1);
-        if constexpr (K >= 3) piece_means_scaled<(K >= 3 ? K - 2 : 1), double>(tm, hh, m2);
-        else m2[0] = 1.0;
-        constexpr double c1 = (double)Fact<K - 1>::v / (double)MeanScale<K - 1>::S;
-        constexpr double c2 = (double)Fact<K - 2>::v / (double)MeanScale<K - 2>::S;
-        double v1 = 0.0, v2 = 0.0;
-#pragma unroll
-        for (int r = 0; r < K; ++r) v1 = fma(m1[r], colm[r], v1);
-#pragma unroll
-        for (int r = 0; r < K - 1; ++r) v2 = fma(m2[r], colq[r], v2);
-        s = fma(2.0 * hs, c1 * v1 + c2 * v2, s);
-    });
+    for (int q = 2; q < N; ++q) s = fma(c[q], S[q - 1], s);
     return s;
+}
+
+// (Ex, Ey) = the path means of e_bar's two components
+template <int K>
+__device__ __forceinline__ void gather_path(const Args2D &A, int2 c, double2 v, double2 d, int n1, int n2, double &Ex,
+                                            double &Ey)
+{
+    Ex = Ey = 0.0;
+    walk2(v.x, v.y, d.x, d.y, n1, n2, [&](double sa, double sb, int k1, int k2) {
+        int cell = c.x * A.M2 + c.y;
+        double x0 = v.x, y0 = v.y;
+        if (k1 != 0 || k2 != 0) {
+            cell = wrapi(c.x + k1, A.M1) * A.M2 + wrapi(c.y + k2, A.M2);
+            x0 -= (double)k1;
+            y0 -= (double)k2;
+        }
+        double ex[K * (K + 1)], ey[K * (K + 1)];
+        load_coef<K * (K + 1)>(A.TEx + (size_t)cell * Dim2<K>::pE, ex);
+        load_coef<K * (K + 1)>(A.TEy + (size_t)cell * Dim2<K>::pE, ey);
+        const double h = sb - sa;
+#pragma unroll
+        for (int g = 0; g < K; ++g) {
+            const double s = fma(h, A.gls[g], sa), wq = h * A.glw[g];
+            const double x = fma(s, d.x, x0), y = fma(s, d.y, y0);
+            double px = 0.0, py = 0.0;
+#pragma unroll
+            for (int a = K; a >= 0; --a) {
+                if (a < K) {
+                    double r = ex[a * (K + 1) + K];
+#pragma unroll
+                    for (int b = K - 1; b >= 0; --b) r = fma(r, y, ex[a * (K + 1) + b]);
+                    px = a == K - 1 ? r : fma(px, x, r);
+                }
+                double r = ey[a * K + K - 1];
+#pragma unroll
+                for (int b = K - 2; b >= 0; --b) r = fma(r, y, ey[a * K + b]);
+                py = a == K ? r : fma(py, x, r);
+            }
+            Ex = fma(wq, px, Ex);
+            Ey = fma(wq, py, Ey);
+        }
+    });
+}
+
+// (wx, wy) x the path moments of the two components to the cells, one addition in global
+// memory per moment and piece
+template <int K>
+__device__ __forceinline__ void deposit_path(const Args2D &A, int2 c, double2 v, double2 d, int n1, int n2, double wx,
+                                             double wy)
+{
+    walk2(v.x, v.y, d.x, d.y, n1, n2, [&](double sa, double sb, int k1, int k2) {
+        int cell = c.x * A.M2 + c.y;
+        double x0 = v.x, y0 = v.y;
+        if (k1 != 0 || k2 != 0) {
+            cell = wrapi(c.x + k1, A.M1) * A.M2 + wrapi(c.y + k2, A.M2);
+            x0 -= (double)k1;
+            y0 -= (double)k2;
+        }
+        const double h = sb - sa;
+        double m[K + 1][K + 1];
+#pragma unroll
+        for (int g = 0; g < K; ++g) {
+            const double s = fma(h, A.gls[g], sa), wq = h * A.glw[g];
+            const double x = fma(s, d.x, x0), y = fma(s, d.y, y0);
+            double yp[K + 1];
+            yp[0] = 1.0;
+#pragma unroll
+            for (int b = 1; b <= K; ++b) yp[b] = b == 1 ? y : yp[b - 1] * y;
+            double xa = wq;
+#pragma unroll
+            for (int a = 0; a <= K; ++a) {
+#pragma unroll
+                for (int b = 0; b <= K; ++b) {
+                    if (a == K && b == K) continue;
+                    const double t = b == 0 ? xa : xa * yp[b];
+                    m[a][b] = g == 0 ? t : (b == 0 ? m[a][b] + xa : fma(xa, yp[b], m[a][b]));
+                }
+                xa *= x;
+            }
+        }
+        double *px = A.mx + (size_t)cell * Dim2<K>::nE, *py = A.my + (size_t)cell * Dim2<K>::nE;
+#pragma unroll
+        for (int a = 0; a <= K; ++a)
+#pragma unroll
+            for (int b = 0; b <= K; ++b) {
+                if (a < K && wx != 0.0) atomicAdd(px + a * (K + 1) + b, wx * m[a][b]);
+                if (b < K && wy != 0.0) atomicAdd(py + a * K + b, wy * m[a][b]);
+            }
+    });
 }
 
 __device__ __forceinline__ void max_bits(unsigned long long *dst, double v)
@@ -376,15 +286,17 @@ __device__ __forceinline__ void max_bits(unsigned long long *dst, double v)
 // predictor delta^(0) = dt p^n / gamma(p^n, A(x^n)) written and the current of
 // x^n -> x^n + delta^(0) deposited, so that the fixed point can start from the
 // field consistent with it; no gather, no momentum update, no increments.
+//
+// Bound by the FP64 pipe.  With basis values at the quadrature points and 24 weights per
+// piece, added to the block's shared rows by compare-and-swap, the sweep took 1068 FP64
+// operations a marker (cubic, path in one cell) and 4.1 ms for 2e6 markers.
 template <int K, bool PRE = false>
 __global__ void __launch_bounds__(256, K <= 3 ? 2 : 1) k2_sweep(Args2D A)
 {
-    extern __shared__ double s_j[];     // 2 * M1 * M2: x then y
+    using Dm = Dim2<K>;
+    constexpr int NC = K + 1;
     __shared__ int s_perm[256];
     __shared__ int s_cnt[8];
-    const int N = A.M1 * A.M2;
-    for (int i = threadIdx.x; i < 2 * N; i += blockDim.x) s_j[i] = 0.0;
-    __syncthreads();
     double dm = 0.0, pm = 0.0;
     bool bad = false;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -399,11 +311,13 @@ __global__ void __launch_bounds__(256, K <= 3 ? 2 : 1) k2_sweep(Args2D A)
             const long long b = base + threadIdx.x;
             bool multi = true;
             if (b < A.np) {
-                // the predicted start's path is within dt p (gamma >= 1)
-                const double vx = A.x[2 * b] * A.idx1, vy = A.x[2 * b + 1] * A.idx2;
-                const double ex = PRE ? A.dt * A.pn[2 * b] : A.d[2 * b];
-                const double ey = PRE ? A.dt * A.pn[2 * b + 1] : A.d[2 * b + 1];
-                multi = floor(vx + ex * A.idx1) != floor(vx) || floor(vy + ey * A.idx2) != floor(vy);
+                const double2 v = A.v[b];
+                double2 d = A.d[b];
+                if (PRE) {                      // the predicted start's path is within dt p (gamma >= 1)
+                    const double2 p = A.pn[b];
+                    d = make_double2(A.dt * p.x * A.idx1, A.dt * p.y * A.idx2);
+                }
+                multi = !within(v.x + d.x, 0.5) || !within(v.y + d.y, 0.5);
             }
             const unsigned one = __ballot_sync(0xffffffffu, !multi);
             if (lane == 0) s_cnt[wid] = __popc(one);
@@ -421,145 +335,306 @@ __global__ void __launch_bounds__(256, K <= 3 ? 2 : 1) k2_sweep(Args2D A)
         const long long a = base + s_perm[threadIdx.x];
         __syncthreads();                    // s_perm and s_cnt are free for the next group
         if (a >= A.np) continue;
-        {
-        const double u0x = A.x[2 * a] * A.idx1, u0y = A.x[2 * a + 1] * A.idx2;
-        const double d0 = A.d[2 * a], d1 = A.d[2 * a + 1];
-        const double p0 = A.pn[2 * a], p1 = A.pn[2 * a + 1];
-        const double dux = d0 * A.idx1, duy = d1 * A.idx2;
+        const int2 c = A.cell[a];
+        const double2 v = A.v[a], p = A.pn[a];
+        double2 d = PRE ? make_double2(0.0, 0.0) : A.d[a];
+        const double pp1 = fma(p.x, p.x, fma(p.y, p.y, 1.0));
+        // beta_b: A contracted over v1 at x1^n; A(x^n) and gamma(p^n, A(x^n)); the same in
+        // every sweep of the step
+        double be[NC], A0, g0;
+        if (PRE || A.first) {
+            contract_cols<NC, NC>(A.TA + (size_t)(c.x * A.M2 + c.y) * Dm::pA, v.x, be);
+            A0 = horner<NC>(be, v.y);
+            g0 = root(fma(A0, A0, pp1));
+#pragma unroll
+            for (int b = 1; b <= K; ++b) A.cache[(size_t)(b - 1) * A.np + a] = be[b];
+            A.cache[(size_t)K * A.np + a] = A0;
+            A.cache[(size_t)(K + 1) * A.np + a] = g0;
+        } else {
+            be[0] = 0.0;
+#pragma unroll
+            for (int b = 1; b <= K; ++b) be[b] = A.cache[(size_t)(b - 1) * A.np + a];
+            A0 = A.cache[(size_t)K * A.np + a];
+            g0 = A.cache[(size_t)(K + 1) * A.np + a];
+        }
         if constexpr (PRE) {
-            const double A0 = value0<K>(A.az, A.M1, A.M2, u0x, u0y);
-            A.a0[a] = A0;
-            const double r = A.dt / sqrt(1.0 + p0 * p0 + p1 * p1 + A0 * A0);
-            const double n0 = r * p0, n1 = r * p1;
-            if (!deposit_path<K>(A, s_j, N, u0x, u0y, n0 * A.idx1, n1 * A.idx2, A.w * n0, A.w * n1)) bad = true;
-            A.d[2 * a] = n0;
-            A.d[2 * a + 1] = n1;
+            const double r = quotient(A.dt, g0);
+            const double x0 = r * p.x, x1 = r * p.y;
+            d = make_double2(x0 * A.idx1, x1 * A.idx2);
+            if (!within(d.x, 1024.0) || !within(d.y, 1024.0)) { bad = true; continue; }
+            int n1, n2;
+            double e1, e2;
+            path_end(v.x, d.x, n1, e1);
+            path_end(v.y, d.y, n2, e2);
+            if (abs(n1) > kMaxCross || abs(n2) > kMaxCross) bad = true;
+            else deposit_path<K>(A, c, v, d, n1, n2, A.w * x0, A.w * x1);
+            A.d[a] = d;
             continue;
         }
-        // A(x^n) is the same in every sweep of the step: evaluated in the first
-        double A0;
-        if (A.first) {
-            A0 = value0<K>(A.az, A.M1, A.M2, u0x, u0y);
-            A.a0[a] = A0;
-        } else {
-            A0 = A.a0[a];
+        int n1, n2;
+        double e1, e2;
+        path_end(v.x, d.x, n1, e1);
+        path_end(v.y, d.y, n2, e2);
+        const bool spin = A.hbar != 0.0;
+        double sx = 0.0, sy = 0.0, sz = 0.0, Z1 = 0.0, Z2 = 0.0;
+        if (spin) {
+            sx = A.s[3 * a] * A.idx2;           // s_x dA/dx2, s_y dA/dx1 in cell units
+            sy = A.s[3 * a + 1] * A.idx1;
+            sz = A.s[3 * a + 2];
         }
-        const double A1 = value0<K>(A.az, A.M1, A.M2, u0x + dux, u0y + duy);
+        // along x1 at x2^(k): alpha_a, A contracted over v2; A(x^(k)) in the last cell
+        double D1 = 0.0, W1 = 0.0, A1 = 0.0;
+        for (int q = 0; q <= abs(n1); ++q) {
+            int cell = c.x * A.M2 + c.y;
+            if (n1 != 0 || n2 != 0)
+                cell = wrapi(c.x + (n1 > 0 ? q : -q), A.M1) * A.M2 + wrapi(c.y + n2, A.M2);
+            double al[NC], S[K];
+            const double *row = A.TA + (size_t)cell * Dm::pA;
+            contract_rows<NC, NC>(row, e2, al);
+            const double h = quotient_piece<K>(q, n1, v.x, e1, S);
+            D1 = fma(h, divided<NC>(al, S), D1);
+            W1 += h;
+            if (q == abs(n1)) A1 = horner<NC>(al, e1);
+            if (spin) {
+                // f = s_x dA/dx2 - s_y dA/dx1 + s_z b_z contracted over v2, its quotient
+                double ady[NC], bz[K], f[NC];
+                contract_rows_dy<NC, NC>(row, e2, ady);
+                contract_rows<K, K>(A.TB + (size_t)cell * Dm::pB, e2, bz);
+#pragma unroll
+                for (int m = 0; m <= K; ++m) {
+                    f[m] = sx * ady[m];
+                    if (m < K) f[m] += sz * bz[m < K ? m : 0] - sy * (double)(m + 1) * al[m < K ? m + 1 : 0];
+                }
+                Z1 = fma(h, divided<NC>(f, S), Z1);
+            }
+        }
+        // along x2 at x1^n
+        double D2 = 0.0, W2 = 0.0;
+        for (int q = 0; q <= abs(n2); ++q) {
+            const int cell = q == 0 ? c.x * A.M2 + c.y : c.x * A.M2 + wrapi(c.y + (n2 > 0 ? q : -q), A.M2);
+            const double *row = A.TA + (size_t)cell * Dm::pA;
+            double bq[NC], S[K];
+            if (q == 0) {
+#pragma unroll
+                for (int b = 0; b <= K; ++b) bq[b] = be[b];
+            } else {
+                contract_cols<NC, NC>(row, v.x, bq);
+            }
+            const double h = quotient_piece<K>(q, n2, v.y, e2, S);
+            D2 = fma(h, divided<NC>(bq, S), D2);
+            W2 += h;
+            if (spin) {
+                double adx[NC], bz[K], f[NC];
+                contract_cols_dx<NC, NC>(row, v.x, adx);
+                contract_cols<K, K>(A.TB + (size_t)cell * Dm::pB, v.x, bz);
+#pragma unroll
+                for (int m = 0; m <= K; ++m) {
+                    f[m] = -sy * adx[m];
+                    if (m < K) f[m] += sz * bz[m < K ? m : 0] + sx * (double)(m + 1) * bq[m < K ? m + 1 : 0];
+                }
+                Z2 = fma(h, divided<NC>(f, S), Z2);
+            }
+        }
+        if (n1 != 0) { D1 = quotient(D1, W1); Z1 = Z1 / W1; }
+        if (n2 != 0) { D2 = quotient(D2, W2); Z2 = Z2 / W2; }
         double Ex, Ey;
-        bool ok = gather_path<K>(A, u0x, u0y, dux, duy, Ex, Ey);
-        const double D1 = dA_mean<K>(A, 0, u0x, dux, u0y + duy);
-        const double D2 = dA_mean<K>(A, 1, u0y, duy, u0x);
-        const double pp = p0 * p0 + p1 * p1;
-        const double g0 = sqrt(1.0 + pp + A0 * A0);
-        const double g1 = sqrt(1.0 + pp + A1 * A1);
-        const double f = A.dt * (A1 + A0) / (g1 + g0);
-        double q0 = p0 + A.dt * Ex - f * D1;
-        double q1 = p1 + A.dt * Ey - f * D2;
-        if (A.hbar != 0.0) {
-            // discrete gradient of hbar s . B, B = (dA/dx2, -dA/dx1, b_z)
-            const double sx = A.s[3 * a], sy = A.s[3 * a + 1], sz = A.s[3 * a + 2];
-            const double Z1 = zee_mean<K>(A, 0, u0x, dux, u0y + duy, A.gxy, sx, A.gxx, -sy, A.gbx, sz);
-            const double Z2 = zee_mean<K>(A, 1, u0y, duy, u0x, A.gxy, -sy, A.gyy, sx, A.gby, sz);
-            q0 -= A.dt * A.hbar * Z1;
-            q1 -= A.dt * A.hbar * Z2;
+        gather_path<K>(A, c, v, d, n1, n2, Ex, Ey);
+        const double g1 = root(fma(A1, A1, pp1));
+        const double f = quotient(A.dt * (A1 + A0), g1 + g0);
+        double q0 = fma(A.dt, Ex, p.x) - f * (D1 * A.idx1);
+        double q1 = fma(A.dt, Ey, p.y) - f * (D2 * A.idx2);
+        if (spin) {
+            q0 -= A.dt * A.hbar * Z1 * A.idx1;
+            q1 -= A.dt * A.hbar * Z2 * A.idx2;
         }
-        const double g2 = sqrt(1.0 + q0 * q0 + q1 * q1 + A1 * A1);
-        const double r = A.dt / (g1 + g2);
-        const double n0 = r * (p0 + q0);
-        const double n1 = r * (p1 + q1);
-        if (!(isfinite(n0) && isfinite(n1))) { bad = true; continue; }
+        const double g2 = root(fma(q0, q0, fma(q1, q1, fma(A1, A1, 1.0))));
+        const double r = quotient(A.dt, g1 + g2);
+        const double x0 = r * (p.x + q0), x1 = r * (p.y + q1);
+        const double2 dn = make_double2(x0 * A.idx1, x1 * A.idx2);
+        if (!within(dn.x, 1024.0) || !within(dn.y, 1024.0)) { bad = true; continue; }
         // the current of the new path
-        ok = ok && deposit_path<K>(A, s_j, N, u0x, u0y, n0 * A.idx1, n1 * A.idx2, A.w * n0, A.w * n1);
-        if (!ok) bad = true;
-        dm = fmax(dm, fmax(fabs(n0 - d0), fabs(n1 - d1)));
-        pm = fmax(pm, fmax(fabs(q0 - A.pk[2 * a]), fabs(q1 - A.pk[2 * a + 1])));
-        A.d[2 * a] = n0;
-        A.d[2 * a + 1] = n1;
-        A.pk[2 * a] = q0;
-        A.pk[2 * a + 1] = q1;
-        }
+        path_end(v.x, dn.x, n1, e1);
+        path_end(v.y, dn.y, n2, e2);
+        if (abs(n1) > kMaxCross || abs(n2) > kMaxCross) bad = true;
+        else deposit_path<K>(A, c, v, dn, n1, n2, A.w * x0, A.w * x1);
+        const double2 po = A.pk[a];
+        dm = max_nonneg(dm, max_nonneg(fabs(dn.x - d.x) * A.dx1, fabs(dn.y - d.y) * A.dx2));
+        pm = max_nonneg(pm, max_nonneg(fabs(q0 - po.x), fabs(q1 - po.y)));
+        A.d[a] = dn;
+        A.pk[a] = make_double2(q0, q1);
     }
     if (bad) atomicOr(A.status, STATUS_NUMERIC);
+    if (PRE) return;
     // block maxima of the increments
     __shared__ double s_m[2][8];
     for (int o = 16; o > 0; o >>= 1) {
-        dm = fmax(dm, __shfl_xor_sync(0xffffffffu, dm, o));
-        pm = fmax(pm, __shfl_xor_sync(0xffffffffu, pm, o));
+        dm = max_nonneg(dm, __shfl_xor_sync(0xffffffffu, dm, o));
+        pm = max_nonneg(pm, __shfl_xor_sync(0xffffffffu, pm, o));
     }
     if ((threadIdx.x & 31) == 0) {
         s_m[0][threadIdx.x >> 5] = dm;
         s_m[1][threadIdx.x >> 5] = pm;
     }
     __syncthreads();
-    if (threadIdx.x == 0 && !PRE) {
+    if (threadIdx.x == 0) {
         double a = 0.0, b = 0.0;
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-            a = fmax(a, s_m[0][w]);
-            b = fmax(b, s_m[1][w]);
+            a = max_nonneg(a, s_m[0][w]);
+            b = max_nonneg(b, s_m[1][w]);
         }
         max_bits(A.dmax_bits, a);
         max_bits(A.pmax_bits, b);
     }
-    for (int i = threadIdx.x; i < 2 * N; i += blockDim.x) {
-        const double v = s_j[i];
-        if (v != 0.0) atomicAdd(i < N ? &A.jx[i] : &A.jy[i - N], v);
-    }
 }
 
-// out[i1, i2] = sum_q g[(i_axis - q) mod M_axis] in[.. q ..] along one axis
-__global__ void k2_circ(int M1, int M2, int axis, const double *g, const double *in, double *out)
+// Coefficient (a, b) of the degree (D1, D2) field with nodes c in every cell: thread per
+// (cell, a, b), coefficients fastest; rows of `pad` numbers.
+template <int D1, int D2>
+__device__ __forceinline__ void table2_at(long long t, int M1, int M2, const double *c, double *tab, int pad)
 {
-    const int N = M1 * M2;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
-        const int i1 = i / M2, i2 = i % M2;
-        double s = 0.0;
-        if (axis == 0) {
-            for (int q = 0; q < M1; ++q) s += g[wrapi(i1 - q, M1)] * in[q * M2 + i2];
-        } else {
-            for (int q = 0; q < M2; ++q) s += g[wrapi(i2 - q, M2)] * in[i1 * M2 + q];
+    constexpr int n = (D1 + 1) * (D2 + 1);
+    const int cell = (int)(t / n), q = (int)(t % n), a = q / (D2 + 1), b = q % (D2 + 1);
+    const int c1 = cell / M2, c2 = cell % M2;
+    int o2[D2 + 1];
+#pragma unroll
+    for (int r = 0; r <= D2; ++r) o2[r] = wrapi(c2 - r, M2);
+    double s = 0.0;
+#pragma unroll
+    for (int r1 = 0; r1 <= D1; ++r1) {
+        const double *row = c + (size_t)wrapi(c1 - r1, M1) * M2;
+        double u = 0.0;
+#pragma unroll
+        for (int r2 = 0; r2 <= D2; ++r2) u = fma(c_spline2.b[D2][r2][b], row[o2[r2]], u);
+        s = fma(c_spline2.b[D1][r1][a], u, s);
+    }
+    tab[(size_t)cell * pad + q] = s;
+}
+
+template <int D1, int D2>
+__global__ void __launch_bounds__(128) k2_table(int M1, int M2, const double *c, double *tab, int pad)
+{
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < (long long)M1 * M2 * (D1 + 1) * (D2 + 1)) table2_at<D1, D2>(t, M1, M2, c, tab, pad);
+}
+
+// both components of e_bar (blockIdx.y)
+template <int K>
+__global__ void __launch_bounds__(128) k2_table_e(int M1, int M2, const double *ebx, const double *eby, double *TEx,
+                                                  double *TEy)
+{
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= (long long)M1 * M2 * K * (K + 1)) return;
+    if (blockIdx.y == 0) table2_at<K - 1, K>(t, M1, M2, ebx, TEx, Dim2<K>::pE);
+    else table2_at<K, K - 1>(t, M1, M2, eby, TEy, Dim2<K>::pE);
+}
+
+// node values of a current component from its moments: degree (D1, D2), moments [a][b]
+template <int D1, int D2>
+__device__ __forceinline__ double node2_at(int M1, int M2, const double *m, int i1, int i2)
+{
+    double s = 0.0;
+#pragma unroll
+    for (int r1 = 0; r1 <= D1; ++r1) {
+        const int c1 = wrapi(i1 + r1, M1) * M2;
+#pragma unroll
+        for (int r2 = 0; r2 <= D2; ++r2) {
+            const double *row = m + (size_t)(c1 + wrapi(i2 + r2, M2)) * ((D1 + 1) * (D2 + 1));
+#pragma unroll
+            for (int a = 0; a <= D1; ++a) {
+                double u = 0.0;
+#pragma unroll
+                for (int b = 0; b <= D2; ++b) u = fma(c_spline2.b[D2][r2][b], row[a * (D2 + 1) + b], u);
+                s = fma(c_spline2.b[D1][r1][a], u, s);
+            }
         }
-        out[i] = s;
     }
+    return s;
 }
 
-// e^(k+1) = e^n - sol (sol = M1^{-1} j); increment max-norm; e_bar for the next sweep
-__global__ void k2_update(int N, const double *en, const double *sol, double *ek, double *eb,
-                          unsigned long long *emax_bits)
+template <int K>
+__global__ void __launch_bounds__(64) k2_nodes(int M1, int M2, const double *mx, const double *my, double *jx, double *jy)
 {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= M1 * M2) return;
+    if (blockIdx.y == 0) jx[i] = node2_at<K - 1, K>(M1, M2, mx, i / M2, i % M2);
+    else jy[i] = node2_at<K, K - 1>(M1, M2, my, i / M2, i % M2);
+}
+
+// sum_q g[(i - q) mod M] in[q stride], four independent chains
+__device__ __forceinline__ double circ_at(int M, int i, const double *g, const double *in, int stride)
+{
+    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+    int k = i, q = 0;
+    auto next = [&]() { const double v = g[k] * in[(size_t)q * stride]; k = k == 0 ? M - 1 : k - 1; ++q; return v; };
+    while (q + 4 <= M) {
+        s0 += next();
+        s1 += next();
+        s2 += next();
+        s3 += next();
+    }
+    while (q < M) s0 += next();
+    return (s0 + s1) + (s2 + s3);
+}
+
+// pass along x2 of both components (blockIdx.y): out[i1, i2] = sum_q g[(i2 - q) mod M2] in[i1, q]
+__global__ void __launch_bounds__(64) k2_circ2(int M1, int M2, const double *gx, const double *gy, const double *jx,
+                                               const double *jy, double *ox, double *oy)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= M1 * M2) return;
+    const int i1 = i / M2, i2 = i % M2;
+    if (blockIdx.y == 0) ox[i] = circ_at(M2, i2, gx, jx + (size_t)i1 * M2, 1);
+    else oy[i] = circ_at(M2, i2, gy, jy + (size_t)i1 * M2, 1);
+}
+
+// pass along x1, then e^(k+1) = e^n - M1^{-1} j, its increment's max-norm, e_bar for the
+// next sweep
+__global__ void __launch_bounds__(64) k2_circ1(int M1, int M2, const double *gx, const double *gy, const double *tx,
+                                               const double *ty, const double *enx, const double *eny, double *ekx,
+                                               double *eky, double *ebx, double *eby, unsigned long long *emax_bits)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
     double m = 0.0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
-        const double v = en[i] - sol[i];
-        m = fmax(m, fabs(v - ek[i]));
-        if (!(v == v)) m = v;
+    if (i < M1 * M2) {
+        const int i1 = i / M2, i2 = i % M2;
+        const bool y = blockIdx.y != 0;
+        const double sol = circ_at(M1, i1, y ? gy : gx, (y ? ty : tx) + i2, M2);
+        const double en = (y ? eny : enx)[i], v = en - sol;
+        double *ek = y ? eky : ekx;
+        m = fabs(v - ek[i]);
         ek[i] = v;
-        eb[i] = 0.5 * (en[i] + v);
+        (y ? eby : ebx)[i] = 0.5 * (en + v);
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        const double t = __shfl_xor_sync(0xffffffffu, m, o);
-        m = (t > m || t != t) ? t : m;
-    }
+    for (int o = 16; o > 0; o >>= 1) m = max_nonneg(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0) max_bits(emax_bits, m);
 }
 
 // acc[0] += sum_a w (g(p_a, A(x_a)) - 1); with spins, acc[1] += sum_a w hbar
-// (s_x dA/dx2 - s_y dA/dx1 + s_z b_z)(x_a) (G_y a on (K, K-1), G_x a on (K-1, K),
-// b_z on (K-1, K-1))
+// (s_x dA/dx2 - s_y dA/dx1 + s_z b_z)(x_a)
 template <int K>
-__global__ void __launch_bounds__(256) k2_energy(long long np, int M1, int M2, double dx1, double dx2, double w,
-                                                  const double *x, const double *p, const double *az, double hbar,
-                                                  const double *sp, const double *gax, const double *gay,
-                                                  const double *bz, double *acc)
+__global__ void __launch_bounds__(256) k2_energy(Args2D A, const double2 *p, double *acc)
 {
+    constexpr int NC = K + 1;
     double s = 0.0, z = 0.0;
-    for (long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x; a < np;
+    for (long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x; a < A.np;
          a += (long long)gridDim.x * blockDim.x) {
-        const double u1 = x[2 * a] / dx1, u2 = x[2 * a + 1] / dx2;
-        const double A = value0<K>(az, M1, M2, u1, u2);
-        s += w * (sqrt(1.0 + p[2 * a] * p[2 * a] + p[2 * a + 1] * p[2 * a + 1] + A * A) - 1.0);
-        if (hbar != 0.0)
-            z += w * hbar * (sp[3 * a] * value_dd<K, K - 1>(gay, M1, M2, u1, u2) -
-                             sp[3 * a + 1] * value_dd<K - 1, K>(gax, M1, M2, u1, u2) +
-                             sp[3 * a + 2] * value_dd<K - 1, K - 1>(bz, M1, M2, u1, u2));
+        const int cell = A.cell[a].x * A.M2 + A.cell[a].y;
+        const double2 v = A.v[a], q = p[a];
+        const double *row = A.TA + (size_t)cell * Dim2<K>::pA;
+        double al[NC];
+        contract_rows<NC, NC>(row, v.y, al);
+        const double Az = horner<NC>(al, v.x);
+        s += A.w * (sqrt(1.0 + q.x * q.x + q.y * q.y + Az * Az) - 1.0);
+        if (A.hbar != 0.0) {
+            double ady[NC], bz[K];
+            contract_rows_dy<NC, NC>(row, v.y, ady);
+            contract_rows<K, K>(A.TB + (size_t)cell * Dim2<K>::pB, v.y, bz);
+            double d1 = (double)K * al[K];
+#pragma unroll
+            for (int m = K - 1; m >= 1; --m) d1 = fma(d1, v.x, (double)m * al[m]);
+            z += A.w * A.hbar * (A.s[3 * a] * horner<NC>(ady, v.x) * A.idx2 - A.s[3 * a + 1] * d1 * A.idx1 +
+                                 A.s[3 * a + 2] * horner<K>(bz, v.x));
+        }
     }
     for (int o = 16; o > 0; o >>= 1) {
         s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -567,25 +642,49 @@ __global__ void __launch_bounds__(256) k2_energy(long long np, int M1, int M2, d
     }
     if ((threadIdx.x & 31) == 0) {
         atomicAdd(acc, s);
-        if (hbar != 0.0) atomicAdd(acc + 1, z);
+        if (A.hbar != 0.0) atomicAdd(acc + 1, z);
     }
 }
 
-// x^{n+1} = x^n + delta wrapped into the box, p^{n+1} = p^(k)
-__global__ void k2_finalize(long long np, double L1, double L2, double *x, double *p, const double *d,
-                            const double *pk)
+// x^{n+1} = x^n + delta (cells wrapped around the box), p^{n+1} = p^(k)
+__global__ void k2_finalize(long long np, int M1, int M2, int2 *cell, double2 *v, double2 *p, const double2 *d,
+                            const double2 *pk)
 {
     for (long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x; a < np;
          a += (long long)gridDim.x * blockDim.x) {
-        for (int q = 0; q < 2; ++q) {
-            const double L = q == 0 ? L1 : L2;
-            double v = x[2 * a + q] + d[2 * a + q];
-            v -= L * floor(v / L);
-            if (v >= L) v -= L;
-            if (v < 0.0) v = 0.0;
-            x[2 * a + q] = v;
-            p[2 * a + q] = pk[2 * a + q];
-        }
+        int n1, n2;
+        double2 u = v[a];
+        const double2 dd = d[a];
+        path_end(u.x, dd.x, n1, u.x);
+        path_end(u.y, dd.y, n2, u.y);
+        const int2 c = cell[a];
+        if (n1 != 0 || n2 != 0) cell[a] = make_int2(wrapi(c.x + n1, M1), wrapi(c.y + n2, M2));
+        v[a] = u;
+        p[a] = pk[a];
+    }
+}
+
+// positions in the box <-> cells and centred offsets
+__global__ void k2_load(long long np, int M1, int M2, double dx1, double dx2, const double2 *x, int2 *cell, double2 *v)
+{
+    for (long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x; a < np;
+         a += (long long)gridDim.x * blockDim.x) {
+        const double u1 = x[a].x / dx1, u2 = x[a].y / dx2;
+        const double f1 = floor(u1), f2 = floor(u2);
+        cell[a] = make_int2(wrapi((int)f1, M1), wrapi((int)f2, M2));
+        v[a] = make_double2((u1 - f1) - 0.5, (u2 - f2) - 0.5);
+    }
+}
+
+__global__ void k2_store(long long np, double L1, double L2, double dx1, double dx2, const int2 *cell, const double2 *v,
+                         double2 *x)
+{
+    for (long long a = blockIdx.x * (long long)blockDim.x + threadIdx.x; a < np;
+         a += (long long)gridDim.x * blockDim.x) {
+        double x1 = (((double)cell[a].x + 0.5) + v[a].x) * dx1, x2 = (((double)cell[a].y + 0.5) + v[a].y) * dx2;
+        x1 = x1 >= L1 ? x1 - L1 : (x1 < 0.0 ? 0.0 : x1);
+        x2 = x2 >= L2 ? x2 - L2 : (x2 < 0.0 ? 0.0 : x2);
+        x[a] = make_double2(x1, x2);
     }
 }
 
@@ -622,22 +721,26 @@ using namespace pic;
 
 struct pic2d_handle {
     pic2d_config cfg{};
-    int device = 0;
+    int device = 0, num_sms = 1;
     cudaStream_t stream = nullptr;
     double dx1 = 0.0, dx2 = 0.0;
     int N = 0;
-    double *x = nullptr, *p = nullptr, *d = nullptr, *pk = nullptr, *a0 = nullptr;
+    int2 *cell = nullptr;
+    double2 *v = nullptr, *p = nullptr, *d = nullptr, *pk = nullptr;
+    double *cache = nullptr;
     double *ex = nullptr, *ey = nullptr, *exk = nullptr, *eyk = nullptr, *ebx = nullptr, *eby = nullptr;
-    double *az = nullptr, *gax = nullptr, *gay = nullptr;
-    double *gxy = nullptr, *gxx = nullptr, *gyy = nullptr;       // second differences of a_z
-    double *spin = nullptr, *bz = nullptr, *gbx = nullptr, *gby = nullptr;   // pic2d_set_spin
-    double *jx = nullptr, *jy = nullptr, *tmp = nullptr, *sol = nullptr;
+    double *az = nullptr, *TA = nullptr, *TEx = nullptr, *TEy = nullptr;   // A_z; cell polynomials of A_z and e_bar
+    double *spin = nullptr, *bz = nullptr, *TB = nullptr;       // pic2d_set_spin
+    double *mom = nullptr;                   // moments of both current components, x then y
+    double *jx = nullptr, *jy = nullptr, *tx = nullptr, *ty = nullptr;
     double *g1x = nullptr, *g0y = nullptr, *g0x = nullptr, *g1y = nullptr;   // inverse rows
-    unsigned long long *bits = nullptr;      // dmax, pmax, emax
-    int *status = nullptr;
+    unsigned long long *bits = nullptr;      // dmax, pmax, emax; then the status word
+    int *status = nullptr;                   // (inside bits' allocation)
+    unsigned long long *h_bits = nullptr;    // page-locked copy of both
     double *acc = nullptr;
     std::vector<double> m0x, m1x, m0y, m1y;  // 1D mass rows (host) for the field energy
-    double glx[5] = {0, 0, 0, 0, 0}, glw[5] = {0, 0, 0, 0, 0};
+    double gls[5] = {0, 0, 0, 0, 0}, glw[5] = {0, 0, 0, 0, 0};
+    pic::HostCopy copy;
     std::string err;
 };
 
@@ -663,29 +766,12 @@ static int fail2d(pic2d_handle *h, int code, const char *fmt, ...)
 
 static void free2d(pic2d_handle *h)
 {
-    double **arrs[] = {&h->x, &h->p, &h->d, &h->pk, &h->a0, &h->ex, &h->ey, &h->exk, &h->eyk, &h->ebx, &h->eby,
-                       &h->az, &h->gax, &h->gay, &h->jx, &h->jy, &h->tmp, &h->sol, &h->g1x, &h->g0y,
-                       &h->g0x, &h->g1y, &h->acc,
-                       &h->gxy, &h->gxx, &h->gyy, &h->spin, &h->bz, &h->gbx, &h->gby};
-    for (double **a : arrs)
-        if (*a) { cudaFree(*a); *a = nullptr; }
-    if (h->bits) cudaFree(h->bits);
-    if (h->status) cudaFree(h->status);
-    h->bits = nullptr;
-    h->status = nullptr;
-}
-
-// backward difference of a grid array along one axis, divided by the cell size
-static std::vector<double> grid_diff(const std::vector<double> &c, int M1, int M2, int axis, double dx)
-{
-    std::vector<double> out(c.size());
-    for (int i1 = 0; i1 < M1; ++i1)
-        for (int i2 = 0; i2 < M2; ++i2) {
-            const int i = i1 * M2 + i2;
-            const int j = axis == 0 ? ((i1 - 1 + M1) % M1) * M2 + i2 : i1 * M2 + (i2 - 1 + M2) % M2;
-            out[i] = (c[i] - c[j]) / dx;
-        }
-    return out;
+    void *arrs[] = {h->cell, h->v, h->p, h->d, h->pk, h->cache, h->ex, h->ey, h->exk, h->eyk, h->ebx, h->eby,
+                    h->az, h->TA, h->TEx, h->TEy, h->mom, h->jx, h->jy, h->tx, h->ty, h->g1x, h->g0y,
+                    h->g0x, h->g1y, h->acc, h->bits, h->spin, h->bz, h->TB};
+    for (void *a : arrs)
+        if (a) cudaFree(a);
+    if (h->h_bits) cudaFreeHost(h->h_bits);
 }
 
 // full periodic circulant row of the degree-d mass matrix (band folded onto M nodes)
@@ -706,21 +792,57 @@ static std::vector<double> inverse_row(int d, int M, double dx)
     return g;
 }
 
-template <int K>
-static cudaError_t smem_optin(size_t smem)
+// the body for the degree K (a compile-time constant in it)
+#define PIC2D_DEGREE(K_, ...)                                                             \
+    switch (K_) {                                                                         \
+    case 2: { constexpr int K = 2; __VA_ARGS__; break; }                                  \
+    case 3: { constexpr int K = 3; __VA_ARGS__; break; }                                  \
+    case 4: { constexpr int K = 4; __VA_ARGS__; break; }                                  \
+    default: { constexpr int K = 5; __VA_ARGS__; break; }                                 \
+    }
+
+static Args2D make_args(pic2d_handle *h)
 {
-    cudaError_t e = cudaFuncSetAttribute(k2_sweep<K, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k2_sweep<K, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    return e;
+    const pic2d_config &c = h->cfg;
+    Args2D a{};
+    a.M1 = c.M1; a.M2 = c.M2; a.np = c.np; a.dx1 = h->dx1; a.dx2 = h->dx2; a.dt = c.dt; a.w = c.weight;
+    a.idx1 = 1.0 / h->dx1; a.idx2 = 1.0 / h->dx2;
+    a.cell = h->cell; a.v = h->v; a.cache = h->cache; a.pn = h->p; a.d = h->d; a.pk = h->pk;
+    a.TA = h->TA; a.TEx = h->TEx; a.TEy = h->TEy; a.TB = h->TB;
+    a.mx = h->mom; a.my = h->mom + (size_t)h->N * c.degree * (c.degree + 1);
+    a.hbar = h->spin ? c.hbar : 0.0;
+    a.s = h->spin;
+    a.dmax_bits = h->bits; a.pmax_bits = h->bits + 1; a.status = h->status;
+    for (int g = 0; g < 5; ++g) { a.gls[g] = h->gls[g]; a.glw[g] = h->glw[g]; }
+    return a;
 }
 
-template <int K>
-static int launch_sweep2d(const Args2D &a, int grid, size_t smem, cudaStream_t s, bool pre)
+static int marker_grid2d(const pic2d_handle *h) { return (int)std::min<long long>((h->cfg.np + 255) / 256, 8LL * h->num_sms); }
+
+// cell polynomials of e_bar
+static int tables_e(pic2d_handle *h)
 {
-    if (pre) k2_sweep<K, true><<<grid, 256, smem, s>>>(a);
-    else k2_sweep<K><<<grid, 256, smem, s>>>(a);
-    return 0;
+    const pic2d_config &c = h->cfg;
+    const dim3 grid((unsigned)(((long long)h->N * c.degree * (c.degree + 1) + 127) / 128), 2);
+    PIC2D_DEGREE(c.degree, (k2_table_e<K><<<grid, 128, 0, h->stream>>>(c.M1, c.M2, h->ebx, h->eby, h->TEx, h->TEy)))
+    CK2(cudaGetLastError());
+    return PIC_OK;
+}
+
+// e^(k+1) = e^n - M1^{-1} j from the sweep's moments, its increment, e_bar and its polynomials
+static int solve2d(pic2d_handle *h)
+{
+    const pic2d_config &c = h->cfg;
+    const Args2D a = make_args(h);
+    const dim3 grid((h->N + 63) / 64, 2);
+    cudaStream_t s = h->stream;
+    PIC2D_DEGREE(c.degree, (k2_nodes<K><<<grid, 64, 0, s>>>(c.M1, c.M2, a.mx, a.my, h->jx, h->jy)))
+    // along x2 with the rows of component x's N^k and y's N^{k-1}, then along x1
+    k2_circ2<<<grid, 64, 0, s>>>(c.M1, c.M2, h->g0y, h->g1y, h->jx, h->jy, h->tx, h->ty);
+    k2_circ1<<<grid, 64, 0, s>>>(c.M1, c.M2, h->g1x, h->g0x, h->tx, h->ty, h->ex, h->ey, h->exk, h->eyk, h->ebx, h->eby,
+                                 h->bits + 2);
+    CK2(cudaGetLastError());
+    return tables_e(h);
 }
 
 extern "C" int pic2d_init(const pic2d_config *cfg, const double *x, const double *p, const double *ex,
@@ -742,96 +864,74 @@ extern "C" int pic2d_init(const pic2d_config *cfg, const double *x, const double
     h->dx1 = c.L1 / c.M1;
     h->dx2 = c.L2 / c.M2;
     h->N = c.M1 * c.M2;
-    const size_t np2 = 2 * (size_t)c.np, N = (size_t)h->N;
+    const size_t np = (size_t)c.np, N = (size_t)h->N;
     auto bail = [&](int rc) {
         g_err2d = h->err.empty() ? "pic2d_init failed" : h->err;
         free2d(h);
         delete h;
         return rc;
     };
-    double **parts[] = {&h->x, &h->p, &h->d, &h->pk};
-    for (double **a : parts)
-        if (cudaMalloc((void **)a, np2 * sizeof(double)) != cudaSuccess) return bail(PIC_ERR_NOMEM);
-    if (cudaMalloc((void **)&h->a0, (size_t)c.np * sizeof(double)) != cudaSuccess) return bail(PIC_ERR_NOMEM);
-    double **grids[] = {&h->ex, &h->ey, &h->exk, &h->eyk, &h->ebx, &h->eby, &h->az, &h->gax, &h->gay,
-                        &h->gxy, &h->gxx, &h->gyy, &h->jx, &h->jy, &h->tmp, &h->sol};
+    cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, h->device);
+    const int K = c.degree;
+    struct { void **p; size_t bytes; } allocs[] = {
+        {(void **)&h->cell, np * sizeof(int2)}, {(void **)&h->v, np * sizeof(double2)},
+        {(void **)&h->p, np * sizeof(double2)}, {(void **)&h->d, np * sizeof(double2)},
+        {(void **)&h->pk, np * sizeof(double2)}, {(void **)&h->cache, np * (K + 2) * sizeof(double)},
+        {(void **)&h->TA, N * pad2((K + 1) * (K + 1)) * sizeof(double)},
+        {(void **)&h->TEx, N * pad2(K * (K + 1)) * sizeof(double)},
+        {(void **)&h->TEy, N * pad2(K * (K + 1)) * sizeof(double)},
+        {(void **)&h->mom, 2 * N * K * (K + 1) * sizeof(double)},
+        {(void **)&h->g1x, c.M1 * sizeof(double)}, {(void **)&h->g0x, c.M1 * sizeof(double)},
+        {(void **)&h->g0y, c.M2 * sizeof(double)}, {(void **)&h->g1y, c.M2 * sizeof(double)},
+        {(void **)&h->bits, 4 * sizeof(unsigned long long)}, {(void **)&h->acc, 2 * sizeof(double)}};
+    for (auto &al : allocs)
+        if (cudaMalloc(al.p, al.bytes) != cudaSuccess) return bail(PIC_ERR_NOMEM);
+    double **grids[] = {&h->ex, &h->ey, &h->exk, &h->eyk, &h->ebx, &h->eby, &h->az, &h->jx, &h->jy, &h->tx, &h->ty};
     for (double **a : grids)
         if (cudaMalloc((void **)a, N * sizeof(double)) != cudaSuccess) return bail(PIC_ERR_NOMEM);
-    if (cudaMalloc((void **)&h->g1x, c.M1 * sizeof(double)) != cudaSuccess ||
-        cudaMalloc((void **)&h->g0x, c.M1 * sizeof(double)) != cudaSuccess ||
-        cudaMalloc((void **)&h->g0y, c.M2 * sizeof(double)) != cudaSuccess ||
-        cudaMalloc((void **)&h->g1y, c.M2 * sizeof(double)) != cudaSuccess ||
-        cudaMalloc((void **)&h->bits, 3 * sizeof(unsigned long long)) != cudaSuccess ||
-        cudaMalloc((void **)&h->status, sizeof(int)) != cudaSuccess ||
-        cudaMalloc((void **)&h->acc, 2 * sizeof(double)) != cudaSuccess)
-        return bail(PIC_ERR_NOMEM);
+    h->status = reinterpret_cast<int *>(h->bits + 3);
+    if (cudaMallocHost((void **)&h->h_bits, 4 * sizeof(unsigned long long)) != cudaSuccess) return bail(PIC_ERR_NOMEM);
     // positions must lie in the box
     const cudaMemcpyKind kind = mem == PIC_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
     if (mem == PIC_MEM_HOST) {
-        for (size_t a = 0; a < (size_t)c.np; ++a)
+        for (size_t a = 0; a < np; ++a)
             if (!(x[2 * a] >= 0.0 && x[2 * a] < c.L1 && x[2 * a + 1] >= 0.0 && x[2 * a + 1] < c.L2) ||
                 !std::isfinite(p[2 * a]) || !std::isfinite(p[2 * a + 1])) {
                 fail2d(h, PIC_ERR_INVALID, "marker %zu outside the box or not finite", a);
                 return bail(PIC_ERR_INVALID);
             }
     }
-    if (cudaMemcpyAsync(h->x, x, np2 * sizeof(double), kind, h->stream) != cudaSuccess ||
-        cudaMemcpyAsync(h->p, p, np2 * sizeof(double), kind, h->stream) != cudaSuccess ||
+    // the positions pass through the displacement array
+    if (cudaMemcpyAsync(h->d, x, np * sizeof(double2), kind, h->stream) != cudaSuccess ||
+        cudaMemcpyAsync(h->p, p, np * sizeof(double2), kind, h->stream) != cudaSuccess ||
         cudaMemcpyAsync(h->ex, ex, N * sizeof(double), kind, h->stream) != cudaSuccess ||
         cudaMemcpyAsync(h->ey, ey, N * sizeof(double), kind, h->stream) != cudaSuccess ||
         cudaMemcpyAsync(h->az, az, N * sizeof(double), kind, h->stream) != cudaSuccess)
         return bail(fail2d(h, PIC_ERR_CUDA, "input copies"));
-    // differences of A_z (host: small grids): (G_x a)_{i1,i2} = (a_{i1,i2} - a_{i1-1,i2}) / dx1,
-    // (G_y a)_{i1,i2} = (a_{i1,i2} - a_{i1,i2-1}) / dx2, and the second differences of the
-    // Zeeman term's quotients
+    k2_load<<<marker_grid2d(h), 256, 0, h->stream>>>(c.np, c.M1, c.M2, h->dx1, h->dx2, h->d, h->cell, h->v);
+    PIC2D_DEGREE(c.degree, (k2_table<K, K><<<(unsigned)((N * Dim2<K>::nA + 127) / 128), 128, 0, h->stream>>>(
+                               c.M1, c.M2, h->az, h->TA, Dim2<K>::pA)))
+    if (cudaGetLastError() != cudaSuccess) return bail(fail2d(h, PIC_ERR_CUDA, "input kernels"));
     {
-        std::vector<double> a(N);
-        if (cudaMemcpyAsync(a.data(), h->az, N * sizeof(double), cudaMemcpyDeviceToHost, h->stream) != cudaSuccess ||
-            cudaStreamSynchronize(h->stream) != cudaSuccess)
-            return bail(fail2d(h, PIC_ERR_CUDA, "a_z readback"));
-        const std::vector<double> gx = grid_diff(a, c.M1, c.M2, 0, h->dx1), gy = grid_diff(a, c.M1, c.M2, 1, h->dx2);
-        const std::vector<double> gxy = grid_diff(gy, c.M1, c.M2, 0, h->dx1);
-        const std::vector<double> gxx = grid_diff(gx, c.M1, c.M2, 0, h->dx1);
-        const std::vector<double> gyy = grid_diff(gy, c.M1, c.M2, 1, h->dx2);
         std::vector<double> g1x = inverse_row(c.degree - 1, c.M1, h->dx1), g0x = inverse_row(c.degree, c.M1, h->dx1);
         std::vector<double> g1y = inverse_row(c.degree - 1, c.M2, h->dx2), g0y = inverse_row(c.degree, c.M2, h->dx2);
         h->m0x = mass_row_full(c.degree, c.M1, h->dx1);
         h->m1x = mass_row_full(c.degree - 1, c.M1, h->dx1);
         h->m0y = mass_row_full(c.degree, c.M2, h->dx2);
         h->m1y = mass_row_full(c.degree - 1, c.M2, h->dx2);
-        if (cudaMemcpy(h->gax, gx.data(), N * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemcpy(h->gxy, gxy.data(), N * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemcpy(h->gxx, gxx.data(), N * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemcpy(h->gyy, gyy.data(), N * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemcpy(h->gay, gy.data(), N * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemcpy(h->g1x, g1x.data(), c.M1 * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemcpy(h->g0x, g0x.data(), c.M1 * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemcpy(h->g1y, g1y.data(), c.M2 * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
-            cudaMemcpy(h->g0y, g0y.data(), c.M2 * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
+        if (cudaMemcpyAsync(h->g1x, g1x.data(), c.M1 * sizeof(double), cudaMemcpyHostToDevice, h->stream) != cudaSuccess ||
+            cudaMemcpyAsync(h->g0x, g0x.data(), c.M1 * sizeof(double), cudaMemcpyHostToDevice, h->stream) != cudaSuccess ||
+            cudaMemcpyAsync(h->g1y, g1y.data(), c.M2 * sizeof(double), cudaMemcpyHostToDevice, h->stream) != cudaSuccess ||
+            cudaMemcpyAsync(h->g0y, g0y.data(), c.M2 * sizeof(double), cudaMemcpyHostToDevice, h->stream) != cudaSuccess ||
+            cudaStreamSynchronize(h->stream) != cudaSuccess)
             return bail(fail2d(h, PIC_ERR_CUDA, "grid uploads"));
     }
-    gauss_legendre(c.degree, h->glx, h->glw);
-    const size_t smem = 2 * N * sizeof(double);
-    cudaError_t e = cudaSuccess;
-    switch (c.degree) {
-    case 2: e = smem_optin<2>(smem); break;
-    case 3: e = smem_optin<3>(smem); break;
-    case 4: e = smem_optin<4>(smem); break;
-    default: e = smem_optin<5>(smem); break;
+    gauss_legendre(c.degree, h->gls, h->glw);
+    for (int g = 0; g < c.degree; ++g) {        // on [0, 1]
+        h->gls[g] = 0.5 * (1.0 + h->gls[g]);
+        h->glw[g] *= 0.5;
     }
-    if (e != cudaSuccess) return bail(fail2d(h, PIC_ERR_CUDA, "shared-memory opt-in: %s", cudaGetErrorString(e)));
-    if (cudaStreamSynchronize(h->stream) != cudaSuccess) return bail(fail2d(h, PIC_ERR_CUDA, "init sync"));
     *out = h;
-    return PIC_OK;
-}
-
-static int solve_axis_pair(pic2d_handle *h, const double *ga, const double *gb, const double *in)
-{
-    // sol = (A_1^{-1} (x) B_2^{-1}) in: first along x2 with gb, then along x1 with ga
-    const int grid = (h->N + 255) / 256;
-    k2_circ<<<grid, 256, 0, h->stream>>>(h->cfg.M1, h->cfg.M2, 1, gb, in, h->tmp);
-    k2_circ<<<grid, 256, 0, h->stream>>>(h->cfg.M1, h->cfg.M2, 0, ga, h->tmp, h->sol);
-    CK2(cudaGetLastError());
     return PIC_OK;
 }
 
@@ -841,77 +941,44 @@ extern "C" int pic2d_substep1(pic2d_handle *h, int32_t *iters)
     const pic2d_config &c = h->cfg;
     if (c.hbar != 0.0 && !h->spin)
         return fail2d(h, PIC_ERR_INVALID, "hbar != 0: pic2d_set_spin must give the spins and b_z first");
-    const size_t np2 = 2 * (size_t)c.np, N = (size_t)h->N;
+    const size_t np = (size_t)c.np, N = (size_t)h->N;
+    const size_t mom_bytes = 2 * N * c.degree * (c.degree + 1) * sizeof(double);
     cudaStream_t s = h->stream;
-    CK2(cudaMemsetAsync(h->d, 0, np2 * sizeof(double), s));
-    CK2(cudaMemcpyAsync(h->pk, h->p, np2 * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    CK2(cudaMemcpyAsync(h->exk, h->ex, N * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    CK2(cudaMemcpyAsync(h->eyk, h->ey, N * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    CK2(cudaMemcpyAsync(h->ebx, h->ex, N * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    CK2(cudaMemcpyAsync(h->eby, h->ey, N * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    CK2(cudaMemsetAsync(h->status, 0, sizeof(int), s));
-    Args2D a{};
-    a.M1 = c.M1; a.M2 = c.M2; a.np = c.np; a.dx1 = h->dx1; a.dx2 = h->dx2; a.dt = c.dt; a.w = c.weight;
-    a.idx1 = 1.0 / h->dx1; a.idx2 = 1.0 / h->dx2; a.a0 = h->a0;
-    a.x = h->x; a.pn = h->p; a.d = h->d; a.pk = h->pk;
-    a.ebx = h->ebx; a.eby = h->eby; a.az = h->az; a.gax = h->gax; a.gay = h->gay;
-    a.hbar = h->spin ? c.hbar : 0.0;
-    a.s = h->spin; a.gxy = h->gxy; a.gxx = h->gxx; a.gyy = h->gyy; a.gbx = h->gbx; a.gby = h->gby;
-    a.jx = h->jx; a.jy = h->jy; a.dmax_bits = h->bits; a.pmax_bits = h->bits + 1; a.status = h->status;
-    for (int g = 0; g < 5; ++g) { a.glx[g] = h->glx[g]; a.glw[g] = h->glw[g]; }
-    int num_sms = 0;
-    cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, h->device);
-    const int grid = (int)std::min<long long>((c.np + 255) / 256, 4LL * (num_sms > 0 ? num_sms : 1));
-    const size_t smem = 2 * N * sizeof(double);
-    unsigned long long hb[3];
-    int hs = 0;
-    int it = 0;
+    CK2(cudaMemsetAsync(h->d, 0, np * sizeof(double2), s));
+    CK2(cudaMemcpyAsync(h->pk, h->p, np * sizeof(double2), cudaMemcpyDeviceToDevice, s));
+    double *copies[][2] = {{h->exk, h->ex}, {h->eyk, h->ey}, {h->ebx, h->ex}, {h->eby, h->ey}};
+    for (auto &q : copies) CK2(cudaMemcpyAsync(q[0], q[1], N * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    CK2(cudaMemsetAsync(h->bits, 0, 4 * sizeof(unsigned long long), s));
+    Args2D a = make_args(h);
+    const int grid = marker_grid2d(h);
+    int rc, it = 0;
     const bool warm = c.warm != 0;
     if (warm) {
         // the predicted start: delta^(0) and its current, then e^(0) = e^n - M1^{-1} j^(0)
         // and e_bar = (e^n + e^(0)) / 2 for the first sweep
-        CK2(cudaMemsetAsync(h->jx, 0, N * sizeof(double), s));
-        CK2(cudaMemsetAsync(h->jy, 0, N * sizeof(double), s));
-        switch (c.degree) {
-        case 2: launch_sweep2d<2>(a, grid, smem, s, true); break;
-        case 3: launch_sweep2d<3>(a, grid, smem, s, true); break;
-        case 4: launch_sweep2d<4>(a, grid, smem, s, true); break;
-        default: launch_sweep2d<5>(a, grid, smem, s, true); break;
-        }
+        CK2(cudaMemsetAsync(h->mom, 0, mom_bytes, s));
+        PIC2D_DEGREE(c.degree, (k2_sweep<K, true><<<grid, 256, 0, s>>>(a)))
         CK2(cudaGetLastError());
-        int rc;
-        if ((rc = solve_axis_pair(h, h->g1x, h->g0y, h->jx))) return rc;
-        k2_update<<<(h->N + 255) / 256, 256, 0, s>>>(h->N, h->ex, h->sol, h->exk, h->ebx, h->bits + 2);
-        if ((rc = solve_axis_pair(h, h->g0x, h->g1y, h->jy))) return rc;
-        k2_update<<<(h->N + 255) / 256, 256, 0, s>>>(h->N, h->ey, h->sol, h->eyk, h->eby, h->bits + 2);
-        CK2(cudaGetLastError());
+        if ((rc = solve2d(h))) return rc;
+    } else if ((rc = tables_e(h))) {
+        return rc;
     }
     for (;;) {
-        CK2(cudaMemsetAsync(h->jx, 0, N * sizeof(double), s));
-        CK2(cudaMemsetAsync(h->jy, 0, N * sizeof(double), s));
+        CK2(cudaMemsetAsync(h->mom, 0, mom_bytes, s));
         CK2(cudaMemsetAsync(h->bits, 0, 3 * sizeof(unsigned long long), s));
-        a.first = !warm && it == 0;          // the predicted start stored A(x^n) already
-        switch (c.degree) {
-        case 2: launch_sweep2d<2>(a, grid, smem, s, false); break;
-        case 3: launch_sweep2d<3>(a, grid, smem, s, false); break;
-        case 4: launch_sweep2d<4>(a, grid, smem, s, false); break;
-        default: launch_sweep2d<5>(a, grid, smem, s, false); break;
-        }
+        a.first = !warm && it == 0;          // the predicted start filled the cache already
+        PIC2D_DEGREE(c.degree, (k2_sweep<K><<<grid, 256, 0, s>>>(a)))
         CK2(cudaGetLastError());
-        int rc;
-        if ((rc = solve_axis_pair(h, h->g1x, h->g0y, h->jx))) return rc;
-        k2_update<<<(h->N + 255) / 256, 256, 0, s>>>(h->N, h->ex, h->sol, h->exk, h->ebx, h->bits + 2);
-        if ((rc = solve_axis_pair(h, h->g0x, h->g1y, h->jy))) return rc;
-        k2_update<<<(h->N + 255) / 256, 256, 0, s>>>(h->N, h->ey, h->sol, h->eyk, h->eby, h->bits + 2);
-        CK2(cudaGetLastError());
-        CK2(cudaMemcpyAsync(hb, h->bits, sizeof(hb), cudaMemcpyDeviceToHost, s));
-        CK2(cudaMemcpyAsync(&hs, h->status, sizeof(int), cudaMemcpyDeviceToHost, s));
+        if ((rc = solve2d(h))) return rc;
+        CK2(cudaMemcpyAsync(h->h_bits, h->bits, 4 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
         CK2(cudaStreamSynchronize(s));
         ++it;
         double dm, pm, em;
-        std::memcpy(&dm, &hb[0], 8);
-        std::memcpy(&pm, &hb[1], 8);
-        std::memcpy(&em, &hb[2], 8);
+        int hs;
+        std::memcpy(&dm, &h->h_bits[0], 8);
+        std::memcpy(&pm, &h->h_bits[1], 8);
+        std::memcpy(&em, &h->h_bits[2], 8);
+        std::memcpy(&hs, &h->h_bits[3], sizeof(int));
         if (hs & STATUS_NUMERIC) return fail2d(h, PIC_ERR_NUMERIC, "2D subsystem I: non-finite value or a path beyond %d cells", kMaxCross);
         if (!(dm == dm && pm == pm && em == em)) return fail2d(h, PIC_ERR_NUMERIC, "2D subsystem I: NaN increment");
         if (dm <= c.tol && pm <= c.tol && em <= c.tol) break;
@@ -921,8 +988,7 @@ extern "C" int pic2d_substep1(pic2d_handle *h, int32_t *iters)
         }
     }
     if (iters) *iters = it;
-    k2_finalize<<<(int)std::min<long long>((c.np + 255) / 256, 1024), 256, 0, s>>>(c.np, c.L1, c.L2, h->x, h->p,
-                                                                                     h->d, h->pk);
+    k2_finalize<<<grid, 256, 0, s>>>(c.np, c.M1, c.M2, h->cell, h->v, h->p, h->d, h->pk);
     CK2(cudaMemcpyAsync(h->ex, h->exk, N * sizeof(double), cudaMemcpyDeviceToDevice, s));
     CK2(cudaMemcpyAsync(h->ey, h->eyk, N * sizeof(double), cudaMemcpyDeviceToDevice, s));
     CK2(cudaGetLastError());
@@ -954,17 +1020,8 @@ extern "C" int pic2d_energy(pic2d_handle *h, double out[4])
     const pic2d_config &c = h->cfg;
     CK2(cudaMemsetAsync(h->acc, 0, 2 * sizeof(double), h->stream));
     const int grid = (int)std::min<long long>((c.np + 255) / 256, 1024);
-    const double hb = h->spin ? c.hbar : 0.0;
-#define PIC2D_ENERGY(K)                                                                                     \
-    k2_energy<K><<<grid, 256, 0, h->stream>>>(c.np, c.M1, c.M2, h->dx1, h->dx2, c.weight, h->x, h->p, h->az, hb, \
-                                              h->spin, h->gax, h->gay, h->bz, h->acc)
-    switch (c.degree) {
-    case 2: PIC2D_ENERGY(2); break;
-    case 3: PIC2D_ENERGY(3); break;
-    case 4: PIC2D_ENERGY(4); break;
-    default: PIC2D_ENERGY(5); break;
-    }
-#undef PIC2D_ENERGY
+    const Args2D args = make_args(h);
+    PIC2D_DEGREE(c.degree, (k2_energy<K><<<grid, 256, 0, h->stream>>>(args, h->p, h->acc)))
     CK2(cudaGetLastError());
     std::vector<double> ex(h->N), ey(h->N);
     double acc[2] = {0.0, 0.0};
@@ -986,19 +1043,17 @@ extern "C" int pic2d_set_spin(pic2d_handle *h, const double *s, const double *bz
     const pic2d_config &c = h->cfg;
     const size_t N = (size_t)h->N, n3 = 3 * (size_t)c.np;
     if (!h->spin) {
-        double *sp = nullptr, *b0 = nullptr, *b1 = nullptr, *b2 = nullptr;
+        double *sp = nullptr, *b0 = nullptr, *tb = nullptr;
         if (cudaMalloc((void **)&sp, n3 * sizeof(double)) != cudaSuccess ||
             cudaMalloc((void **)&b0, N * sizeof(double)) != cudaSuccess ||
-            cudaMalloc((void **)&b1, N * sizeof(double)) != cudaSuccess ||
-            cudaMalloc((void **)&b2, N * sizeof(double)) != cudaSuccess) {
-            for (double *q : {sp, b0, b1, b2})
+            cudaMalloc((void **)&tb, N * pad2(c.degree * c.degree) * sizeof(double)) != cudaSuccess) {
+            for (double *q : {sp, b0, tb})
                 if (q) cudaFree(q);
             return fail2d(h, PIC_ERR_NOMEM, "spin and b_z arrays");
         }
         h->spin = sp;
         h->bz = b0;
-        h->gbx = b1;
-        h->gby = b2;
+        h->TB = tb;
     }
     const cudaMemcpyKind kind = mem == PIC_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
     std::vector<double> b(N);
@@ -1008,9 +1063,9 @@ extern "C" int pic2d_set_spin(pic2d_handle *h, const double *s, const double *bz
     CK2(cudaStreamSynchronize(h->stream));
     for (size_t i = 0; i < N; ++i)
         if (!std::isfinite(b[i])) return fail2d(h, PIC_ERR_INVALID, "b_z not finite at node %zu", i);
-    const std::vector<double> gbx = grid_diff(b, c.M1, c.M2, 0, h->dx1), gby = grid_diff(b, c.M1, c.M2, 1, h->dx2);
-    CK2(cudaMemcpyAsync(h->gbx, gbx.data(), N * sizeof(double), cudaMemcpyHostToDevice, h->stream));
-    CK2(cudaMemcpyAsync(h->gby, gby.data(), N * sizeof(double), cudaMemcpyHostToDevice, h->stream));
+    PIC2D_DEGREE(c.degree, (k2_table<K - 1, K - 1><<<(unsigned)((N * Dim2<K>::nB + 127) / 128), 128, 0, h->stream>>>(
+                               c.M1, c.M2, h->bz, h->TB, Dim2<K>::pB)))
+    CK2(cudaGetLastError());
     CK2(cudaStreamSynchronize(h->stream));
     return PIC_OK;
 }
@@ -1019,9 +1074,30 @@ extern "C" int pic2d_get_state(pic2d_handle *h, double *x, double *p, double *ex
 {
     if (!h || (mem != PIC_MEM_HOST && mem != PIC_MEM_DEVICE)) return PIC_ERR_INVALID;
     const cudaMemcpyKind kind = mem == PIC_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
-    const size_t np2 = 2 * (size_t)h->cfg.np, N = (size_t)h->N;
-    if (x) CK2(cudaMemcpyAsync(x, h->x, np2 * sizeof(double), kind, h->stream));
-    if (p) CK2(cudaMemcpyAsync(p, h->p, np2 * sizeof(double), kind, h->stream));
+    const size_t bytes = (size_t)h->cfg.np * sizeof(double2), N = (size_t)h->N;
+    // markers to the host: by several threads where the memory is pageable
+    auto markers = [&](double *dst, const double2 *src) -> int {
+        if (mem == PIC_MEM_HOST) {
+            cudaPointerAttributes at{};
+            const bool pageable = cudaPointerGetAttributes(&at, dst) != cudaSuccess || at.type == cudaMemoryTypeUnregistered;
+            cudaGetLastError();
+            if (pageable) {
+                CK2(cudaStreamSynchronize(h->stream));
+                if (h->copy.run(dst, src, bytes, h->device)) return PIC_OK;
+            }
+        }
+        CK2(cudaMemcpyAsync(dst, src, bytes, kind, h->stream));
+        return PIC_OK;
+    };
+    int rc;
+    if (x) {
+        // host positions pass through the displacement array (free between substeps)
+        double2 *dst = mem == PIC_MEM_HOST ? h->d : reinterpret_cast<double2 *>(x);
+        k2_store<<<marker_grid2d(h), 256, 0, h->stream>>>(h->cfg.np, h->cfg.L1, h->cfg.L2, h->dx1, h->dx2, h->cell, h->v, dst);
+        CK2(cudaGetLastError());
+        if (mem == PIC_MEM_HOST && (rc = markers(x, dst))) return rc;
+    }
+    if (p && (rc = markers(p, h->p))) return rc;
     if (ex) CK2(cudaMemcpyAsync(ex, h->ex, N * sizeof(double), kind, h->stream));
     if (ey) CK2(cudaMemcpyAsync(ey, h->ey, N * sizeof(double), kind, h->stream));
     CK2(cudaStreamSynchronize(h->stream));

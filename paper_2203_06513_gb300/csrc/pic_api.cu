@@ -1289,13 +1289,16 @@ extern "C" int pic_get_state(pic_handle *h, const pic_arrays *o, int32_t mem)
         stage_doubles(h, 1 - h->cur, o->x ? &dx_out : nullptr, o->p ? &dp_out : nullptr);
         launch_store(h->fp32, h->np, h->M, h->dx, cur_parts(h), dx_out, dp_out, particle_grid(h), 256, h->stream);
         cudaError_t e = cudaGetLastError();
-        if (e == cudaSuccess) {
-            if (o->x) e = cudaMemcpyAsync(o->x, dx_out, np * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
-            if (e == cudaSuccess && o->p)
-                e = cudaMemcpyAsync(o->p, dp_out, np * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
-            cudaError_t e2 = cudaStreamSynchronize(h->stream);
-            if (e == cudaSuccess) e = e2;
-        }
+        if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+        // pageable arrays by several threads, page-locked ones by the copy engine
+        auto out = [&](double *dst, double *src, bool pageable) {
+            if (!dst || e != cudaSuccess) return;
+            if (pageable && h->copy.run(dst, src, np * sizeof(double), h->device)) return;
+            e = cudaMemcpyAsync(dst, src, np * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+        };
+        out(o->x, dx_out, !px);
+        out(o->p, dp_out, !pp);
         if (e != cudaSuccess) return fail(h, PIC_ERR_CUDA, "get_state: %s", cudaGetErrorString(e));
         ++h->launches;
     }

@@ -6,6 +6,7 @@
 #include <vector>
 
 #include "pic.h"
+#include "pic_hostcopy.h"
 #include "pic_internal.h"
 
 using pic::PartPtrs;
@@ -95,6 +96,8 @@ struct pic_handle {
     double t_warm = 0;
     long long n_warm = 0;
     pic_mlp *mlp = nullptr;         // borrowed warm-start network
+
+    pic::HostCopy copy;             // pageable host transfers
 
     std::string err;
 };
