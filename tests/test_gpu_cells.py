@@ -130,3 +130,92 @@ def test_one_kernel_steps_report_no_convergence():
     with pytest.raises(pic.NoConvergence):
         g.step(3)
     g.close()
+
+
+# rows of the scratch: 32 replicas, fewer than 32 blocks, 2 replicas, one replica; paths of several laps
+@pytest.mark.parametrize("nx,k,n,reach", [(8, 3, 900, 64.0), (33, 5, 1, 0.3), (100, 2, 700, 0.5), (1000, 4, 12000, 2.5),
+                                          (4099, 5, 900, 1.0), (8192, 4, 700, 20.0)])
+def test_noalloc_replicas_vs_oracle(nx, k, n, reach):
+    """The handle-free deposit at its replica counts; half of the markers in one cell.
+    Double sums on both sides: 1e-13 of w sum |disp|, as for the handle's deposit."""
+    import ctypes
+    import torch
+    L = 4 * np.pi
+    dx, w = L / nx, L / n
+    rng = np.random.default_rng(nx + k)
+    x = rng.uniform(0, L, n)
+    x[: n // 2] = (nx // 2 + rng.random(n // 2)) * dx
+    x[-1] = -3.25 * L                                              # wrapped into the box
+    disp = rng.uniform(-reach, reach, n) * dx
+    xd, dd = torch.from_numpy(x).cuda(), torch.from_numpy(disp).cuda()
+    out = torch.full((nx,), float("nan"), dtype=torch.float64, device="cuda")
+    ptr = [ctypes.c_void_p(t.data_ptr()) for t in (xd, dd, out)]
+    f = pic.load().pic_deposit_current_noalloc
+    f.argtypes = [ctypes.c_double, ctypes.c_int32, ctypes.c_int32, ctypes.c_int64, ctypes.c_double] + [ctypes.c_void_p] * 4
+    assert f(L, nx, k, n, w, *ptr, None) == 0
+    want = np.zeros(nx)
+    if n <= 1000:
+        for xa, da in zip(x, disp):
+            want += w * O.path_integral(k, nx, dx, float(xa), float(xa + da))[1]
+    else:                                                          # the handle's deposit
+        ay = np.zeros(nx)
+        g = pic.Pic(pic.Config(L, nx, k, n, w, 8 * dx), np.mod(x, L), np.zeros(n), ay, ay)
+        ref = torch.zeros(nx, dtype=torch.float64, device="cuda")
+        g.deposit(pic.PIC_DEP_CURRENT, dd, ref)
+        want = ref.cpu().numpy()
+        g.close()
+    assert np.max(np.abs(out.cpu().numpy() - want)) < 1e-13 * w * np.sum(np.abs(disp))
+
+
+#                         M1  M2  k  np   vth  dt   spin
+@pytest.mark.parametrize("M1,M2,k,n,vth,dt,spin", [
+    (1, 11, 3, 40, 0.2, 0.1, False), (5, 1, 2, 33, 0.2, 0.1, True), (13, 9, 5, 300, 0.2, 0.1, False),
+    (40, 3, 3, 200, 1.5, 0.12, True),                              # paths over more than a cell
+    (9, 10, 4, 257, 0.1, 0.02, True), (6, 7, 2, 1, 0.5, 0.05, False)])
+def test_2d_awkward_shapes(M1, M2, k, n, vth, dt, spin):
+    """Subsystem I in two dimensions against the oracle where blocks, cells and paths have
+    edges; half of the markers in one cell, some on knots.  Both sides stop at the same
+    increment: 1e-10, as in the 2D parity tests."""
+    from oracle import oracle2d as O2
+    from paper_2203_06513_gb300 import pic2d as P2
+    rng = np.random.default_rng(100 * M1 + M2)
+    L1, L2 = 4.0, 3.0
+    x = np.column_stack([rng.uniform(0, L1, n), rng.uniform(0, L2, n)])
+    x[: n // 2] = (np.array([M1 // 2, M2 // 2]) + rng.random((n // 2, 2))) * [L1 / M1, L2 / M2]
+    x[-1] = [0.0, (M2 - 1) * L2 / M2]
+    p = rng.normal(0, vth, (n, 2))
+    a, ex, ey, bz = (0.05 * rng.normal(0, 1, M1 * M2) for _ in range(4))
+    s = rng.normal(0, 1, (n, 3))
+    s /= np.linalg.norm(s, axis=1, keepdims=True)
+    cfg = P2.Config2D(L1, L2, M1, M2, k, n, L1 * L2 / n, dt)
+    orc = O2.Oracle2D(L1, L2, M1, M2, k, w=L1 * L2 / n, dt=dt)
+    if spin:
+        cfg.hbar = orc.hbar = 0.1
+    g = P2.Pic2D(cfg, x, p, ex, ey, a)
+    if spin:
+        g.set_spin(s, bz)
+    sx, sp, sex, sey = x, p, ex, ey
+    for _ in range(2):
+        sx, sp, sex, sey, it = orc.substep1(sx, sp, sex, sey, a, s=s if spin else None, bz=bz if spin else None)
+        assert abs(g.substep1() - it) <= 1
+    st = g.state()
+    d = np.abs(np.mod(st["x"] - sx + 0.5 * np.array([L1, L2]), [L1, L2]) - 0.5 * np.array([L1, L2]))
+    assert np.max(d / [L1, L2]) < 1e-10
+    for got, ref in ((st["p"], sp), (st["ex"], sex), (st["ey"], sey)):
+        assert np.max(np.abs(got - ref)) <= 1e-10 * max(np.max(np.abs(ref)), 1e-3)
+    g.close()
+
+
+def test_2d_large_state_copy():
+    """A state larger than one copy piece comes back to pageable memory whole."""
+    from paper_2203_06513_gb300 import pic2d as P2
+    n, L1, L2 = 700001, 4.0, 3.0
+    rng = np.random.default_rng(7)
+    x = np.column_stack([rng.uniform(0, L1, n), rng.uniform(0, L2, n)])
+    p = rng.normal(0, 0.1, (n, 2))
+    f = np.zeros(30)
+    g = P2.Pic2D(P2.Config2D(L1, L2, 6, 5, 3, n, L1 * L2 / n, 0.1), x, p, f, f, f)
+    st = g.state()
+    np.testing.assert_array_equal(st["p"], p)
+    assert np.max(np.abs(st["x"] - x)) < 4e-15                      # cell + offset, a few roundings of L
+    g.close()
