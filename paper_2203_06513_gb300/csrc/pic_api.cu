@@ -732,7 +732,7 @@ static WarmArgs warm_args(pic_handle *h, double dt)
     WarmArgs wa{};
     wa.M = h->M; wa.K = h->K; wa.fp32 = h->fp32; wa.np = h->np; wa.dx = h->dx; wa.dt = dt;
     wa.P = cur_parts(h);
-    wa.ex = h->ex; wa.ay = h->ay; wa.az = h->az;
+    wa.ex = h->ex; wa.coefA = h->T.A;
     wa.params = mlp_params(h->mlp); wa.norm = mlp_norm(h->mlp);
     wa.status = &h->ctrl->status;
     return wa;

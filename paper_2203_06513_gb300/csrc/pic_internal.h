@@ -383,7 +383,8 @@ struct WarmArgs {
     long long np;
     double dx, dt;
     PartPtrs P;
-    const double *ex, *ay, *az;
+    const double *ex;
+    const void *coefA;  // a^n's table (CoefTables)
     const float *params, *norm;
     int *status;        // error bits (STATUS_TIMEOUT)
 };

@@ -27,6 +27,7 @@
 
 #include "pic.h"
 #include "pic_internal.h"
+#include "pic_poly.cuh"
 
 namespace pic {
 
@@ -51,32 +52,49 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
     return u;
 }
 
-// ReLU of two pre-activations, rounded to bf16 and packed: one packed max a pair.
+// ReLU of two pre-activations, rounded to bf16 and packed.  NaN = true: a NaN becomes 0 (one
+// packed max more); false: it stays a NaN, one conversion does both.
+template <bool NaN>
 __device__ __forceinline__ uint32_t relu_bf16x2(float z0, float z1)
 {
-    const __nv_bfloat162 out = __hmax2(__floats2bfloat162_rn(z0, z1), __float2bfloat162_rn(0.f));
     uint32_t o;
-    memcpy(&o, &out, 4);
+    if (NaN) {
+        const __nv_bfloat162 out = __hmax2(__floats2bfloat162_rn(z0, z1), __float2bfloat162_rn(0.f));
+        memcpy(&o, &out, 4);
+    } else {
+        asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(o) : "f"(z1), "f"(z0));
+    }
     return o;
 }
 
 // ---------------------------------------------------------------------------
 // Tensor-core inference with tcgen05 (5th-generation tensor cores, accumulators
-// in tensor memory).  One block of 1024 threads per SM runs 8 independent chains,
+// in tensor memory).  One block of 640 threads per SM runs 5 independent chains,
 // one per warpgroup; a chain takes 128 markers at a time, one row per thread.  Per
-// layer the chain writes its rows' bf16 activations to shared memory in the
-// canonical K-major layout (8-row x 16-byte core matrices), one of its threads
-// issues the layer's tcgen05.mma instructions (M = 128, N = 64, K = 16 each) and
-// commits them to the chain's mbarrier, every thread of the chain waits (bounded),
-// loads its row of the fp32 accumulator from the chain's 64 tensor-memory columns
-// and applies the ReLU.  While one chain waits for the tensor
-// cores, the other seven run their epilogues.  Weights are staged once per block,
-// in the same layout, and shared by the chains.
+// layer every thread stores its row's bf16 activations to the chain's operand columns
+// of tensor memory, one thread issues the layer's tcgen05.mma instructions (M = 128,
+// N = 64, K = 16 each) and commits them to the chain's mbarrier, every thread waits
+// (bounded), loads its row of the fp32 accumulator and applies the ReLU.  While one
+// chain waits for the tensor cores, the others run their epilogues.  Weights are staged
+// once per block, in the canonical K-major layout (8-row x 16-byte core matrices) in
+// shared memory, and shared by the chains.
+//
+// Activations stay out of shared memory: as the A operand there they cost 48 KB written
+// and 48 KB read back a tile at 128 bytes a clock, more than the products themselves
+// (32 clocks a step).  Warm start of 2e7 markers: 666 us with 8 chains on operands in
+// shared memory, 582 us so, 562 us with the next tile's features formed beside the
+// second layer (605 us with the ReLU as a packed maximum of its own).  What bounds it:
+// the tensor pipe is busy half of the time, the rest is the chains' own latency.
+// The tensor memory holds 5 chains: 64 accumulator and 32 operand columns each, and 8
+// columns of the constant operand for the biases.
 // ---------------------------------------------------------------------------
 constexpr int kRows = 128;                       // markers per tile (UMMA M) = threads per chain
-constexpr int kChains = 8;                       // warpgroups per block
-constexpr int kMlpThreads = kRows * kChains;     // 1024
-constexpr int kTmemCols = 512;                   // chain g: columns 64 g .. 64 g + 63
+constexpr int kChains = 5;                       // warpgroups per block
+constexpr int kMlpThreads = kRows * kChains;     // 640
+constexpr int kTmemCols = 512;
+constexpr int kChainCols = 96;                   // chain g: columns 96 g .. : 64 accumulators, 32 operands
+constexpr int kOnesCol = kChains * kChainCols;   // 8 columns: 1 in operand column 0, else 0
+static_assert(kOnesCol + 8 <= kTmemCols, "tensor memory");
 constexpr int kOutN = 16;                        // output layer padded to the smallest N for M = 128
 
 // byte offset of element (r, k) in a K-major no-swizzle operand with K columns:
@@ -87,28 +105,26 @@ __host__ __device__ constexpr int kmaj_off(int r, int k, int K)
 }
 
 struct MlpChain {
-    __nv_bfloat16 A0[kRows * 16];   // features (K = 16, 6 used)
-    __nv_bfloat16 A[kRows * 64];    // hidden activations (reused per layer)
     unsigned long long bar;         // MMA completion
-    int abort;
-    int pad[5];
+    int abort;                      // a wait gave up
+    int pad;
 };
 
 // The biases of layers 1-3 ride on the tensor cores: layer 1 takes b1 as weight
-// column 6 against a constant feature 1; layers 2 and 3 add one K = 16 step of a
-// shared block whose column 0 is 1 against a bias block whose column 0 is b.
+// column 6 against a constant feature 1; layers 2 and 3 add one K = 16 step of the
+// constant operand, whose column 0 is 1, against a bias block whose column 0 is b.
 struct MlpUmma {
     __nv_bfloat16 W1[64 * 16];      // [n][k], K = 16: 6 weights, b1, zeros
     __nv_bfloat16 W2[64 * 64];
     __nv_bfloat16 W3[64 * 64];
     __nv_bfloat16 W4[kOutN * 64];   // rows 0, 1 used
-    __nv_bfloat16 ONES[kRows * 16]; // column 0 = 1
     __nv_bfloat16 B2[64 * 16];      // column 0 = b2
     __nv_bfloat16 B3[64 * 16];      // column 0 = b3
     MlpChain C[kChains];
     float b4[2];
     float norm[kNorm];
     uint32_t tmem;                  // tensor-memory base address
+    int last_ok;                    // the output layer's row 0 has no NaN
 };
 
 // shared-memory matrix descriptor (tcgen05): start, leading (K-direction core
@@ -126,12 +142,13 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N)
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc)
+// D (tensor memory) = A (tensor memory: lane = row, two bf16 a column) x B (shared memory)
+__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint32_t a_tmem, uint64_t b, uint32_t idesc, uint32_t acc)
 {
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-        "l"(a), "l"(b), "r"(idesc), "r"(acc));
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(b), "r"(idesc), "r"(acc));
 }
 
 __device__ __forceinline__ void umma_commit(unsigned long long *bar)
@@ -150,24 +167,45 @@ __device__ __forceinline__ void chain_sync(int g)
     asm volatile("bar.sync %0, %1;" ::"r"(1 + g), "r"(kRows) : "memory");
 }
 
-// 32 consecutive fp32 columns of this thread's tensor-memory lane, and the wait
+// 64 consecutive fp32 columns of this thread's tensor-memory lane, and the wait
 // for them, in one statement (the registers are valid only after the wait)
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32])
+__device__ __forceinline__ void tmem_ld64(uint32_t taddr, uint32_t (&r)[64])
 {
-    uint32_t r[32];
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x64.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,"
+        "%32,%33,%34,%35,%36,%37,%38,%39,%40,%41,%42,%43,%44,%45,%46,%47,%48,%49,%50,%51,%52,%53,%54,%55,%56,%57,%58,%59,%60,%61,%62,%63}, [%64];\n"
         "tcgen05.wait::ld.sync.aligned;\n"
         : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
           "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]),
+          "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]),
+          "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]),
+          "=r"(r[48]), "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]),
+          "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63])
         : "r"(taddr)
         : "memory");
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
+
+// 32 and 8 consecutive columns of this thread's lane; complete after tmem_st_wait
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32])
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31};\n" ::
+          "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),
+          "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),
+          "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),
+          "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31]),
+        "r"(taddr)
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%5,%5,%5};\n" ::"r"(taddr), "r"(a), "r"(b),
+                 "r"(c), "r"(d), "r"(0u)
+                 : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 __device__ __forceinline__ void tmem_ld2(uint32_t taddr, float (&v)[2])
 {
@@ -197,10 +235,6 @@ __device__ void stage_umma(MlpUmma &S, const float *params, const float *norm)
         put_bf16(S.B2, kmaj_off(n, k, 16), k == 0 ? params[kOffB2 + n] : 0.f);
         put_bf16(S.B3, kmaj_off(n, k, 16), k == 0 ? params[kOffB3 + n] : 0.f);
     }
-    for (int i = threadIdx.x; i < kRows * 16; i += blockDim.x) {
-        const int r = i >> 4, k = i & 15;
-        put_bf16(S.ONES, kmaj_off(r, k, 16), k == 0 ? 1.f : 0.f);
-    }
     for (int i = threadIdx.x; i < 64 * 64; i += blockDim.x) {
         const int n = i >> 6, k = i & 63;
         put_bf16(S.W2, kmaj_off(n, k, 64), params[kOffW2 + n * kHid + k]);
@@ -212,9 +246,11 @@ __device__ void stage_umma(MlpUmma &S, const float *params, const float *norm)
     }
     if (threadIdx.x < kOut) S.b4[threadIdx.x] = params[kOffB4 + threadIdx.x];
     if (threadIdx.x < kNorm) S.norm[threadIdx.x] = norm[threadIdx.x];
-    // the padding half of every feature row (k = 8..15) stays zero
-    const int g = threadIdx.x / kRows, r = threadIdx.x % kRows;
-    *reinterpret_cast<uint4 *>(reinterpret_cast<char *>(S.C[g].A0) + kmaj_off(r, 8, 16)) = make_uint4(0, 0, 0, 0);
+    if (threadIdx.x < 32) {
+        const float w = params[kOffW4 + threadIdx.x] + params[kOffW4 + 32 + threadIdx.x];
+        const int ok = __all_sync(0xffffffffu, !isnan(w)) && !isnan(params[kOffB4]) && !isnan(norm[2 * kIn]);
+        if (threadIdx.x == 0) S.last_ok = ok;
+    }
 }
 
 // Block prologue: chain barriers, tensor memory (warp 0 allocates all 512
@@ -233,15 +269,29 @@ __device__ __forceinline__ void umma_begin(MlpUmma &S, const float *params, cons
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     stage_umma(S, params, norm);
-    fence_proxy_async();           // weights and zero padding: visible to the tensor cores
+    fence_proxy_async();           // weights: visible to the tensor cores
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (threadIdx.x < kRows) {     // the constant operand, a lane a thread
+        tmem_st8(S.tmem + ((threadIdx.x & ~31u) << 16) + kOnesCol, pack_bf16(1.f, 0.f), 0u, 0u, 0u);
+        tmem_st_wait();
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
 }
 
-__device__ __forceinline__ void umma_end(MlpUmma &S)
+// Block epilogue: report chains that gave up, and give their MMAs in flight one more
+// bounded wait before the tensor memory is freed.
+__device__ __forceinline__ void umma_end(MlpUmma &S, int g, unsigned phase, int *status)
 {
     tc_fence_before();
+    __syncthreads();
+    if (*reinterpret_cast<volatile int *>(&S.C[g].abort)) {
+        atomicOr(status, STATUS_TIMEOUT);
+        mbar_wait(&S.C[g].bar, phase ^ 1u);
+    }
     __syncthreads();
     tc_fence_after();
     if (threadIdx.x < 32)
@@ -249,96 +299,83 @@ __device__ __forceinline__ void umma_end(MlpUmma &S)
                      : "memory");
 }
 
-// Write this thread's feature row (normalised, bf16) into its chain's tile.
-__device__ __forceinline__ void umma_put_features(MlpUmma &S, int g, int r, const float f[kIn])
+// This thread's lane of its chain's columns.  Warp w reaches lanes 32 (w % 4) .. + 31.
+__device__ __forceinline__ uint32_t umma_cols(const MlpUmma &S, int g, int r)
 {
-    uint4 v;
-    v.x = pack_bf16((f[0] - S.norm[0]) * S.norm[kIn + 0], (f[1] - S.norm[1]) * S.norm[kIn + 1]);
-    v.y = pack_bf16((f[2] - S.norm[2]) * S.norm[kIn + 2], (f[3] - S.norm[3]) * S.norm[kIn + 3]);
-    v.z = pack_bf16((f[4] - S.norm[4]) * S.norm[kIn + 4], (f[5] - S.norm[5]) * S.norm[kIn + 5]);
-    v.w = pack_bf16(1.f, 0.f);     // feature 6 = 1 (carries b1)
-    *reinterpret_cast<uint4 *>(reinterpret_cast<char *>(S.C[g].A0) + kmaj_off(r, 0, 16)) = v;
+    return S.tmem + ((uint32_t)(r & ~31) << 16) + (uint32_t)(kChainCols * g);
 }
 
-// One layer of chain g: issue (the chain's first thread), wait (all of its
-// threads); false after a bounded wait gave up.
-__device__ __forceinline__ bool umma_layer(MlpUmma &S, int g, int r, const __nv_bfloat16 *Aop, int K,
-                                           const __nv_bfloat16 *Bop, const __nv_bfloat16 *bias,
-                                           uint32_t idesc, unsigned &phase)
+// Write this thread's feature row (normalised, bf16) into its chain's operand.
+__device__ __forceinline__ void umma_put_features(MlpUmma &S, int g, int r, const float f[kIn])
+{
+    tmem_st8(umma_cols(S, g, r) + 64,
+             pack_bf16((f[0] - S.norm[0]) * S.norm[kIn + 0], (f[1] - S.norm[1]) * S.norm[kIn + 1]),
+             pack_bf16((f[2] - S.norm[2]) * S.norm[kIn + 2], (f[3] - S.norm[3]) * S.norm[kIn + 3]),
+             pack_bf16((f[4] - S.norm[4]) * S.norm[kIn + 4], (f[5] - S.norm[5]) * S.norm[kIn + 5]),
+             pack_bf16(1.f, 0.f));     // feature 6 = 1 (carries b1)
+}
+
+// One layer of chain g: issue (the chain's first thread), wait (all of its threads).
+// A wait that gives up marks the chain; its threads all leave at the next layer's
+// barrier (false), before anything else is issued.  beside() runs while the layer does.
+template <typename Beside>
+__device__ __forceinline__ bool umma_layer(MlpUmma &S, int g, int r, int K, const __nv_bfloat16 *Bop,
+                                           const __nv_bfloat16 *bias, uint32_t idesc, unsigned &phase, Beside &&beside)
 {
     MlpChain &C = S.C[g];
-    fence_proxy_async();           // this thread's activations: visible to the tensor cores
+    tmem_st_wait();                // this thread's activations
     tc_fence_before();
     chain_sync(g);
     tc_fence_after();
+    if (*reinterpret_cast<volatile int *>(&C.abort)) return false;
     if (r == 0) {
         const uint32_t sbo = (uint32_t)K * 16;    // K/8 core matrices of 128 bytes per 8-row group
-        for (int kt = 0; kt < K / 16; ++kt)
-            umma_bf16(S.tmem + 64u * g, umma_desc(reinterpret_cast<const char *>(Aop) + kt * 256, 128, sbo),
-                      umma_desc(reinterpret_cast<const char *>(Bop) + kt * 256, 128, sbo), idesc, kt > 0);
+        const uint32_t d = S.tmem + (uint32_t)(kChainCols * g);
+        for (int kt = 0; kt < K / 16; ++kt)       // 16 bf16 = 8 operand columns a step
+            umma_bf16(d, d + 64 + 8 * kt, umma_desc(reinterpret_cast<const char *>(Bop) + kt * 256, 128, sbo), idesc,
+                      kt > 0);
         if (bias)      // + ones x bias^T
-            umma_bf16(S.tmem + 64u * g, umma_desc(S.ONES, 128, 256), umma_desc(bias, 128, 256), idesc, 1u);
+            umma_bf16(d, S.tmem + kOnesCol, umma_desc(bias, 128, 256), idesc, 1u);
         umma_commit(&C.bar);
     }
-    // warp 0 of the chain waits for the MMAs (bounded); the other warps block at
-    // the chain barrier instead of polling
-    bool ok = true;
-    if (r < 32) {
-        ok = mbar_wait(&C.bar, phase);
-        if (!ok) atomicExch(&C.abort, 1);
-        tc_fence_before();
-    }
-    chain_sync(g);
-    if (*reinterpret_cast<volatile int *>(&C.abort)) {
-        // gave up: give the MMAs in flight one more bounded wait before the block
-        // frees its tensor memory and leaves
-        mbar_wait(&C.bar, phase);
-        ok = false;
-    }
+    __syncwarp();
+    beside();
+    if (!mbar_wait(&C.bar, phase)) atomicExch(&C.abort, 1);
+    __syncwarp();
     phase ^= 1u;
     tc_fence_after();
-    return ok;
+    return true;
 }
 
 // ReLU of this thread's accumulator row (the chain's 64 columns, bias included)
-// into its row of the next layer's operand.  Warp w reads tensor-memory lanes
-// 32 (w % 4) .. + 31.
+// into its row of the next layer's operand.
+template <bool NaN>
 __device__ __forceinline__ void umma_epilogue(MlpUmma &S, int g, int r)
 {
-    const uint32_t taddr = S.tmem + ((uint32_t)(r & ~31) << 16) + 64u * g;
-    char *row = reinterpret_cast<char *>(S.C[g].A);
+    const uint32_t cols = umma_cols(S, g, r);
+    uint32_t v[64], o[32];
+    tmem_ld64(cols, v);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        float v[32];
-        tmem_ld32(taddr + 32 * h, v);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) {      // 8 columns = one 16-byte chunk of the row
-            uint4 o;
-            const int k0 = 32 * h + 8 * c;
-            o.x = relu_bf16x2(v[8 * c + 0], v[8 * c + 1]);
-            o.y = relu_bf16x2(v[8 * c + 2], v[8 * c + 3]);
-            o.z = relu_bf16x2(v[8 * c + 4], v[8 * c + 5]);
-            o.w = relu_bf16x2(v[8 * c + 6], v[8 * c + 7]);
-            *reinterpret_cast<uint4 *>(row + kmaj_off(r, k0, 64)) = o;
-        }
-    }
+    for (int i = 0; i < 32; ++i) o[i] = relu_bf16x2<NaN>(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+    tmem_st32(cols + 64, o);
 }
 
 // The network on chain g's 128 feature rows.  Returns false after a bounded wait
-// gave up; y = this row's scaled outputs.
-__device__ __forceinline__ bool umma_network(MlpUmma &S, int g, int r, unsigned &phase, float (&y)[2])
+// gave up; y = this row's scaled outputs.  beside() runs while the tensor cores work.
+template <bool NaN, typename Beside>
+__device__ __forceinline__ bool umma_network(MlpUmma &S, int g, int r, unsigned &phase, float (&y)[2], Beside &&beside)
 {
+    auto nothing = [] {};
     constexpr uint32_t kHidDesc = idesc_bf16(kRows, kHid), kOutDesc = idesc_bf16(kRows, kOutN);
-    MlpChain &C = S.C[g];
-    if (!umma_layer(S, g, r, C.A0, 16, S.W1, nullptr, kHidDesc, phase)) return false;
-    umma_epilogue(S, g, r);
-    if (!umma_layer(S, g, r, C.A, 64, S.W2, S.B2, kHidDesc, phase)) return false;
-    umma_epilogue(S, g, r);
-    if (!umma_layer(S, g, r, C.A, 64, S.W3, S.B3, kHidDesc, phase)) return false;
-    umma_epilogue(S, g, r);
-    if (!umma_layer(S, g, r, C.A, 64, S.W4, nullptr, kOutDesc, phase)) return false;
+    if (!umma_layer(S, g, r, 16, S.W1, nullptr, kHidDesc, phase, nothing)) return false;
+    umma_epilogue<NaN>(S, g, r);
+    if (!umma_layer(S, g, r, 64, S.W2, S.B2, kHidDesc, phase, beside)) return false;
+    umma_epilogue<NaN>(S, g, r);
+    if (!umma_layer(S, g, r, 64, S.W3, S.B3, kHidDesc, phase, nothing)) return false;
+    umma_epilogue<NaN>(S, g, r);
+    if (!umma_layer(S, g, r, 64, S.W4, nullptr, kOutDesc, phase, nothing)) return false;
     float o[2];
-    tmem_ld2(S.tmem + ((uint32_t)(r & ~31) << 16) + 64u * g, o);
+    tmem_ld2(umma_cols(S, g, r), o);
     y[0] = (o[0] + S.b4[0]) * S.norm[2 * kIn];
     y[1] = (o[1] + S.b4[1]) * S.norm[2 * kIn + 1];
     return true;
@@ -371,36 +408,30 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp_infer(const float *param
         for (int i = 0; i < kIn; ++i) nx[i] = an < B ? X[an * kIn + i] : 0.f;
         umma_put_features(S, g, r, f);
         float y[2];
-        if (!umma_network(S, g, r, phase, y)) {
-            if (r == 0) atomicOr(status, STATUS_TIMEOUT);
-            break;
-        }
+        if (!umma_network<true>(S, g, r, phase, y, [] {})) break;
         if (a < B) {
             Y[2 * a] = y[0];
             Y[2 * a + 1] = y[1];
         }
     }
-    umma_end(S);
+    umma_end(S, g, phase, status);
 }
 
 // ---------------------------------------------------------------------------
-// Warm start of subsystem I: delta^(0) = tau p/g0 + y0 dt^2/dx for every marker,
-// with the features gathered at x^n from e_x^n and a^n (staged in shared memory).
+// Warm start of subsystem I: delta^(0) = tau p/g0 + y0 dt^2/dx for every marker, with the
+// features at x^n: a^n from the cells' polynomials (the preparation of the substep writes
+// them), e_x^n from the nodes staged in shared memory.  The features of a chain's next
+// tile are formed while the tensor cores run the second layer of this one.
 // ---------------------------------------------------------------------------
 template <int K, typename R>
 __global__ void __launch_bounds__(kMlpThreads, 1) k_warm_mlp(WarmArgs A)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
     MlpUmma &S = *reinterpret_cast<MlpUmma *>(smem);
-    const int H = K + 1;
+    constexpr int H = K + 1, kPad = CoefPad<R, K + 1>::v;
     const int W = A.M + 2 * H;
     float *s_e = reinterpret_cast<float *>(smem + ((sizeof(MlpUmma) + 127) & ~size_t(127)));
-    float2 *s_a = reinterpret_cast<float2 *>(s_e + ((W + 1) & ~1));
-    for (int i = threadIdx.x; i < W; i += blockDim.x) {
-        const int gg = wrap_cell(i - H, A.M);
-        s_e[i] = (float)A.ex[gg];
-        s_a[i] = make_float2((float)A.ay[gg], (float)A.az[gg]);
-    }
+    for (int i = threadIdx.x; i < W; i += blockDim.x) s_e[i] = (float)A.ex[wrap_cell(i - H, A.M)];
     umma_begin(S, A.params, A.norm);
     const int g = threadIdx.x / kRows, r = threadIdx.x % kRows;
     const R *tp = static_cast<const R *>(A.P.t);
@@ -410,55 +441,55 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_warm_mlp(WarmArgs A)
     const float c2 = (float)(A.dt * A.dt / A.dx);
     unsigned phase = 0;
     const long long stride = (long long)gridDim.x * kChains * kRows;
-    // the next tile's markers are loaded while the network runs on this one
-    const long long base0 = ((long long)blockIdx.x * kChains + g) * kRows;
-    int nc = 0;
-    R nt = R(0), np_ = R(0);
-    if (base0 + r < A.np) {
-        nc = A.P.cell[base0 + r];
-        nt = tp[base0 + r];
-        np_ = pp[base0 + r];
-    }
-    for (long long base = base0; base < A.np; base += stride) {
-        const long long a = base + r;
-        const bool act = a < A.np;
-        float f[kIn], pn = 0.f, g0 = 1.f;
-        const int c = nc;
-        const float t = (float)nt + 0.5f;             // cell-relative position
-        pn = act ? (float)np_ : 0.f;
-        if (a + stride < A.np) {
-            nc = A.P.cell[a + stride];
-            nt = tp[a + stride];
-            np_ = pp[a + stride];
-        }
-        if (act) {
-            float v[K + 1], u[K];
-            bspline_vals<K, float>(t, v);
-            bspline_vals<K - 1, float>(t, u);
-            float Ay = 0.f, Az = 0.f, Ex = 0.f;
-#pragma unroll
-            for (int q = 0; q <= K; ++q) {
-                const float2 av = s_a[c - q + H];
-                Ay += av.x * v[q];
-                Az += av.y * v[q];
-            }
-#pragma unroll
-            for (int q = 0; q < K; ++q) Ex += s_e[c - q + H] * u[q];
-            g0 = sqrtf(1.f + pn * pn + Ay * Ay + Az * Az);
-            f[0] = t; f[1] = pn; f[2] = Ex; f[3] = Ay; f[4] = Az; f[5] = (float)A.dt;
-        } else {
+    int c = 0;
+    R t = R(0), p = R(0);
+    auto fetch = [&](long long a) {
+        if (a >= A.np) return;
+        c = A.P.cell[a];
+        t = tp[a];
+        p = pp[a];
+    };
+    float f[kIn], expl = 0.f;
+    auto features = [&](long long a) {
+        if (a >= A.np) {
 #pragma unroll
             for (int i = 0; i < kIn; ++i) f[i] = S.norm[i];
+            return;
         }
+        const float v = (float)t, pn = (float)p, tc = v + 0.5f;      // tc: cell-relative position
+        float u[K];
+        bspline_vals<K - 1, float>(tc, u);
+        float Ex = 0.f, Af[2];
+#pragma unroll
+        for (int q = 0; q < K; ++q) Ex += s_e[c - q + H] * u[q];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            R co[K + 1];
+            load_coef<K + 1>(static_cast<const R *>(A.coefA) + ((size_t)2 * c + i) * kPad, co);
+            Af[i] = (float)horner(co, t);
+        }
+        f[0] = tc; f[1] = pn; f[2] = Ex; f[3] = Af[0]; f[4] = Af[1]; f[5] = (float)A.dt;
+        expl = quotient(tau * pn, root(fmaf(pn, pn, fmaf(Af[0], Af[0], fmaf(Af[1], Af[1], 1.f)))));
+    };
+    const long long base0 = ((long long)blockIdx.x * kChains + g) * kRows;
+    fetch(base0 + r);
+    features(base0 + r);
+    fetch(base0 + r + stride);
+    for (long long base = base0; base < A.np; base += stride) {
+        const long long a = base + r;
         umma_put_features(S, g, r, f);
+        const float now = expl;
         float y[2];
-        if (!umma_network(S, g, r, phase, y)) {
-            if (r == 0) atomicOr(A.status, STATUS_TIMEOUT);
-            break;
-        }
-        if (act) dp[a] = (R)(tau * pn / g0 + y[0] * c2);
+        auto next = [&] {
+            features(a + stride);
+            fetch(a + 2 * stride);
+        };
+        if (!umma_network<false>(S, g, r, phase, y, next)) break;
+        // a hidden value that is no number proposes nothing (the inference takes it as 0)
+        if (isnan(y[0]) && S.last_ok) y[0] = 0.f;
+        if (a < A.np) dp[a] = (R)(now + y[0] * c2);
     }
-    umma_end(S);
+    umma_end(S, g, phase, A.status);
 }
 
 // ---------------------------------------------------------------------------
@@ -720,16 +751,19 @@ constexpr size_t kMinUmmaSmem = 120 * 1024;
 
 size_t mlp_infer_smem() { return sizeof(MlpUmma) > kMinUmmaSmem ? sizeof(MlpUmma) : kMinUmmaSmem; }
 
+// Grids up to this many staged nodes (M + 2 (K + 1)); larger ones are refused.
+constexpr size_t kMaxWarmNodes = 3296;
+
 size_t warm_mlp_smem(int M, int K)
 {
     const size_t W = (size_t)M + 2 * (size_t)(K + 1);
-    const size_t s = ((sizeof(MlpUmma) + 127) & ~size_t(127)) + ((W + 1) & ~size_t(1)) * sizeof(float) +
-                     W * sizeof(float2);
+    const size_t s = ((sizeof(MlpUmma) + 127) & ~size_t(127)) + W * sizeof(float);
     return s > kMinUmmaSmem ? s : kMinUmmaSmem;
 }
 
 int launch_warm_mlp(const WarmArgs &a, int grid, cudaStream_t s)
 {
+    if ((size_t)a.M + 2 * (size_t)(a.K + 1) > kMaxWarmNodes) return 1;
     const size_t smem = warm_mlp_smem(a.M, a.K);
     static size_t opted = 0;
     if (smem > opted) {

@@ -29,3 +29,33 @@ def test_training_gradient_at_ragged_batches(B):
     print(f"\nB {B}: gradient off by {err:.2e}, loss by {abs(loss / ref_loss - 1):.2e}")
     assert abs(loss - ref_loss) <= 1e-5 * ref_loss
     assert err <= 1e-4
+
+
+@pytest.mark.parametrize("n,k,fp32", [(1, 3, False), (127, 2, False), (641, 4, False), (5001, 5, True),
+                                      (100003, 3, True), (100003, 3, False)])
+def test_network_start_reaches_the_fixed_point(n, k, fp32):
+    """Steps from the network's proposal at partial tiles, several tiles a chain and every
+    degree against steps from x^n: the same fixed point, to the tolerances of the parity
+    tests."""
+    pytest.importorskip("torch")
+    from paper_2203_06513_gb300 import inputs as I
+    from paper_2203_06513_gb300 import pic
+    w = I.Workload("n", nx=51, degree=k, np=n, vth=0.1, pump=0.1, seed=n)
+    x, p = I.particles(w)
+    ay, az, ey, ez = I.fields(w)
+    az = 0.05 * np.random.default_rng(k).normal(size=w.nx)
+    norm = np.array([0.5, 0, 0, 0, 0, 0.05, 4.0, 5.0, 10.0, 3.0, 3.0, 10.0, 1.0, 1.0], np.float32)
+    net = pic.Mlp(norm, (0.3 * R.init(11)).astype(np.float32))
+    prec = pic.PIC_FP32 if fp32 else pic.PIC_FP64
+    a = pic.Pic(pic.Config.from_workload(w, precision=prec, warm_start=pic.PIC_WARM_MLP), x, p, ay, az, ey, ez)
+    net.attach(a)
+    b = pic.Pic(pic.Config.from_workload(w, precision=prec), x, p, ay, az, ey, ez)
+    a.step(2)
+    b.step(2)
+    got, ref = a.state_numpy(), b.state_numpy()
+    d = np.mod(got["x"] - ref["x"] + 0.5 * w.L, w.L) - 0.5 * w.L
+    assert np.max(np.abs(d)) / w.L <= (1e-5 if fp32 else 1e-11)
+    for key in ("p", "ex", "ey", "ez", "ay", "az"):
+        assert np.max(np.abs(got[key] - ref[key])) <= (1e-4 if fp32 else 1e-10) * max(np.max(np.abs(ref[key])), 1e-3), key
+    a.close()
+    b.close()
