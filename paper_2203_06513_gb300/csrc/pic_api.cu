@@ -187,7 +187,7 @@ static int read_ctrl(pic_handle *h)
     return PIC_OK;
 }
 
-static int particle_grid(pic_handle *h) { return h->num_sms * 4; }
+static int particle_grid(pic_handle *h) { return h->num_sms * 8; }
 
 // Split runs: a sum or max over the processes that hold the plasma's markers.
 static int reduce(pic_handle *h, int op, double *buf, long long n)
@@ -249,7 +249,7 @@ static int sort_markers(pic_handle *h)
     dst.delta = h->delta;
     dst.pnew = h->pnew;
     if (launch_sort(h->fp32, h->np, h->M, h->cfg.dt / h->dx, bins_per_cell(h->np, h->M), src, dst, h->counts,
-                    particle_grid(h), 256, h->stream))
+                    h->num_sms, h->stream))
         return fail(h, PIC_ERR_CUDA, "sort launch failed");
     CKL_N("launch_sort");
     h->cur = 1 - h->cur;
@@ -473,7 +473,7 @@ extern "C" int pic_init_split(const pic_config *cfg, const pic_arrays *in, int32
             (rc = dalloc(h, &h->gtab, M * coef_pad(0, c.degree + 1))))
             return bail(rc);
     }
-    if ((rc = dalloc(h, &h->counts, 2 * M * kVelBinsBase * bins_per_cell((long long)np, (int)M)))) return bail(rc);
+    if ((rc = dalloc(h, &h->counts, sort_counts(M * kVelBinsBase * bins_per_cell((long long)np, (int)M))))) return bail(rc);
     if ((rc = dalloc(h, &h->ctrl, 1))) return bail(rc);
     if (cudaMallocHost((void **)&h->h_flag, sizeof(int)) != cudaSuccess) return bail(PIC_ERR_NOMEM);
     if (cudaMallocHost((void **)&h->h_ctrl, sizeof(DevCtrl)) != cudaSuccess) return bail(PIC_ERR_NOMEM);

@@ -14,9 +14,10 @@ namespace pic {
 // together after they move (fewer deposit-window misses): measured on C2 (48,828
 // markers a cell) with sorting every second step, 64 quarter-cell bins 13.1 ms a step
 // against 13.4 ms for 16 whole-cell bins.  With few markers a cell they buy nothing and
-// the key count (M x bins) costs the single-block scan time, so sparse runs keep whole
-// cells.
+// the keys cost the scan time, so sparse runs keep whole cells.
 constexpr int kVelBinsBase = 16;
+constexpr int kScanTile = 2048;      // keys a block of the sort's scan takes
+constexpr size_t sort_counts(size_t nkeys) { return 2 * nkeys + (nkeys + kScanTile - 1) / kScanTile; }
 inline int bins_per_cell(long long np, int M) { return np >= 8192LL * M ? 4 : 1; }
 // most threads per block of the marker kernels that split their range by warps
 constexpr int kSweepThreads = 256;
@@ -181,11 +182,11 @@ struct SortRun {
     int M, nbins;
     float taup;             // dt / dx times the bins per cell
     PartPtrs src, dst;
-    int32_t *counts;        // 2 M nbins: histogram, then cursors
+    int32_t *counts;        // sort_counts(M nbins): histogram, cursors, tile totals
 };
 int launch_sort_ens(int fp32, const SortRun *runs, int nruns, int grid_x, cudaStream_t s);
 int launch_sort(int fp32, long long np, int M, double tau, int per, PartPtrs src, PartPtrs dst,
-                int32_t *counts, int grid, int block, cudaStream_t s);
+                int32_t *counts, int num_sms, cudaStream_t s);
 
 // ---------------------------------------------------------------- grid
 // FP32 form, subsystem I: the last field increment must be below this fraction of

@@ -28,16 +28,6 @@
 
 namespace pic {
 
-// Contiguous chunk of markers owned by one block (a multiple of 32, so every
-// warp's lanes see consecutive, sorted markers).
-__device__ __forceinline__ void block_chunk(long long np, long long &beg, long long &end)
-{
-    long long chunk = (np + gridDim.x - 1) / gridDim.x;
-    chunk = (chunk + 31) & ~31LL;
-    beg = (long long)blockIdx.x * chunk;
-    end = beg + chunk < np ? beg + chunk : np;
-}
-
 template <int K, typename R, int ACC>
 __global__ void __launch_bounds__(SweepShape<R, K>::threads1, SweepShape<R, K>::blocks1) k_sweep1(Sweep1Args A)
 {
@@ -833,7 +823,7 @@ int launch_store_ordered(int fp32, long long np, int M, double dx, PartPtrs P, i
 // p_new are not carried (each step's first sweep or warm start writes them
 // before they are read, and delta is all zero where the iteration starts from
 // it).  Atomics are aggregated per warp over equal keys.
-// counts: 2 * nkeys int32 (histogram, then cursors).
+// counts: sort_counts(nkeys) int32 (histogram, cursors, the scan's tile totals).
 // ---------------------------------------------------------------------------
 template <typename R>
 __device__ __forceinline__ int sort_key(int c, R p, float taup, int nbins)
@@ -847,13 +837,25 @@ __device__ __forceinline__ int sort_key(int c, R p, float taup, int nbins)
 // nearly sorted (they were sorted a few steps ago), so the blocks running at the
 // same time then touch different keys' counters; in a grid-stride order every
 // block would work on the same few cells at once and serialise on their counters.
-// chunk [beg, end) of block b among nb blocks (a multiple of 32 markers)
+// chunk [beg, end) of block b among nb blocks (a multiple of 128 markers)
 __device__ __forceinline__ void chunk_of(long long np, int b, int nb, long long &beg, long long &end)
 {
     long long chunk = (np + nb - 1) / nb;
-    chunk = (chunk + 31) & ~31LL;
+    chunk = (chunk + 127) & ~127LL;
     beg = (long long)b * chunk;
     end = beg + chunk < np ? beg + chunk : np;
+}
+
+// four consecutive markers' numbers (none beyond end)
+template <typename T>
+__device__ __forceinline__ void load4_to(const T *q, long long a, long long end, T (&v)[4])
+{
+    if (a + 4 <= end) {
+        load4(q + a, v);
+    } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = a + u < end ? q[a + u] : T(0);
+    }
 }
 
 template <typename R>
@@ -862,12 +864,18 @@ __device__ __forceinline__ void hist_range(long long beg, long long end, float t
 {
     const R *ps = static_cast<const R *>(S.p);
     const int lane = threadIdx.x & 31;
-    for (long long base = beg; base < end; base += blockDim.x) {
-        const long long a = base + threadIdx.x;
-        const bool act = a < end;
-        const int key = act ? sort_key(S.cell[a], ps[a], tau, nbins) : -1;
-        const unsigned grp = __match_any_sync(0xffffffffu, key);
-        if (act && lane == __ffs(grp) - 1) atomicAdd(&counts[key], __popc(grp));
+    for (long long base = beg; base < end; base += 4 * blockDim.x) {
+        const long long a = base + 4 * threadIdx.x;
+        int c[4];
+        R p[4];
+        load4_to(S.cell, a, end, c);
+        load4_to(ps, a, end, p);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int key = a + u < end ? sort_key(c[u], p[u], tau, nbins) : -1;
+            const unsigned grp = __match_any_sync(0xffffffffu, key);
+            if (key >= 0 && lane == __ffs(grp) - 1) atomicAdd(&counts[key], __popc(grp));
+        }
     }
 }
 
@@ -875,31 +883,68 @@ template <typename R>
 __global__ void __launch_bounds__(256) k_hist(long long np, float tau, int nbins, PartPtrs S, int32_t *counts)
 {
     long long beg, end;
-    block_chunk(np, beg, end);
+    chunk_of(np, blockIdx.x, gridDim.x, beg, end);
     hist_range<R>(beg, end, tau, nbins, S, counts);
 }
 
-__device__ __forceinline__ void scan_block(int nkeys, int32_t *counts)
+// Exclusive scan of nkeys counts into the cursors behind them: a block a tile of
+// kScanTile keys sums it into the totals behind the cursors, then a block a tile adds the
+// totals before its own and scans it.  (One block with a range of keys a thread, whose
+// loads are strided, took 227 us for 131072 keys.)
+__device__ __forceinline__ int block_sum(int v)
 {
-    // exclusive scan of nkeys counts into cursors (single block)
-    __shared__ int s_part[1024];
-    const int per = (nkeys + blockDim.x - 1) / blockDim.x;
-    const int lo = threadIdx.x * per, hi = min(nkeys, lo + per);
-    int s = 0;
-    for (int i = lo; i < hi; ++i) s += counts[i];
-    s_part[threadIdx.x] = s;
+    __shared__ int s_part[32];
+    v = __reduce_add_sync(0xffffffffu, v);
     __syncthreads();
-    for (int off = 1; off < (int)blockDim.x; off <<= 1) {
-        const int v = threadIdx.x >= (unsigned)off ? s_part[threadIdx.x - off] : 0;
-        __syncthreads();
-        s_part[threadIdx.x] += v;
-        __syncthreads();
-    }
-    int run = s_part[threadIdx.x] - s;     // exclusive prefix of this thread's range
-    for (int i = lo; i < hi; ++i) { const int v = counts[i]; counts[nkeys + i] = run; run += v; }
+    if ((threadIdx.x & 31) == 0) s_part[threadIdx.x >> 5] = v;
+    __syncthreads();
+    int t = 0;
+    for (int w = 0; w < (int)blockDim.x / 32; ++w) t += s_part[w];
+    return t;
 }
 
-__global__ void __launch_bounds__(1024) k_scan(int nkeys, int32_t *counts) { scan_block(nkeys, counts); }
+__device__ __forceinline__ void scan_totals(int nkeys, int tile, int32_t *counts)
+{
+    int s = 0;
+    const int end = min(nkeys, (tile + 1) * kScanTile);
+    for (int i = tile * kScanTile + threadIdx.x; i < end; i += blockDim.x) s += counts[i];
+    s = block_sum(s);
+    if (threadIdx.x == 0) counts[2 * (size_t)nkeys + tile] = s;
+}
+
+__device__ __forceinline__ void scan_tile(int nkeys, int tile, int32_t *counts)
+{
+    __shared__ int s_warp[32];
+    int before = 0;
+    for (int i = threadIdx.x; i < tile; i += blockDim.x) before += counts[2 * (size_t)nkeys + i];
+    before = block_sum(before);
+    constexpr int kPer = kScanTile / 256;      // consecutive keys a thread
+    const int lane = threadIdx.x & 31, lo = tile * kScanTile + threadIdx.x * kPer;
+    int v[kPer], s = 0;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        v[i] = lo + i < nkeys ? counts[lo + i] : 0;
+        s += v[i];
+    }
+    int incl = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += u;
+    }
+    if (lane == 31) s_warp[threadIdx.x >> 5] = incl;
+    __syncthreads();
+    int run = before + incl - s;
+    for (int w = 0; w < (int)threadIdx.x / 32; ++w) run += s_warp[w];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        if (lo + i < nkeys) counts[nkeys + lo + i] = run;
+        run += v[i];
+    }
+}
+
+__global__ void __launch_bounds__(256) k_scan_totals(int nkeys, int32_t *counts) { scan_totals(nkeys, blockIdx.x, counts); }
+__global__ void __launch_bounds__(256) k_scan(int nkeys, int32_t *counts) { scan_tile(nkeys, blockIdx.x, counts); }
 
 template <typename R>
 __device__ __forceinline__ void scatter_range(long long beg, long long end, float tau, int nbins, const PartPtrs &S,
@@ -910,37 +955,33 @@ __device__ __forceinline__ void scatter_range(long long beg, long long end, floa
     R *td = static_cast<R *>(D.t);
     R *pd = static_cast<R *>(D.p);
     const int lane = threadIdx.x & 31;
-    // kSortU markers a thread per pass: their cursor atomics are independent, so
+    // four markers a thread per pass: their loads and cursor atomics are independent, so
     // the warp waits for the returned slots once per pass instead of once a marker
-    constexpr int kSortU = 4;
-    for (long long base = beg; base < end; base += kSortU * (long long)blockDim.x) {
-        int c[kSortU], key[kSortU], first[kSortU];
-        R p[kSortU];
-        unsigned grp[kSortU];
+    for (long long base = beg; base < end; base += 4 * blockDim.x) {
+        const long long a = base + 4 * threadIdx.x;
+        int c[4], id[4], key[4], first[4];
+        R p[4], t[4];
+        unsigned grp[4];
+        load4_to(S.cell, a, end, c);
+        load4_to(ps, a, end, p);
+        load4_to(ts, a, end, t);
+        load4_to(S.id, a, end, id);
 #pragma unroll
-        for (int u = 0; u < kSortU; ++u) {
-            const long long a = base + u * (long long)blockDim.x + threadIdx.x;
-            const bool act = a < end;
-            c[u] = act ? S.cell[a] : 0;
-            p[u] = act ? ps[a] : R(0);
-            key[u] = act ? sort_key(c[u], p[u], tau, nbins) : -1;
-        }
-#pragma unroll
-        for (int u = 0; u < kSortU; ++u) {
+        for (int u = 0; u < 4; ++u) {
+            key[u] = a + u < end ? sort_key(c[u], p[u], tau, nbins) : -1;
             grp[u] = __match_any_sync(0xffffffffu, key[u]);
             first[u] = 0;
             if (key[u] >= 0 && lane == __ffs(grp[u]) - 1) first[u] = atomicAdd(&cursor[key[u]], __popc(grp[u]));
         }
 #pragma unroll
-        for (int u = 0; u < kSortU; ++u) {
-            const long long a = base + u * (long long)blockDim.x + threadIdx.x;
+        for (int u = 0; u < 4; ++u) {
             const int f = __shfl_sync(0xffffffffu, first[u], __ffs(grp[u]) - 1);
             if (key[u] < 0) continue;
             const long long j = (long long)f + __popc(grp[u] & ((1u << lane) - 1u));
             D.cell[j] = c[u];
-            td[j] = ts[a];
+            td[j] = t[u];
             pd[j] = p[u];
-            D.id[j] = S.id[a];
+            D.id[j] = id[u];
         }
     }
 }
@@ -950,16 +991,16 @@ __global__ void __launch_bounds__(256) k_scatter(long long np, float tau, int nb
                                                  int32_t *cursor)
 {
     long long beg, end;
-    block_chunk(np, beg, end);
+    chunk_of(np, blockIdx.x, gridDim.x, beg, end);
     scatter_range<R>(beg, end, tau, nbins, S, D, cursor);
 }
 
 // Batched sorts (ensembles): block row y = run, its counts zeroed, histogrammed,
-// scanned (one block a run) and scattered in four launches for all runs due.
+// scanned and scattered in five launches for all runs due.
 __global__ void __launch_bounds__(256) k_sort_zero_ens(const SortRun *runs)
 {
     const SortRun &r = runs[blockIdx.y];
-    const int n = 2 * r.M * r.nbins;
+    const int n = r.M * r.nbins;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) r.counts[i] = 0;
 }
 
@@ -972,10 +1013,18 @@ __global__ void __launch_bounds__(256) k_hist_ens(const SortRun *runs)
     hist_range<R>(beg, end, r.taup, r.nbins, r.src, r.counts);
 }
 
-__global__ void __launch_bounds__(1024) k_scan_ens(const SortRun *runs)
+__global__ void __launch_bounds__(256) k_scan_totals_ens(const SortRun *runs)
 {
-    const SortRun &r = runs[blockIdx.x];
-    scan_block(r.M * r.nbins, r.counts);
+    const SortRun &r = runs[blockIdx.y];
+    for (int t = blockIdx.x; t * kScanTile < r.M * r.nbins; t += gridDim.x) scan_totals(r.M * r.nbins, t, r.counts);
+}
+__global__ void __launch_bounds__(256) k_scan_ens(const SortRun *runs)
+{
+    const SortRun &r = runs[blockIdx.y];
+    for (int t = blockIdx.x; t * kScanTile < r.M * r.nbins; t += gridDim.x) {
+        scan_tile(r.M * r.nbins, t, r.counts);
+        __syncthreads();
+    }
 }
 
 template <typename R>
@@ -994,24 +1043,31 @@ int launch_sort_ens(int fp32, const SortRun *runs, int nruns, int grid_x, cudaSt
     k_sort_zero_ens<<<g, 256, 0, s>>>(runs);
     if (fp32) k_hist_ens<float><<<g, 256, 0, s>>>(runs);
     else k_hist_ens<double><<<g, 256, 0, s>>>(runs);
-    k_scan_ens<<<nruns, 1024, 0, s>>>(runs);
+    k_scan_totals_ens<<<dim3(8, nruns), 256, 0, s>>>(runs);
+    k_scan_ens<<<dim3(8, nruns), 256, 0, s>>>(runs);
     if (fp32) k_scatter_ens<float><<<g, 256, 0, s>>>(runs);
     else k_scatter_ens<double><<<g, 256, 0, s>>>(runs);
     return 0;
 }
 
 int launch_sort(int fp32, long long np, int M, double tau, int per, PartPtrs src, PartPtrs dst,
-                int32_t *counts, int grid, int block, cudaStream_t s)
+                int32_t *counts, int num_sms, cudaStream_t s)
 {
+    // more blocks than fit: their chunks are short, so the blocks running together write a
+    // narrow range of the sorted order (2e7 float markers: scatter 180 us at 4 blocks a SM,
+    // 176 at 8, 150 at 16; histogram 41, 32, 32)
+    const int grid = 16 * num_sms;
     const int nbins = kVelBinsBase * per;
     const int nkeys = M * nbins;
     const float taup = (float)(tau * per);
-    if (cudaMemsetAsync(counts, 0, sizeof(int32_t) * 2 * (size_t)nkeys, s) != cudaSuccess) return 1;
-    if (fp32) k_hist<float><<<grid, block, 0, s>>>(np, taup, nbins, src, counts);
-    else k_hist<double><<<grid, block, 0, s>>>(np, taup, nbins, src, counts);
-    k_scan<<<1, 1024, 0, s>>>(nkeys, counts);
-    if (fp32) k_scatter<float><<<grid, block, 0, s>>>(np, taup, nbins, src, dst, counts + nkeys);
-    else k_scatter<double><<<grid, block, 0, s>>>(np, taup, nbins, src, dst, counts + nkeys);
+    if (cudaMemsetAsync(counts, 0, sizeof(int32_t) * (size_t)nkeys, s) != cudaSuccess) return 1;
+    if (fp32) k_hist<float><<<grid, 256, 0, s>>>(np, taup, nbins, src, counts);
+    else k_hist<double><<<grid, 256, 0, s>>>(np, taup, nbins, src, counts);
+    const int tiles = (nkeys + kScanTile - 1) / kScanTile;
+    k_scan_totals<<<tiles, 256, 0, s>>>(nkeys, counts);
+    k_scan<<<tiles, 256, 0, s>>>(nkeys, counts);
+    if (fp32) k_scatter<float><<<grid, 256, 0, s>>>(np, taup, nbins, src, dst, counts + nkeys);
+    else k_scatter<double><<<grid, 256, 0, s>>>(np, taup, nbins, src, dst, counts + nkeys);
     return 0;
 }
 

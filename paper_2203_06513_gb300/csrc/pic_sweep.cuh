@@ -610,7 +610,29 @@ __device__ __forceinline__ void finalize1_range(long long np, int M, const PartP
     R *pp = static_cast<R *>(P.p);
     R *dp = static_cast<R *>(P.delta);
     const R *pnp = static_cast<const R *>(P.pnew);
-    for (long long a = a0; a < np; a += stride) {
+    // four markers a thread and pass: the kernel only moves memory (28 bytes a marker in the
+    // float form), and one marker's loads did not keep enough of it in flight (2e7 float
+    // markers: 162 us one at a time, 80 us so, 7.0 TB/s)
+    for (long long i = a0; i < np / 4; i += stride) {
+        const int4 c = reinterpret_cast<const int4 *>(P.cell)[i];
+        R t[4], d[4], p[4];
+        load4(tp + 4 * i, t);
+        load4(dp + 4 * i, d);
+        load4(pnp + 4 * i, p);
+        int g[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            int n;
+            path_end(t[j], d[j], n, t[j]);
+            g[j] = wrap_cell(g[j] + n, M);
+            d[j] = R(0);
+        }
+        reinterpret_cast<int4 *>(P.cell)[i] = make_int4(g[0], g[1], g[2], g[3]);
+        store4(tp + 4 * i, t);
+        store4(pp + 4 * i, p);
+        if (zero_delta) store4(dp + 4 * i, d);
+    }
+    for (long long a = (np & ~3LL) + a0; a < np; a += stride) {
         int n;
         R v;
         path_end(tp[a], dp[a], n, v);

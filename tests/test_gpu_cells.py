@@ -25,7 +25,9 @@ SHAPES = [(33, 3, 2001, 0.05, 0.1, 0, True),
           (9, 4, 1000, 0.5, 0.5, 1, False),
           (250, 3, 3000, 0.3, 0.8, 0, True),     # paths over several cells, unsorted
           (127, 5, 31, 0.1, 0.2, 0, False),
-          (64, 4, 20011, 0.05, 0.1, 2, True)]
+          (64, 4, 20011, 0.05, 0.1, 2, True),
+          (128, 3, 3002, 0.05, 0.1, 1, False),   # one tile of sort keys, then one and a few
+          (129, 2, 3003, 0.05, 0.1, 1, True)]
 
 
 def _check(st, s, L, tol_x, tol):
