@@ -461,7 +461,6 @@ extern "C" int pic_init_split(const pic_config *cfg, const pic_arrays *in, int32
         cudaMemcpyAsync(h->spx, in->sx, np * sizeof(double), k, h->stream);
         cudaMemcpyAsync(h->spy, in->sy, np * sizeof(double), k, h->stream);
         cudaMemcpyAsync(h->spz, in->sz, np * sizeof(double), k, h->stream);
-        if (spin_optin(h->M)) return bail(fail(h, PIC_ERR_CUDA, "spin deposit shared-memory opt-in failed"));
     }
     {
         const size_t pa = coef_pad(h->fp32, c.degree + 1), pe = coef_pad(h->fp32, c.degree);
@@ -648,6 +647,27 @@ static SpinArgs spin_args(pic_handle *h)
     a.dy = h->sdy; a.dz = h->sdz;
     a.acc = h->diag + 6;
     return a;
+}
+
+// Zeeman source of subsystem II's right side (constant during its loop: x, s frozen).
+static int spin_source(pic_handle *h, cudaStream_t s)
+{
+    const SpinArgs sa = spin_args(h);
+    const size_t bytes = sizeof(double) * (size_t)h->M * h->K;
+    CK(cudaMemsetAsync(h->sdy, 0, bytes, s));
+    CK(cudaMemsetAsync(h->sdz, 0, bytes, s));
+    if (launch_spin_deposit(sa, particle_grid(h), s)) return fail(h, PIC_ERR_INVALID, "bad degree");
+    if (!h->reduce) {
+        launch_spin_source(h->M, h->K, h->cfg.dt * h->cfg.hbar * h->cfg.weight / h->dx, h->sdy, h->sdz, h->by, h->bz, s);
+        return PIC_OK;
+    }
+    // split runs sum the nodes over the processes
+    int rc;
+    launch_moments_to_nodes(h->M, h->K - 1, false, h->cfg.weight, h->sdy, h->sy[0], s);
+    launch_moments_to_nodes(h->M, h->K - 1, false, h->cfg.weight, h->sdz, h->sz[0], s);
+    if ((rc = reduce(h, PIC_REDUCE_SUM, h->sy[0], h->M)) || (rc = reduce(h, PIC_REDUCE_SUM, h->sz[0], h->M))) return rc;
+    launch_spin_rhs(h->M, h->dx, h->cfg.dt, h->cfg.hbar, h->sy[0], h->sz[0], h->by, h->bz, s);
+    return PIC_OK;
 }
 
 // Subsystem III: the exact rotation of every spin (markers and fields frozen).
@@ -837,16 +857,9 @@ static int substep2(pic_handle *h, int *iters)
     launch_prep2(desc, h->stream);
     CKL_N("launch_prep2");
     if (h->cfg.hbar != 0.0) {
-        // Zeeman source of the right side (constant during the loop: x, s frozen)
-        SpinArgs sa = spin_args(h);
-        CK(cudaMemsetAsync(h->sdy, 0, sizeof(double) * h->M, h->stream));
-        CK(cudaMemsetAsync(h->sdz, 0, sizeof(double) * h->M, h->stream));
-        if (launch_spin_deposit(sa, particle_grid(h), h->stream)) return fail(h, PIC_ERR_INVALID, "bad degree");
-        CKL_N("launch_spin_deposit");
-        if ((rc = reduce(h, PIC_REDUCE_SUM, h->sdy, h->M)) || (rc = reduce(h, PIC_REDUCE_SUM, h->sdz, h->M)))
-            return rc;
-        launch_spin_rhs(h->M, h->dx, h->cfg.dt, h->cfg.hbar, h->sdy, h->sdz, h->by, h->bz, h->stream);
-        CKL_N("launch_spin_rhs");
+        if ((rc = spin_source(h, h->stream))) return rc;
+        CKL_N("spin source");
+        ++h->launches;
     }
     Sweep2Args a = make_sweep2_args(h);
     ConvArgs c = make_conv2_args(h);
@@ -900,10 +913,10 @@ extern "C" int pic_substep(pic_handle *h, int32_t which, int32_t *iters)
 // decision on the device (no host round trip per sweep).  The markers' buffers
 // enter the kernel arguments, so there is one graph per marker copy (the sort
 // alternates them).  Host loops are kept for split runs (their reductions call
-// back into the host), spin runs, kernel timing and PIC_DEBUG_SYNC.
+// back into the host), kernel timing and PIC_DEBUG_SYNC.
 static bool graph_eligible(const pic_handle *h)
 {
-    return !h->reduce && h->cfg.hbar == 0.0 && !h->timing && !debug_sync() &&
+    return !h->reduce && !h->timing && !debug_sync() &&
            (h->cfg.warm_start != PIC_WARM_MLP || h->mlp) && getenv("PIC_NO_GRAPH") == nullptr;
 }
 
@@ -952,6 +965,11 @@ static int seg_sub2_head(pic_handle *h, cudaStream_t s, int *nodes)
 {
     launch_prep2(handle_desc(h), s);
     *nodes += 1;
+    if (h->cfg.hbar != 0.0) {
+        int rc;
+        if ((rc = spin_source(h, s))) return rc;
+        *nodes += 2;
+    }
     return PIC_OK;
 }
 
@@ -959,6 +977,10 @@ static int seg_sub2_tail(pic_handle *h, cudaStream_t s, int *nodes)
 {
     launch_commit(handle_desc(h), 2, s);
     *nodes += 1;
+    if (h->cfg.hbar != 0.0) {      // Lie--Trotter steps: subsystem III ends the step
+        if (launch_spin_rotate(spin_args(h), particle_grid(h), s)) return fail(h, PIC_ERR_INVALID, "bad degree");
+        *nodes += 1;
+    }
     return PIC_OK;
 }
 

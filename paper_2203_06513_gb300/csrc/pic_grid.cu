@@ -594,7 +594,20 @@ __global__ void k_spin_rhs(int M, double dx, double c, const double *dy, const d
     bz[j] += c * (dy[j] - dy[jp]) / dx;
 }
 
+__global__ void k_spin_source(int M, int K, double c, const double *mom_y, const double *mom_z, double *by, double *bz)
+{
+    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q < 2 * M) pic::spin_source_at(M, K, c, mom_y, mom_z, by, bz, q % M, q / M);
+}
+
 namespace pic {
+int launch_spin_source(int M, int K, double c, const double *mom_y, const double *mom_z, double *by, double *bz,
+                       cudaStream_t s)
+{
+    k_spin_source<<<(2 * M + 63) / 64, 64, 0, s>>>(M, K, c, mom_y, mom_z, by, bz);
+    return 0;
+}
+
 int launch_spin_rhs(int M, double dx, double dt, double hbar, const double *dy, const double *dz, double *by,
                     double *bz, cudaStream_t s)
 {

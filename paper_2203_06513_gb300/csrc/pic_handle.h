@@ -35,7 +35,7 @@ struct pic_handle {
     void *a0 = nullptr;             // start-point cache of a fixed-point loop (4 reals a marker; FP64 form)
     // spin (hbar != 0, FP64 form): components in caller order, and the spin deposits
     double *spx = nullptr, *spy = nullptr, *spz = nullptr;
-    double *sdy = nullptr, *sdz = nullptr;      // M x K each (moments, or M nodes)
+    double *sdy = nullptr, *sdz = nullptr;      // spin moments, M x K each
 
     // split run: the markers of one plasma spread over several processes; marker
     // sums and maxima go through this reduction (NULL: all markers are here)

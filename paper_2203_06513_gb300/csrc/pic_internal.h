@@ -247,10 +247,11 @@ struct SpinArgs {
     PartPtrs P;                 // markers in stored order (cell, t as double, id)
     const double *ay, *az;
     double *sx, *sy, *sz;
-    double *dy, *dz;            // spin deposit outputs (M each)
+    double *dy, *dz;            // spin deposit outputs (M x K moments each)
     double *acc;                // Zeeman energy sum (without hbar)
 };
-// d_y,i = sum_a w s_y,a Lambda^1_i(x_a), d_z likewise (Lambda_1(X)^T W S of subsystem II)
+// moments sum_a s_y,a v_a^m per cell, s_z likewise: d_y,i = sum_a w s_y,a Lambda^1_i(x_a) follows
+// from them (Lambda_1(X)^T W S of subsystem II)
 int launch_spin_deposit(const SpinArgs &a, int grid, cudaStream_t s);
 // subsystem III: exact rotation of every spin
 int launch_spin_rotate(const SpinArgs &a, int grid, cudaStream_t s);
@@ -259,8 +260,9 @@ int launch_spin_energy(const SpinArgs &a, int grid, cudaStream_t s);
 // b_y -= dt hbar (G^T d_z), b_z += dt hbar (G^T d_y), (G^T v)_j = (v_j - v_{j+1}) / dx
 int launch_spin_rhs(int M, double dx, double dt, double hbar, const double *dy, const double *dz,
                     double *by, double *bz, cudaStream_t s);
-// raise the spin deposit's dynamic shared-memory limit for a grid of M cells
-int spin_optin(int M);
+// the same from the moments
+int launch_spin_source(int M, int K, double c, const double *mom_y, const double *mom_z, double *by, double *bz,
+                       cudaStream_t s);
 
 // split runs: buf[0..2] = (max increment, numeric bit, timeout bit) of the control block
 int launch_split_pack(const DevCtrl *c, double *buf, cudaStream_t s);

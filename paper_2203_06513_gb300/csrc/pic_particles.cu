@@ -24,6 +24,7 @@
 
 #include "pic_internal.h"
 #include "pic_poly.cuh"
+#include "pic_solve.cuh"
 #include "pic_sweep.cuh"
 
 namespace pic {
@@ -434,38 +435,75 @@ __device__ __forceinline__ void spin_field_grad(const SpinArgs &A, int c, double
     Z /= A.dx;
 }
 
+// Moments s_y v^m, s_z v^m (m < K) per cell: windows of cells in registers as in k_charge
+// (adding each marker's 2 K basis values to nodes in shared memory, where a double addition
+// is a compare-and-swap loop, took 36 us for 1e4 markers).
 template <int K>
-__global__ void __launch_bounds__(256) k_spin_deposit(SpinArgs A)
+__global__ void __launch_bounds__(kSweepThreads) k_spin_deposit(SpinArgs A)
 {
-    extern __shared__ __align__(16) double s_dep[];
-    double *sy = s_dep, *sz = s_dep + A.M;
-    for (int i = threadIdx.x; i < 2 * A.M; i += blockDim.x) s_dep[i] = 0.0;
-    __syncthreads();
-    const double *tp = static_cast<const double *>(A.P.t);
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long a = (long long)blockIdx.x * blockDim.x + threadIdx.x; a < A.np; a += stride) {
-        const int c = A.P.cell[a];
-        const int id = A.P.id[a];
-        double v[K];
-        bspline_vals<K - 1, double>(tp[a] + 0.5, v);
-        const double wy = A.w * A.sy[id], wz = A.w * A.sz[id];
+    const int32_t *__restrict__ cp = A.P.cell;
+    const double *__restrict__ vp = static_cast<const double *>(A.P.t);
+    const int lane = threadIdx.x & 31, M = A.M;
+    long long wb, we;
+    grid_warp_chunk(A.np, wb, we);
+    if (wb >= we) return;
+    MomentWindow<kWin2, K, AccNative<double>> wy, wz;
+    wy.clear();
+    wz.clear();
+    int base = cp[wb];
+    unsigned used = 0u;
+    for (long long s = wb; s < we; s += 32) {
+        const long long a = s + lane;
+        const bool act = a < we;
+        const unsigned amask = __ballot_sync(0xffffffffu, act);
+        const int c = act ? cp[a] : 0;
+        const double v = act ? vp[a] : 0.0;
+        const int id = act ? A.P.id[a] : 0;
+        double y[K], z[K];
+        y[0] = act ? A.sy[id] : 0.0;
+        z[0] = act ? A.sz[id] : 0.0;
 #pragma unroll
-        for (int r = 0; r < K; ++r) {
-            const int i = wrap_cell(c - r, A.M);
-            atomicAdd(&sy[i], wy * v[r]);
-            atomicAdd(&sz[i], wz * v[r]);
+        for (int m = 1; m < K; ++m) {
+            y[m] = y[m - 1] * v;
+            z[m] = z[m - 1] * v;
+        }
+        int rel = rel_cell(c, base, M);
+        bool in = act && (unsigned)rel < (unsigned)kWin2;
+        if (__popc(__ballot_sync(0xffffffffu, act && !in)) > kWindowMisses) {
+            int off = window_move<kWin2>(rel, rel, act, amask);
+            if (off > 0 && off < kWin2) {
+                for (; off > 0; --off) {
+                    wy.shift(A.dy, base, used);
+                    wz.shift(A.dz, base, used);
+                    used >>= 1;
+                    base = base + 1 == M ? 0 : base + 1;
+                }
+            } else if (off != 0) {
+                wy.flush(A.dy, base, used, M);
+                wz.flush(A.dz, base, used, M);
+                used = 0u;
+                base = wrap_cell(base + off, M);
+            }
+            rel = rel_cell(c, base, M);
+            in = act && (unsigned)rel < (unsigned)kWin2;
+        }
+        const unsigned mask = __reduce_or_sync(0xffffffffu, in ? 1u << rel : 0u);
+        used |= mask;
+        wy.add(mask, in ? rel : -1, y);
+        wz.add(mask, in ? rel : -1, z);
+        if (act && !in) {
+#pragma unroll
+            for (int m = 0; m < K; ++m) {
+                atomicAdd(&A.dy[(size_t)c * K + m], y[m]);
+                atomicAdd(&A.dz[(size_t)c * K + m], z[m]);
+            }
         }
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < A.M; i += blockDim.x) {
-        if (sy[i] != 0.0) atomicAdd(&A.dy[i], sy[i]);
-        if (sz[i] != 0.0) atomicAdd(&A.dz[i], sz[i]);
-    }
+    wy.flush(A.dy, base, used, M);
+    wz.flush(A.dz, base, used, M);
 }
 
-// Subsystem III (Eq. spin_rodrigue): s <- s + sin(dt|r|)/|r| (r x s)
-//                                         + (1/2) (sin(dt|r|/2)/(|r|/2))^2 r x (r x s),
-// r = (0, Z, -Y), Y = dA_y/dx, Z = dA_z/dx at the marker.
+// Subsystem III
 template <int K>
 __global__ void __launch_bounds__(256) k_spin_rotate(SpinArgs A)
 {
@@ -475,24 +513,7 @@ __global__ void __launch_bounds__(256) k_spin_rotate(SpinArgs A)
         const int id = A.P.id[a];
         double Y, Z;
         spin_field_grad<K>(A, A.P.cell[a], tp[a], Y, Z);
-        const double r1 = Z, r2 = -Y;
-        const double nr = sqrt(r1 * r1 + r2 * r2);
-        const double s0 = A.sx[id], s1 = A.sy[id], s2 = A.sz[id];
-        // c1 = r x s, c2 = r x c1, with r0 = 0
-        const double c1x = r1 * s2 - r2 * s1, c1y = r2 * s0, c1z = -r1 * s0;
-        const double c2x = r1 * c1z - r2 * c1y, c2y = r2 * c1x, c2z = -r1 * c1x;
-        double f1, f2;
-        if (nr > 0.0) {
-            f1 = sin(A.dt * nr) / nr;
-            const double hh = sin(0.5 * A.dt * nr) / (0.5 * nr);
-            f2 = 0.5 * hh * hh;
-        } else {
-            f1 = A.dt;
-            f2 = 0.5 * A.dt * A.dt;
-        }
-        A.sx[id] = s0 + f1 * c1x + f2 * c2x;
-        A.sy[id] = s1 + f1 * c1y + f2 * c2y;
-        A.sz[id] = s2 + f1 * c1z + f2 * c2z;
+        spin_turn(A.dt, Y, Z, A.sx[id], A.sy[id], A.sz[id]);
     }
 }
 
@@ -512,25 +533,27 @@ __global__ void __launch_bounds__(256) k_spin_energy(SpinArgs A)
     block_sum_to(A.acc, acc, s_red);
 }
 
-#define PIC_SPIN_LAUNCH(NAME, SMEM)                                                      \
+#define PIC_SPIN_LAUNCH(NAME)                                                            \
     switch (a.K) {                                                                       \
-    case 2: NAME<2><<<grid, 256, SMEM, s>>>(a); break;                                   \
-    case 3: NAME<3><<<grid, 256, SMEM, s>>>(a); break;                                   \
-    case 4: NAME<4><<<grid, 256, SMEM, s>>>(a); break;                                   \
-    case 5: NAME<5><<<grid, 256, SMEM, s>>>(a); break;                                   \
+    case 2: NAME<2><<<grid, 256, 0, s>>>(a); break;                                      \
+    case 3: NAME<3><<<grid, 256, 0, s>>>(a); break;                                      \
+    case 4: NAME<4><<<grid, 256, 0, s>>>(a); break;                                      \
+    case 5: NAME<5><<<grid, 256, 0, s>>>(a); break;                                      \
     default: return 1;                                                                   \
     }                                                                                    \
     return 0;
 
 int launch_spin_deposit(const SpinArgs &a, int grid, cudaStream_t s)
 {
-    const size_t smem = 2 * (size_t)a.M * sizeof(double);
-    PIC_SPIN_LAUNCH(k_spin_deposit, smem)
+    // at least 128 markers a warp: a warp's windows cost it a reduction of their cells
+    const int most = (int)std::max<long long>(1, a.np / (128 * kSweepWarps));
+    if (grid > most) grid = most;
+    PIC_SPIN_LAUNCH(k_spin_deposit)
 }
 
-int launch_spin_rotate(const SpinArgs &a, int grid, cudaStream_t s) { PIC_SPIN_LAUNCH(k_spin_rotate, 0) }
+int launch_spin_rotate(const SpinArgs &a, int grid, cudaStream_t s) { PIC_SPIN_LAUNCH(k_spin_rotate) }
 
-int launch_spin_energy(const SpinArgs &a, int grid, cudaStream_t s) { PIC_SPIN_LAUNCH(k_spin_energy, 0) }
+int launch_spin_energy(const SpinArgs &a, int grid, cudaStream_t s) { PIC_SPIN_LAUNCH(k_spin_energy) }
 
 #undef PIC_SPIN_LAUNCH
 
@@ -1194,28 +1217,6 @@ int launch_finalize1_ens(int fp32, const RunDesc *R, int nruns, int grid_x, cuda
 {
     if (fp32) k_finalize1_ens<float><<<dim3(grid_x, nruns), 256, 0, s>>>(R);
     else k_finalize1_ens<double><<<dim3(grid_x, nruns), 256, 0, s>>>(R);
-    return 0;
-}
-
-static int set_attrs_spin(size_t smem)
-{
-    int rc = 0;
-    rc |= cudaFuncSetAttribute(k_spin_deposit<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess;
-    rc |= cudaFuncSetAttribute(k_spin_deposit<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess;
-    rc |= cudaFuncSetAttribute(k_spin_deposit<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess;
-    rc |= cudaFuncSetAttribute(k_spin_deposit<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess;
-    return rc;
-}
-
-int spin_optin(int M)
-{
-    static std::mutex mu;
-    static size_t have = 0;
-    std::lock_guard<std::mutex> lock(mu);
-    const size_t need = 2 * (size_t)M * sizeof(double);
-    if (need <= have) return 0;
-    if (set_attrs_spin(need)) return 1;
-    have = need;
     return 0;
 }
 

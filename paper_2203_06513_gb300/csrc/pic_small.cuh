@@ -104,21 +104,7 @@ __device__ __forceinline__ bool loop_decision(const ConvArgs &C, unsigned long l
     return s_stop != 0;
 }
 
-// Zeeman source of subsystem II: b_y -= dt hbar (G^T d_z)_j, b_z += dt hbar (G^T d_y)_j,
-// d = Lambda_1(X)^T W S from the moments s v^m of the markers (degree K - 1).
-__device__ __forceinline__ void spin_source_at(int j, int comp, const SmallArgs &A)
-{
-    const int M = A.d.M, K = A.d.K, jp = j + 1 == M ? 0 : j + 1;
-    const double c = A.d.dt * A.hbar * A.w / A.d.dx;
-    const double *sm = comp ? A.sm_y : A.sm_z;
-    const double v = c * (node_value(M, K - 1, false, sm, j) - node_value(M, K - 1, false, sm, jp));
-    if (comp) A.d.bz[j] += v;
-    else A.d.by[j] -= v;
-}
-
-// Subsystem III (Eq. spin_rodrigue): s <- s + sin(dt|r|)/|r| (r x s)
-// + 2 (sin(dt|r|/2)/|r|)^2 r x (r x s), r = (0, dA_z/dx, -dA_y/dx), from the coefficients of
-// a^{n+1} in the marker's cell.
+// Subsystem III from the coefficients of a^{n+1} in the marker's cell.
 template <int K>
 __device__ __forceinline__ void spin_rotate_one(const SmallArgs &A, const double (&cy)[K + 1], const double (&cz)[K + 1],
                                                 double v, int id)
@@ -129,22 +115,7 @@ __device__ __forceinline__ void spin_rotate_one(const SmallArgs &A, const double
         Y = fma(Y, v, m * cy[m]);
         Z = fma(Z, v, m * cz[m]);
     }
-    const double r1 = Z / A.d.dx, r2 = -Y / A.d.dx;
-    const double nr = sqrt(r1 * r1 + r2 * r2), dt = A.d.dt;
-    const double s0 = A.sx[id], s1 = A.sy[id], s2 = A.sz[id];
-    const double c1x = r1 * s2 - r2 * s1, c1y = r2 * s0, c1z = -r1 * s0;
-    const double c2x = r1 * c1z - r2 * c1y, c2y = r2 * c1x, c2z = -r1 * c1x;
-    double f1 = dt, f2 = 0.5 * dt * dt;
-    if (nr > 0.0) {
-        double sn, cs;
-        sincos(0.5 * dt * nr, &sn, &cs);
-        const double q = sn / nr;
-        f1 = 2.0 * q * cs;
-        f2 = 2.0 * q * q;
-    }
-    A.sx[id] = s0 + f1 * c1x + f2 * c2x;
-    A.sy[id] = s1 + f1 * c1y + f2 * c2y;
-    A.sz[id] = s2 + f1 * c1z + f2 * c2z;
+    spin_turn(A.d.dt, Y / A.d.dx, Z / A.d.dx, A.sx[id], A.sy[id], A.sz[id]);
 }
 
 template <int K, typename R>
@@ -293,7 +264,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constan
                 // ---- subsystem II
                 if (me < 9) S->maxima[0][me / 3][me % 3] = 0ull;
                 if (spin)
-                    for (int q = me; q < 2 * M; q += all) spin_source_at(q % M, q / M, A);
+                    for (int q = me; q < 2 * M; q += all) spin_source_at(M, K, A.d.dt * A.hbar * A.w / A.d.dx, A.sm_y, A.sm_z, D.by, D.bz, q % M, q / M);
                 const R *TA = static_cast<const R *>(T.A), *TK = static_cast<const R *>(T.Kt);
                 const size_t row = (size_t)c * (2 * PA);
                 R cy[NC], cz[NC];

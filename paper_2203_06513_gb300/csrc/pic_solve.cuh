@@ -442,6 +442,40 @@ __device__ __forceinline__ void prep1_task(int i, int t, const RunDesc &R)
     }
 }
 
+// Zeeman source of subsystem II at a node: b_y -= dt hbar (G^T d_z)_j, b_z += dt hbar
+// (G^T d_y)_j, d = Lambda_1(X)^T W S from the moments s v^m of the markers (degree K - 1);
+// c = dt hbar w / dx.
+__device__ __forceinline__ void spin_source_at(int M, int K, double c, const double *mom_y, const double *mom_z,
+                                               double *by, double *bz, int j, int comp)
+{
+    const int jp = j + 1 == M ? 0 : j + 1;
+    const double *m = comp ? mom_y : mom_z;
+    const double v = c * (node_value(M, K - 1, false, m, j) - node_value(M, K - 1, false, m, jp));
+    if (comp) bz[j] += v;
+    else by[j] -= v;
+}
+
+// Subsystem III (Eq. spin_rodrigue): s <- s + sin(dt|r|)/|r| (r x s)
+// + 2 (sin(dt|r|/2)/|r|)^2 r x (r x s), r = (0, Z, -Y), Y = dA_y/dx, Z = dA_z/dx at the marker.
+__device__ __forceinline__ void spin_turn(double dt, double Y, double Z, double &sx, double &sy, double &sz)
+{
+    const double r1 = Z, r2 = -Y, nr = sqrt(r1 * r1 + r2 * r2);
+    const double s0 = sx, s1 = sy, s2 = sz;
+    const double c1x = r1 * s2 - r2 * s1, c1y = r2 * s0, c1z = -r1 * s0;
+    const double c2x = r1 * c1z - r2 * c1y, c2y = r2 * c1x, c2z = -r1 * c1x;
+    double f1 = dt, f2 = 0.5 * dt * dt;
+    if (nr > 0.0) {
+        double sn, cs;
+        sincos(0.5 * dt * nr, &sn, &cs);
+        const double q = sn / nr;
+        f1 = 2.0 * q * cs;
+        f2 = 2.0 * q * q;
+    }
+    sx = s0 + f1 * c1x + f2 * c2x;
+    sy = s1 + f1 * c1y + f2 * c2y;
+    sz = s2 + f1 * c1z + f2 * c2z;
+}
+
 // Subsystem II: b = (M0 - dt^2/4 K) e^n + dt K a^n (banded circulant products), e^(0),
 // a^(0) = a^n - dt/2 (e^n + e^(0)), cleared moments, the cells' polynomials.
 template <int K> constexpr int prep2_tasks = 2 * (K + 1) + 2;

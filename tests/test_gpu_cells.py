@@ -94,7 +94,8 @@ def test_device_state_equals_host_state(n, precision):
     (1, 3, {}), (31, 2, dict(warm_start=1, warm_field=1)), (33, 5, dict(splitting=1)),
     (5003, 4, dict(sort_every=2, warm_start=1)), (38912, 3, dict(warm_start=1, warm_field=1, sort_every=3)),
     (38913, 3, dict(warm_start=1, warm_field=1)), (4001, 3, dict(splitting=1, warm_start=1, warm_field=1)),
-    (2003, 3, dict(hbar=0.1)), (2003, 2, dict(hbar=0.1, sort_every=1))])
+    (2003, 3, dict(hbar=0.1)), (2003, 2, dict(hbar=0.1, sort_every=1)),
+    (40001, 3, dict(hbar=0.1)), (65537, 5, dict(hbar=0.1, sort_every=2))])
 def test_one_kernel_steps_equal_host_loops(n, k, kw, monkeypatch):
     """Steps of a small plasma (one cooperative kernel, or just above its limit the graph)
     against the same steps driven from the host: the same iteration, so rounding order
