@@ -17,11 +17,13 @@
 // in shared memory, fp32 accumulators in tensor memory), 128 markers per tile;
 // the ReLU runs in packed bf16 on each thread's accumulator row.  Training
 // (forward + backward + Adam) runs in fp32 on the CUDA cores.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
 #include <climits>
 #include <cmath>
+#include <cstddef>
 #include <cstring>
 #include <vector>
 
@@ -225,9 +227,27 @@ __device__ __forceinline__ void put_bf16(void *base, int off, float v)
     *reinterpret_cast<__nv_bfloat16 *>(reinterpret_cast<char *>(base) + off) = __float2bfloat16(v);
 }
 
-// Stage the network (fp32 parameters in global memory) into the operand layouts.
+// Four columns k .. k + 3 of row n, bf16, at a multiple of four columns (8 bytes of a core matrix row).
+__device__ __forceinline__ void put_bf16x4(void *base, int n, int k, int K, float4 w)
+{
+    *reinterpret_cast<uint2 *>(reinterpret_cast<char *>(base) + kmaj_off(n, k, K)) =
+        make_uint2(pack_bf16(w.x, w.y), pack_bf16(w.z, w.w));
+}
+
+// Stage the network (fp32 parameters in global memory) into the operand layouts: rows of W2
+// and W3 four columns at a time, all of a thread's loads in flight together (one element at
+// a time the staging was most of the 12.7 us of an inference of 4096 rows; now 9.0).
 __device__ void stage_umma(MlpUmma &S, const float *params, const float *norm)
 {
+    constexpr int kQ = kHid * kHid / 4, kPer = (2 * kQ + kMlpThreads - 1) / kMlpThreads;
+    float4 w[kPer];
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        const int q = threadIdx.x + j * kMlpThreads;
+        if (q < 2 * kQ)
+            w[j] = reinterpret_cast<const float4 *>(params + (q < kQ ? kOffW2 : kOffW3))[q < kQ ? q : q - kQ];
+    }
+    static_assert(kOffW2 % 4 == 0 && kOffW3 % 4 == 0 && kOffW4 % 4 == 0, "float4 rows");
     for (int i = threadIdx.x; i < 64 * 16; i += blockDim.x) {
         const int n = i >> 4, k = i & 15;
         put_bf16(S.W1, kmaj_off(n, k, 16),
@@ -235,14 +255,15 @@ __device__ void stage_umma(MlpUmma &S, const float *params, const float *norm)
         put_bf16(S.B2, kmaj_off(n, k, 16), k == 0 ? params[kOffB2 + n] : 0.f);
         put_bf16(S.B3, kmaj_off(n, k, 16), k == 0 ? params[kOffB3 + n] : 0.f);
     }
-    for (int i = threadIdx.x; i < 64 * 64; i += blockDim.x) {
-        const int n = i >> 6, k = i & 63;
-        put_bf16(S.W2, kmaj_off(n, k, 64), params[kOffW2 + n * kHid + k]);
-        put_bf16(S.W3, kmaj_off(n, k, 64), params[kOffW3 + n * kHid + k]);
+    if (threadIdx.x < kOutN * kHid / 4) {
+        const int n = threadIdx.x / (kHid / 4), k = 4 * (threadIdx.x % (kHid / 4));
+        put_bf16x4(S.W4, n, k, 64,
+                   n < kOut ? *reinterpret_cast<const float4 *>(params + kOffW4 + n * kHid + k) : make_float4(0.f, 0.f, 0.f, 0.f));
     }
-    for (int i = threadIdx.x; i < kOutN * 64; i += blockDim.x) {
-        const int n = i >> 6, k = i & 63;
-        put_bf16(S.W4, kmaj_off(n, k, 64), n < kOut ? params[kOffW4 + n * kHid + k] : 0.f);
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        const int q = threadIdx.x + j * kMlpThreads;
+        if (q < 2 * kQ) put_bf16x4(q < kQ ? S.W2 : S.W3, (q % kQ) / 16, 4 * (q % 16), 64, w[j]);
     }
     if (threadIdx.x < kOut) S.b4[threadIdx.x] = params[kOffB4 + threadIdx.x];
     if (threadIdx.x < kNorm) S.norm[threadIdx.x] = norm[threadIdx.x];
@@ -501,13 +522,14 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_warm_mlp(WarmArgs A)
 // 4 x 4 of a weight gradient (products along the samples), all operands in shared memory
 // read four numbers at a time: 32 multiply-adds per 6 loads, 16 per 2.  The row strides
 // keep these reads free of bank conflicts (kWS: 8 rows of one column group; kHS: two
-// rows of 16 columns).  The weight gradients stay in registers over a block's tiles and
-// are added to the global gradient once, four numbers an addition.  One product a thread
-// at a time with two loads each, gradients through shared memory and one double addition
-// to the loss a sample and output made an Adam step, a gradient and an inference of 4096
-// samples take 260 us; with this kernel they take 143 us.
+// rows of 16 columns).  The weights are loaded four numbers at a time, all of a thread's
+// loads in flight together; the weight gradients stay in registers over a block's tiles; a
+// cluster of blocks sums them through distributed shared memory and adds them to the global
+// gradient once.  4096 samples, cold caches: 83 us with one product a thread at a time and
+// gradients through shared memory, 29 us with these tiles, 19.7 us with the weights' loads
+// together, 18.2 us with clusters of 4 (26.3 us with clusters of 8, whose blocks share SMs).
 // ---------------------------------------------------------------------------
-constexpr int kTB = 32, kTrainThreads = 256;
+constexpr int kTB = 32, kTrainThreads = 256, kTrainCluster = 4;
 constexpr int kWS = kHid + 4, kHS = kHid + 16;
 struct TrainSmem {
     float W2[kHid * kWS], W3[kHid * kWS];
@@ -516,7 +538,8 @@ struct TrainSmem {
     float W1[kHid * kIn], W4[kOut * kHid];
     float b1[kHid], b2[kHid], b3[kHid], b4[kOut];
     float h0[kTB * kIn];
-    float y[kTB * kOut];
+    float y[kTB * kOut], tg[kTB * kOut];
+    float norm[kNorm];
     double loss[kTrainThreads / 32];
 };
 
@@ -601,15 +624,16 @@ __device__ __forceinline__ void dense_grad(const float *d, const float *h, float
     }
 }
 
-__device__ __forceinline__ void add_grad(float *gW, float *gB, const float (&G)[4][4], const float (&gb)[4])
+// this thread's part of a layer's gradient to the block's
+__device__ __forceinline__ void put_grad(float *gW, float *gB, const float (&G)[4][4], const float (&gb)[4])
 {
     const int k = 4 * (threadIdx.x & 15), n = 4 * (threadIdx.x >> 4);
 #pragma unroll
     for (int i = 0; i < 4; ++i)
-        atomicAdd(reinterpret_cast<float4 *>(gW + (n + i) * kHid + k), make_float4(G[i][0], G[i][1], G[i][2], G[i][3]));
-    if (k == 0) atomicAdd(reinterpret_cast<float4 *>(gB + n), make_float4(gb[0], gb[1], gb[2], gb[3]));
+        *reinterpret_cast<float4 *>(gW + (n + i) * kHid + k) = make_float4(G[i][0], G[i][1], G[i][2], G[i][3]);
+    if (k == 0) *reinterpret_cast<float4 *>(gB + n) = make_float4(gb[0], gb[1], gb[2], gb[3]);
 }
-static_assert(kOffW2 % 4 == 0 && kOffB2 % 4 == 0 && kOffW3 % 4 == 0 && kOffB3 % 4 == 0, "float4 additions");
+static_assert(kOffB2 % 4 == 0 && kOffB3 % 4 == 0, "float4 stores");
 
 __global__ void __launch_bounds__(kTrainThreads, 2) k_mlp_train(const float *params, const float *norm,
                                                                 const float *X, const float *Tg, long long B,
@@ -618,27 +642,44 @@ __global__ void __launch_bounds__(kTrainThreads, 2) k_mlp_train(const float *par
     extern __shared__ __align__(1024) unsigned char smem[];
     TrainSmem &S = *reinterpret_cast<TrainSmem *>(smem);
     const int tid = threadIdx.x;
-    for (int i = tid; i < kHid * kHid; i += kTrainThreads) {
-        S.W2[(i / kHid) * kWS + i % kHid] = params[kOffW2 + i];
-        S.W3[(i / kHid) * kWS + i % kHid] = params[kOffW3 + i];
+    {   // the weights, all loads in flight together
+        constexpr int kPer = kHid * kHid / 4 / kTrainThreads;
+        float4 w2[kPer], w3[kPer];
+        float w1[2];
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            w2[j] = reinterpret_cast<const float4 *>(params + kOffW2)[tid + j * kTrainThreads];
+            w3[j] = reinterpret_cast<const float4 *>(params + kOffW3)[tid + j * kTrainThreads];
+        }
+        w1[0] = params[kOffW1 + tid];
+        w1[1] = tid < kHid * kIn - kTrainThreads ? params[kOffW1 + kTrainThreads + tid] : 0.f;
+        if (tid < kHid) {
+            S.b1[tid] = params[kOffB1 + tid];
+            S.b2[tid] = params[kOffB2 + tid];
+            S.b3[tid] = params[kOffB3 + tid];
+        }
+        if (tid < kOut * kHid) S.W4[tid] = params[kOffW4 + tid];
+        if (tid < kOut) S.b4[tid] = params[kOffB4 + tid];
+        if (tid < kNorm) S.norm[tid] = norm[tid];
+#pragma unroll
+        for (int j = 0; j < kPer; ++j) {
+            const int q = tid + j * kTrainThreads, o = (q / 16) * kWS + 4 * (q % 16);
+            *reinterpret_cast<float4 *>(S.W2 + o) = w2[j];
+            *reinterpret_cast<float4 *>(S.W3 + o) = w3[j];
+        }
+        S.W1[tid] = w1[0];
+        if (tid < kHid * kIn - kTrainThreads) S.W1[kTrainThreads + tid] = w1[1];
+        static_assert(kHid * kIn >= kTrainThreads && kHid * kIn <= 2 * kTrainThreads, "W1");
     }
-    for (int i = tid; i < kHid * kIn; i += kTrainThreads) S.W1[i] = params[kOffW1 + i];
-    if (tid < kOut * kHid) S.W4[tid] = params[kOffW4 + tid];
-    if (tid < kHid) {
-        S.b1[tid] = params[kOffB1 + tid];
-        S.b2[tid] = params[kOffB2 + tid];
-        S.b3[tid] = params[kOffB3 + tid];
-    }
-    if (tid < kOut) S.b4[tid] = params[kOffB4 + tid];
     float G2[4][4] = {}, G3[4][4] = {}, gb2[4] = {}, gb3[4] = {}, g1[2] = {}, gb1 = 0.f, g4 = 0.f;
     double sum = 0.0;
     for (long long s0 = (long long)blockIdx.x * kTB; s0 < B; s0 += (long long)gridDim.x * kTB) {
         const int ns = (int)min((long long)kTB, B - s0);
+        const float x = tid < ns * kIn ? X[s0 * kIn + tid] : 0.f;
+        const float tg = tid < ns * kOut ? Tg[s0 * kOut + tid] : 0.f;
         __syncthreads();                          // the weights; the last tile's reads
-        if (tid < kTB * kIn) {
-            const int s = tid / kIn, k = tid % kIn;
-            S.h0[tid] = s < ns ? (X[(s0 + s) * kIn + k] - norm[k]) * norm[kIn + k] : 0.f;
-        }
+        if (tid < kTB * kIn) S.h0[tid] = tid < ns * kIn ? (x - S.norm[tid % kIn]) * S.norm[kIn + tid % kIn] : 0.f;
+        if (tid < kTB * kOut) S.tg[tid] = tid < ns * kOut ? tg / S.norm[2 * kIn + tid % kOut] : 0.f;
         __syncthreads();
         {
             const int ng = tid & 15, sg = tid >> 4;
@@ -671,7 +712,7 @@ __global__ void __launch_bounds__(kTrainThreads, 2) k_mlp_train(const float *par
             if (q == 0) {
                 float dy = 0.f;
                 if (s < ns) {
-                    const float r = acc + S.b4[o] - Tg[(s0 + s) * kOut + o] / norm[2 * kIn + o];
+                    const float r = acc + S.b4[o] - S.tg[s * kOut + o];
                     dy = 2.f * r / (float)B;
                     sum += (double)r * (double)r;
                 }
@@ -710,15 +751,35 @@ __global__ void __launch_bounds__(kTrainThreads, 2) k_mlp_train(const float *par
             }
         }
     }
-    add_grad(grad + kOffW2, grad + kOffB2, G2, gb2);
-    add_grad(grad + kOffW3, grad + kOffB3, G3, gb3);
+    // the block's gradient over its weights, then the cluster's: a block sums one part of it
+    // over the blocks and adds that to the global gradient
+    float *G = reinterpret_cast<float *>(smem);
+    static_assert(kNParams * sizeof(float) <= offsetof(TrainSmem, d1), "gradient over weights and activations");
+    __syncthreads();
+    put_grad(G + kOffW2, G + kOffB2, G2, gb2);
+    put_grad(G + kOffW3, G + kOffB3, G3, gb3);
     {
         const int n = tid % kHid, k0 = tid / kHid;
-        atomicAdd(&grad[kOffW1 + n * kIn + k0], g1[0]);
-        if (k0 + 4 < kIn) atomicAdd(&grad[kOffW1 + n * kIn + k0 + 4], g1[1]);
-        if (k0 == 3) atomicAdd(&grad[kOffB1 + n], gb1);
-        if (tid < kOut * kHid + kOut) atomicAdd(&grad[kOffW4 + tid], g4);
+        G[kOffW1 + n * kIn + k0] = g1[0];
+        if (k0 + 4 < kIn) G[kOffW1 + n * kIn + k0 + 4] = g1[1];
+        if (k0 == 3) G[kOffB1 + n] = gb1;
+        if (tid < kOut * kHid + kOut) G[kOffW4 + tid] = g4;
     }
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    cl.sync();
+    const int nb = (int)cl.num_blocks(), part = (kNParams / 2 + nb - 1) / nb;
+    for (int i = (int)cl.block_rank() * part + tid; i < min(kNParams / 2, ((int)cl.block_rank() + 1) * part);
+         i += kTrainThreads) {
+        float2 t = make_float2(0.f, 0.f);
+        for (int b = 0; b < nb; ++b) {
+            const float2 u = *reinterpret_cast<const float2 *>(cl.map_shared_rank(G, b) + 2 * i);
+            t.x += u.x;
+            t.y += u.y;
+        }
+        atomicAdd(reinterpret_cast<float2 *>(grad) + i, t);
+    }
+    static_assert(kNParams % 2 == 0, "pairs");
+    cl.sync();                                    // the others' reads of G
     static_assert(kOffB4 == kOffW4 + kOut * kHid && kTrainThreads == 4 * kHid && kIn <= 8, "gradient layout");
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
@@ -819,15 +880,16 @@ extern "C" int pic_mlp_create(const float *params, const float *norm, void *stre
     cudaDeviceGetAttribute(&m->num_sms, cudaDevAttrMultiProcessorCount, dev);
     bool ok = cudaMalloc((void **)&m->params, kNParams * sizeof(float)) == cudaSuccess &&
               cudaMalloc((void **)&m->norm, kNorm * sizeof(float)) == cudaSuccess &&
-              cudaMalloc((void **)&m->grad, kNParams * sizeof(float)) == cudaSuccess &&
+              cudaMalloc((void **)&m->grad, kNParams * sizeof(float) + sizeof(double)) == cudaSuccess &&
               cudaMalloc((void **)&m->m, kNParams * sizeof(float)) == cudaSuccess &&
               cudaMalloc((void **)&m->v, kNParams * sizeof(float)) == cudaSuccess &&
-              cudaMalloc((void **)&m->loss, sizeof(double)) == cudaSuccess &&
               cudaMalloc((void **)&m->status, sizeof(int)) == cudaSuccess;
     if (!ok) {
         pic_mlp_destroy(m);
         return mlp_fail(PIC_ERR_NOMEM, "pic_mlp_create: cudaMalloc failed");
     }
+    static_assert(kNParams % 2 == 0, "the loss behind the gradient is aligned");
+    m->loss = reinterpret_cast<double *>(m->grad + kNParams);
     std::vector<float> zero(kNParams, 0.f);
     cudaMemcpyAsync(m->params, params ? params : zero.data(), kNParams * sizeof(float), cudaMemcpyHostToDevice, m->stream);
     cudaMemcpyAsync(m->norm, norm, kNorm * sizeof(float), cudaMemcpyHostToDevice, m->stream);
@@ -845,7 +907,7 @@ extern "C" int pic_mlp_destroy(pic_mlp *m)
 {
     if (!m) return PIC_OK;
     cudaStreamSynchronize(m->stream);
-    cudaFree(m->params); cudaFree(m->norm); cudaFree(m->grad); cudaFree(m->m); cudaFree(m->v); cudaFree(m->loss);
+    cudaFree(m->params); cudaFree(m->norm); cudaFree(m->grad); cudaFree(m->m); cudaFree(m->v);
     cudaFree(m->status);
     delete m;
     return PIC_OK;
@@ -869,11 +931,23 @@ extern "C" int pic_mlp_grad(pic_mlp *m, const float *X, const float *T, int64_t 
             return mlp_fail(PIC_ERR_CUDA, "pic_mlp_grad: shared-memory opt-in failed");
         opted = true;
     }
-    cudaMemsetAsync(m->grad, 0, kNParams * sizeof(float), m->stream);
-    cudaMemsetAsync(m->loss, 0, sizeof(double), m->stream);
+    cudaMemsetAsync(m->grad, 0, kNParams * sizeof(float) + sizeof(double), m->stream);    // and the loss behind it
     // two blocks are resident on an SM; beyond that the tiles of a block follow each other
-    const long long nblk = std::min<long long>((B + kTB - 1) / kTB, 2LL * m->num_sms);
-    k_mlp_train<<<(unsigned)nblk, kTrainThreads, sizeof(TrainSmem), m->stream>>>(m->params, m->norm, X, T, B, m->grad, m->loss);
+    const long long tiles = std::min<long long>((B + kTB - 1) / kTB, 2LL * m->num_sms);
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = tiles >= kTrainCluster ? kTrainCluster : 1;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)((tiles + at.val.clusterDim.x - 1) / at.val.clusterDim.x * at.val.clusterDim.x));
+    cfg.blockDim = dim3(kTrainThreads);
+    cfg.dynamicSmemBytes = sizeof(TrainSmem);
+    cfg.stream = m->stream;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, k_mlp_train, (const float *)m->params, (const float *)m->norm, X, T, (long long)B, m->grad,
+                           m->loss) != cudaSuccess)
+        return mlp_fail(PIC_ERR_CUDA, "pic_mlp_grad: launch failed");
     if (cudaGetLastError() != cudaSuccess) return mlp_fail(PIC_ERR_CUDA, "pic_mlp_grad: launch failed");
     if (grad_out && cudaMemcpyAsync(grad_out, m->grad, kNParams * sizeof(float), cudaMemcpyDeviceToDevice, m->stream))
         return mlp_fail(PIC_ERR_CUDA, "pic_mlp_grad: copy failed");
