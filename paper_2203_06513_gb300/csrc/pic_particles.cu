@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(256) k_kinetic(DiagArgs A)
             Ay += A.c0[i] * v[r];
             Az += A.c1[i] * v[r];
         }
-        const double p = (double)pp[a];
+        const double p = as_double(pp[a]);
         const double q = p * p + Ay * Ay + Az * Az;
         acc += A.w * q / (1.0 + sqrt(1.0 + q));      // w (gamma - 1) without cancellation
     }
@@ -639,12 +639,15 @@ int launch_load(int fp32, long long np, int M, double dx, const double *x, const
 }
 
 // position of a marker in [0, L): the centre of its cell plus its offset (an offset of a
-// whole half cell may reach L)
+// whole half cell may reach L).  Two FP64 operations a marker: with conversions and the
+// comparison on the FP64 pipe (ten) the stores were bound by it (2e7 dealt float markers:
+// 374 us, the pipe 86 % busy; now 224).
 template <typename R>
 __device__ __forceinline__ double position(int c, R v, double dx, double L)
 {
-    const double x = (((double)c + 0.5) + (double)v) * dx;
-    return x >= L ? x - L : x;
+    const double x = (cell_centre(c) + as_double(v)) * dx;
+    // x >= L, as integers (L > 0)
+    return __double_as_longlong(x) >= __double_as_longlong(L) ? x - L : x;
 }
 
 template <typename R>
@@ -656,7 +659,7 @@ __global__ void __launch_bounds__(256) k_store(long long np, int M, double dx, P
     for (long long a = (long long)blockIdx.x * blockDim.x + threadIdx.x; a < np; a += stride) {
         const long long i = P.id[a];
         if (x) x[i] = position(P.cell[a], tp[a], dx, M * dx);
-        if (p) p[i] = (double)pp[a];
+        if (p) p[i] = as_double(pp[a]);
     }
 }
 
@@ -681,7 +684,7 @@ __global__ void __launch_bounds__(256) k_store_state(long long np, int M, double
         for (long long a = first; a < np; a += stride) {
             const long long i = P.id[a];
             if (o.x) o.x[i] = position(P.cell[a], vp[a], dx, L);
-            if (o.p) o.p[i] = (double)pp[a];
+            if (o.p) o.p[i] = as_double(pp[a]);
         }
     for (int f = 0; f < o.n; ++f)
         for (long long a = first; a < o.len[f]; a += stride) o.dst[f][a] = o.src[f][a];
@@ -695,18 +698,31 @@ int launch_store_state(int fp32, long long np, int M, double dx, PartPtrs P, con
     return 0;
 }
 
+// four consecutive markers' numbers (none beyond end)
+template <typename T>
+__device__ __forceinline__ void load4_to(const T *q, long long a, long long end, T (&v)[4])
+{
+    if (a + 4 <= end) {
+        load4(q + a, v);
+    } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = a + u < end ? q[a + u] : T(0);
+    }
+}
+
 // Stored order to caller order for more markers than L2 holds outputs for.  Scattered
 // directly, every 8-byte write is a sector of its own by the time it leaves L2 (1e8
 // markers: 6.8 ms).  Instead the markers are first dealt into at most 256 buckets of
-// 2^shift consecutive caller indices (a tile of 4096 markers is ordered by bucket in shared
-// memory, so a bucket's part of it is one run of a few hundred bytes), then each bucket
+// 2^shift consecutive caller indices (a tile of 2048 markers is ordered by bucket in shared
+// memory, so a bucket's part of it is one run of some 128 bytes), then each bucket
 // is written out while its range of x and p stays in L2.  Every bucket is full (the
 // indices are a permutation), so bucket b starts at b 2^shift and needs no histogram.
-// 1e8 markers, float: 6.8 -> 1.6 ms.
+// 2e7 float markers: deal 175 us (512 threads 202, 1024 271; loading cell, v and p only after
+// the ranks 257), store 224 us; 1e8: 6.8 -> 2.0 ms.
 template <typename R> struct StoreRec;
 template <> struct StoreRec<float> { int id, cell; float v, p; };
 template <> struct StoreRec<double> { double v, p; int id, cell; };
-constexpr int kDealThreads = 512, kDealPer = 8, kDealTile = kDealThreads * kDealPer, kDealBuckets = 256;
+constexpr int kDealThreads = 256, kDealPer = 8, kDealTile = kDealThreads * kDealPer, kDealBuckets = 256;
 
 __global__ void k_deal_start(int *cursor, int shift) { cursor[threadIdx.x] = (int)((long long)threadIdx.x << shift); }
 
@@ -722,27 +738,31 @@ __global__ void __launch_bounds__(kDealThreads) k_deal(long long np, int shift, 
     const int n = (int)min((long long)kDealTile, np - base);
     if (threadIdx.x < kDealBuckets) s_cnt[threadIdx.x] = 0;
     __syncthreads();
-    int id[kDealPer], rank[kDealPer];
+    int id[kDealPer], c[kDealPer], rank[kDealPer];
+    R v[kDealPer], p[kDealPer];
 #pragma unroll
-    for (int j = 0; j < kDealPer; ++j) {
-        const int i = j * kDealThreads + threadIdx.x;
-        if (i < n) {
-            id[j] = P.id[base + i];
-            rank[j] = atomicAdd(&s_cnt[id[j] >> shift], 1);
-        }
+    for (int j = 0; j < kDealPer; j += 4) {
+        const long long a = base + j * kDealThreads + 4 * threadIdx.x;
+        load4_to(P.id, a, np, *reinterpret_cast<int (*)[4]>(id + j));
+        load4_to(P.cell, a, np, *reinterpret_cast<int (*)[4]>(c + j));
+        load4_to(vp, a, np, *reinterpret_cast<R (*)[4]>(v + j));
+        load4_to(pp, a, np, *reinterpret_cast<R (*)[4]>(p + j));
     }
+#pragma unroll
+    for (int j = 0; j < kDealPer; ++j)
+        if ((j & ~3) * kDealThreads + 4 * threadIdx.x + (j & 3) < n) rank[j] = atomicAdd(&s_cnt[id[j] >> shift], 1);
     __syncthreads();
     if (threadIdx.x < kDealBuckets) {          // exclusive scan of the counts, and the runs' places
-        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, c = s_cnt[threadIdx.x];
-        int v = c;
+        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, m = s_cnt[threadIdx.x];
+        int sum = m;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
-            const int u = __shfl_up_sync(0xffffffffu, v, o);
-            if (lane >= o) v += u;
+            const int u = __shfl_up_sync(0xffffffffu, sum, o);
+            if (lane >= o) sum += u;
         }
-        if (lane == 31) s_warp[w] = v;
-        s_off[threadIdx.x] = v - c;
-        s_dst[threadIdx.x] = c ? atomicAdd(&cursor[threadIdx.x], c) : 0;
+        if (lane == 31) s_warp[w] = sum;
+        s_off[threadIdx.x] = sum - m;
+        s_dst[threadIdx.x] = m ? atomicAdd(&cursor[threadIdx.x], m) : 0;
     }
     __syncthreads();
     if (threadIdx.x < kDealBuckets) {
@@ -753,13 +773,12 @@ __global__ void __launch_bounds__(kDealThreads) k_deal(long long np, int shift, 
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < kDealPer; ++j) {
-        const int i = j * kDealThreads + threadIdx.x;
-        if (i < n) {
+        if ((j & ~3) * kDealThreads + 4 * threadIdx.x + (j & 3) < n) {
             StoreRec<R> r;
             r.id = id[j];
-            r.cell = P.cell[base + i];
-            r.v = vp[base + i];
-            r.p = pp[base + i];
+            r.cell = c[j];
+            r.v = v[j];
+            r.p = p[j];
             s_rec[s_off[id[j] >> shift] + rank[j]] = r;
         }
     }
@@ -772,14 +791,14 @@ __global__ void __launch_bounds__(kDealThreads) k_deal(long long np, int shift, 
 }
 
 template <typename R>
-__global__ void __launch_bounds__(256) k_store_dealt(long long np, int M, double dx, const StoreRec<R> *rec, double *x,
-                                                     double *p)
+__global__ void __launch_bounds__(256) k_store_dealt(long long np, double dx, double L, const StoreRec<R> *rec,
+                                                     double *x, double *p)
 {
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= np) return;
     const StoreRec<R> r = rec[i];
-    if (x) x[r.id] = position(r.cell, r.v, dx, M * dx);
-    if (p) p[r.id] = (double)r.p;
+    if (x) x[r.id] = position(r.cell, r.v, dx, L);
+    if (p) p[r.id] = as_double(r.p);
 }
 
 template <typename R>
@@ -793,7 +812,7 @@ static int launch_store_dealt_t(long long np, int M, double dx, PartPtrs P, void
     k_deal_start<<<1, kDealBuckets, 0, s>>>(cursor, shift);
     k_deal<R><<<(unsigned)((np + kDealTile - 1) / kDealTile), kDealThreads, smem, s>>>(
         np, shift, P, static_cast<StoreRec<R> *>(rec), cursor);
-    k_store_dealt<R><<<(unsigned)((np + 255) / 256), 256, 0, s>>>(np, M, dx, static_cast<StoreRec<R> *>(rec), x, p);
+    k_store_dealt<R><<<(unsigned)((np + 255) / 256), 256, 0, s>>>(np, dx, M * dx, static_cast<StoreRec<R> *>(rec), x, p);
     return 0;
 }
 
@@ -826,7 +845,7 @@ __global__ void __launch_bounds__(256) k_store_ordered(long long np, int M, doub
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < np; i += stride) {
         const long long a = inv[i];
         if (x) x[i] = position(P.cell[a], tp[a], dx, M * dx);
-        if (p) p[i] = (double)pp[a];
+        if (p) p[i] = as_double(pp[a]);
     }
 }
 
@@ -867,18 +886,6 @@ __device__ __forceinline__ void chunk_of(long long np, int b, int nb, long long 
     chunk = (chunk + 127) & ~127LL;
     beg = (long long)b * chunk;
     end = beg + chunk < np ? beg + chunk : np;
-}
-
-// four consecutive markers' numbers (none beyond end)
-template <typename T>
-__device__ __forceinline__ void load4_to(const T *q, long long a, long long end, T (&v)[4])
-{
-    if (a + 4 <= end) {
-        load4(q + a, v);
-    } else {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = a + u < end ? q[a + u] : T(0);
-    }
 }
 
 template <typename R>
