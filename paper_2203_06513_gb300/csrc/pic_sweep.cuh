@@ -253,7 +253,8 @@ __device__ __forceinline__ void sweep1_range_z(const Sweep1Args &A, long long be
     R dmax = R(0);
     bool bad = false;
     if (beg >= end) return;
-    PathDeposit<K, U, typename AccOf<R, ACC>::T> dep;
+    constexpr bool kFixed = !Real<R>::fp32 && ACC == ACC_NATIVE;
+    PathDeposit<K, U, typename std::conditional<kFixed, AccFixed, typename AccOf<R, ACC>::T>::type> dep;
     dep.start(mom, flux, M, cp[beg]);
 
     // the next step's markers are loaded while this one's are computed
@@ -385,7 +386,8 @@ __device__ __forceinline__ void sweep1_range(const Sweep1Args &A, long long beg,
 // deposited as the moments f v^m of each cell.  Same warp ranges as subsystem I.
 // us a launch, float (1e8 markers, cubic) and double (1e7): basis values and node windows
 // 1260 and 2060, cell polynomials and moments 767 and 830, as here (centred offsets, the
-// short root and quotient, two markers a lane) 570 and 672.
+// short root and quotient, two markers a lane) 570 and 672, with their seeds refined off the
+// FP64 pipe 610 in double.
 // Z: the z component is not identically zero, as in subsystem I.
 // f = (s + L) / G, s = A^n + A^(k) of a component, G = g0 + g1, L the float form's residue.
 // The float rounding of a coefficient is the same for every marker of its cell, so it
