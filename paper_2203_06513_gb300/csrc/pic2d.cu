@@ -70,7 +70,7 @@ struct Args2D {
     const double *s;        // np x 3 spins
     unsigned long long *dmax_bits, *pmax_bits;
     int *status;
-    double gls[5], glw[5];  // K-point Gauss--Legendre on [0, 1]
+    long long gls[5], glw[5];   // K-point Gauss--Legendre on [0, 1], times 2^62
 };
 
 __device__ __forceinline__ int wrapi(int i, int M)
@@ -95,13 +95,16 @@ __device__ __forceinline__ void walk2(double v1, double v2, double d1, double d2
     }
     for (int guard = 0; guard < 2 * kMaxCross + 2; ++guard) {
         double b1 = 2.0, b2 = 2.0;
+        bool go = true, last = true;        // a path in one cell compares nothing
         if (multi) {
             if (k1 != n1) b1 = ((double)k1 + 0.5 * g1 - v1) * r1;
             if (k2 != n2) b2 = ((double)k2 + 0.5 * g2 - v2) * r2;
             sb = fmin(fmin(b1, b2), 1.0);
+            go = sb > sa;
+            last = sb >= 1.0;
         }
-        if (sb > sa) f(sa, sb, k1, k2);
-        if (sb >= 1.0) return;
+        if (go) f(sa, sb, k1, k2);
+        if (last) return;
         if (b1 <= sb) k1 += g1;
         if (b2 <= sb) k2 += g2;
         sa = fmax(sa, sb);
@@ -186,91 +189,107 @@ __device__ __forceinline__ double divided(const double (&c)[N], const double (&S
     return s;
 }
 
-// (Ex, Ey) = the path means of e_bar's two components
+// The means of x^a y^b (a, b <= K, not both K) over a path piece in one cell, from (xa, ya)
+// to (xb, yb) (offsets, below 1 in size), by K Gauss points, which are exact.  In integers
+// of 64 bits (offsets 2^62, means 2^60): the values are at most 1, so the absolute error of
+// a few 2^-60 is below that of a double, and the products run beside the FP64 pipe.
 template <int K>
-__device__ __forceinline__ void gather_path(const Args2D &A, int2 c, double2 v, double2 d, int n1, int n2, double &Ex,
-                                            double &Ey)
+__device__ __forceinline__ void piece_means2(const Args2D &A, double xa, double ya, double xb, double yb,
+                                             double (&md)[K + 1][K + 1])
 {
-    Ex = Ey = 0.0;
+    const long long x0 = to_fixed(xa), y0 = to_fixed(ya), dx = to_fixed(xb) - x0, dy = to_fixed(yb) - y0;
+    long long m[K + 1][K + 1];
+#pragma unroll
+    for (int g = 0; g < K; ++g) {
+        const long long x = x0 + (__mul64hi(dx, A.gls[g]) << 2), y = y0 + (__mul64hi(dy, A.gls[g]) << 2);
+        long long yp[K + 1];
+        yp[0] = 0;
+        yp[1] = y;
+#pragma unroll
+        for (int b = 2; b <= K; ++b) yp[b] = __mul64hi(yp[b - 1], y) << 2;
+        long long xw = A.glw[g];
+#pragma unroll
+        for (int a = 0; a <= K; ++a) {
+            if (a > 0) xw = __mul64hi(xw, x) << 2;
+#pragma unroll
+            for (int b = 0; b <= K; ++b) {
+                if (a == K && b == K) continue;
+                const long long t = b == 0 ? xw >> 2 : __mul64hi(xw, yp[b]);
+                m[a][b] = g == 0 ? t : m[a][b] + t;
+            }
+        }
+    }
+#pragma unroll
+    for (int a = 0; a <= K; ++a)
+#pragma unroll
+        for (int b = 0; b <= K; ++b)
+            if (a < K || b < K) md[a][b] = from_fixed60(m[a][b]);
+}
+
+// f(cell, h, means) for the pieces of the path from v over d, which ends at (e1, e2) n1 and
+// n2 cells over; h: the fraction of the path in the piece
+template <int K, class F>
+__device__ __forceinline__ void path_pieces(const Args2D &A, int2 c, double2 v, double2 d, int n1, int n2, double e1,
+                                            double e2, F &&f)
+{
     walk2(v.x, v.y, d.x, d.y, n1, n2, [&](double sa, double sb, int k1, int k2) {
         int cell = c.x * A.M2 + c.y;
-        double x0 = v.x, y0 = v.y;
-        if (k1 != 0 || k2 != 0) {
+        double xa = v.x, ya = v.y, xb = e1, yb = e2, h = 1.0;
+        if (n1 != 0 || n2 != 0) {
             cell = wrapi(c.x + k1, A.M1) * A.M2 + wrapi(c.y + k2, A.M2);
-            x0 -= (double)k1;
-            y0 -= (double)k2;
+            const double x0 = v.x - (double)k1, y0 = v.y - (double)k2;
+            xa = fma(sa, d.x, x0);
+            ya = fma(sa, d.y, y0);
+            xb = fma(sb, d.x, x0);
+            yb = fma(sb, d.y, y0);
+            h = sb - sa;
         }
+        double md[K + 1][K + 1];
+        piece_means2<K>(A, xa, ya, xb, yb, md);
+        f(cell, h, md);
+    });
+}
+
+// (Ex, Ey) = the path means of e_bar's two components
+template <int K>
+__device__ __forceinline__ void gather_path(const Args2D &A, int2 c, double2 v, double2 d, int n1, int n2, double e1,
+                                            double e2, double &Ex, double &Ey)
+{
+    Ex = Ey = 0.0;
+    path_pieces<K>(A, c, v, d, n1, n2, e1, e2, [&](int cell, double h, const double (&md)[K + 1][K + 1]) {
         double ex[K * (K + 1)], ey[K * (K + 1)];
         load_coef<K * (K + 1)>(A.TEx + (size_t)cell * Dim2<K>::pE, ex);
         load_coef<K * (K + 1)>(A.TEy + (size_t)cell * Dim2<K>::pE, ey);
-        const double h = sb - sa;
+        double sx = ex[0] * md[0][0], sy = ey[0] * md[0][0];
 #pragma unroll
-        for (int g = 0; g < K; ++g) {
-            const double s = fma(h, A.gls[g], sa), wq = h * A.glw[g];
-            const double x = fma(s, d.x, x0), y = fma(s, d.y, y0);
-            double px = 0.0, py = 0.0;
+        for (int a = 0; a <= K; ++a)
 #pragma unroll
-            for (int a = K; a >= 0; --a) {
-                if (a < K) {
-                    double r = ex[a * (K + 1) + K];
-#pragma unroll
-                    for (int b = K - 1; b >= 0; --b) r = fma(r, y, ex[a * (K + 1) + b]);
-                    px = a == K - 1 ? r : fma(px, x, r);
-                }
-                double r = ey[a * K + K - 1];
-#pragma unroll
-                for (int b = K - 2; b >= 0; --b) r = fma(r, y, ey[a * K + b]);
-                py = a == K ? r : fma(py, x, r);
+            for (int b = 0; b <= K; ++b) {
+                if (a + b == 0) continue;
+                if (a < K) sx = fma(ex[a < K ? a * (K + 1) + b : 0], md[a][b], sx);
+                if (b < K) sy = fma(ey[b < K ? a * K + b : 0], md[a][b], sy);
             }
-            Ex = fma(wq, px, Ex);
-            Ey = fma(wq, py, Ey);
-        }
+        Ex = fma(h, sx, Ex);
+        Ey = fma(h, sy, Ey);
     });
 }
 
 // (wx, wy) x the path moments of the two components to the cells, one addition in global
 // memory per moment and piece
 template <int K>
-__device__ __forceinline__ void deposit_path(const Args2D &A, int2 c, double2 v, double2 d, int n1, int n2, double wx,
-                                             double wy)
+__device__ __forceinline__ void deposit_path(const Args2D &A, int2 c, double2 v, double2 d, int n1, int n2, double e1,
+                                             double e2, double wx, double wy)
 {
-    walk2(v.x, v.y, d.x, d.y, n1, n2, [&](double sa, double sb, int k1, int k2) {
-        int cell = c.x * A.M2 + c.y;
-        double x0 = v.x, y0 = v.y;
-        if (k1 != 0 || k2 != 0) {
-            cell = wrapi(c.x + k1, A.M1) * A.M2 + wrapi(c.y + k2, A.M2);
-            x0 -= (double)k1;
-            y0 -= (double)k2;
-        }
-        const double h = sb - sa;
-        double m[K + 1][K + 1];
-#pragma unroll
-        for (int g = 0; g < K; ++g) {
-            const double s = fma(h, A.gls[g], sa), wq = h * A.glw[g];
-            const double x = fma(s, d.x, x0), y = fma(s, d.y, y0);
-            double yp[K + 1];
-            yp[0] = 1.0;
-#pragma unroll
-            for (int b = 1; b <= K; ++b) yp[b] = b == 1 ? y : yp[b - 1] * y;
-            double xa = wq;
-#pragma unroll
-            for (int a = 0; a <= K; ++a) {
-#pragma unroll
-                for (int b = 0; b <= K; ++b) {
-                    if (a == K && b == K) continue;
-                    const double t = b == 0 ? xa : xa * yp[b];
-                    m[a][b] = g == 0 ? t : (b == 0 ? m[a][b] + xa : fma(xa, yp[b], m[a][b]));
-                }
-                xa *= x;
-            }
-        }
+    const bool bx = wx != 0.0, by = wy != 0.0;
+    path_pieces<K>(A, c, v, d, n1, n2, e1, e2, [&](int cell, double h, const double (&md)[K + 1][K + 1]) {
         double *px = A.mx + (size_t)cell * Dim2<K>::nE, *py = A.my + (size_t)cell * Dim2<K>::nE;
+        const double hx = h * wx, hy = h * wy;
 #pragma unroll
         for (int a = 0; a <= K; ++a)
 #pragma unroll
             for (int b = 0; b <= K; ++b) {
-                if (a < K && wx != 0.0) atomicAdd(px + a * (K + 1) + b, wx * m[a][b]);
-                if (b < K && wy != 0.0) atomicAdd(py + a * K + b, wy * m[a][b]);
+                if (a < K && bx) atomicAdd(px + a * (K + 1) + b, hx * md[a][b]);
+                if (b < K && by) atomicAdd(py + a * K + b, hy * md[a][b]);
             }
     });
 }
@@ -290,27 +309,35 @@ __device__ __forceinline__ void max_bits(unsigned long long *dst, double v)
 // Bound by the FP64 pipe.  With basis values at the quadrature points and 24 weights per
 // piece, added to the block's shared rows by compare-and-swap, the sweep took 1068 FP64
 // operations a marker (cubic, path in one cell) and 4.1 ms for 2e6 markers.
+constexpr int kTile2 = 256;          // markers a warp groups at a time
+template <int K> constexpr int sweep2d_blocks = K <= 3 ? 2 : 1;      // resident on an SM
 template <int K, bool PRE = false>
-__global__ void __launch_bounds__(256, K <= 3 ? 2 : 1) k2_sweep(Args2D A)
+__global__ void __launch_bounds__(256, sweep2d_blocks<K>) k2_sweep(Args2D A)
 {
     using Dm = Dim2<K>;
     constexpr int NC = K + 1;
-    __shared__ int s_perm[256];
-    __shared__ int s_cnt[8];
+    __shared__ unsigned char s_perm[8][kTile2];
     double dm = 0.0, pm = 0.0;
     bool bad = false;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
-    for (long long base = blockIdx.x * 256LL; base < A.np; base += gridDim.x * 256LL) {
-        // The block's 256 markers in two groups, paths within one cell first and
-        // paths across a knot last (by the current iterate; the new path mostly
-        // follows it): a warp then runs the extra pieces of a crossing only when
-        // it holds crossing markers, instead of nearly every warp running them
-        // for one lane.
-        {
-            const long long b = base + threadIdx.x;
+    // a run of markers per warp
+    const long long warps = gridDim.x * 8LL, run = ((A.np + warps - 1) / warps + 31) & ~31LL;
+    const long long beg = (blockIdx.x * 8LL + wid) * run, end = beg + run < A.np ? beg + run : A.np;
+    for (long long base = beg; base < end; base += kTile2) {
+        // The warp's next markers in two groups, paths within one cell first and paths
+        // across a knot last (by the current iterate; the new path mostly follows it): the
+        // extra pieces of a crossing then run only in the steps that hold crossing markers,
+        // instead of nearly every step running them for one lane.  By warps, not blocks:
+        // the warps of a block with the crossings kept the others waiting (388 us for 5e5
+        // cubic markers, 289 so).
+        const int n = (int)(end - base < kTile2 ? end - base : kTile2);
+        int front = 0, back = n;
+        for (int q = 0; q < n; q += 32) {
+            const long long b = base + q + lane;
+            const bool act = q + lane < n;
             bool multi = true;
-            if (b < A.np) {
+            if (act) {
                 const double2 v = A.v[b];
                 double2 d = A.d[b];
                 if (PRE) {                      // the predicted start's path is within dt p (gamma >= 1)
@@ -319,149 +346,143 @@ __global__ void __launch_bounds__(256, K <= 3 ? 2 : 1) k2_sweep(Args2D A)
                 }
                 multi = !within(v.x + d.x, 0.5) || !within(v.y + d.y, 0.5);
             }
-            const unsigned one = __ballot_sync(0xffffffffu, !multi);
-            if (lane == 0) s_cnt[wid] = __popc(one);
-            __syncthreads();
-            int before = 0, total = 0;
-#pragma unroll
-            for (int w = 0; w < 8; ++w) {
-                const int c = s_cnt[w];
-                before += w < wid ? c : 0;
-                total += c;
+            const unsigned one = __ballot_sync(0xffffffffu, !multi), more = __ballot_sync(0xffffffffu, act && multi);
+            if (act) s_perm[wid][multi ? back - 1 - __popc(more & lt) : front + __popc(one & lt)] = (unsigned char)(q + lane);
+            front += __popc(one);
+            back -= __popc(more);
+        }
+        __syncwarp();
+        for (int q = lane; q < n; q += 32) {
+            const long long a = base + s_perm[wid][q];
+            const int2 c = A.cell[a];
+            const double2 v = A.v[a], p = A.pn[a];
+            double2 d = PRE ? make_double2(0.0, 0.0) : A.d[a];
+            const double pp1 = fma(p.x, p.x, fma(p.y, p.y, 1.0));
+            // beta_b: A contracted over v1 at x1^n; A(x^n) and gamma(p^n, A(x^n)); the same in
+            // every sweep of the step
+            double be[NC], A0, g0;
+            if (PRE || A.first) {
+                contract_cols<NC, NC>(A.TA + (size_t)(c.x * A.M2 + c.y) * Dm::pA, v.x, be);
+                A0 = horner<NC>(be, v.y);
+                g0 = root(fma(A0, A0, pp1));
+    #pragma unroll
+                for (int b = 1; b <= K; ++b) A.cache[(size_t)(b - 1) * A.np + a] = be[b];
+                A.cache[(size_t)K * A.np + a] = A0;
+                A.cache[(size_t)(K + 1) * A.np + a] = g0;
+            } else {
+                be[0] = 0.0;
+    #pragma unroll
+                for (int b = 1; b <= K; ++b) be[b] = A.cache[(size_t)(b - 1) * A.np + a];
+                A0 = A.cache[(size_t)K * A.np + a];
+                g0 = A.cache[(size_t)(K + 1) * A.np + a];
             }
-            s_perm[multi ? total + (wid * 32 - before) + __popc(~one & lt) : before + __popc(one & lt)] = threadIdx.x;
-            __syncthreads();
-        }
-        const long long a = base + s_perm[threadIdx.x];
-        __syncthreads();                    // s_perm and s_cnt are free for the next group
-        if (a >= A.np) continue;
-        const int2 c = A.cell[a];
-        const double2 v = A.v[a], p = A.pn[a];
-        double2 d = PRE ? make_double2(0.0, 0.0) : A.d[a];
-        const double pp1 = fma(p.x, p.x, fma(p.y, p.y, 1.0));
-        // beta_b: A contracted over v1 at x1^n; A(x^n) and gamma(p^n, A(x^n)); the same in
-        // every sweep of the step
-        double be[NC], A0, g0;
-        if (PRE || A.first) {
-            contract_cols<NC, NC>(A.TA + (size_t)(c.x * A.M2 + c.y) * Dm::pA, v.x, be);
-            A0 = horner<NC>(be, v.y);
-            g0 = root(fma(A0, A0, pp1));
-#pragma unroll
-            for (int b = 1; b <= K; ++b) A.cache[(size_t)(b - 1) * A.np + a] = be[b];
-            A.cache[(size_t)K * A.np + a] = A0;
-            A.cache[(size_t)(K + 1) * A.np + a] = g0;
-        } else {
-            be[0] = 0.0;
-#pragma unroll
-            for (int b = 1; b <= K; ++b) be[b] = A.cache[(size_t)(b - 1) * A.np + a];
-            A0 = A.cache[(size_t)K * A.np + a];
-            g0 = A.cache[(size_t)(K + 1) * A.np + a];
-        }
-        if constexpr (PRE) {
-            const double r = quotient(A.dt, g0);
-            const double x0 = r * p.x, x1 = r * p.y;
-            d = make_double2(x0 * A.idx1, x1 * A.idx2);
-            if (!within(d.x, 1024.0) || !within(d.y, 1024.0)) { bad = true; continue; }
+            if constexpr (PRE) {
+                const double r = quotient(A.dt, g0);
+                const double x0 = r * p.x, x1 = r * p.y;
+                d = make_double2(x0 * A.idx1, x1 * A.idx2);
+                if (!within(d.x, 1024.0) || !within(d.y, 1024.0)) { bad = true; continue; }
+                int n1, n2;
+                double e1, e2;
+                path_end(v.x, d.x, n1, e1);
+                path_end(v.y, d.y, n2, e2);
+                if (abs(n1) > kMaxCross || abs(n2) > kMaxCross) bad = true;
+                else deposit_path<K>(A, c, v, d, n1, n2, e1, e2, A.w * x0, A.w * x1);
+                A.d[a] = d;
+                continue;
+            }
             int n1, n2;
             double e1, e2;
             path_end(v.x, d.x, n1, e1);
             path_end(v.y, d.y, n2, e2);
+            const bool spin = A.hbar != 0.0;
+            double sx = 0.0, sy = 0.0, sz = 0.0, Z1 = 0.0, Z2 = 0.0;
+            if (spin) {
+                sx = A.s[3 * a] * A.idx2;           // s_x dA/dx2, s_y dA/dx1 in cell units
+                sy = A.s[3 * a + 1] * A.idx1;
+                sz = A.s[3 * a + 2];
+            }
+            // along x1 at x2^(k): alpha_a, A contracted over v2; A(x^(k)) in the last cell
+            double D1 = 0.0, W1 = 0.0, A1 = 0.0;
+            for (int q = 0; q <= abs(n1); ++q) {
+                int cell = c.x * A.M2 + c.y;
+                if (n1 != 0 || n2 != 0)
+                    cell = wrapi(c.x + (n1 > 0 ? q : -q), A.M1) * A.M2 + wrapi(c.y + n2, A.M2);
+                double al[NC], S[K];
+                const double *row = A.TA + (size_t)cell * Dm::pA;
+                contract_rows<NC, NC>(row, e2, al);
+                const double h = quotient_piece<K>(q, n1, v.x, e1, S);
+                D1 = fma(h, divided<NC>(al, S), D1);
+                W1 += h;
+                if (q == abs(n1)) A1 = horner<NC>(al, e1);
+                if (spin) {
+                    // f = s_x dA/dx2 - s_y dA/dx1 + s_z b_z contracted over v2, its quotient
+                    double ady[NC], bz[K], f[NC];
+                    contract_rows_dy<NC, NC>(row, e2, ady);
+                    contract_rows<K, K>(A.TB + (size_t)cell * Dm::pB, e2, bz);
+    #pragma unroll
+                    for (int m = 0; m <= K; ++m) {
+                        f[m] = sx * ady[m];
+                        if (m < K) f[m] += sz * bz[m < K ? m : 0] - sy * (double)(m + 1) * al[m < K ? m + 1 : 0];
+                    }
+                    Z1 = fma(h, divided<NC>(f, S), Z1);
+                }
+            }
+            // along x2 at x1^n
+            double D2 = 0.0, W2 = 0.0;
+            for (int q = 0; q <= abs(n2); ++q) {
+                const int cell = q == 0 ? c.x * A.M2 + c.y : c.x * A.M2 + wrapi(c.y + (n2 > 0 ? q : -q), A.M2);
+                const double *row = A.TA + (size_t)cell * Dm::pA;
+                double bq[NC], S[K];
+                if (q == 0) {
+    #pragma unroll
+                    for (int b = 0; b <= K; ++b) bq[b] = be[b];
+                } else {
+                    contract_cols<NC, NC>(row, v.x, bq);
+                }
+                const double h = quotient_piece<K>(q, n2, v.y, e2, S);
+                D2 = fma(h, divided<NC>(bq, S), D2);
+                W2 += h;
+                if (spin) {
+                    double adx[NC], bz[K], f[NC];
+                    contract_cols_dx<NC, NC>(row, v.x, adx);
+                    contract_cols<K, K>(A.TB + (size_t)cell * Dm::pB, v.x, bz);
+    #pragma unroll
+                    for (int m = 0; m <= K; ++m) {
+                        f[m] = -sy * adx[m];
+                        if (m < K) f[m] += sz * bz[m < K ? m : 0] + sx * (double)(m + 1) * bq[m < K ? m + 1 : 0];
+                    }
+                    Z2 = fma(h, divided<NC>(f, S), Z2);
+                }
+            }
+            if (n1 != 0) { D1 = quotient(D1, W1); Z1 = Z1 / W1; }
+            if (n2 != 0) { D2 = quotient(D2, W2); Z2 = Z2 / W2; }
+            double Ex, Ey;
+            gather_path<K>(A, c, v, d, n1, n2, e1, e2, Ex, Ey);
+            const double g1 = root(fma(A1, A1, pp1));
+            const double f = quotient(A.dt * (A1 + A0), g1 + g0);
+            double q0 = fma(A.dt, Ex, p.x) - f * (D1 * A.idx1);
+            double q1 = fma(A.dt, Ey, p.y) - f * (D2 * A.idx2);
+            if (spin) {
+                q0 -= A.dt * A.hbar * Z1 * A.idx1;
+                q1 -= A.dt * A.hbar * Z2 * A.idx2;
+            }
+            const double g2 = root(fma(q0, q0, fma(q1, q1, fma(A1, A1, 1.0))));
+            const double r = quotient(A.dt, g1 + g2);
+            const double x0 = r * (p.x + q0), x1 = r * (p.y + q1);
+            const double2 dn = make_double2(x0 * A.idx1, x1 * A.idx2);
+            if (!within(dn.x, 1024.0) || !within(dn.y, 1024.0)) { bad = true; continue; }
+            // the current of the new path
+            path_end(v.x, dn.x, n1, e1);
+            path_end(v.y, dn.y, n2, e2);
             if (abs(n1) > kMaxCross || abs(n2) > kMaxCross) bad = true;
-            else deposit_path<K>(A, c, v, d, n1, n2, A.w * x0, A.w * x1);
-            A.d[a] = d;
-            continue;
+            else deposit_path<K>(A, c, v, dn, n1, n2, e1, e2, A.w * x0, A.w * x1);
+            const double2 po = A.pk[a];
+            dm = max_nonneg(dm, max_nonneg(fabs(dn.x - d.x) * A.dx1, fabs(dn.y - d.y) * A.dx2));
+            pm = max_nonneg(pm, max_nonneg(fabs(q0 - po.x), fabs(q1 - po.y)));
+            A.d[a] = dn;
+            A.pk[a] = make_double2(q0, q1);
         }
-        int n1, n2;
-        double e1, e2;
-        path_end(v.x, d.x, n1, e1);
-        path_end(v.y, d.y, n2, e2);
-        const bool spin = A.hbar != 0.0;
-        double sx = 0.0, sy = 0.0, sz = 0.0, Z1 = 0.0, Z2 = 0.0;
-        if (spin) {
-            sx = A.s[3 * a] * A.idx2;           // s_x dA/dx2, s_y dA/dx1 in cell units
-            sy = A.s[3 * a + 1] * A.idx1;
-            sz = A.s[3 * a + 2];
-        }
-        // along x1 at x2^(k): alpha_a, A contracted over v2; A(x^(k)) in the last cell
-        double D1 = 0.0, W1 = 0.0, A1 = 0.0;
-        for (int q = 0; q <= abs(n1); ++q) {
-            int cell = c.x * A.M2 + c.y;
-            if (n1 != 0 || n2 != 0)
-                cell = wrapi(c.x + (n1 > 0 ? q : -q), A.M1) * A.M2 + wrapi(c.y + n2, A.M2);
-            double al[NC], S[K];
-            const double *row = A.TA + (size_t)cell * Dm::pA;
-            contract_rows<NC, NC>(row, e2, al);
-            const double h = quotient_piece<K>(q, n1, v.x, e1, S);
-            D1 = fma(h, divided<NC>(al, S), D1);
-            W1 += h;
-            if (q == abs(n1)) A1 = horner<NC>(al, e1);
-            if (spin) {
-                // f = s_x dA/dx2 - s_y dA/dx1 + s_z b_z contracted over v2, its quotient
-                double ady[NC], bz[K], f[NC];
-                contract_rows_dy<NC, NC>(row, e2, ady);
-                contract_rows<K, K>(A.TB + (size_t)cell * Dm::pB, e2, bz);
-#pragma unroll
-                for (int m = 0; m <= K; ++m) {
-                    f[m] = sx * ady[m];
-                    if (m < K) f[m] += sz * bz[m < K ? m : 0] - sy * (double)(m + 1) * al[m < K ? m + 1 : 0];
-                }
-                Z1 = fma(h, divided<NC>(f, S), Z1);
-            }
-        }
-        // along x2 at x1^n
-        double D2 = 0.0, W2 = 0.0;
-        for (int q = 0; q <= abs(n2); ++q) {
-            const int cell = q == 0 ? c.x * A.M2 + c.y : c.x * A.M2 + wrapi(c.y + (n2 > 0 ? q : -q), A.M2);
-            const double *row = A.TA + (size_t)cell * Dm::pA;
-            double bq[NC], S[K];
-            if (q == 0) {
-#pragma unroll
-                for (int b = 0; b <= K; ++b) bq[b] = be[b];
-            } else {
-                contract_cols<NC, NC>(row, v.x, bq);
-            }
-            const double h = quotient_piece<K>(q, n2, v.y, e2, S);
-            D2 = fma(h, divided<NC>(bq, S), D2);
-            W2 += h;
-            if (spin) {
-                double adx[NC], bz[K], f[NC];
-                contract_cols_dx<NC, NC>(row, v.x, adx);
-                contract_cols<K, K>(A.TB + (size_t)cell * Dm::pB, v.x, bz);
-#pragma unroll
-                for (int m = 0; m <= K; ++m) {
-                    f[m] = -sy * adx[m];
-                    if (m < K) f[m] += sz * bz[m < K ? m : 0] + sx * (double)(m + 1) * bq[m < K ? m + 1 : 0];
-                }
-                Z2 = fma(h, divided<NC>(f, S), Z2);
-            }
-        }
-        if (n1 != 0) { D1 = quotient(D1, W1); Z1 = Z1 / W1; }
-        if (n2 != 0) { D2 = quotient(D2, W2); Z2 = Z2 / W2; }
-        double Ex, Ey;
-        gather_path<K>(A, c, v, d, n1, n2, Ex, Ey);
-        const double g1 = root(fma(A1, A1, pp1));
-        const double f = quotient(A.dt * (A1 + A0), g1 + g0);
-        double q0 = fma(A.dt, Ex, p.x) - f * (D1 * A.idx1);
-        double q1 = fma(A.dt, Ey, p.y) - f * (D2 * A.idx2);
-        if (spin) {
-            q0 -= A.dt * A.hbar * Z1 * A.idx1;
-            q1 -= A.dt * A.hbar * Z2 * A.idx2;
-        }
-        const double g2 = root(fma(q0, q0, fma(q1, q1, fma(A1, A1, 1.0))));
-        const double r = quotient(A.dt, g1 + g2);
-        const double x0 = r * (p.x + q0), x1 = r * (p.y + q1);
-        const double2 dn = make_double2(x0 * A.idx1, x1 * A.idx2);
-        if (!within(dn.x, 1024.0) || !within(dn.y, 1024.0)) { bad = true; continue; }
-        // the current of the new path
-        path_end(v.x, dn.x, n1, e1);
-        path_end(v.y, dn.y, n2, e2);
-        if (abs(n1) > kMaxCross || abs(n2) > kMaxCross) bad = true;
-        else deposit_path<K>(A, c, v, dn, n1, n2, A.w * x0, A.w * x1);
-        const double2 po = A.pk[a];
-        dm = max_nonneg(dm, max_nonneg(fabs(dn.x - d.x) * A.dx1, fabs(dn.y - d.y) * A.dx2));
-        pm = max_nonneg(pm, max_nonneg(fabs(q0 - po.x), fabs(q1 - po.y)));
-        A.d[a] = dn;
-        A.pk[a] = make_double2(q0, q1);
+        __syncwarp();
     }
     if (bad) atomicOr(A.status, STATUS_NUMERIC);
     if (PRE) return;
@@ -560,45 +581,50 @@ __global__ void __launch_bounds__(64) k2_nodes(int M1, int M2, const double *mx,
     else jy[i] = node2_at<K, K - 1>(M1, M2, my, i / M2, i % M2);
 }
 
-// sum_q g[(i - q) mod M] in[q stride], four independent chains
-__device__ __forceinline__ double circ_at(int M, int i, const double *g, const double *in, int stride)
+// sum_q g[(i - q) mod M] in[q stride]: a quarter of the terms a thread, kCirc outputs a block
+// of 4 kCirc threads (a whole sum a thread is one chain of M dependent reads: 28 us along
+// x1 of 64 x 64 nodes, 11 so).  The sum is returned to the block's first kCirc threads.
+constexpr int kCirc = 16;
+__device__ __forceinline__ double circ_at(int M, int i, const double *__restrict__ g, const double *__restrict__ in,
+                                          int stride)
 {
-    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-    int k = i, q = 0;
-    auto next = [&]() { const double v = g[k] * in[(size_t)q * stride]; k = k == 0 ? M - 1 : k - 1; ++q; return v; };
-    while (q + 4 <= M) {
-        s0 += next();
-        s1 += next();
-        s2 += next();
-        s3 += next();
+    __shared__ double s_part[3][kCirc];
+    const int part = threadIdx.x / kCirc, o = threadIdx.x % kCirc;
+    const int q1 = (part + 1) * M / 4;
+    double s[2] = {0.0, 0.0};
+    int q = part * M / 4, k = i - q < 0 ? i - q + M : i - q;
+    for (; q < q1; ++q) {
+        s[q & 1] = fma(g[k], in[(size_t)q * stride], s[q & 1]);
+        k = k == 0 ? M - 1 : k - 1;
     }
-    while (q < M) s0 += next();
-    return (s0 + s1) + (s2 + s3);
+    const double t = s[0] + s[1];
+    if (part > 0) s_part[part - 1][o] = t;
+    __syncthreads();
+    return part > 0 ? 0.0 : (t + s_part[0][o]) + (s_part[1][o] + s_part[2][o]);
 }
 
 // pass along x2 of both components (blockIdx.y): out[i1, i2] = sum_q g[(i2 - q) mod M2] in[i1, q]
-__global__ void __launch_bounds__(64) k2_circ2(int M1, int M2, const double *gx, const double *gy, const double *jx,
+__global__ void __launch_bounds__(4 * kCirc) k2_circ2(int M1, int M2, const double *gx, const double *gy, const double *jx,
                                                const double *jy, double *ox, double *oy)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= M1 * M2) return;
-    const int i1 = i / M2, i2 = i % M2;
-    if (blockIdx.y == 0) ox[i] = circ_at(M2, i2, gx, jx + (size_t)i1 * M2, 1);
-    else oy[i] = circ_at(M2, i2, gy, jy + (size_t)i1 * M2, 1);
+    const int i = blockIdx.x * kCirc + threadIdx.x % kCirc, n = min(i, M1 * M2 - 1);
+    const int i1 = n / M2, i2 = n % M2;
+    const bool y = blockIdx.y != 0;
+    const double v = circ_at(M2, i2, y ? gy : gx, (y ? jy : jx) + (size_t)i1 * M2, 1);
+    if (threadIdx.x < kCirc && i < M1 * M2) (y ? oy : ox)[i] = v;
 }
 
 // pass along x1, then e^(k+1) = e^n - M1^{-1} j, its increment's max-norm, e_bar for the
 // next sweep
-__global__ void __launch_bounds__(64) k2_circ1(int M1, int M2, const double *gx, const double *gy, const double *tx,
+__global__ void __launch_bounds__(4 * kCirc) k2_circ1(int M1, int M2, const double *gx, const double *gy, const double *tx,
                                                const double *ty, const double *enx, const double *eny, double *ekx,
                                                double *eky, double *ebx, double *eby, unsigned long long *emax_bits)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = blockIdx.x * kCirc + threadIdx.x % kCirc, n = min(i, M1 * M2 - 1);
+    const bool y = blockIdx.y != 0;
+    const double sol = circ_at(M1, n / M2, y ? gy : gx, (y ? ty : tx) + n % M2, M2);
     double m = 0.0;
-    if (i < M1 * M2) {
-        const int i1 = i / M2, i2 = i % M2;
-        const bool y = blockIdx.y != 0;
-        const double sol = circ_at(M1, i1, y ? gy : gx, (y ? ty : tx) + i2, M2);
+    if (threadIdx.x < kCirc && i < M1 * M2) {
         const double en = (y ? eny : enx)[i], v = en - sol;
         double *ek = y ? eky : ekx;
         m = fabs(v - ek[i]);
@@ -606,7 +632,7 @@ __global__ void __launch_bounds__(64) k2_circ1(int M1, int M2, const double *gx,
         (y ? eby : ebx)[i] = 0.5 * (en + v);
     }
     for (int o = 16; o > 0; o >>= 1) m = max_nonneg(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) max_bits(emax_bits, m);
+    if (threadIdx.x == 0) max_bits(emax_bits, m);
 }
 
 // acc[0] += sum_a w (g(p_a, A(x_a)) - 1); with spins, acc[1] += sum_a w hbar
@@ -813,7 +839,7 @@ static Args2D make_args(pic2d_handle *h)
     a.hbar = h->spin ? c.hbar : 0.0;
     a.s = h->spin;
     a.dmax_bits = h->bits; a.pmax_bits = h->bits + 1; a.status = h->status;
-    for (int g = 0; g < 5; ++g) { a.gls[g] = h->gls[g]; a.glw[g] = h->glw[g]; }
+    for (int g = 0; g < 5; ++g) { a.gls[g] = std::llrint(std::ldexp(h->gls[g], 62)); a.glw[g] = std::llrint(std::ldexp(h->glw[g], 62)); }
     return a;
 }
 
@@ -834,12 +860,12 @@ static int solve2d(pic2d_handle *h)
 {
     const pic2d_config &c = h->cfg;
     const Args2D a = make_args(h);
-    const dim3 grid((h->N + 63) / 64, 2);
+    const dim3 grid((h->N + 63) / 64, 2), circ((h->N + kCirc - 1) / kCirc, 2);
     cudaStream_t s = h->stream;
     PIC2D_DEGREE(c.degree, (k2_nodes<K><<<grid, 64, 0, s>>>(c.M1, c.M2, a.mx, a.my, h->jx, h->jy)))
     // along x2 with the rows of component x's N^k and y's N^{k-1}, then along x1
-    k2_circ2<<<grid, 64, 0, s>>>(c.M1, c.M2, h->g0y, h->g1y, h->jx, h->jy, h->tx, h->ty);
-    k2_circ1<<<grid, 64, 0, s>>>(c.M1, c.M2, h->g1x, h->g0x, h->tx, h->ty, h->ex, h->ey, h->exk, h->eyk, h->ebx, h->eby,
+    k2_circ2<<<circ, 4 * kCirc, 0, s>>>(c.M1, c.M2, h->g0y, h->g1y, h->jx, h->jy, h->tx, h->ty);
+    k2_circ1<<<circ, 4 * kCirc, 0, s>>>(c.M1, c.M2, h->g1x, h->g0x, h->tx, h->ty, h->ex, h->ey, h->exk, h->eyk, h->ebx, h->eby,
                                  h->bits + 2);
     CK2(cudaGetLastError());
     return tables_e(h);
@@ -957,7 +983,7 @@ extern "C" int pic2d_substep1(pic2d_handle *h, int32_t *iters)
         // the predicted start: delta^(0) and its current, then e^(0) = e^n - M1^{-1} j^(0)
         // and e_bar = (e^n + e^(0)) / 2 for the first sweep
         CK2(cudaMemsetAsync(h->mom, 0, mom_bytes, s));
-        PIC2D_DEGREE(c.degree, (k2_sweep<K, true><<<grid, 256, 0, s>>>(a)))
+        PIC2D_DEGREE(c.degree, (k2_sweep<K, true><<<std::min(grid, sweep2d_blocks<K> * h->num_sms), 256, 0, s>>>(a)))
         CK2(cudaGetLastError());
         if ((rc = solve2d(h))) return rc;
     } else if ((rc = tables_e(h))) {
@@ -967,7 +993,7 @@ extern "C" int pic2d_substep1(pic2d_handle *h, int32_t *iters)
         CK2(cudaMemsetAsync(h->mom, 0, mom_bytes, s));
         CK2(cudaMemsetAsync(h->bits, 0, 3 * sizeof(unsigned long long), s));
         a.first = !warm && it == 0;          // the predicted start filled the cache already
-        PIC2D_DEGREE(c.degree, (k2_sweep<K><<<grid, 256, 0, s>>>(a)))
+        PIC2D_DEGREE(c.degree, (k2_sweep<K><<<std::min(grid, sweep2d_blocks<K> * h->num_sms), 256, 0, s>>>(a)))
         CK2(cudaGetLastError());
         if ((rc = solve2d(h))) return rc;
         CK2(cudaMemcpyAsync(h->h_bits, h->bits, 4 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, s));
