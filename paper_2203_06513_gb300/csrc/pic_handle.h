@@ -69,7 +69,7 @@ struct pic_handle {
     int32_t *counts = nullptr;
 
     // circulant bands and inverse taps
-    double *d_rowM0 = nullptr, *d_rowM1 = nullptr, *d_rowK = nullptr;
+    double *d_rowM0 = nullptr, *d_rowM1 = nullptr;
     double *d_tapM1 = nullptr, *d_tapP = nullptr;
     int tapM1_start = 0, tapM1_n = 0, tapP_start = 0, tapP_n = 0;
 

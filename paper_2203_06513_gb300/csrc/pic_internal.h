@@ -39,8 +39,8 @@ template <> struct SweepU<float> { static constexpr int v = 2; };
 //            256 x 2 (128)            992 /  770              128 x 5 (102)    - / 378
 //            128 x 7 (73)               - /  570              128 x 4 (128)  833 / 440
 //            128 x 5 (102)           1606 /  662              128 x 3 (170)  624 /   -
-// The double form is bound by the FP64 pipe and does not mind (1060 / 610 us for 1e7
-// markers at 16 warps, cubic).
+// The double form is bound by the FP64 pipe and does not mind (1057 / 318 us for 1e7
+// markers at 16 warps, cubic; 24 warps 1104 / 613 before the last change of sweep II).
 template <typename R, int K> struct SweepShape {
     static constexpr int threads1 = 256, blocks1 = 2, threads2 = 256, blocks2 = 2;
 };
@@ -374,10 +374,9 @@ int launch_cell_coefs(int M, int D, bool path, const double *c, double *tab, cud
 int launch_tables2(int M, int K, int fp32, const double *an_y, const double *an_z, const double *ak_y,
                    const double *ak_z, CoefTables T, cudaStream_t s);
 int launch_poisson_rhs(int M, double dx, const double *rho, double *d, cudaStream_t s);
-int launch_energy_grid(int M, int K, double dx, const double *rowM0, const double *rowM1,
-                       const double *rowK, const double *ex, const double *ey, const double *ez,
-                       const double *ay, const double *az, const double *rho, double *diag,
-                       cudaStream_t s);
+int launch_energy_grid(int M, int K, double dx, const double *rowM0, const double *rowM1, const double *ex,
+                       const double *ey, const double *ez, const double *ay, const double *az, const double *rho,
+                       double *diag, cudaStream_t s);
 int launch_ctrl_reset(DevCtrl *ctrl, cudaStream_t s);
 
 // learned warm start (pic_mlp.cu)
