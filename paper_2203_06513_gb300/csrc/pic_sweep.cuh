@@ -96,6 +96,7 @@ __device__ __forceinline__ void start_cache_load(const void *base, long long a, 
 //   cell polynomials, path moments h S_m in every cell visited  1680   2680
 //   end-point moments and knot counts, centred offsets, roots
 //   and quotients without exception paths, two markers a lane    992   1513
+//   double: path ends, moments and seeds off the FP64 pipe         -   1057
 // PRE: the predicted start instead of a sweep -- the proposal delta^(0) (the
 // explicit predictor when A.warm, else the one already in delta) is written back
 // and its path current deposited into A.mom; no gather walk, no momentum update.
@@ -387,7 +388,7 @@ __device__ __forceinline__ void sweep1_range(const Sweep1Args &A, long long beg,
 // us a launch, float (1e8 markers, cubic) and double (1e7): basis values and node windows
 // 1260 and 2060, cell polynomials and moments 767 and 830, as here (centred offsets, the
 // short root and quotient, two markers a lane) 570 and 672, with their seeds refined off the
-// FP64 pipe 610 in double.
+// FP64 pipe 610 in double, with the moments as 64-bit integers 318.
 // Z: the z component is not identically zero, as in subsystem I.
 // f = (s + L) / G, s = A^n + A^(k) of a component, G = g0 + g1, L the float form's residue.
 // The float rounding of a coefficient is the same for every marker of its cell, so it
@@ -432,15 +433,18 @@ __device__ __forceinline__ void sweep2_range_z(const Sweep2Args &A, long long be
     const bool keep = !Real<R>::fp32 && first && A.a0 != nullptr;
     const int lane = threadIdx.x & 31;
     if (beg >= end) return;
-    using Acc = typename AccOf<R, ACC>::T;
+    constexpr bool kFixed = !Real<R>::fp32 && ACC == ACC_NATIVE;
+    using Acc = typename std::conditional<kFixed, AccFixed, typename AccOf<R, ACC>::T>::type;
     MomentWindow<NW, NC, Acc> wy, wz;
     wy.clear();
     if (Z) wz.clear();
     int base = cp[beg], adds = 0;
     unsigned used = 0u;
+    int ewy = 0, ewz = 0;               // AccFixed: exponents of the windows' scales
+    double scy = 1.0, scz = 1.0;
     auto flush = [&]() {
-        wy.flush(my, base, used, M);
-        if (Z) wz.flush(mz, base, used, M);
+        wy.flush(my, base, used, M, scy);
+        if (Z) wz.flush(mz, base, used, M, scz);
         used = 0u;
         adds = 0;
     };
@@ -517,6 +521,8 @@ __device__ __forceinline__ void sweep2_range_z(const Sweep2Args &A, long long be
             exchange<R, Z>(A0y + A1y, A0z + A1z, g0 + root(q1), Ly, Lz, fy[u], fz[u]);
             rel[u] = rel_cell(cw[u], base, M);
             in[u] = act[u] && (unsigned)rel[u] < (unsigned)NW;
+            // infinities, NaN: to global memory as they are
+            if constexpr (kFixed) in[u] = in[u] && exponent_of(fy[u]) < 2000 && (!Z || exponent_of(fz[u]) < 2000);
             miss += __popc(__ballot_sync(0xffffffffu, act[u] && !in[u]));
         }
         if (miss > kWindowMisses) {
@@ -527,8 +533,8 @@ __device__ __forceinline__ void sweep2_range_z(const Sweep2Args &A, long long be
             int off = window_move<NW>(lo, rel[0], act[0], amask);
             if (off > 0 && off < NW) {
                 for (; off > 0; --off) {
-                    wy.shift(my, base, used);
-                    if (Z) wz.shift(mz, base, used);
+                    wy.shift(my, base, used, scy);
+                    if (Z) wz.shift(mz, base, used, scz);
                     used >>= 1;
                     base = base + 1 == M ? 0 : base + 1;
                 }
@@ -540,6 +546,18 @@ __device__ __forceinline__ void sweep2_range_z(const Sweep2Args &A, long long be
             for (int u = 0; u < U; ++u) {
                 rel[u] = rel_cell(cw[u], base, M);
                 in[u] = act[u] && (unsigned)rel[u] < (unsigned)NW;
+                if constexpr (kFixed) in[u] = in[u] && exponent_of(fy[u]) < 2000 && (!Z || exponent_of(fz[u]) < 2000);
+            }
+        }
+        if constexpr (kFixed) {
+            const int ey = __reduce_max_sync(0xffffffffu, in[0] ? exponent_of(fy[0]) : 0);
+            const int ez = Z ? __reduce_max_sync(0xffffffffu, in[0] ? exponent_of(fz[0]) : 0) : -1;
+            if (ey >= ewy || ez >= ewz) {
+                flush();
+                ewy = max(ewy, ey + 1);
+                ewz = max(ewz, ez + 1);
+                scy = exponent_scale(ewy);
+                scz = exponent_scale(ewz);
             }
         }
         unsigned bits = 0u;
@@ -549,30 +567,54 @@ __device__ __forceinline__ void sweep2_range_z(const Sweep2Args &A, long long be
         used |= mask;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            R x[NC], pw = one;
-            x[0] = fy[u];
-            R pws[NC];
-            pws[0] = one;
-#pragma unroll
-            for (int m = 1; m < NC; ++m) { pw = m == 1 ? v[u] : pw * v[u]; pws[m] = pw; x[m] = fy[u] * pw; }
             const int r = in[u] ? rel[u] : -1;
-            wy.add(mask, r, x);
-            if (act[u] && !in[u]) {
-                double *dst = my + (size_t)cw[u] * NC;
+            if constexpr (kFixed) {
+                const long long q = to_fixed(v[u]);
+                long long x[NC];
+                moments_fixed<NC>(in[u] ? to_fixed(fy[u], ewy) : 0, q, x);
+                wy.add(mask, r, x);
+                if (Z) {
+                    moments_fixed<NC>(in[u] ? to_fixed(fz[u], ewz) : 0, q, x);
+                    wz.add(mask, r, x);
+                }
+            } else {
+                R x[NC], pw = one;
+                x[0] = fy[u];
+                R pws[NC];
+                pws[0] = one;
 #pragma unroll
-                for (int m = 0; m < NC; ++m)
-                    if (x[m] != R(0)) atomicAdd(&dst[m], (double)x[m]);
-            }
-            if (Z) {
-                x[0] = fz[u];
-#pragma unroll
-                for (int m = 1; m < NC; ++m) x[m] = fz[u] * pws[m];
-                wz.add(mask, r, x);
+                for (int m = 1; m < NC; ++m) { pw = m == 1 ? v[u] : pw * v[u]; pws[m] = pw; x[m] = fy[u] * pw; }
+                wy.add(mask, r, x);
                 if (act[u] && !in[u]) {
-                    double *dst = mz + (size_t)cw[u] * NC;
+                    double *dst = my + (size_t)cw[u] * NC;
 #pragma unroll
                     for (int m = 0; m < NC; ++m)
                         if (x[m] != R(0)) atomicAdd(&dst[m], (double)x[m]);
+                }
+                if (Z) {
+                    x[0] = fz[u];
+#pragma unroll
+                    for (int m = 1; m < NC; ++m) x[m] = fz[u] * pws[m];
+                    wz.add(mask, r, x);
+                    if (act[u] && !in[u]) {
+                        double *dst = mz + (size_t)cw[u] * NC;
+#pragma unroll
+                        for (int m = 0; m < NC; ++m)
+                            if (x[m] != R(0)) atomicAdd(&dst[m], (double)x[m]);
+                    }
+                }
+            }
+            if constexpr (kFixed) {
+                if (act[u] && !in[u]) {
+                    double *dy = my + (size_t)cw[u] * NC, *dz = mz + (size_t)cw[u] * NC;
+                    R xy = fy[u], xz = Z ? fz[u] : R(0);
+#pragma unroll
+                    for (int m = 0; m < NC; ++m) {
+                        if (xy != R(0)) atomicAdd(&dy[m], (double)xy);
+                        if (Z && xz != R(0)) atomicAdd(&dz[m], (double)xz);
+                        xy *= v[u];
+                        if (Z) xz *= v[u];
+                    }
                 }
             }
         }
