@@ -88,12 +88,25 @@ int launch_sweep1(const Sweep1Args &a, int grid, cudaStream_t s)
     return 1;
 }
 
+// four consecutive markers' numbers (none beyond end)
+template <typename T>
+__device__ __forceinline__ void load4_to(const T *q, long long a, long long end, T (&v)[4])
+{
+    if (a + 4 <= end) {
+        load4(q + a, v);
+    } else {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = a + u < end ? q[a + u] : T(0);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Path-integrated current of given displacements (pic_deposit CURRENT): the
 // deposit half of the sweep above, in the form's precision.  A path inside one cell
 // has length d exactly, a path across knots ends at the offset of t0 + d.  Adding every
 // basis value to a shared-memory row by a double atomic (a compare-and-swap loop) took
-// 4.2 ms for 1e7 markers; the register window takes 0.32 ms.
+// 4.2 ms for 1e7 markers; the register window takes 0.32 ms, bound by the displacements'
+// scattered loads and the FP64 pipe.
 // ---------------------------------------------------------------------------
 // The deposit is the path's pieces cell by cell, h S_m in each (displacements may be tiny
 // here, which the difference of the end points' moments would not resolve).
@@ -238,7 +251,10 @@ int launch_sweep2(const Sweep2Args &a, int grid, cudaStream_t s)
 // ---------------------------------------------------------------------------
 // Diagnostics, evaluated in double from the stored state.
 // ---------------------------------------------------------------------------
-// charge moments sum_a v^m per cell
+// charge moments sum_a v^m per cell, as 64-bit integers (AccFixed; the count as 2^53, so a
+// lane adds at most kChargeAdds markers between flushes): with double sums the FP64 pipe
+// bounds it (1e7 float markers: 274 us, 85 now)
+constexpr int kChargeAdds = 512;
 template <int K, typename R>
 __global__ void __launch_bounds__(kSweepThreads) k_charge(DiagArgs A)
 {
@@ -248,16 +264,17 @@ __global__ void __launch_bounds__(kSweepThreads) k_charge(DiagArgs A)
     long long wb, we;
     grid_warp_chunk(A.np, wb, we);
     if (wb >= we) return;
-    MomentWindow<kWin2, K + 1, AccNative<double>> win;
+    MomentWindow<kWin2, K + 1, AccFixed> win;
     win.clear();
     int base = cp[wb];
     unsigned used = 0u;
+    int adds = 0;
     for (long long s = wb; s < we; s += 32) {
         const long long a = s + lane;
         const bool act = a < we;
         const unsigned amask = __ballot_sync(0xffffffffu, act);
         const int c = act ? cp[a] : 0;
-        const double v = act ? (double)vp[a] : 0.0;
+        const double v = act ? as_double(vp[a]) : 0.0;
         int rel = rel_cell(c, base, M);
         bool in = act && (unsigned)rel < (unsigned)kWin2;
         if (__popc(__ballot_sync(0xffffffffu, act && !in)) > kWindowMisses) {
@@ -278,15 +295,17 @@ __global__ void __launch_bounds__(kSweepThreads) k_charge(DiagArgs A)
         }
         const unsigned mask = __reduce_or_sync(0xffffffffu, in ? 1u << rel : 0u);
         used |= mask;
-        double x[K + 1];
-        x[0] = 1.0;
+        long long x[K + 1], y[K];
+        point_moments_fixed<K>(v, y);
+        x[0] = 1LL << 53;
 #pragma unroll
-        for (int m = 1; m <= K; ++m) x[m] = m == 1 ? v : x[m - 1] * v;
+        for (int m = 1; m <= K; ++m) x[m] = y[m - 1];
         win.add(mask, in ? rel : -1, x);
         if (act && !in) {
 #pragma unroll
-            for (int m = 0; m <= K; ++m) atomicAdd(&A.mom[(size_t)c * (K + 1) + m], x[m]);
+            for (int m = 0; m <= K; ++m) atomicAdd(&A.mom[(size_t)c * (K + 1) + m], (double)x[m] * 1.1102230246251565e-16);
         }
+        if (++adds == kChargeAdds) { win.flush(A.mom, base, used, M); used = 0u; adds = 0; }
     }
     win.flush(A.mom, base, used, M);
 }
@@ -300,7 +319,7 @@ __global__ void __launch_bounds__(256) k_gather(DiagArgs A)
     for (long long a = (long long)blockIdx.x * blockDim.x + threadIdx.x; a < A.np; a += stride) {
         double c[D + 1];
         load_coef<D + 1>(A.tab + (size_t)A.P.cell[a] * CoefPad<double, D + 1>::v, c);
-        A.out[A.P.id[a]] = horner<D + 1>(c, (double)tp[a]);
+        A.out[A.P.id[a]] = horner<D + 1>(c, as_double(tp[a]));
     }
 }
 
@@ -315,7 +334,7 @@ __global__ void __launch_bounds__(256) k_kinetic(DiagArgs A)
     for (long long a = (long long)blockIdx.x * blockDim.x + threadIdx.x; a < A.np; a += stride) {
         const int c = A.P.cell[a];
         double v[K + 1];
-        bspline_vals<K, double>((double)tp[a] + 0.5, v);
+        bspline_vals<K, double>(as_double(tp[a]) + 0.5, v);
         double Ay = 0.0, Az = 0.0;
 #pragma unroll
         for (int r = 0; r <= K; ++r) {
@@ -325,7 +344,7 @@ __global__ void __launch_bounds__(256) k_kinetic(DiagArgs A)
         }
         const double p = as_double(pp[a]);
         const double q = p * p + Ay * Ay + Az * Az;
-        acc += A.w * q / (1.0 + sqrt(1.0 + q));      // w (gamma - 1) without cancellation
+        acc += quotient(A.w * q, 1.0 + root(1.0 + q));      // w (gamma - 1) without cancellation
     }
     block_sum_to(A.acc, acc, s_red);
 }
@@ -372,7 +391,8 @@ int launch_gather(const DiagArgs &a, int d, int grid, int block, cudaStream_t s)
 // (1/dt) int Lambda_1(X(tau)) dtau . e of subsystem I), in double: the path is
 // split at the knots and each piece contributes (h/d) sum_m E_m S_m (A.tab holds
 // E_m / (m + 1)); a zero displacement gives E_x,h(x_a).  On entry
-// out[id] holds d (length units); it is overwritten with the mean.
+// out[id] holds d (length units); it is overwritten with the mean.  Bound by the FP64 pipe:
+// 32 operations a marker took 604 us for 1e7 float markers, cubic; 450 us now.
 template <int K, typename R>
 __global__ void __launch_bounds__(256) k_gather_path(DiagArgs A)
 {
@@ -380,34 +400,45 @@ __global__ void __launch_bounds__(256) k_gather_path(DiagArgs A)
     bool bad = false;
     constexpr int PE = CoefPad<double, K>::v;
     const double inv = 1.0 / A.dx;
+    const long long lim = __double_as_longlong((double)A.Dlim);
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long a = (long long)blockIdx.x * blockDim.x + threadIdx.x; a < A.np; a += stride) {
         int g = A.P.cell[a];
         const int id = A.P.id[a];
         const double d = A.out[id] * inv;
-        if (!(fabs(d) <= (double)A.Dlim)) { bad = true; A.out[id] = 0.0; continue; }
-        const double v0 = (double)tp[a];
+        // |d| <= Dlim, as integers (a NaN is larger)
+        if ((__double_as_longlong(d) & LLONG_MAX) > lim) { bad = true; A.out[id] = 0.0; continue; }
+        const double v0 = as_double(tp[a]);
         int n;
         double v1;
         path_end(v0, d, n, v1);
         const int an = abs(n);
         const bool right = n > 0;
-        double sum = 0.0, W = 0.0;
-        for (int q = 0; q <= an; ++q) {
-            const double va = q == 0 ? v0 : (right ? -0.5 : 0.5);
-            const double vb = q == an ? v1 : (right ? 0.5 : -0.5);
-            double S[K], c[K];
-            path_sums<K, double>(va, vb, S);
-            load_coef<K>(A.tab + (size_t)g * PE, c);
-            double e = c[0];
+        const double edge = right ? 0.5 : -0.5;
+        double S[K], c[K];
+        const double vb = an == 0 ? v1 : edge;
+        path_sums<K, double>(v0, vb, S);
+        load_coef<K>(A.tab + (size_t)g * PE, c);
+        double e = c[0];
 #pragma unroll
-            for (int m = 1; m < K; ++m) e = fma(c[m], S[m], e);
-            const double h = an == 0 ? 1.0 : vb - va;
-            sum = fma(h, e, sum);
-            W += h;
-            g = wrap_once(g + (right ? 1 : -1), A.M);
+        for (int m = 1; m < K; ++m) e = fma(c[m], S[m], e);
+        if (an > 0) {
+            double W = vb - v0, sum = W * e;
+            for (int q = 1; q <= an; ++q) {
+                g = wrap_once(g + (right ? 1 : -1), A.M);
+                const double ve = q == an ? v1 : edge;
+                edge_sums<K, double>(right, -edge, ve, S);
+                load_coef<K>(A.tab + (size_t)g * PE, c);
+                e = c[0];
+#pragma unroll
+                for (int m = 1; m < K; ++m) e = fma(c[m], S[m], e);
+                const double h = ve + edge;
+                sum = fma(h, e, sum);
+                W += h;
+            }
+            e = quotient(sum, W);
         }
-        A.out[id] = an == 0 ? sum : sum / W;
+        A.out[id] = e;
     }
     if (bad) atomicOr(A.status, STATUS_NUMERIC);
 }
@@ -696,18 +727,6 @@ int launch_store_state(int fp32, long long np, int M, double dx, PartPtrs P, con
     if (fp32) k_store_state<float><<<grid, block, 0, s>>>(np, M, dx, P, o);
     else k_store_state<double><<<grid, block, 0, s>>>(np, M, dx, P, o);
     return 0;
-}
-
-// four consecutive markers' numbers (none beyond end)
-template <typename T>
-__device__ __forceinline__ void load4_to(const T *q, long long a, long long end, T (&v)[4])
-{
-    if (a + 4 <= end) {
-        load4(q + a, v);
-    } else {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = a + u < end ? q[a + u] : T(0);
-    }
 }
 
 // Stored order to caller order for more markers than L2 holds outputs for.  Scattered
