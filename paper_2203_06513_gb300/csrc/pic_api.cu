@@ -139,7 +139,6 @@ static void release(pic_handle *h)
     f(h->T.A); f(h->T.E); f(h->T.Kt); f(h->T.L);
     for (int m = 0; m < kMaxStartOrder; ++m) { f(h->fh.x[m]); f(h->fh.y[m]); f(h->fh.z[m]); }
     cudaStreamSynchronize(s);
-    if (h->h_flag) cudaFreeHost(h->h_flag);
     if (h->h_ctrl) cudaFreeHost(h->h_ctrl);
     if (h->h_count) cudaFreeHost(h->h_count);
     if (h->cap) cudaStreamDestroy(h->cap);
@@ -474,7 +473,6 @@ extern "C" int pic_init_split(const pic_config *cfg, const pic_arrays *in, int32
     }
     if ((rc = dalloc(h, &h->counts, sort_counts(M * kVelBinsBase * bins_per_cell((long long)np, (int)M))))) return bail(rc);
     if ((rc = dalloc(h, &h->ctrl, 1))) return bail(rc);
-    if (cudaMallocHost((void **)&h->h_flag, sizeof(int)) != cudaSuccess) return bail(PIC_ERR_NOMEM);
     if (cudaMallocHost((void **)&h->h_ctrl, sizeof(DevCtrl)) != cudaSuccess) return bail(PIC_ERR_NOMEM);
 
     // circulant bands: M0 (degree k), M1 (degree k-1), K = G^T M1 G, P = M0 + dt^2/4 K

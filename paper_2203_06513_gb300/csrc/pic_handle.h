@@ -76,7 +76,6 @@ struct pic_handle {
     CoefTables T{};                 // cell polynomials of the sweeps' fields
     pic::FieldHist fh{};            // field changes of the last solves (starting fields)
     DevCtrl *ctrl = nullptr;
-    int *h_flag = nullptr;          // pinned: converged flag readback
     DevCtrl *h_ctrl = nullptr;      // pinned: full control block readback
 
     int grid1 = 0, grid2 = 0;       // blocks of the sweeps of subsystems I and II
