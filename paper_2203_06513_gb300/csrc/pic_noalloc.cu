@@ -15,7 +15,7 @@
 // result; order them on one stream.
 //
 // The markers come in any order, so their moments go straight to the scratch by double
-// additions in L2, K per path piece, which is what bounds the call: 104 us for 1e6 markers
+// additions in L2, K per path piece, which is what bounds the call: 91 us for 1e6 markers
 // on 1000 cells, reach 1.5 cells, degree 3.  (Rows of nodes per block in shared memory,
 // where a double addition is a compare-and-swap loop, and one thread per node to add the
 // rows: 529 us.)

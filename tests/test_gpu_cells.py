@@ -222,3 +222,24 @@ def test_2d_large_state_copy():
     np.testing.assert_array_equal(st["p"], p)
     assert np.max(np.abs(st["x"] - x)) < 4e-15                      # cell + offset, a few roundings of L
     g.close()
+
+
+@pytest.mark.parametrize("nx,k,n", [(65, 2, 1), (65, 3, 3001), (40, 5, 2050)])
+def test_scaled_moments_of_uneven_fields(nx, k, n, monkeypatch):
+    """The double form's sweeps (driven from the host) on potentials that differ by ten
+    orders of magnitude between neighbouring nodes, markers in no order: a warp raises its
+    scale many times.  Against the oracle to the parity tests' tolerances."""
+    monkeypatch.setenv("PIC_NO_GRAPH", "1")
+    w = I.Workload("u", nx=nx, degree=k, np=n, dt=0.02, vth=0.1, pump=0.1, seed=nx + k)
+    x, p = I.particles(w)
+    _, _, ey, ez = I.fields(w)
+    rng = np.random.default_rng(n)
+    ay, az = (0.1 * rng.choice([-1, 1], nx) * 10.0 ** rng.uniform(-10, 0, nx) for _ in range(2))
+    orc = O.Oracle(w.L, nx, k, w.weight, w.dt, w.tol, 200)
+    s = O.initial_state(orc, x, p, ay, az, ey, ez)
+    g = pic.Pic(pic.Config.from_workload(w, sort_every=0, max_iter=200), x, p, ay, az, ey, ez)
+    for _ in range(2):
+        s = orc.step(s)
+    g.step(2)
+    _check(g.state_numpy(), s, w.L, 1e-11, 1e-10)
+    g.close()
