@@ -275,8 +275,9 @@ __global__ void __launch_bounds__(kSweepThreads) k_charge(DiagArgs A)
         const unsigned amask = __ballot_sync(0xffffffffu, act);
         const int c = act ? cp[a] : 0;
         const double v = act ? as_double(vp[a]) : 0.0;
+        const bool num = is_offset(v);          // what is none goes to global memory as it is
         int rel = rel_cell(c, base, M);
-        bool in = act && (unsigned)rel < (unsigned)kWin2;
+        bool in = act && num && (unsigned)rel < (unsigned)kWin2;
         if (__popc(__ballot_sync(0xffffffffu, act && !in)) > kWindowMisses) {
             int off = window_move<kWin2>(rel, rel, act, amask);
             if (off > 0 && off < kWin2) {
@@ -291,7 +292,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_charge(DiagArgs A)
                 base = wrap_cell(base + off, M);
             }
             rel = rel_cell(c, base, M);
-            in = act && (unsigned)rel < (unsigned)kWin2;
+            in = act && num && (unsigned)rel < (unsigned)kWin2;
         }
         const unsigned mask = __reduce_or_sync(0xffffffffu, in ? 1u << rel : 0u);
         used |= mask;
@@ -302,8 +303,12 @@ __global__ void __launch_bounds__(kSweepThreads) k_charge(DiagArgs A)
         for (int m = 1; m <= K; ++m) x[m] = y[m - 1];
         win.add(mask, in ? rel : -1, x);
         if (act && !in) {
+            double pw = 1.0;
 #pragma unroll
-            for (int m = 0; m <= K; ++m) atomicAdd(&A.mom[(size_t)c * (K + 1) + m], (double)x[m] * 1.1102230246251565e-16);
+            for (int m = 0; m <= K; ++m) {
+                atomicAdd(&A.mom[(size_t)c * (K + 1) + m], pw);
+                pw *= v;
+            }
         }
         if (++adds == kChargeAdds) { win.flush(A.mom, base, used, M); used = 0u; adds = 0; }
     }

@@ -78,6 +78,21 @@ def test_current_of_a_position_that_is_not_finite(precision, bad, k):
     g.close()
 
 
+@pytest.mark.parametrize("precision", FORMS)
+@pytest.mark.parametrize("bad", BAD)
+@pytest.mark.parametrize("k", [2, 5])
+def test_charge_of_a_position_that_is_not_finite(precision, bad, k):
+    """Its nodes are NaN, and with them the field of the discrete Poisson equation."""
+    w, x, p, ay, az, ey, ez = _inputs(500, k, bad)
+    g = pic.Pic(pic.Config.from_workload(w, precision=precision), x, p, ay, az, ey, ez)
+    out = torch.zeros(w.nx, dtype=torch.float64, device="cuda")
+    g.deposit(pic.PIC_DEP_CHARGE, None, out)
+    assert np.count_nonzero(np.isnan(out.cpu().numpy())) == k + 1
+    assert not np.any(np.isfinite(g.state_numpy()["ex"]))
+    assert np.isnan(g.energy()["ex"])
+    g.close()
+
+
 @pytest.mark.parametrize("bad", BAD)
 @pytest.mark.parametrize("warm", [0, 1])
 def test_2d_substep_reports_positions_that_are_not_finite(bad, warm):
