@@ -251,10 +251,8 @@ int launch_sweep2(const Sweep2Args &a, int grid, cudaStream_t s)
 // ---------------------------------------------------------------------------
 // Diagnostics, evaluated in double from the stored state.
 // ---------------------------------------------------------------------------
-// charge moments sum_a v^m per cell, as 64-bit integers (AccFixed; the count as 2^53, so a
-// lane adds at most kChargeAdds markers between flushes): with double sums the FP64 pipe
-// bounds it (1e7 float markers: 274 us, 85 now)
-constexpr int kChargeAdds = 512;
+// charge moments sum_a v^m per cell, halved, as 64-bit integers (AccFixed): with double sums
+// the FP64 pipe bounds it (1e7 float markers: 274 us, 85 now)
 template <int K, typename R>
 __global__ void __launch_bounds__(kSweepThreads) k_charge(DiagArgs A)
 {
@@ -282,12 +280,12 @@ __global__ void __launch_bounds__(kSweepThreads) k_charge(DiagArgs A)
             int off = window_move<kWin2>(rel, rel, act, amask);
             if (off > 0 && off < kWin2) {
                 for (; off > 0; --off) {
-                    win.shift(A.mom, base, used);
+                    win.shift(A.mom, base, used, 2.0);
                     used >>= 1;
                     base = base + 1 == M ? 0 : base + 1;
                 }
             } else if (off != 0) {
-                win.flush(A.mom, base, used, M);
+                win.flush(A.mom, base, used, M, 2.0);
                 used = 0u;
                 base = wrap_cell(base + off, M);
             }
@@ -298,7 +296,7 @@ __global__ void __launch_bounds__(kSweepThreads) k_charge(DiagArgs A)
         used |= mask;
         long long x[K + 1], y[K];
         point_moments_fixed<K>(v, y);
-        x[0] = 1LL << 53;
+        x[0] = 1LL << 55;
 #pragma unroll
         for (int m = 1; m <= K; ++m) x[m] = y[m - 1];
         win.add(mask, in ? rel : -1, x);
@@ -310,9 +308,9 @@ __global__ void __launch_bounds__(kSweepThreads) k_charge(DiagArgs A)
                 pw *= v;
             }
         }
-        if (++adds == kChargeAdds) { win.flush(A.mom, base, used, M); used = 0u; adds = 0; }
+        if (++adds == kFixedAdds) { win.flush(A.mom, base, used, M, 2.0); used = 0u; adds = 0; }
     }
-    win.flush(A.mom, base, used, M);
+    win.flush(A.mom, base, used, M, 2.0);
 }
 
 // A.tab: the field's polynomial of each cell in double (launch_cell_coefs)

@@ -391,7 +391,8 @@ __device__ __forceinline__ void sweep1_range(const Sweep1Args &A, long long beg,
 // us a launch, float (1e8 markers, cubic) and double (1e7): basis values and node windows
 // 1260 and 2060, cell polynomials and moments 767 and 830, as here (centred offsets, the
 // short root and quotient, two markers a lane) 570 and 672, with their seeds refined off the
-// FP64 pipe 610 in double, with the moments as 64-bit integers 318.
+// FP64 pipe 610 in double, with the moments as 64-bit integers 318 (one scale a warp, which
+// took the digits of weak fields in its range; 323 with a scale a cell).
 // Z: the z component is not identically zero, as in subsystem I.
 // f = (s + L) / G, s = A^n + A^(k) of a component, G = g0 + g1, L the float form's residue.
 // The float rounding of a coefficient is the same for every marker of its cell, so it
@@ -437,17 +438,15 @@ __device__ __forceinline__ void sweep2_range_z(const Sweep2Args &A, long long be
     const int lane = threadIdx.x & 31;
     if (beg >= end) return;
     constexpr bool kFixed = !Real<R>::fp32 && ACC == ACC_NATIVE;
-    using Acc = typename std::conditional<kFixed, AccFixed, typename AccOf<R, ACC>::T>::type;
-    MomentWindow<NW, NC, Acc> wy, wz;
+    using Window = typename std::conditional<kFixed, ScaledWindow<NW, NC>, MomentWindow<NW, NC, typename AccOf<R, ACC>::T>>::type;
+    Window wy, wz;
     wy.clear();
     if (Z) wz.clear();
     int base = cp[beg], adds = 0;
     unsigned used = 0u;
-    int ewy = 0, ewz = 0;               // AccFixed: exponents of the windows' scales
-    double scy = 1.0, scz = 1.0;
     auto flush = [&]() {
-        wy.flush(my, base, used, M, scy);
-        if (Z) wz.flush(mz, base, used, M, scz);
+        wy.flush(my, base, used, M);
+        if (Z) wz.flush(mz, base, used, M);
         used = 0u;
         adds = 0;
     };
@@ -536,8 +535,8 @@ __device__ __forceinline__ void sweep2_range_z(const Sweep2Args &A, long long be
             int off = window_move<NW>(lo, rel[0], act[0], amask);
             if (off > 0 && off < NW) {
                 for (; off > 0; --off) {
-                    wy.shift(my, base, used, scy);
-                    if (Z) wz.shift(mz, base, used, scz);
+                    wy.shift(my, base, used);
+                    if (Z) wz.shift(mz, base, used);
                     used >>= 1;
                     base = base + 1 == M ? 0 : base + 1;
                 }
@@ -552,34 +551,17 @@ __device__ __forceinline__ void sweep2_range_z(const Sweep2Args &A, long long be
                 if constexpr (kFixed) in[u] = in[u] && exponent_of(fy[u]) < 2000 && (!Z || exponent_of(fz[u]) < 2000);
             }
         }
-        if constexpr (kFixed) {
-            const int ey = __reduce_max_sync(0xffffffffu, in[0] ? exponent_of(fy[0]) : 0);
-            const int ez = Z ? __reduce_max_sync(0xffffffffu, in[0] ? exponent_of(fz[0]) : 0) : -1;
-            if (ey >= ewy || ez >= ewz) {
-                flush();
-                ewy = max(ewy, ey + 1);
-                ewz = max(ewz, ez + 1);
-                scy = exponent_scale(ewy);
-                scz = exponent_scale(ewz);
-            }
-        }
         unsigned bits = 0u;
 #pragma unroll
         for (int u = 0; u < U; ++u) bits |= in[u] ? 1u << rel[u] : 0u;
         const unsigned mask = __reduce_or_sync(0xffffffffu, bits);
-        used |= mask;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
             const int r = in[u] ? rel[u] : -1;
             if constexpr (kFixed) {
-                const long long q = to_fixed(v[u]);
-                long long x[NC];
-                moments_fixed<NC>(in[u] ? to_fixed(fy[u], ewy) : 0, q, x);
-                wy.add(mask, r, x);
-                if (Z) {
-                    moments_fixed<NC>(in[u] ? to_fixed(fz[u], ewz) : 0, q, x);
-                    wz.add(mask, r, x);
-                }
+                const long long q = to_fixed<63>(v[u]);
+                wy.add(my, base, used, M, mask, r, fy[u], q);
+                if (Z) wz.add(mz, base, used, M, mask, r, fz[u], q);
             } else {
                 R x[NC], pw = one;
                 x[0] = fy[u];
@@ -621,7 +603,8 @@ __device__ __forceinline__ void sweep2_range_z(const Sweep2Args &A, long long be
                 }
             }
         }
-        if (++adds == kMaxLaneAdds / U) flush();
+        used |= mask;
+        if (++adds == (kFixed ? kFixedAdds : kMaxLaneAdds) / U) flush();
     }
     flush();
 }
