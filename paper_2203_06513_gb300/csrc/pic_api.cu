@@ -128,7 +128,7 @@ static void release(pic_handle *h)
     f(h->spx); f(h->spy); f(h->spz); f(h->sdy); f(h->sdz); f(h->red);
     double *arr[] = {h->ex, h->ey, h->ez, h->ay, h->az, h->ek, h->ebar,
                      h->eky, h->ekz, h->aky, h->akz, h->by, h->bz, h->m0, h->mdep, h->gtab, h->rho,
-                     h->work, h->diag, h->d_rowM0, h->d_rowM1,
+                     h->work, h->diag, h->node, h->d_rowM0, h->d_rowM1,
                      h->d_tapM1, h->d_tapP};
     for (double *a : arr) f(a);
     f(h->counts);
@@ -522,6 +522,9 @@ extern "C" int pic_init_split(const pic_config *cfg, const pic_arrays *in, int32
         taps[-h->tapP_start] += r / m[0];
     }
     if ((rc = dalloc(h, &h->d_tapP, h->tapP_n))) return bail(rc);
+    // split runs form the nodes for their sums over the processes anyway
+    h->node_pass = !reduce_fn && conv_node_ops(h->M, K, h->tapP_n) >= kNodePassOps;
+    if (!reduce_fn && (rc = dalloc(h, &h->node, 2 * M))) return bail(rc);
     if (cudaMemcpy(h->d_tapP, taps.data(), sizeof(double) * h->tapP_n, cudaMemcpyHostToDevice) != cudaSuccess)
         return bail(PIC_ERR_CUDA);
 
@@ -757,6 +760,7 @@ ConvArgs pic::make_conv2_args(pic_handle *h)
     c.max_iter = h->cfg.max_iter; c.fp32 = h->fp32; c.subsystem = 2; c.ctrl = h->ctrl;
     c.pair[0][0] = h->my[0]; c.pair[0][1] = h->my[1];
     c.pair[1][0] = h->mz[0]; c.pair[1][1] = h->mz[1];
+    if (h->node_pass) { c.node[0] = h->node; c.node[1] = h->node + h->M; }
     return c;
 }
 
@@ -893,6 +897,7 @@ static int substep2(pic_handle *h, int *iters)
         if ((rc = timed_begin(h))) return rc;
         if (launch_conv(c, h->stream)) return fail(h, PIC_ERR_CUDA, "k_conv shared-memory opt-in failed");
         CKL_N("launch_conv");
+        if (c.node[0]) ++h->launches;
         if ((rc = timed_end(h, 2))) return rc;
         ++it;
         if ((rc = read_ctrl(h))) return rc;
@@ -1181,7 +1186,7 @@ static int step_graphs(pic_handle *h, int nsteps, long long *s1, long long *s2)
     if ((rc = read_ctrl(h))) return rc;
     *s1 = h->h_count[0];
     *s2 = h->h_count[1];
-    h->launches += 2 * (*s1 + *s2);
+    h->launches += 2 * (*s1 + *s2) + (h->node_pass ? *s2 : 0);
     h->marker_sweeps += *s1 * h->np;
     for (int which = 1; which <= 2; ++which)
         if ((rc = check_status(h, which))) return rc;

@@ -55,6 +55,7 @@ struct pic_ensemble {
     int *h_buf = nullptr;               // pinned readback: sweeps (2 nruns), status (nruns), Q fields
 
     int grid1 = 1, grid2 = 1;           // launch grids of the sweeps: SMs x resident blocks
+    bool node_pass = false;             // subsystem II's nodes in a pass before its solves
     int bps_max = 1;                    // blocks per SM of the schedule: the smaller of both
     int item_markers = 65536, bps = 1;  // schedule (the autotuner's choice)
     int fin_grid = 1;
@@ -142,8 +143,11 @@ static void build_tables(pic_ensemble *e)
 
         e->a2[r] = make_sweep2_args(h);
         e->a2[r].graph = 1;
-        e->c2[r] = make_conv2_args(h);
-        e->c2[r].graph = 1;
+        ConvArgs &d = e->c2[r];
+        d = make_conv2_args(h);
+        d.graph = 1;
+        // all runs or none: by the work of all of them
+        for (int k = 0; k < 2; ++k) d.node[k] = e->node_pass ? h->node + (size_t)k * h->M : nullptr;
 
         e->er[r].np = h->np;
         e->er[r].ctrl = h->ctrl;
@@ -180,11 +184,11 @@ static int loop_body(pic_ensemble *e, int which, cudaStream_t s, unsigned long l
     ELAUNCH(launch_ens_plan(e->d_q, e->d_er, e->nruns, cond, s), "ensemble plan");
     if (which == 1) {
         ELAUNCH(launch_sweep1_ens(e->K, e->fp32, e->d_a1, e->nruns, e->d_q, e->grid1, s), "ensemble sweep I");
-        ELAUNCH(launch_conv_ens(e->d_c1, e->nruns, e->Mmax, e->K, 1, e->ntap1, e->d_q, e->d_sweeps, cond, s),
+        ELAUNCH(launch_conv_ens(e->d_c1, e->nruns, e->Mmax, e->K, 1, e->ntap1, false, e->d_q, e->d_sweeps, cond, s),
                 "ensemble solve I");
     } else {
         ELAUNCH(launch_sweep2_ens(e->K, e->fp32, e->d_a2, e->nruns, e->d_q, e->grid2, s), "ensemble sweep II");
-        ELAUNCH(launch_conv_ens(e->d_c2, e->nruns, e->Mmax, e->K, 2, e->ntap2, e->d_q, e->d_sweeps, cond, s),
+        ELAUNCH(launch_conv_ens(e->d_c2, e->nruns, e->Mmax, e->K, 2, e->ntap2, e->node_pass, e->d_q, e->d_sweeps, cond, s),
                 "ensemble solve II");
     }
     return PIC_OK;
@@ -199,7 +203,7 @@ static int seg_prep1(pic_ensemble *e, cudaStream_t s)
         ELAUNCH(launch_ens_plan(e->d_q, e->d_er, e->nruns, 0ull, s), "ensemble plan");
         ELAUNCH(launch_predeposit_ens(e->K, e->fp32, e->d_a1p, e->nruns, e->d_q, e->grid1, s),
                 "ensemble predicted start");
-        ELAUNCH(launch_conv_ens(e->d_c1p, e->nruns, e->Mmax, e->K, 1, e->ntap1, e->d_q, e->d_sweeps, 0ull, s),
+        ELAUNCH(launch_conv_ens(e->d_c1p, e->nruns, e->Mmax, e->K, 1, e->ntap1, false, e->d_q, e->d_sweeps, 0ull, s),
                 "ensemble start field");
     }
     return PIC_OK;
@@ -365,14 +369,16 @@ extern "C" int pic_ensemble_create(const pic_config *cfgs, const pic_arrays *ins
     e->K = h0->K;
     e->fp32 = h0->fp32;
     e->num_sms = h0->num_sms;
-    long long npmax = 0, total = 0;
+    long long npmax = 0, total = 0, node_ops = 0;
     for (pic_handle *h : e->runs) {
         total += h->np;
+        node_ops += conv_node_ops(h->M, h->K, h->tapP_n);
         e->Mmax = std::max(e->Mmax, h->M);
         e->ntap1 = std::max(e->ntap1, h->tapM1_n);
         e->ntap2 = std::max(e->ntap2, h->tapP_n);
         npmax = std::max(npmax, h->np);
     }
+    e->node_pass = node_ops >= kNodePassOps;
     e->fin_grid = (int)std::min<long long>(std::max<long long>((npmax + 255) / 256, 1), 64);
     {
         const int b1 = sweep_blocks_per_sm(e->K, e->fp32, e->fp32 ? ACC_COMP : ACC_NATIVE, 1);
@@ -403,7 +409,7 @@ extern "C" int pic_ensemble_create(const pic_config *cfgs, const pic_arrays *ins
     if (cudaMemsetAsync(e->d_q, 0, sizeof(EnsQueue), e->stream) != cudaSuccess ||
         cudaMemsetAsync(e->d_sweeps, 0, 2 * n * sizeof(int), e->stream) != cudaSuccess)
         return bail(PIC_ERR_CUDA);
-    if (conv_ens_optin(e->K, std::max(e->ntap1, e->ntap2)))
+    if (conv_ens_optin(e->K, e->ntap1, e->ntap2, e->node_pass))
         return bail(efail(e, PIC_ERR_CUDA, "solve kernel shared-memory opt-in failed"));
     build_tables(e);
     if ((rc = upload_tables(e)) || (rc = upload_schedule(e))) return bail(rc);
@@ -483,7 +489,8 @@ extern "C" int pic_ensemble_step(pic_ensemble *e, int32_t nsteps, int64_t *sweep
     {
         const long long l1 = e->h_buf[3 * n], l2 = e->h_buf[3 * n + 1];
         e->launches += (long long)nsteps * (kStepLaunches + (e->warm_field ? kStartLaunches : 0)) +
-                       kLoopLaunches * ((l1 - e->loops_seen[0]) + (l2 - e->loops_seen[1]));
+                       kLoopLaunches * ((l1 - e->loops_seen[0]) + (l2 - e->loops_seen[1])) +
+                       (e->node_pass ? l2 - e->loops_seen[1] : 0);
         e->loops_seen[0] = l1;
         e->loops_seen[1] = l2;
     }

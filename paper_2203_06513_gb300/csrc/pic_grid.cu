@@ -162,7 +162,7 @@ template <int K>
 __global__ void __launch_bounds__(kConvThreads) k_conv(ConvArgs A)
 {
     extern __shared__ __align__(16) double s_conv[];
-    conv_block<K>(A, A.T, conv_iter(A), blockIdx.x, blockIdx.y, s_conv, nullptr);
+    conv_block<K>(A, A.node[blockIdx.y], A.T, conv_iter(A), blockIdx.x, blockIdx.y, s_conv, nullptr);
 }
 
 // Batched solves of an ensemble: block (bx, run, comp).  Runs that are not in
@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(kConvThreads) k_conv_ens(const ConvArgs *runs,
     const ConvArgs &A = runs[r];
     if (A.mode != CONV_PLAIN && !Q->active[r]) return;
     if (comp >= A.ncomp || (int)blockIdx.x * (kConvOut - K) >= A.M) return;
-    const bool last = conv_block<K>(A, A.T, conv_iter(A), blockIdx.x, comp, s_conv, nullptr);
+    const bool last = conv_block<K>(A, A.node[comp], A.T, conv_iter(A), blockIdx.x, comp, s_conv, nullptr);
     if (!last || threadIdx.x != 0) return;
     atomicAdd(&sweeps[2 * r + A.subsystem - 1], 1);
     if (!A.ctrl->converged) atomicAdd(&Q->n_continue, 1);
@@ -191,6 +191,28 @@ __global__ void __launch_bounds__(kConvThreads) k_conv_ens(const ConvArgs *runs,
         Q->loops[A.subsystem - 1] += 1;
         if (cond) cudaGraphSetConditional((cudaGraphConditionalHandle)cond, (unsigned)go);
     }
+}
+
+// The nodes of a solve of subsystem II, each formed once (ConvArgs::node).
+constexpr int kNodeThreads = 64;
+
+template <int K>
+__global__ void __launch_bounds__(kNodeThreads) k_nodes(ConvArgs A)
+{
+    node_pass<K>(A, conv_iter(A), blockIdx.x * kNodeThreads + threadIdx.x, blockIdx.y);
+}
+
+template <int K>
+__global__ void __launch_bounds__(kNodeThreads) k_nodes_ens(const ConvArgs *runs, const EnsQueue *Q)
+{
+    if (!Q->active[blockIdx.y]) return;
+    const ConvArgs &A = runs[blockIdx.y];
+    node_pass<K>(A, conv_iter(A), blockIdx.x * kNodeThreads + threadIdx.x, blockIdx.z);
+}
+
+long long conv_node_ops(int M, int K, int ntap)
+{
+    return 2LL * conv_blocks(M, K) * (kConvOut + ntap - 1) * (K + 1) * (K + 1);
 }
 
 // Raises a solve kernel's dynamic shared-memory limit (never lowers it).  Inverse rows
@@ -210,17 +232,22 @@ static int conv_optin(const void *fn, size_t smem, size_t &opted)
 static size_t g_conv_ens_opted[kMaxDegree + 1];
 
 // raise the shared-memory limit of k_conv_ens before any capture of it
-int conv_ens_optin(int K_, int ntap_max)
+int conv_ens_optin(int K_, int ntap1, int ntap2, bool nodes)
 {
-    PIC_FOR_DEGREE(K_, return conv_optin((const void *)k_conv_ens<K>, conv_smem(K, ntap_max), g_conv_ens_opted[K]))
+    const size_t smem = std::max(conv_smem(K_, ntap1, false), conv_smem(K_, ntap2, nodes));
+    PIC_FOR_DEGREE(K_, return conv_optin((const void *)k_conv_ens<K>, smem, g_conv_ens_opted[K]))
     return 1;
 }
 
-int launch_conv_ens(const ConvArgs *runs, int nruns, int Mmax, int K_, int ncomp, int ntap_max, EnsQueue *Q,
+int launch_conv_ens(const ConvArgs *runs, int nruns, int Mmax, int K_, int ncomp, int ntap_max, bool nodes, EnsQueue *Q,
                     int *sweeps, unsigned long long cond, cudaStream_t s)
 {
-    const size_t smem = conv_smem(K_, ntap_max);
+    const size_t smem = conv_smem(K_, ntap_max, nodes);
     if (smem > 48 * 1024 && smem > g_conv_ens_opted[K_]) return 1;   // conv_ens_optin first
+    if (nodes) {
+        const dim3 ngrid((Mmax + kNodeThreads - 1) / kNodeThreads, nruns, ncomp);
+        PIC_FOR_DEGREE(K_, (k_nodes_ens<K><<<ngrid, kNodeThreads, 0, s>>>(runs, Q)))
+    }
     dim3 grid(conv_blocks(Mmax, K_), nruns, ncomp);
     PIC_FOR_DEGREE(K_, (k_conv_ens<K><<<grid, kConvThreads, smem, s>>>(runs, Q, sweeps, cond)))
     return 0;
@@ -228,11 +255,12 @@ int launch_conv_ens(const ConvArgs *runs, int nruns, int Mmax, int K_, int ncomp
 
 int launch_conv(const ConvArgs &a, cudaStream_t s)
 {
-    const size_t smem = conv_smem(a.K, a.ntap);
+    const size_t smem = conv_smem(a.K, a.ntap, a.node[0] != nullptr);
     static size_t opted[kMaxDegree + 1];   // largest dynamic shared memory opted in so far
-    const dim3 grid(conv_blocks(a.M, a.K), a.ncomp);
+    const dim3 grid(conv_blocks(a.M, a.K), a.ncomp), ngrid((a.M + kNodeThreads - 1) / kNodeThreads, a.ncomp);
     PIC_FOR_DEGREE(a.K, {
         if (conv_optin((const void *)k_conv<K>, smem, opted[K])) return 1;
+        if (a.node[0]) k_nodes<K><<<ngrid, kNodeThreads, 0, s>>>(a);
         k_conv<K><<<grid, kConvThreads, smem, s>>>(a);
     })
     return 0;

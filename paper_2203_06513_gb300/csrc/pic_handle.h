@@ -66,6 +66,8 @@ struct pic_handle {
     double *m1[2] = {nullptr, nullptr}, *my[2] = {nullptr, nullptr}, *mz[2] = {nullptr, nullptr};
     double *mdep = nullptr, *gtab = nullptr;
     double *rho = nullptr, *work = nullptr, *diag = nullptr;
+    double *node = nullptr;         // 2 M: nodes of subsystem II's deposits, formed in a pass of
+    bool node_pass = false;         // their own before its solves (long inverse rows)
     int32_t *counts = nullptr;
 
     // circulant bands and inverse taps

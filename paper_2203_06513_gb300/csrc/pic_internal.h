@@ -211,6 +211,7 @@ struct ConvArgs {
     const double *mom0;     // subsystem I: moments of the start points
     const int *flux;
     const double *in[2];
+    double *node[2];        // SOLVE2 with long rows: the nodes, formed once by a pass before the solve
     double scale;
     double *out[2];
     const double *en[2];    // e^n
@@ -236,7 +237,22 @@ struct ConvArgs {
     int *count;         // graph mode of single runs: sweeps counted by the decision (or NULL)
 };
 
+// the solve, after a pass that forms its nodes when a.node is given (two launches)
 int launch_conv(const ConvArgs &a, cudaStream_t s);
+// FP64 operations a solve of subsystem II (all runs of an ensemble) spends on its nodes when
+// every block forms those of its own tap window: long rows (large dt/dx) repeat a node some
+// ntap / (16 - K) times.  From kNodePassOps on the nodes are formed once, in a pass before
+// the solve, which costs a launch (or a barrier).  us a step, blocks and pass, double form:
+//   M, k, dt/dx    operations   4e3 markers (one kernel)   6e4 (graph)
+//   128, 3, 8        0.05e6          164   169               383   388
+//   2048, 3, 1       0.60e6          252   249               338   343
+//   512, 3, 16       0.68e6          200   189               387   367
+//   2048, 3, 4       0.88e6          273   262               364   357
+//   2048, 3, 8       1.67e6          301   265               374   348
+//   4000, 5, 16      16.9e6          792   506               733   544
+//   4000, 5, 64      66.1e6         1725   723              2206   942
+long long conv_node_ops(int M, int K, int ntap);
+constexpr long long kNodePassOps = 800000;
 
 // ---------------------------------------------------------------- spin (double form)
 // Spin components are kept in caller order (sx[id], sy[id], sz[id]).
@@ -321,8 +337,9 @@ struct RunDesc {
 
 int launch_ens_plan(EnsQueue *Q, const EnsRun *runs, int nruns, unsigned long long cond, cudaStream_t s);
 int launch_ens_status(const EnsRun *runs, int nruns, int *status, cudaStream_t s);
-int conv_ens_optin(int K, int ntap_max);
-int launch_conv_ens(const ConvArgs *runs, int nruns, int Mmax, int K, int ncomp, int ntap_max, EnsQueue *Q,
+int conv_ens_optin(int K, int ntap1, int ntap2, bool nodes);
+// nodes: a pass that forms the runs' nodes comes first (ConvArgs::node)
+int launch_conv_ens(const ConvArgs *runs, int nruns, int Mmax, int K, int ncomp, int ntap_max, bool nodes, EnsQueue *Q,
                     int *sweeps, unsigned long long cond, cudaStream_t s);
 int launch_prep1_ens(const RunDesc *R, int nruns, int K, int Mmax, cudaStream_t s);
 int launch_prep2_ens(const RunDesc *R, int nruns, int K, int Mmax, cudaStream_t s);

@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constan
                     if (bad) atomicOr(&ctrl->status, STATUS_NUMERIC);
                     PIC_BARRIER();
                     for (int b = blockIdx.x; b < nconv; b += gridDim.x) {
-                        conv_block<K>(A.c1p, T, 0, b, 0, s_conv, nullptr);
+                        conv_block<K>(A.c1p, nullptr, T, 0, b, 0, s_conv, nullptr);
                         __syncthreads();
                     }
                     PIC_BARRIER();
@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constan
                     }
                     PIC_BARRIER();
                     for (int b = blockIdx.x; b < nconv; b += gridDim.x) {
-                        conv_block<K>(A.c1, T, L.it, b, 0, s_conv, S->maxima[0][L.it % 3] + 1);
+                        conv_block<K>(A.c1, nullptr, T, L.it, b, 0, s_conv, S->maxima[0][L.it % 3] + 1);
                         __syncthreads();
                     }
                     PIC_BARRIER();
@@ -300,8 +300,12 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constan
                         }
                     }
                     PIC_BARRIER();
+                    if (A.c2.node[0]) {
+                        for (int q = me; q < 2 * M; q += all) node_pass<K>(A.c2, L.it, q % M, q / M);
+                        PIC_BARRIER();
+                    }
                     for (int b = blockIdx.x; b < 2 * nconv; b += gridDim.x) {
-                        conv_block<K>(A.c2, T, L.it, b % nconv, b / nconv, s_conv, S->maxima[1][L.it % 3] + 1);
+                        conv_block<K>(A.c2, A.c2.node[b / nconv], T, L.it, b % nconv, b / nconv, s_conv, S->maxima[1][L.it % 3] + 1);
                         __syncthreads();
                     }
                     PIC_BARRIER();
@@ -364,7 +368,7 @@ int launch_small_r(const SmallArgs &a, int num_sms, cudaStream_t s)
     const long long want = std::max<long long>((a.d.np + 31) / 32, 2 * conv_blocks(a.d.M, a.d.K));
     const int grid = (int)std::min<long long>(num_sms, want);
     if (a.d.np > (long long)grid * kSmallThreads) return 1;
-    const size_t smem = conv_smem(a.d.K, std::max(a.c1.ntap, a.c2.ntap));
+    const size_t smem = std::max(conv_smem(a.d.K, a.c1.ntap, false), conv_smem(a.d.K, a.c2.ntap, a.c2.node[0] != nullptr));
     switch (a.d.K) {
     case 2: return launch_small_kr<2, R>(a, grid, smem, s);
     case 3: return launch_small_kr<3, R>(a, grid, smem, s);

@@ -177,13 +177,16 @@ __device__ __forceinline__ float sum_residue(double n, double k)
 // to event: 20.8 us with 32 nodes a block and the degree at run time, 12 us so.
 // Returns true in the one block that finished the run's solve last (after the
 // convergence decision, in the solve modes).  With max_e != NULL the maxima go to
-// max_e[0 .. 1] (increment, field) and no decision is taken.
+// max_e[0 .. 1] (increment, field) and no decision is taken.  given: the nodes of the component
+// when a pass has formed them (ConvArgs::node), else null.
 constexpr int kConvOut = 16, kConvThreads = 160, kConvMaxWarps = 8;
 
-inline size_t conv_smem(int K, int ntap)
+// nodes: they are given (conv_block), no moments are staged
+inline size_t conv_smem(int K, int ntap, bool nodes)
 {
     const int nq = kConvOut + ntap - 1;
-    return ((size_t)nq + ntap + (size_t)(nq + K) * (K + 1) + kConvMaxWarps * kConvOut + 2 * kConvOut) * sizeof(double) +
+    return ((size_t)nq + ntap + (nodes ? 0 : (size_t)(nq + K) * (K + 1)) + kConvMaxWarps * kConvOut + 2 * kConvOut) *
+               sizeof(double) +
            (size_t)(nq + K + 1) * sizeof(int);
 }
 inline int conv_blocks(int M, int K) { return (M + kConvOut - K - 1) / (kConvOut - K); }
@@ -200,16 +203,40 @@ __device__ __forceinline__ double warp_max_nonneg(double v)
     return __longlong_as_double(x);
 }
 
+// Node j of subsystem II's deposit: r-th cell's moments at(r, m).
+template <int K, class At>
+__device__ __forceinline__ double solve2_node(const ConvArgs &A, At &&at)
+{
+    double s0 = 0.0, s1 = 0.0;
+#pragma unroll
+    for (int r = 0; r <= K; ++r)
+#pragma unroll
+        for (int m = 0; m <= K; ++m) {
+            double &s = (m & 1) ? s1 : s0;
+            s = fma(c_spline.b[K][r][m], at(r, m), s);
+        }
+    return A.scale * (s0 + s1);
+}
+
+// Node j of component comp into A.node (sweep `it` of the loop).
 template <int K>
-static __device__ __forceinline__ bool conv_block(const ConvArgs &A, CoefTables T, int it, int bx, int comp, double *sm,
-                                                  unsigned long long *max_e)
+__device__ __forceinline__ void node_pass(const ConvArgs &A, int it, int j, int comp)
+{
+    if (j >= A.M) return;
+    const double *mom = A.graph ? A.pair[comp][it & 1] : A.mom[comp];
+    A.node[comp][j] = solve2_node<K>(A, [&](int r, int m) { return mom[(size_t)wrap_once(j + r, A.M) * (K + 1) + m]; });
+}
+
+template <int K>
+static __device__ __forceinline__ bool conv_block(const ConvArgs &A, const double *given, CoefTables T, int it, int bx,
+                                                  int comp, double *sm, unsigned long long *max_e)
 {
     const int M = A.M, i0 = bx * (kConvOut - K), ntap = A.ntap;
     const int nq = kConvOut + ntap - 1;
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
-    double *s_in = sm, *s_tap = s_in + nq, *s_mom = s_tap + ntap, *s_part = s_mom + (size_t)(nq + K) * (K + 1);
-    double *s_val = s_part + kConvMaxWarps * kConvOut, *s_an = s_val + kConvOut;
-    int *s_flux = reinterpret_cast<int *>(s_an + kConvOut);
+    double *s_in = sm, *s_tap = s_in + nq, *s_part = s_tap + ntap;
+    double *s_val = s_part + kConvMaxWarps * kConvOut, *s_an = s_val + kConvOut, *s_mom = s_an + kConvOut;
+    int *s_flux = reinterpret_cast<int *>(s_mom + (size_t)(nq + K) * K);       // (subsystem I)
     const double *mom = A.mom[comp];
     double *zero = A.zero[comp];
     const int *flux = A.flux;
@@ -220,6 +247,7 @@ static __device__ __forceinline__ bool conv_block(const ConvArgs &A, CoefTables 
         flux = A.fpair[it & 1];
         zflux = A.fpair[(it + 1) & 1];
     }
+    if (given) mom = nullptr;
     // the epilogue's loads (lanes 0 .. 15 of warp 0: one node each)
     const int o = lane & (kConvOut - 1), i = i0 - K + o;
     const int iw = wrap_cell(i, M);
@@ -248,21 +276,14 @@ static __device__ __forceinline__ bool conv_block(const ConvArgs &A, CoefTables 
         for (int q = tid; q < (nq + K) * (K + 1); q += nt)
             s_mom[q] = mom[(size_t)node(q / (K + 1)) * (K + 1) + q % (K + 1)];
         __syncthreads();
-        for (int q = tid; q < nq; q += nt) {
-            double s0 = 0.0, s1 = 0.0;
-#pragma unroll
-            for (int r = 0; r <= K; ++r)
-#pragma unroll
-                for (int m = 0; m <= K; ++m) {
-                    double &s = (m & 1) ? s1 : s0;
-                    s = fma(c_spline.b[K][r][m], s_mom[(q + r) * (K + 1) + m], s);
-                }
-            s_in[q] = fma(A.dt, A.scale * (s0 + s1), A.b[comp][node(q)]);
-        }
+        for (int q = tid; q < nq; q += nt)
+            s_in[q] = fma(A.dt, solve2_node<K>(A, [&](int r, int m) { return s_mom[(q + r) * (K + 1) + m]; }),
+                          A.b[comp][node(q)]);
     } else {
+        const double *in = given ? given : A.in[comp];
         for (int q = tid; q < nq; q += nt) {
             const int g = node(q);
-            const double s = A.in[comp][g];
+            const double s = in[g];
             s_in[q] = A.mode == CONV_SOLVE2 ? fma(A.dt, s, A.b[comp][g]) : s;
         }
     }
