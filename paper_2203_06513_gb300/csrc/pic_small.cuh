@@ -63,6 +63,7 @@ __device__ __forceinline__ bool grid_barrier(SmallSync *S, unsigned &gen, DevCtr
 struct LoopState {
     double dprev, eprev;
     int it;                 // sweeps done
+    bool failed;            // a marker went bad in this launch, or an error was there before it
     __device__ __forceinline__ void reset()
     {
         dprev = eprev = bits_to_double(0x7ff0000000000000ull);
@@ -73,22 +74,26 @@ struct LoopState {
 // After the barrier behind the solve of sweep L.it: true when the loop ends.  Each
 // subsystem has its maxima, slot s of them for the sweeps s, s + 3, ..: the slot of the next
 // sweep is cleared two barriers before it is used, and a subsystem's slots after the
-// barrier that ends it (a slower block may be reading them until then).
+// barrier that ends it (a slower block may be reading them until then).  A marker that goes
+// bad publishes a NaN increment in the sweep's slot: the control block's status is for the
+// host alone, since a block that has gone on to the next sweep may set its bits before a slower
+// one has taken this decision, and all have to take the same.
 __device__ __forceinline__ bool loop_decision(const ConvArgs &C, unsigned long long (*maxima)[3], LoopState &L)
 {
     __shared__ int s_stop;
     if (threadIdx.x == 0) {
         const int slot = L.it % 3;
         volatile unsigned long long *m = maxima[slot];
-        const double d = bits_to_double(m[0]), e = bits_to_double(m[1]), mag = bits_to_double(m[2]);
-        const int status = *reinterpret_cast<volatile int *>(&C.ctrl->status);
+        const unsigned long long moved = m[0];
+        const double d = bits_to_double(moved), e = bits_to_double(m[1]), mag = bits_to_double(m[2]);
         L.it += 1;
         bool stop = fixed_point_reached(C, L.it, d, L.dprev, e, L.eprev, mag);
         if (!stop && L.it >= C.max_iter) {
             stop = true;
             if (blockIdx.x == 0) atomicOr(&C.ctrl->status, STATUS_NOCONV);
         }
-        if (status & (STATUS_NUMERIC | STATUS_TIMEOUT)) stop = true;
+        L.failed = L.failed || moved > 0x7ff0000000000000ull;     // a NaN
+        if (L.failed) stop = true;
         L.dprev = d;
         L.eprev = e;
         if (blockIdx.x == 0) {
@@ -145,6 +150,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constan
         if (spin) id = D.P.id[me];
     }
     CoefTables T = D.T;             // A and Kt change places after every subsystem II
+    LoopState L;
+    L.failed = (*reinterpret_cast<volatile int *>(&ctrl->status) & (STATUS_NUMERIC | STATUS_TIMEOUT)) != 0;
     int hist2 = ctrl->hist2;
 #define PIC_BARRIER() do { if (!grid_barrier(S, gen, ctrl)) return; } while (0)
     // ---- what a step finds prepared: the polynomials of a^n and of ebar^(0) = e^n, cleared
@@ -158,7 +165,6 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constan
     PIC_BARRIER();
     for (int step = 0; step < A.nsteps; ++step) {
         for (int part = 0; part < (A.strang ? 3 : 2); ++part) {
-            LoopState L;
             L.reset();
             if (part != 1) {
                 // ---- subsystem I
@@ -215,7 +221,10 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constan
                         d = dnew;
                         const double big = warp_max_nonneg((double)inc);
                         if (lane == 0 && big != 0.0) atomic_max_nonneg(&S->maxima[0][L.it % 3][0], big);
-                        if (bad) atomicOr(&ctrl->status, STATUS_NUMERIC);
+                        if (bad) {
+                            atomicOr(&ctrl->status, STATUS_NUMERIC);
+                            atomicMax(&S->maxima[0][L.it % 3][0], 0x7ff8000000000000ull);
+                        }
                     }
                     PIC_BARRIER();
                     for (int b = blockIdx.x; b < nconv; b += gridDim.x) {

@@ -111,3 +111,27 @@ def test_2d_substep_reports_positions_that_are_not_finite(bad, warm):
                           pic.PIC_MEM_DEVICE, None, ctypes.byref(h)) == 0
     assert lib.pic2d_substep1(h, ctypes.byref(it)) == pic.PIC_ERR_NUMERIC
     lib.pic2d_destroy(h)
+
+
+@pytest.mark.parametrize("precision", FORMS)
+@pytest.mark.parametrize("no_graph", [False, True])
+def test_a_marker_that_goes_bad_in_a_later_sweep(precision, no_graph, monkeypatch):
+    """A potential that is NaN in a few cells: no marker starts there, and the iterate of the
+    second sweep walks into them.  Every block of the one-kernel step has to stop with that
+    sweep (a block that went on alone would wait at its barrier for seconds)."""
+    if no_graph:
+        monkeypatch.setenv("PIC_NO_GRAPH", "1")
+    nx, k, n, L = 256, 3, 20003, 8.0
+    dx = L / nx
+    x = (np.arange(n) + 0.5) / n * 0.5 * L          # cells 0 .. 127; node 131 reaches cells 131 .. 134
+    p = np.zeros(n)
+    p[-64:] = 3.0                                   # to the right by 0.95 dt = 7.6 cells
+    ay = np.full(nx, 0.01)
+    ay[131] = np.nan
+    z = np.zeros(nx)
+    for _ in range(10):
+        g = pic.Pic(pic.Config(L, nx, k, n, L / n, 8 * dx, precision=precision), x, p, ay, z)
+        with pytest.raises(pic.PicError) as e:
+            g.step(3)
+        assert e.value.code == pic.PIC_ERR_NUMERIC
+        g.close()
