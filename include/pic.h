@@ -218,7 +218,9 @@ int pic_substep(pic_handle *h, int32_t which, int32_t *iters);
  * Phi_III(dt) o Phi_II(dt) o Phi_I(dt)), or with
  * splitting = PIC_SPLIT_STRANG the symmetric Phi_I(dt/2) o Phi_II(dt) o
  * Phi_I(dt/2), each substep the paper's energy-conserving scheme.  Sweep counts
- * summed over the steps go to *iters_I / *iters_II (may be NULL). */
+ * summed over the steps go to *iters_I / *iters_II (may be NULL).  After
+ * PIC_ERR_CUDA from a wait that gave up the handle has no state to go on from:
+ * pic_step and pic_substep refuse it with PIC_ERR_CUDA. */
 int pic_step(pic_handle *h, int32_t nsteps, int64_t *iters_I, int64_t *iters_II);
 
 /* Discrete Hamiltonian (Eq. discrete_H) and Gauss-law residual, evaluated in

@@ -911,9 +911,12 @@ static int substep2(pic_handle *h, int *iters)
     return PIC_OK;
 }
 
+static const char *kLost = "an earlier step gave up at a barrier: the handle has no state to go on from";
+
 extern "C" int pic_substep(pic_handle *h, int32_t which, int32_t *iters)
 {
     if (!h) return PIC_ERR_INVALID;
+    if (h->lost) return fail(h, PIC_ERR_CUDA, "%s", kLost);
     int it = 0, rc;
     if (which == PIC_SUBSYSTEM_I) rc = substep1(h, &it, h->cfg.dt);
     else if (which == PIC_SUBSYSTEM_II) rc = substep2(h, &it);
@@ -1100,7 +1103,7 @@ static int build_step_graph(pic_handle *h)
 // With a thread a marker the steps run in one cooperative kernel (pic_small.cuh).
 static bool small_eligible(const pic_handle *h)
 {
-    return h->np <= (long long)h->num_sms * kSmallThreads && !h->reduce && !h->timing && !debug_sync() &&
+    return !h->small_refused && h->np <= (long long)h->num_sms * kSmallThreads && !h->reduce && !h->timing && !debug_sync() &&
            h->cfg.warm_start != PIC_WARM_MLP && h->acc == (h->fp32 ? ACC_COMP : ACC_NATIVE) &&
            getenv("PIC_NO_GRAPH") == nullptr;
 }
@@ -1114,9 +1117,11 @@ static int step_counts(pic_handle *h)
     return PIC_OK;
 }
 
-static int step_small(pic_handle *h, int nsteps, long long *s1, long long *s2)
+// *done: the steps taken, fewer than nsteps when the launch was refused
+static int step_small(pic_handle *h, int nsteps, int *done, long long *s1, long long *s2)
 {
     int rc;
+    *done = 0;
     if ((rc = step_counts(h))) return rc;
     if (!h->small && (rc = dalloc(h, &h->small, 1))) return rc;
     GCK(cudaMemsetAsync(h->d_count, 0, 2 * sizeof(int), h->stream));
@@ -1151,9 +1156,15 @@ static int step_small(pic_handle *h, int nsteps, long long *s1, long long *s2)
         a.sx = h->spx; a.sy = h->spy; a.sz = h->spz;
         a.sm_y = h->sdy; a.sm_z = h->sdz;
         GCK(cudaMemsetAsync(h->small, 0, sizeof(SmallSync), h->stream));
-        if ((h->fp32 ? launch_small_f32 : launch_small_f64)(a, h->num_sms, h->stream)) return fail(h, PIC_ERR_CUDA, "step kernel: launch failed");
+        const int e = (h->fp32 ? launch_small_f32 : launch_small_f64)(a, h->num_sms, h->stream);
+        if (e == kSmallRefused) {
+            h->small_refused = true;
+            break;
+        }
+        if (e) return fail(h, PIC_ERR_CUDA, "step kernel: launch failed");
         CKL_N("launch_small");
         n += m;
+        *done = n;
         h->steps_done += m;
         if (every > 0 && h->steps_done % every == 0)
             if ((rc = sort_markers(h))) return rc;
@@ -1163,6 +1174,8 @@ static int step_small(pic_handle *h, int nsteps, long long *s1, long long *s2)
     *s1 = h->h_count[0];
     *s2 = h->h_count[1];
     h->marker_sweeps += *s1 * h->np;
+    // fields of the step are there, its markers were in registers
+    if (h->h_ctrl->status & STATUS_TIMEOUT) h->lost = true;
     for (int which = 1; which <= 2; ++which)
         if ((rc = check_status(h, which))) return rc;
     return PIC_OK;
@@ -1197,15 +1210,18 @@ extern "C" int pic_step(pic_handle *h, int32_t nsteps, int64_t *iters_I, int64_t
 {
     if (!h) return PIC_ERR_INVALID;
     if (nsteps < 0) return fail(h, PIC_ERR_INVALID, "nsteps < 0");
+    if (h->lost) return fail(h, PIC_ERR_CUDA, "%s", kLost);
     long long s1 = 0, s2 = 0;
     int rc = PIC_OK;
     for (int n = 0; n < nsteps; ++n) {
         if (small_eligible(h)) {
             long long g1 = 0, g2 = 0;
-            rc = step_small(h, nsteps - n, &g1, &g2);
+            int done = 0;
+            rc = step_small(h, nsteps - n, &done, &g1, &g2);
             s1 += g1;
             s2 += g2;
-            break;
+            n += done;
+            if (rc || n >= nsteps) break;       // else refused: the other paths take the rest
         }
         // graph steps once a host-loop step has opted the kernels in to their shared memory
         if (h->host_steps > 0 && graph_eligible(h)) {

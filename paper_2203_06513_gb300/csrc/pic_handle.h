@@ -51,6 +51,8 @@ struct pic_handle {
     int *h_count = nullptr;             // pinned readback of d_count
     int host_steps = 0;                 // steps taken by host loops (the first one opts kernels in)
     pic::SmallSync *small = nullptr;    // barrier of the one-kernel steps of small plasmas
+    bool small_refused = false;         // the device would not hold their grid at once
+    bool lost = false;                  // a one-kernel step gave up at a barrier: no state to go on from
 
     // grid state (double)
     double *ex = nullptr, *ey = nullptr, *ez = nullptr, *ay = nullptr, *az = nullptr;

@@ -370,6 +370,8 @@ struct SmallArgs {
     double *sx, *sy, *sz;   // spins, caller order (hbar != 0)
     double *sm_y, *sm_z;    // M x K moments of the spin deposit
 };
+// kSmallRefused: the device does not hold the grid at once (nothing was launched)
+constexpr int kSmallRefused = 2;
 int launch_small_f32(const SmallArgs &a, int num_sms, cudaStream_t s);
 int launch_small_f64(const SmallArgs &a, int num_sms, cudaStream_t s);
 int launch_prep1(const RunDesc &R, cudaStream_t s);

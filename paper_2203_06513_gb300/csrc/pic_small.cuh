@@ -12,7 +12,8 @@
 //
 // The barrier is bounded: a block that waits longer than its limit sets STATUS_TIMEOUT
 // and an abort flag, and every block returns at its next barrier.  The launch is
-// cooperative, so all blocks are resident.
+// cooperative, so all blocks are resident; where the device does not hold them at once (fewer
+// SMs for this process than it reports) the launch is refused and the steps go on as graphs.
 #pragma once
 
 #include <algorithm>
@@ -366,8 +367,13 @@ int launch_small_kr(const SmallArgs &a, int grid, size_t smem, cudaStream_t s)
         }
     }
     void *args[] = {const_cast<SmallArgs *>(&a)};
-    return cudaLaunchCooperativeKernel((const void *)k_small<K, R>, dim3(grid), dim3(kSmallThreads), args, smem, s) !=
-           cudaSuccess;
+    const cudaError_t e =
+        cudaLaunchCooperativeKernel((const void *)k_small<K, R>, dim3(grid), dim3(kSmallThreads), args, smem, s);
+    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorLaunchOutOfResources || e == cudaErrorNotSupported) {
+        cudaGetLastError();
+        return kSmallRefused;
+    }
+    return e != cudaSuccess;
 }
 
 template <typename R>
