@@ -215,27 +215,15 @@ long long conv_node_ops(int M, int K, int ntap)
     return 2LL * conv_blocks(M, K) * (kConvOut + ntap - 1) * (K + 1) * (K + 1);
 }
 
-// Raises a solve kernel's dynamic shared-memory limit (never lowers it).  Inverse rows
-// that decay slowly (large dt/dx in subsystem II) may keep as many taps as nodes.
-static int conv_optin(const void *fn, size_t smem, size_t &opted)
-{
-    static std::mutex mu;
-    std::lock_guard<std::mutex> lock(mu);
-    if (smem > 48 * 1024 && smem > opted) {
-        if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-            return 1;
-        opted = smem;
-    }
-    return 0;
-}
-
-static size_t g_conv_ens_opted[kMaxDegree + 1];
+// Inverse rows that decay slowly (large dt/dx in subsystem II) may keep as many taps as
+// nodes, which takes more shared memory than the default.
+static SmemOptin g_conv_optin[kMaxDegree + 1], g_conv_ens_optin[kMaxDegree + 1];
 
 // raise the shared-memory limit of k_conv_ens before any capture of it
 int conv_ens_optin(int K_, int ntap1, int ntap2, bool nodes)
 {
     const size_t smem = std::max(conv_smem(K_, ntap1, false), conv_smem(K_, ntap2, nodes));
-    PIC_FOR_DEGREE(K_, return conv_optin((const void *)k_conv_ens<K>, smem, g_conv_ens_opted[K]))
+    PIC_FOR_DEGREE(K_, return g_conv_ens_optin[K].raise((const void *)k_conv_ens<K>, smem) ? 0 : 1)
     return 1;
 }
 
@@ -243,7 +231,7 @@ int launch_conv_ens(const ConvArgs *runs, int nruns, int Mmax, int K_, int ncomp
                     int *sweeps, unsigned long long cond, cudaStream_t s)
 {
     const size_t smem = conv_smem(K_, ntap_max, nodes);
-    if (smem > 48 * 1024 && smem > g_conv_ens_opted[K_]) return 1;   // conv_ens_optin first
+    if (!g_conv_ens_optin[K_].allowed(smem)) return 1;   // conv_ens_optin first
     if (nodes) {
         const dim3 ngrid((Mmax + kNodeThreads - 1) / kNodeThreads, nruns, ncomp);
         PIC_FOR_DEGREE(K_, (k_nodes_ens<K><<<ngrid, kNodeThreads, 0, s>>>(runs, Q)))
@@ -256,10 +244,9 @@ int launch_conv_ens(const ConvArgs *runs, int nruns, int Mmax, int K_, int ncomp
 int launch_conv(const ConvArgs &a, cudaStream_t s)
 {
     const size_t smem = conv_smem(a.K, a.ntap, a.node[0] != nullptr);
-    static size_t opted[kMaxDegree + 1];   // largest dynamic shared memory opted in so far
     const dim3 grid(conv_blocks(a.M, a.K), a.ncomp), ngrid((a.M + kNodeThreads - 1) / kNodeThreads, a.ncomp);
     PIC_FOR_DEGREE(a.K, {
-        if (conv_optin((const void *)k_conv<K>, smem, opted[K])) return 1;
+        if (!g_conv_optin[K].raise((const void *)k_conv<K>, smem)) return 1;
         if (a.node[0]) k_nodes<K><<<ngrid, kNodeThreads, 0, s>>>(a);
         k_conv<K><<<grid, kConvThreads, smem, s>>>(a);
     })

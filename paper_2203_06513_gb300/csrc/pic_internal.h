@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include "pic_device.cuh"
+#include "pic_optin.h"
 
 namespace pic {
 

@@ -826,16 +826,11 @@ int launch_warm_mlp(const WarmArgs &a, int grid, cudaStream_t s)
 {
     if ((size_t)a.M + 2 * (size_t)(a.K + 1) > kMaxWarmNodes) return 1;
     const size_t smem = warm_mlp_smem(a.M, a.K);
-    static size_t opted = 0;
-    if (smem > opted) {
-        cudaError_t e = cudaSuccess;
-#define ATTR(KK, RR) e = e ? e : cudaFuncSetAttribute(k_warm_mlp<KK, RR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        ATTR(2, float) ATTR(3, float) ATTR(4, float) ATTR(5, float)
-        ATTR(2, double) ATTR(3, double) ATTR(4, double) ATTR(5, double)
-#undef ATTR
-        if (e != cudaSuccess) return 1;
-        opted = smem;
-    }
+    static SmemOptin optin;
+#define FN(KK) (const void *)k_warm_mlp<KK, float>, (const void *)k_warm_mlp<KK, double>
+    const void *const fn[] = {FN(2), FN(3), FN(4), FN(5)};
+#undef FN
+    if (!optin.raise(fn, smem)) return 1;
 #define LAUNCH(KK)                                                                               \
     case KK:                                                                                     \
         if (a.fp32) k_warm_mlp<KK, float><<<grid, kMlpThreads, smem, s>>>(a);                          \
@@ -925,12 +920,9 @@ extern "C" int pic_mlp_get_params(pic_mlp *m, float *params_host)
 extern "C" int pic_mlp_grad(pic_mlp *m, const float *X, const float *T, int64_t B, float *grad_out, double *loss_out)
 {
     if (!m || !X || !T || B < 1) return mlp_fail(PIC_ERR_INVALID, "pic_mlp_grad: invalid argument");
-    static bool opted = false;
-    if (!opted) {
-        if (cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmem)))
-            return mlp_fail(PIC_ERR_CUDA, "pic_mlp_grad: shared-memory opt-in failed");
-        opted = true;
-    }
+    static SmemOptin optin;
+    if (!optin.raise((const void *)k_mlp_train, sizeof(TrainSmem)))
+        return mlp_fail(PIC_ERR_CUDA, "pic_mlp_grad: shared-memory opt-in failed");
     cudaMemsetAsync(m->grad, 0, kNParams * sizeof(float) + sizeof(double), m->stream);    // and the loss behind it
     // two blocks are resident on an SM; beyond that the tiles of a block follow each other
     const long long tiles = std::min<long long>((B + kTB - 1) / kTB, 2LL * m->num_sms);
@@ -982,12 +974,9 @@ extern "C" int pic_mlp_infer(pic_mlp *m, const float *X, int64_t B, float *Y)
     if (!m || !X || !Y || B < 0) return mlp_fail(PIC_ERR_INVALID, "pic_mlp_infer: invalid argument");
     if (B == 0) return PIC_OK;
     const size_t smem = mlp_infer_smem();
-    static bool opted = false;
-    if (!opted) {
-        if (cudaFuncSetAttribute(k_mlp_infer, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem))
-            return mlp_fail(PIC_ERR_CUDA, "pic_mlp_infer: shared-memory opt-in failed");
-        opted = true;
-    }
+    static SmemOptin optin;
+    if (!optin.raise((const void *)k_mlp_infer, smem))
+        return mlp_fail(PIC_ERR_CUDA, "pic_mlp_infer: shared-memory opt-in failed");
     long long blocks = (B + kMlpThreads - 1) / kMlpThreads;
     if (blocks > (long long)m->num_sms) blocks = (long long)m->num_sms;
     if (cudaMemsetAsync(m->status, 0, sizeof(int), m->stream) != cudaSuccess)

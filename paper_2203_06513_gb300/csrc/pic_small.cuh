@@ -17,7 +17,6 @@
 #pragma once
 
 #include <algorithm>
-#include <mutex>
 
 #include "pic_internal.h"
 #include "pic_poly.cuh"
@@ -356,16 +355,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_small(const __grid_constan
 template <int K, typename R>
 int launch_small_kr(const SmallArgs &a, int grid, size_t smem, cudaStream_t s)
 {
-    static std::mutex mu;
-    static size_t opted = 0;
-    {
-        std::lock_guard<std::mutex> lock(mu);
-        if (smem > 48 * 1024 && smem > opted) {
-            if (cudaFuncSetAttribute(k_small<K, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-                return 1;
-            opted = smem;
-        }
-    }
+    static SmemOptin optin;
+    if (!optin.raise((const void *)k_small<K, R>, smem)) return 1;
     void *args[] = {const_cast<SmallArgs *>(&a)};
     const cudaError_t e =
         cudaLaunchCooperativeKernel((const void *)k_small<K, R>, dim3(grid), dim3(kSmallThreads), args, smem, s);
