@@ -450,8 +450,7 @@ extern "C" int pic_ensemble_step(pic_ensemble *e, int32_t nsteps, int64_t *sweep
         } else if ((rc = host_step(e))) {
             return rc;
         }
-        // periodic marker sort of the runs due, all in one batched sort (four
-        // launches instead of four per run), then fresh tables
+        // periodic marker sort of the runs due, all in one batched sort, then fresh tables
         e->sorts.clear();
         for (pic_handle *h : e->runs) {
             ++h->steps_done;
@@ -476,7 +475,7 @@ extern "C" int pic_ensemble_step(pic_ensemble *e, int32_t nsteps, int64_t *sweep
                                 cudaMemcpyHostToDevice, e->stream));
             ELAUNCH(launch_sort_ens(e->fp32, e->d_sorts, (int)e->sorts.size(), e->sort_grid, e->stream),
                     "ensemble sort");
-            e->launches += 4;
+            e->launches += kSortEnsLaunches;
             build_tables(e);
             if ((rc = upload_tables(e))) return rc;
         }

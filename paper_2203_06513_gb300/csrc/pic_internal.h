@@ -185,6 +185,7 @@ struct SortRun {
     PartPtrs src, dst;
     int32_t *counts;        // sort_counts(M nbins): histogram, cursors, tile totals
 };
+constexpr int kSortEnsLaunches = 5;
 int launch_sort_ens(int fp32, const SortRun *runs, int nruns, int grid_x, cudaStream_t s);
 int launch_sort(int fp32, long long np, int M, double tau, int per, PartPtrs src, PartPtrs dst,
                 int32_t *counts, int num_sms, cudaStream_t s);
