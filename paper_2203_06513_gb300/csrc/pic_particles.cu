@@ -252,9 +252,11 @@ int launch_sweep2(const Sweep2Args &a, int grid, cudaStream_t s)
 // Diagnostics, evaluated in double from the stored state.
 // ---------------------------------------------------------------------------
 // charge moments sum_a v^m per cell, halved, as 64-bit integers (AccFixed): with double sums
-// the FP64 pipe bounds it (1e7 float markers: 274 us, 85 now)
+// the FP64 pipe bounds it (1e7 float markers: 274 us, 88 now, the pipe 30 % busy).  Four blocks
+// an SM: left alone the compiler takes 70 registers in degrees 2 and 3, which leaves three
+// (112 us).
 template <int K, typename R>
-__global__ void __launch_bounds__(kSweepThreads) k_charge(DiagArgs A)
+__global__ void __launch_bounds__(kSweepThreads, K <= 3 ? 4 : 1) k_charge(DiagArgs A)
 {
     const int32_t *__restrict__ cp = A.P.cell;
     const R *__restrict__ vp = static_cast<const R *>(A.P.t);
