@@ -67,7 +67,7 @@ NCU_DRAM_PER_MARKER = {"k_sweep1<3,float>": 22.33, "k_sweep2<3,float>": 12.20, "
 # Warp instructions x 32 per marker from the same captures: the kernels are bound by
 # instruction issue, which the "issue" entry compares with the issue-slot peak
 # (SMs x 4 schedulers x 1 warp instruction a cycle x the sampled SM clock).
-NCU_INST_PER_MARKER = {"k_sweep1<3,float>": 295, "k_sweep2<3,float>": 170, "k_warm_mlp<3,float>": 461}
+NCU_INST_PER_MARKER = {"k_sweep1<3,float>": 293, "k_sweep2<3,float>": 171, "k_warm_mlp<3,float>": 461}
 
 
 def peaks():

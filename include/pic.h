@@ -83,7 +83,10 @@ extern "C" {
 
 /* deposit accumulation (pic_config.deposit): how the sweeps of the FP32 form
  * sum the float contributions of the markers a lane holds before they reach the
- * double grid row.  The FP64 form always accumulates in double. */
+ * double grid row.  The FP64 form (also with PIC_ACC_DOUBLE) sums the moments
+ * f v^m of a cell exactly, as 64-bit integers of 2^(56 + m) with f scaled to at
+ * most 1/2 by a power of two per cell: each term is good to 2^-57 2^-m of that
+ * scale (a double near the largest term to 2^-55 2^-m). */
 #define PIC_ACC_DEFAULT      0  /* FP32: PIC_ACC_COMPENSATED                                  */
 #define PIC_ACC_FLOAT        1  /* FP32, k = 3 or 5: plain float lane sums, float warp sums    */
 #define PIC_ACC_COMPENSATED  2  /* FP32: compensated float pair per lane (two-sum), double warp sums */
@@ -254,8 +257,8 @@ int pic_destroy(pic_handle *h);
  * small network can propose x^(0) instead.  The iteration still runs to the
  * same tolerance, so the converged state does not depend on the proposal.
  * Network: 6 inputs (cell-relative x, p, E_x(x^n), A_y(x^n), A_z(x^n), dt),
- * normalised by (v - shift) * scale; three hidden layers of width 64, GELU
- * (tanh form); 2 outputs times out_scale, read as
+ * normalised by (v - shift) * scale; three hidden layers of width 64, ReLU;
+ * 2 outputs times out_scale, read as
  *   y0 = (x^{n+1} - x^n - dt p / gamma(p, A(x^n))) / dt^2,
  *   y1 = (p^{n+1} - p^n - dt E_x(x^n)) / dt^2.
  * Parameters: 8898 floats, W1 (64x6 row-major [out][in]), b1, W2 (64x64), b2,
@@ -295,10 +298,10 @@ const char *pic_last_error(const pic_handle *h);
  * device array inside the library (one per GPU that loads the library, kept
  * until the process exits).
  *   out[nx] (device)  = sum_a weight * int_{x_a}^{x_a + disp_a} Lambda^1_i,
- * the same quantity as pic_deposit(PIC_DEP_CURRENT), computed in double.  Each
- * block sums its markers with shared-memory atomics (so repeated calls may
- * differ in the last bits) and the blocks' partial rows are then added in a
- * fixed order.  x[np], disp[np]: device arrays of positions (any finite value,
+ * the same quantity as pic_deposit(PIC_DEP_CURRENT), computed in double.  The
+ * markers' path moments are added to one of several replicas of the cells by
+ * atomic additions (so repeated calls may differ in the last bits), and the
+ * replicas are then added in a fixed order.  x[np], disp[np]: device arrays of positions (any finite value,
  * read periodically; normally in [0, L)) and signed displacements (length
  * units, at most 64 cells).  L > 0, 8 <= nx <= 8192 (larger grids exceed the
  * scratch and are rejected with PIC_ERR_INVALID), 2 <= degree <= 5 (degree of

@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(256, sweep2d_blocks<K>) k2_sweep(Args2D A)
         // extra pieces of a crossing then run only in the steps that hold crossing markers,
         // instead of nearly every step running them for one lane.  By warps, not blocks:
         // the warps of a block with the crossings kept the others waiting (388 us for 5e5
-        // cubic markers, 289 so).
+        // cubic markers, 293 so).
         const int n = (int)(end - base < kTile2 ? end - base : kTile2);
         int front = 0, back = n;
         for (int q = 0; q < n; q += 32) {

@@ -406,8 +406,7 @@ extern "C" int pic_init_split(const pic_config *cfg, const pic_arrays *in, int32
         return bail(PIC_ERR_CUDA);
 
     const size_t np = (size_t)h->np, M = (size_t)h->M;
-    // marker arrays are padded by 64 entries: the sweeps' bulk copies round a
-    // tile's byte count up to a multiple of 16 and may read up to 3 entries past N_p
+    // 64 spare entries behind the markers (no kernel reads past N_p)
     const size_t npa = np + 64;
     // each copy: cell, t, p, id back to back, every array 256-byte aligned; at least
     // 16 bytes a marker, room for the staged (x, p) doubles of a host transfer

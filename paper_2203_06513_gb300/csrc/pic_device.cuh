@@ -1,8 +1,8 @@
 // pic_device.cuh -- device-side building blocks of libpic (sm_103a).
 //
-// Positions are stored as (cell c, offset t in [0,1)) in cell units: x = (c + t) dx.
-// In cell c the degree-d periodic basis functions j = c - r (r = 0..d) are nonzero
-// with values N^d(r + t), N^d the cardinal B-spline on the integer knots (Sec. 3.1:
+// Positions are stored as (cell c, offset v in [-1/2, 1/2] from its centre) in cell units:
+// x = (c + 1/2 + v) dx.  In cell c the degree-d periodic basis functions j = c - r
+// (r = 0..d) are nonzero with values N^d(r + 1/2 + v), N^d the cardinal B-spline on the integer knots (Sec. 3.1:
 // Lambda^0_j = N^k_j, Lambda^1_j = N^{k-1}_j, supp N^d_j = [x_j, x_{j+d+1})).
 #pragma once
 
@@ -37,7 +37,7 @@ struct DevCtrl {
 enum : int {
     STATUS_NUMERIC = 1,    // NaN/Inf or displacement beyond the halo
     STATUS_NOCONV  = 2,
-    STATUS_TIMEOUT = 4,    // a bounded wait on a bulk copy gave up
+    STATUS_TIMEOUT = 4,    // a bounded wait (tensor cores, grid barrier) gave up
 };
 
 // accumulator kinds of the sweeps (pic_config.deposit)
@@ -48,10 +48,9 @@ enum : int { ACC_NATIVE = 0, ACC_COMP = 1, ACC_DOUBLE = 2 };
 __host__ __device__ inline int coef_pad(int fp32, int n) { return fp32 ? (n <= 4 ? 4 : 8) : ((n + 1) & ~1); }
 
 // ---------------------------------------------------------------------------
-// Bulk asynchronous copies (the TMA engine's 1-D bulk mode) into shared memory,
-// completed on an mbarrier.  Every wait is bounded: after kMaxWaitTries polls it
-// returns false and the caller records STATUS_TIMEOUT and leaves.  Addresses and
-// sizes must be multiples of 16 bytes.
+// mbarriers in shared memory (completion of the tensor cores' work).  Every wait is
+// bounded: after kMaxWaitTries polls it returns false and the caller records
+// STATUS_TIMEOUT and leaves.
 // ---------------------------------------------------------------------------
 constexpr unsigned long long kMaxWaitTries = 1ull << 26;
 

@@ -117,10 +117,10 @@ private:
         }
     };
 
-    // lives until the process exits; nothing is freed then that a handle still uses
+    // (nothing is given back at the process's exit: a handle may still be there)
     static Set &set(int device)
     {
-        static Set *sets = new Set[kDevices];
+        static Set sets[kDevices];
         return sets[device];
     }
 

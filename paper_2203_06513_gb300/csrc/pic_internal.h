@@ -40,8 +40,8 @@ template <> struct SweepU<float> { static constexpr int v = 2; };
 //            256 x 2 (128)            992 /  770              128 x 5 (102)    - / 378
 //            128 x 7 (73)               - /  570              128 x 4 (128)  833 / 440
 //            128 x 5 (102)           1606 /  662              128 x 3 (170)  624 /   -
-// The double form is bound by the FP64 pipe and does not mind (1057 / 318 us for 1e7
-// markers at 16 warps, cubic; 24 warps 1104 / 613 before the last change of sweep II).
+// The double form is bound by the FP64 pipe and does not mind (1042 / 303 us for 1e7
+// markers, cubic, at 16 warps an SM; with 24 warps sweep I 4 % slower).
 template <typename R, int K> struct SweepShape {
     static constexpr int threads1 = 256, blocks1 = 2, threads2 = 256, blocks2 = 2;
 };

@@ -13,9 +13,9 @@
 // Parameters: one float vector W1 (64x6, row-major [out][in]), b1, W2 (64x64),
 // b2, W3, b3, W4 (2x64), b4 -- 8898 numbers.
 //
-// Inference runs on the 5th-generation tensor cores (tcgen05.mma, bf16 operands
-// in shared memory, fp32 accumulators in tensor memory), 128 markers per tile;
-// the ReLU runs in packed bf16 on each thread's accumulator row.  Training
+// Inference runs on the 5th-generation tensor cores (tcgen05.mma, bf16 activations
+// and fp32 accumulators in tensor memory, weights in shared memory), 128 markers per
+// tile; the ReLU is part of each thread's conversion of its accumulator row to bf16.  Training
 // (forward + backward + Adam) runs in fp32 on the CUDA cores.
 #include <cooperative_groups.h>
 #include <cuda_bf16.h>

@@ -1,6 +1,6 @@
 // pic_solve.cuh -- grid-side device functions: circulant solves with the convergence
 // decision, preparation and end of the substeps (launched by pic_grid.cu, and all in
-// one kernel by pic_small.cu).
+// one kernel by pic_small.cuh).
 #pragma once
 
 #include "pic_internal.h"

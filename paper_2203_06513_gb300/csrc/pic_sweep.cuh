@@ -1,6 +1,6 @@
 // pic_sweep.cuh -- the marker sweeps of subsystems I and II and the end of subsystem I, as
 // device functions over a warp's range of markers (launched by pic_particles.cu, and all
-// in one kernel by pic_small.cu).
+// in one kernel by pic_small.cuh).
 #pragma once
 
 #include <climits>
@@ -96,7 +96,7 @@ __device__ __forceinline__ void start_cache_load(const void *base, long long a, 
 //   cell polynomials, path moments h S_m in every cell visited  1680   2680
 //   end-point moments and knot counts, centred offsets, roots
 //   and quotients without exception paths, two markers a lane    992   1513
-//   double: path ends, moments and seeds off the FP64 pipe         -   1057
+//   double: path ends, moments and seeds off the FP64 pipe         -   1042
 // PRE: the predicted start instead of a sweep -- the proposal delta^(0) (the
 // explicit predictor when A.warm, else the one already in delta) is written back
 // and its path current deposited into A.mom; no gather walk, no momentum update.
@@ -391,8 +391,8 @@ __device__ __forceinline__ void sweep1_range(const Sweep1Args &A, long long beg,
 // us a launch, float (1e8 markers, cubic) and double (1e7): basis values and node windows
 // 1260 and 2060, cell polynomials and moments 767 and 830, as here (centred offsets, the
 // short root and quotient, two markers a lane) 570 and 672, with their seeds refined off the
-// FP64 pipe 610 in double, with the moments as 64-bit integers 318 (one scale a warp, which
-// took the digits of weak fields in its range; 323 with a scale a cell).
+// FP64 pipe 610 in double, with the moments as 64-bit integers 303 (301 with one scale a
+// warp instead of one a cell, which took the digits of weak fields in its range).
 // Z: the z component is not identically zero, as in subsystem I.
 // f = (s + L) / G, s = A^n + A^(k) of a component, G = g0 + g1, L the float form's residue.
 // The float rounding of a coefficient is the same for every marker of its cell, so it
