@@ -256,6 +256,7 @@ static int sort_markers(pic_handle *h)
 }
 
 int pic::handle_sort(pic_handle *h) { return sort_markers(h); }
+int pic::handle_nodes(pic_handle *h) { return h->node ? PIC_OK : dalloc(h, &h->node, 2 * (size_t)h->M); }
 PartPtrs pic::handle_parts(pic_handle *h) { return cur_parts(h); }
 
 pic::RunDesc pic::handle_desc(pic_handle *h)
@@ -523,7 +524,7 @@ extern "C" int pic_init_split(const pic_config *cfg, const pic_arrays *in, int32
     if ((rc = dalloc(h, &h->d_tapP, h->tapP_n))) return bail(rc);
     // split runs form the nodes for their sums over the processes anyway
     h->node_pass = !reduce_fn && conv_node_ops(h->M, K, h->tapP_n) >= kNodePassOps;
-    if (!reduce_fn && (rc = dalloc(h, &h->node, 2 * M))) return bail(rc);
+    if (h->node_pass && (rc = handle_nodes(h))) return bail(rc);
     if (cudaMemcpy(h->d_tapP, taps.data(), sizeof(double) * h->tapP_n, cudaMemcpyHostToDevice) != cudaSuccess)
         return bail(PIC_ERR_CUDA);
 

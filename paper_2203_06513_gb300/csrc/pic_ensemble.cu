@@ -379,6 +379,9 @@ extern "C" int pic_ensemble_create(const pic_config *cfgs, const pic_arrays *ins
         npmax = std::max(npmax, h->np);
     }
     e->node_pass = node_ops >= kNodePassOps;
+    if (e->node_pass)
+        for (pic_handle *h : e->runs)
+            if (const int rc = handle_nodes(h)) return bail(efail(e, rc, "%s", h->err.c_str()));
     e->fin_grid = (int)std::min<long long>(std::max<long long>((npmax + 255) / 256, 1), 64);
     {
         const int b1 = sweep_blocks_per_sm(e->K, e->fp32, e->fp32 ? ACC_COMP : ACC_NATIVE, 1);

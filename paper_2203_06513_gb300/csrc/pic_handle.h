@@ -108,6 +108,8 @@ struct pic_handle {
 namespace pic {
 // marker sort of one handle (swaps its current buffer); its current marker arrays
 int handle_sort(pic_handle *h);
+// room for the nodes of a pass before the solves (pic_handle::node)
+int handle_nodes(pic_handle *h);
 PartPtrs handle_parts(pic_handle *h);
 // the grid-side pointers of one handle (preparation and commit kernels)
 RunDesc handle_desc(pic_handle *h);
